@@ -74,7 +74,8 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
     __shared__ uint32_t s_tmem;
     __shared__ volatile uint32_t s_fail;
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // (warp number, tensor-memory base and go-ahead through a shuffle: uniform to the compiler, as in the product kernel)
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const int S = p.stages;
     const uint32_t ring = sm32(smem);
     const uint32_t tbuf = ring + (uint32_t)(S * p.stage_bytes);          // the tensor between the layers: n_c2 chunks
@@ -113,8 +114,8 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t tmem = s_tmem;
-    const bool run = s_fail == 0u;
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, s_tmem, 0);
+    const bool run = __shfl_sync(0xFFFFFFFFu, s_fail, 0) == 0u;
     const uint32_t full0 = sm32(&s_full[0]), empty0 = sm32(&s_empty[0]);
 
     if (warp == 0) {
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
             const uint32_t tx1 = (uint32_t)(p.a_bytes + p.O1p * 128), tx2 = (uint32_t)(kCtBN2 * 128);
             const int cpt128 = p.cpt1 * 128, Kw = p.K;
             uint32_t slot = 0, epar = 1, issued = 0, dst = ring;      // (a fresh barrier counts as released)
-            bool ok = true;
+            bool ok = true, free_now = true;
             // layer one of a tile: the activation box shifted by the tap and that tap's weights, per 128-byte chunk of channels
             auto load_layer_one = [&](int tile) {
                 int n0, y0, x0;
@@ -132,9 +133,9 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
                 const int xi0 = x0 * p.sw - p.pw;
                 int c128 = 0, kx = xi0, hy = y0 * p.sh - p.ph, tap = 0, kk = 0;
                 for (int ks = 0; ks < p.n_ks1; ++ks) {
-                    bool got = gt_poll(empty0 + slot * 8u, epar);
-                    got = __all_sync(0xFFFFFFFFu, got);
-                    if (!got) { ok = false; return; }
+                    if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; return; }
+                    const bool wrap = slot + 1u == (uint32_t)S;
+                    const uint32_t next_free = gt_test(empty0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? epar ^ 1u : epar);
                     asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xFFFFFFFF;\n"
                                  " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
                                  " @e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6, %7}], [%0];\n"
@@ -142,7 +143,8 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
                                  ::"r"(full0 + slot * 8u), "r"(tx1), "r"(dst), "l"(&p.tmx), "r"(c128), "r"(kx), "r"(hy), "r"(n0),
                                    "r"(dst + (uint32_t)kGtABytes), "l"(&p.tmw1), "r"(tap), "r"(0) : "memory");
                     ++issued;
-                    if (++slot == (uint32_t)S) { slot = 0; epar ^= 1u; dst = ring; } else dst += stage_bytes;
+                    free_now = __all_sync(0xFFFFFFFFu, next_free != 0u);
+                    if (wrap) { slot = 0; epar ^= 1u; dst = ring; } else { ++slot; dst += stage_bytes; }
                     c128 += 128;
                     if (c128 == cpt128) {
                         c128 = 0; ++tap; ++kx;
@@ -154,15 +156,16 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
             auto load_layer_two = [&]() {
                 for (int t2 = 0; t2 < p.n_t2; ++t2)
                     for (int c2 = 0; c2 < p.n_c2; ++c2) {
-                        bool got = gt_poll(empty0 + slot * 8u, epar);
-                        got = __all_sync(0xFFFFFFFFu, got);
-                        if (!got) { ok = false; return; }
+                        if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; return; }
+                        const bool wrap = slot + 1u == (uint32_t)S;
+                        const uint32_t next_free = gt_test(empty0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? epar ^ 1u : epar);
                         asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xFFFFFFFF;\n"
                                      " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
                                      " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6}], [%0];\n}\n"
                                      ::"r"(full0 + slot * 8u), "r"(tx2), "r"(dst), "l"(&p.tmw2), "r"(c2 * 128), "r"(0), "r"(t2 * kCtBN2) : "memory");
                         ++issued;
-                        if (++slot == (uint32_t)S) { slot = 0; epar ^= 1u; dst = ring; } else dst += stage_bytes;
+                        free_now = __all_sync(0xFFFFFFFFu, next_free != 0u);
+                        if (wrap) { slot = 0; epar ^= 1u; dst = ring; } else { ++slot; dst += stage_bytes; }
                     }
             };
             // the stages follow the order in which the MMA warp consumes them: with double buffers, layer one of the next
@@ -193,7 +196,7 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
             const uint32_t idesc2 = (dfmt << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kCtBN2 >> 3) << 17) | ((128u >> 4) << 24);
             const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4;
             uint32_t slot = 0, par = 0, a16 = ring >> 4, tile_i = 0, u2 = 0;
-            bool ok = true;
+            bool ok = true, full_now = false;
             // layer one of the CTA's i-th tile into accumulator one (buffer b, used for the u-th time)
             auto layer_one = [&](uint32_t i) {
                 const uint32_t b = p.db ? (i & 1u) : 0u, u = p.db ? (i >> 1) : i;
@@ -204,13 +207,14 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t d = tmem + b * 128u;
                 for (int ks = 0; ks < p.n_ks1; ++ks) {
-                    bool got = gt_poll(full0 + slot * 8u, par);
-                    got = __all_sync(0xFFFFFFFFu, got);
-                    if (!got) { ok = false; return; }
+                    if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
+                    const bool wrap = slot + 1u == (uint32_t)S;
+                    const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint64_t da = kGtDesc | (uint64_t)(a16 & 0x3FFFu), db = kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu);
-                    gt_issue_stage<false>(kWt, d, da, db, idesc1, empty0 + slot * 8u, ks != 0 ? 1u : 0u);
-                    if (++slot == (uint32_t)S) { slot = 0; par ^= 1u; a16 = ring >> 4; } else a16 += stage16;
+                    gt_issue_stage<kWt, false>(d, da, db, idesc1, empty0 + slot * 8u, ks != 0 ? 1u : 0u);
+                    full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+                    if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
                 }
                 gt_commit_elected<false>(sm32(&s_acc1_full[b]));
             };
@@ -229,14 +233,15 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint32_t d = tmem + 256u + buf * (uint32_t)kCtBN2;
                     for (int c2 = 0; c2 < p.n_c2; ++c2) {
-                        bool got = gt_poll(full0 + slot * 8u, par);
-                        got = __all_sync(0xFFFFFFFFu, got);
-                        if (!got) { ok = false; return; }
+                        if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
+                        const bool wrap = slot + 1u == (uint32_t)S;
+                        const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
                         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                         const uint64_t da = kGtDesc | (uint64_t)(((tbuf + b * tbytes + (uint32_t)(c2 * kCtChunk)) >> 4) & 0x3FFFu);
                         const uint64_t db = kGtDesc | (uint64_t)(a16 & 0x3FFFu);
-                        gt_issue_stage<false>(kWt, d, da, db, idesc2, empty0 + slot * 8u, c2 != 0 ? 1u : 0u);
-                        if (++slot == (uint32_t)S) { slot = 0; par ^= 1u; a16 = ring >> 4; } else a16 += stage16;
+                        gt_issue_stage<kWt, false>(d, da, db, idesc2, empty0 + slot * 8u, c2 != 0 ? 1u : 0u);
+                        full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+                        if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
                     }
                     gt_commit_elected<false>(sm32(&s_acc2_full[buf]));
                 }

@@ -65,7 +65,7 @@ __device__ __forceinline__ uint32_t gt_bias(const GtParams &p, int ch)
     return (p.bias != nullptr && ch < p.O) ? __ldg((const uint32_t *)p.bias + ch) : 0u;
 }
 
-template <bool kPair>
+template <int kWT, bool kPair>
 __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_constant__ GtParams p)
 {
     extern __shared__ __align__(16) uint8_t gt_smem_raw[];
@@ -75,7 +75,10 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     __shared__ uint32_t s_tmem;
     __shared__ volatile uint32_t s_fail;
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // (the warp's number, the tensor-memory base and the go-ahead below come through a shuffle, which makes them uniform to
+    // the compiler: the role branches and the loops under them are then warp-uniform code.  Without it every MMA cost about
+    // 100 cycles of issue and every poll 150, against 48 / 64 / 127 for the MMA itself at 64 / 128 / 256 channels and 90.)
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const int S = p.stages, n_ks = p.n_ks, BN = p.BN;
     const uint32_t ring = sm32(smem);
     const uint32_t staging = ring + (uint32_t)(S * p.stage_bytes);
@@ -124,8 +127,8 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     gt_sync_all<kPair>();                   // (a pair: both CTAs' barriers are initialised before either signals the other)
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t tmem = s_tmem;
-    const bool run = s_fail == 0u;
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, s_tmem, 0);
+    const bool run = __shfl_sync(0xFFFFFFFFu, s_fail, 0) == 0u;
 
     if (warp == 0) {
         // ================= producer =================
@@ -139,7 +142,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             const int cpt128 = p.cpt * 128, Kw = p.K, ntn = p.n_tiles_n;
             // (a fresh barrier counts as released: the wait on parity 1 of the first round returns at once)
             uint32_t slot = 0, epar = 1, issued = 0, dst = ring;
-            bool ok = true;
+            bool ok = true, free_now = true;
             for (int tile = t_first; tile < t_count && ok; tile += t_step) {
                 int mt, tn;
                 gt_divmod(tile, ntn, p.m_ntn, mt, tn);
@@ -152,9 +155,9 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 int c128 = 0, kx = xi0, hy = y0 * p.sh - p.ph, tap = 0, kk = 0;
                 if (s_fail) { ok = false; break; }
                 for (int ks = 0; ks < n_ks; ++ks) {
-                    bool got = gt_poll(empty0 + slot * 8u, epar);
-                    got = __all_sync(0xFFFFFFFFu, got);
-                    if (!got) { ok = false; break; }
+                    if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; break; }
+                    const bool wrap = slot + 1u == (uint32_t)S;
+                    const uint32_t next_free = gt_test(empty0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? epar ^ 1u : epar);
                     if constexpr (kPair) {
                         asm volatile("{\n .reg .pred e, l;\n elect.sync _|e, 0xFFFFFFFF;\n setp.eq.u32 l, %12, 0;\n and.pred l, l, e;\n"
                                      " @l mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
@@ -171,7 +174,8 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                                        "r"(dst + (uint32_t)p.a_stride), "l"(&p.tmw), "r"(tap), "r"(ch0) : "memory");
                     }
                     ++issued;
-                    if (++slot == (uint32_t)S) { slot = 0; epar ^= 1u; dst = ring; } else dst += stage_bytes;
+                    free_now = __all_sync(0xFFFFFFFFu, next_free != 0u);
+                    if (wrap) { slot = 0; epar ^= 1u; dst = ring; } else { ++slot; dst += stage_bytes; }
                     // next K-stage: the next 128-byte chunk of channels, then the next tap (columns first)
                     c128 += 128;
                     if (c128 == cpt128) {
@@ -198,14 +202,14 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
         if (run && rank == 0) {               // (of a pair, the leader issues for both CTAs)
             // instruction descriptor: D fp32 (int32 for int8), A and B bf16 / signed int8 / tf32, K-major both, M = 128
             // (256 over a pair), N = BN
-            const uint32_t dfmt = p.wtype == BSP_I8 ? 2u : 1u, abfmt = p.wtype == BSP_F32 ? 2u : 1u;
+            const uint32_t dfmt = kWT == BSP_I8 ? 2u : 1u, abfmt = kWT == BSP_F32 ? 2u : 1u;
             const uint32_t idesc = (dfmt << 4) | (abfmt << 7) | (abfmt << 10) | ((uint32_t)(BN >> 3) << 17) | (((kPair ? 256u : 128u) >> 4) << 24);
             const uint32_t full0 = sm32(&s_full[0]), empty0 = sm32(&s_empty[0]);
             const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, astride16 = (uint32_t)p.a_stride >> 4;
             const uint64_t desc0 = p.kbytes == 64 ? kGtDesc64 : kGtDesc;
             const uint32_t nk = (uint32_t)p.kbytes >> 5;            // MMAs per stage: 32 bytes of K each
             uint32_t slot = 0, par = 0, a16 = ring >> 4, tile_i = 0;
-            bool ok = true;
+            bool ok = true, full_now = false;
             for (int tile = t_first; tile < t_count && ok; tile += t_step, ++tile_i) {
                 const uint32_t buf = tile_i & 1u, use = tile_i >> 1;
                 if (!gt_poll(sm32(&s_acc_empty[buf]), (use & 1u) ^ 1u) || s_fail != 0u) ok = false;   // (a fresh barrier counts as released)
@@ -214,13 +218,14 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t d = tmem + buf * 256u;
                 for (int ks = 0; ks < n_ks; ++ks) {
-                    bool got = gt_poll(full0 + slot * 8u, par);
-                    got = __all_sync(0xFFFFFFFFu, got);
-                    if (!got) { ok = false; break; }
+                    if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; break; }
+                    const bool wrap = slot + 1u == (uint32_t)S;
+                    const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint64_t da = desc0 | (uint64_t)(a16 & 0x3FFFu), db = desc0 | (uint64_t)((a16 + astride16) & 0x3FFFu);
-                    gt_issue_stage<kPair>(p.wtype, d, da, db, idesc, empty0 + slot * 8u, ks != 0 ? 1u : 0u, nk);
-                    if (++slot == (uint32_t)S) { slot = 0; par ^= 1u; a16 = ring >> 4; } else a16 += stage16;
+                    gt_issue_stage<kWT, kPair>(d, da, db, idesc, empty0 + slot * 8u, ks != 0 ? 1u : 0u, nk);
+                    full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+                    if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
                 }
                 if (ok) gt_commit_elected<kPair>(sm32(&s_acc_full[buf]));
             }
@@ -259,7 +264,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                         uint32_t v[32];
                         gt_load32(tbase + (uint32_t)c0, v);
                         const uint32_t bl = gt_bias(p, n0 + c0 + lane);      // lane e holds the bias of channel c0 + e
-                        if (p.wtype == BSP_I8) {
+                        if (kWT == BSP_I8) {
 #pragma unroll
                             for (int e = 0; e < 32; ++e) out[e] = (uint32_t)((int)v[e] + (int)__shfl_sync(0xFFFFFFFFu, bl, e));
                         } else {
@@ -397,14 +402,21 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     p.kbytes = (long long)wd.I * esz <= 64 ? 64 : 128;
     p.a_stride = kGtBM * p.kbytes;
     p.a_bytes = p.rows_tile * p.kbytes;
+    // kernels by operand type (in the order of bsp_dtype) and by CTA pairs
+    typedef void (*Kernel)(const GtParams);
+    static const Kernel kernels[3][2] = {{gemm_tc_kernel<BSP_F32, false>, gemm_tc_kernel<BSP_F32, true>},
+                                         {gemm_tc_kernel<BSP_BF16, false>, gemm_tc_kernel<BSP_BF16, true>},
+                                         {gemm_tc_kernel<BSP_I8, false>, gemm_tc_kernel<BSP_I8, true>}};
+    static_assert(BSP_F32 == 0 && BSP_BF16 == 1 && BSP_I8 == 2, "the table is indexed by type");
     static bool opted[kGtMaxDevices] = {};
     static int n_sm[kGtMaxDevices] = {};
     int dev = 0;
     BSP_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
     if (!opted[dev]) {
-        BSP_CUDA_OK(cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
-        BSP_CUDA_OK(cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        for (int t = 0; t < 3; ++t)
+            for (int q = 0; q < 2; ++q)
+                BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t][q], cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
         BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
         opted[dev] = true;
     }
@@ -489,11 +501,11 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
-        BSP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<true>, p));
+        BSP_CUDA_OK(cudaLaunchKernelEx(&cfg, kernels[wd.wtype][1], p));
         return BSP_OK;
     }
     const int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
-    gemm_tc_kernel<false><<<grid, kGtThreads, smem, st>>>(p);
+    kernels[wd.wtype][0]<<<grid, kGtThreads, smem, st>>>(p);
     BSP_CUDA_OK(cudaGetLastError());
     return BSP_OK;
 }

@@ -32,6 +32,16 @@ __device__ __forceinline__ bool gt_poll(uint32_t bar, uint32_t parity)
     }
     return false;
 }
+// One look at the barrier, without waiting: non-zero once the phase has completed.  The result of a poll reaches the
+// branch that depends on it after about 90 cycles, so the producer and the MMA warp look at the barrier of the next
+// stage before they issue the current one and fall back to gt_poll only when that look came too early.
+__device__ __forceinline__ uint32_t gt_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.b32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done;
+}
 // The same wait for the threads of the epilogue warps: try_wait suspends the thread for a while.
 __device__ __forceinline__ bool gt_wait(uint32_t bar, uint32_t parity)
 {
@@ -70,17 +80,18 @@ constexpr uint64_t kGtDesc64 = (1ull << 16) | ((uint64_t)(512u >> 4) << 32) | (1
 
 // kPair: the MMAs span a pair of CTAs (cta_group::2, M = 256: each CTA its own 128 positions and half of the weight
 // tile); the commits then arrive on the barrier at the same shared-memory offset in both CTAs.
-template <bool kPair>
-__device__ __forceinline__ void gt_issue_stage(int wtype, uint32_t d, uint64_t da, uint64_t db, uint32_t idesc,
-                                               uint32_t bar_empty, uint32_t acc, uint32_t nk = 4u)
+// The operand type is a template argument: a choice at run time costs a branch around every stage.
+template <int kWT, bool kPair>
+__device__ __forceinline__ void gt_issue_stage(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t bar_empty,
+                                               uint32_t acc, uint32_t nk = 4u)
 {
     if constexpr (kPair) {
-        if (wtype == BSP_BF16) GT_ISSUE_STAGE("f16", "2", ".multicast::cluster.b64 [%4], %6");
-        else if (wtype == BSP_I8) GT_ISSUE_STAGE("i8", "2", ".multicast::cluster.b64 [%4], %6");
+        if constexpr (kWT == BSP_BF16) GT_ISSUE_STAGE("f16", "2", ".multicast::cluster.b64 [%4], %6");
+        else if constexpr (kWT == BSP_I8) GT_ISSUE_STAGE("i8", "2", ".multicast::cluster.b64 [%4], %6");
         else GT_ISSUE_STAGE("tf32", "2", ".multicast::cluster.b64 [%4], %6");
     } else {
-        if (wtype == BSP_BF16) GT_ISSUE_STAGE("f16", "1", ".b64 [%4]");
-        else if (wtype == BSP_I8) GT_ISSUE_STAGE("i8", "1", ".b64 [%4]");
+        if constexpr (kWT == BSP_BF16) GT_ISSUE_STAGE("f16", "1", ".b64 [%4]");
+        else if constexpr (kWT == BSP_I8) GT_ISSUE_STAGE("i8", "1", ".b64 [%4]");
         else GT_ISSUE_STAGE("tf32", "1", ".b64 [%4]");
     }
 }
