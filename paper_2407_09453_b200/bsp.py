@@ -46,6 +46,15 @@ class Bcsr(C.Structure):
                 ("packed", C.c_void_p), ("nnz", C.c_int64)]
 
 
+# Argument types of the calls that return a status, one letter per argument: p pointer, i int, l int64.  Declared types let
+# the calls below pass plain Python integers and None, which costs a fraction of building a ctypes object per argument
+# (a product call of a few microseconds on the GPU was bound by that).
+_ARG = {"p": C.c_void_p, "i": C.c_int, "l": C.c_int64}
+_ARGS = {"bsp_mask": "ppiilpppp", "bsp_mask_static": "ppiilpp", "bsp_compact_nnz": "ppppp", "bsp_compact": "pppppppl" "pp",
+         "bsp_gemm": "ppplppipp", "bsp_conv2d": "ppppppipp", "bsp_gemm_q8": "ppplppppp", "bsp_conv2d_q8": "ppppppppp",
+         "bsp_conv2d_chain": "ppppppp" "ippipp", "bsp_conv2d_chain_q8": "pppppppp" "ippppp", "bsp_spgemm": "ppppppp",
+         "bsp_index_to_relative": "ipppp", "bsp_index_from_relative": "ipppp", "bsp_check": "pp"}
+
 _lib = None
 
 
@@ -62,9 +71,9 @@ def lib():
             getattr(L, n).restype = C.c_size_t
         L.bsp_status_string.restype = C.c_char_p
         L.bsp_conv_kernel_name.restype = C.c_char_p
-        for n in ("bsp_mask", "bsp_mask_static", "bsp_compact_nnz", "bsp_compact", "bsp_gemm", "bsp_conv2d",
-                  "bsp_gemm_q8", "bsp_conv2d_q8", "bsp_conv2d_chain", "bsp_conv2d_chain_q8", "bsp_spgemm", "bsp_index_to_relative", "bsp_index_from_relative", "bsp_check"):
+        for n, a in _ARGS.items():
             getattr(L, n).restype = C.c_int
+            getattr(L, n).argtypes = [_ARG[c] for c in a]
         _lib = L
     return _lib
 
@@ -81,12 +90,21 @@ def dtype_code(t: torch.dtype) -> int:
 
 
 def _ptr(t):
-    return C.c_void_p(0 if t is None else t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# Address of the current stream of the current device: what torch.cuda.current_stream().cuda_stream gives, without the
+# Stream object around it (3.4 us a call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _raw_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_raw_device())
 
 
 def _raise(rc, what):
@@ -108,7 +126,7 @@ def bsp_mask_workspace_bytes(wd: WDesc) -> int:
 
 
 def bsp_mask(wd: WDesc, W, norm, scope, n_zero, gamma, scores_opt, ws, stream=None):
-    _raise(lib().bsp_mask(C.byref(wd), _ptr(W), C.c_int(norm), C.c_int(scope), C.c_int64(n_zero), _ptr(gamma),
+    _raise(lib().bsp_mask(C.byref(wd), _ptr(W), norm, scope, n_zero, _ptr(gamma),
                           _ptr(scores_opt), _ptr(ws), _stream(stream)), "bsp_mask")
 
 
@@ -129,11 +147,11 @@ def bsp_compact_nnz(wd: WDesc, gamma, ws, stream=None) -> int:
 
 def bsp_compact(wd: WDesc, W, gamma, row_ptr, col_idx, payload, packed, capacity_blocks, ws, stream=None):
     _raise(lib().bsp_compact(C.byref(wd), _ptr(W), _ptr(gamma), _ptr(row_ptr), _ptr(col_idx), _ptr(payload),
-                             _ptr(packed), C.c_int64(capacity_blocks), _ptr(ws), _stream(stream)), "bsp_compact")
+                             _ptr(packed), capacity_blocks, _ptr(ws), _stream(stream)), "bsp_compact")
 
 
 def bcsr(row_ptr, col_idx, payload, packed, nnz) -> Bcsr:
-    return Bcsr(_ptr(row_ptr).value, _ptr(col_idx).value, _ptr(payload).value, _ptr(packed).value, int(nnz))
+    return Bcsr(_ptr(row_ptr), _ptr(col_idx), _ptr(payload), _ptr(packed), int(nnz))
 
 
 def bsp_conv_workspace_bytes(wd: WDesc, xd: XDesc) -> int:
@@ -141,12 +159,12 @@ def bsp_conv_workspace_bytes(wd: WDesc, xd: XDesc) -> int:
 
 
 def bsp_gemm(wd: WDesc, w: Bcsr, X, P, bias, Y, ytype, ws, stream=None):
-    _raise(lib().bsp_gemm(C.byref(wd), C.byref(w), _ptr(X), C.c_int64(P), _ptr(bias), _ptr(Y), C.c_int(ytype),
+    _raise(lib().bsp_gemm(C.byref(wd), C.byref(w), _ptr(X), P, _ptr(bias), _ptr(Y), ytype,
                           _ptr(ws), _stream(stream)), "bsp_gemm")
 
 
 def bsp_conv2d(wd: WDesc, w: Bcsr, xd: XDesc, X, bias, Y, ytype, ws, stream=None):
-    _raise(lib().bsp_conv2d(C.byref(wd), C.byref(w), C.byref(xd), _ptr(X), _ptr(bias), _ptr(Y), C.c_int(ytype),
+    _raise(lib().bsp_conv2d(C.byref(wd), C.byref(w), C.byref(xd), _ptr(X), _ptr(bias), _ptr(Y), ytype,
                             _ptr(ws), _stream(stream)), "bsp_conv2d")
 
 
@@ -156,19 +174,19 @@ def bsp_conv2d_q8(wd: WDesc, w: Bcsr, xd: XDesc, X, bias, shift, Y, ws, stream=N
 
 
 def bsp_gemm_q8(wd: WDesc, w: Bcsr, X, P, bias, shift, Y, ws, stream=None):
-    _raise(lib().bsp_gemm_q8(C.byref(wd), C.byref(w), _ptr(X), C.c_int64(P), _ptr(bias), _ptr(shift), _ptr(Y), _ptr(ws),
+    _raise(lib().bsp_gemm_q8(C.byref(wd), C.byref(w), _ptr(X), P, _ptr(bias), _ptr(shift), _ptr(Y), _ptr(ws),
                              _stream(stream)), "bsp_gemm_q8")
 
 
 def bsp_conv2d_chain(wd1: WDesc, w1: Bcsr, wd2: WDesc, w2: Bcsr, xd: XDesc, X, bias1, relu, bias2, Y, ytype, ws, stream=None):
     _raise(lib().bsp_conv2d_chain(C.byref(wd1), C.byref(w1), C.byref(wd2), C.byref(w2), C.byref(xd), _ptr(X), _ptr(bias1),
-                                  C.c_int(1 if relu else 0), _ptr(bias2), _ptr(Y), C.c_int(ytype), _ptr(ws), _stream(stream)),
+                                  1 if relu else 0, _ptr(bias2), _ptr(Y), ytype, _ptr(ws), _stream(stream)),
            "bsp_conv2d_chain")
 
 
 def bsp_conv2d_chain_q8(wd1: WDesc, w1: Bcsr, wd2: WDesc, w2: Bcsr, xd: XDesc, X, bias1, shift1, relu, bias2, shift2, Y, ws, stream=None):
     _raise(lib().bsp_conv2d_chain_q8(C.byref(wd1), C.byref(w1), C.byref(wd2), C.byref(w2), C.byref(xd), _ptr(X), _ptr(bias1),
-                                     _ptr(shift1), C.c_int(1 if relu else 0), _ptr(bias2), _ptr(shift2), _ptr(Y), _ptr(ws),
+                                     _ptr(shift1), 1 if relu else 0, _ptr(bias2), _ptr(shift2), _ptr(Y), _ptr(ws),
                                      _stream(stream)), "bsp_conv2d_chain_q8")
 
 
@@ -177,16 +195,16 @@ def bsp_spgemm(wa: WDesc, a: Bcsr, wb: WDesc, b: Bcsr, Cm, ws, stream=None):
 
 
 def bsp_index_to_relative(NBo, row_ptr, col_idx, rel, stream=None):
-    _raise(lib().bsp_index_to_relative(C.c_int(NBo), _ptr(row_ptr), _ptr(col_idx), _ptr(rel), _stream(stream)), "bsp_index_to_relative")
+    _raise(lib().bsp_index_to_relative(NBo, _ptr(row_ptr), _ptr(col_idx), _ptr(rel), _stream(stream)), "bsp_index_to_relative")
 
 
 def bsp_index_from_relative(NBo, row_ptr, rel, col_idx, stream=None):
-    _raise(lib().bsp_index_from_relative(C.c_int(NBo), _ptr(row_ptr), _ptr(rel), _ptr(col_idx), _stream(stream)),
+    _raise(lib().bsp_index_from_relative(NBo, _ptr(row_ptr), _ptr(rel), _ptr(col_idx), _stream(stream)),
            "bsp_index_from_relative")
 
 
 def bsp_mask_static(wd: WDesc, W, norm, scope, n_zero, gamma, stream=None):
-    _raise(lib().bsp_mask_static(C.byref(wd), _ptr(W), C.c_int(norm), C.c_int(scope), C.c_int64(n_zero), _ptr(gamma),
+    _raise(lib().bsp_mask_static(C.byref(wd), _ptr(W), norm, scope, n_zero, _ptr(gamma),
                                  _stream(stream)), "bsp_mask_static")
 
 

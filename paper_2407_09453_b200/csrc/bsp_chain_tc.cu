@@ -459,7 +459,7 @@ bool chain_tc_eligible(const bsp_wdesc &wd1, const bsp_wdesc &wd2, const bsp_xde
     const int M = (xd.L + 2 * xd.pad_h - wd1.H) / xd.stride_h + 1, Nw = (xd.J + 2 * xd.pad_w - wd1.K) / xd.stride_w + 1;
     if (M <= 0 || Nw <= 0) return false;
     if ((long long)xd.N * M * Nw > 0x7FFFFFFF - 4096 || (long long)xd.N * xd.L * xd.J > 0x7FFFFFFF) return false;
-    return gt_pick_tile(xd.N, M, Nw, xd.stride_h, xd.stride_w).tiles > 0;
+    return xd.stride_h <= 256 && xd.stride_w <= 256;       // (a box of one position then fits: gt_pick_tile)
 }
 
 bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_wdesc &wd2, const void *packed2,

@@ -371,7 +371,7 @@ bool gemm_tc_eligible(const bsp_wdesc &wd, const bsp_xdesc &xd0, bsp_dtype ytype
     if (M <= 0 || Nw <= 0) return false;
     if ((long long)xd.N * M * Nw > 0x7FFFFFFF || (long long)xd.N * xd.L * xd.J > 0x7FFFFFFF) return false;
     if ((long long)xd.N * M * Nw * wd.O * ey >= (1LL << 46)) return false;
-    return gt_pick_tile(xd.N, M, Nw, xd.stride_h, xd.stride_w).tiles > 0;
+    return xd.stride_h <= 256 && xd.stride_w <= 256;       // (a box of one position then fits: gt_pick_tile)
 }
 
 bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void *packed, const void *X,
