@@ -81,7 +81,7 @@ typedef struct {
  *   payload [nnz][b_o][H][K][b_i]  the surviving weights in canonical order
  *   packed            the same weights in the kernels' own tile order, written by bsp_compact and
  *                     opaque to the caller (bsp_packed_bytes() gives its size)
- *   nnz               number of stored blocks (host copy; used for size checks only)
+ *   nnz               number of stored blocks (host copy; used for size checks and, by bsp_spgemm, to choose a kernel)
  * The product kernels read `packed`; row_ptr/col_idx/payload are the portable form. */
 typedef struct {
     const int32_t *row_ptr;
@@ -227,7 +227,9 @@ bsp_status bsp_conv2d_chain_q8(const bsp_wdesc *wd1, const bsp_bcsr *w1, const b
  *             8x8 blocks and the same type (F32 or BF16); `a` and `b` are their compact forms from bsp_compact (row_ptr,
  *             col_idx and the canonical payload are read; `packed` is not).  C is dense float32 [wa->O][wb->O], 8-byte
  *             aligned (the two payloads 16-byte aligned), written in full (blocks without a common column are zero).  Products are accumulated in float32
- *             in ascending order of k.  A column index outside the matrix is skipped and latches BSP_ERR_INDEX.
+ *             in ascending order of k (bfloat16 operands with enough common columns run as a dense product over masked
+ *             blocks: sums of 16 products inside the tensor core, and of up to eight column ranges).  A column index outside
+ *             the matrix is skipped and latches BSP_ERR_INDEX.
  *             ws: any workspace of at least 256 bytes (status word only).
  * bsp_index_to_relative / bsp_index_from_relative: within each row of Gamma the first kept block keeps its column, every
  *             further one stores its distance (>= 1) to the previous kept block of the row; and back.  int32 in, int32

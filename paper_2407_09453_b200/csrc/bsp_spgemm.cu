@@ -8,8 +8,9 @@
 // turn: 32 entries of B's column list are looked up at once, a ballot gives the common columns in ascending order, and
 // for each of them the warp adds the 8 x 8 x 8 product, lane (r, c) holding C[r][2c], C[r][2c + 1] in fp32 (fp32 blocks:
 // fused multiply-adds; bfloat16 blocks: one m16n8k16 tensor-core instruction per two common columns).  Work and
-// traffic follow the kept blocks only: nothing is read or multiplied where either mask has a zero.
-#include "bsp_internal.cuh"
+// traffic follow the kept blocks only: nothing is read or multiplied where either mask has a zero.  bfloat16 operands whose
+// masks leave enough common columns take the dense form on tcgen05 below.
+#include "bsp_tc.cuh"
 
 namespace bsp {
 namespace {
@@ -23,14 +24,57 @@ __device__ __forceinline__ void sp_row(const float *p, float (&v)[8])
     const float4 a = __ldg((const float4 *)p), b = __ldg((const float4 *)p + 1);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
-__device__ __forceinline__ void sp_row(const __nv_bfloat16 *p, float (&v)[8])
+// The 8 x 8 block of C of one row of A and one row of B: acc0, acc1 are this lane's entries (r, 2c), (r, 2c + 1) with
+// r = lane / 4, c = lane % 4.  `pos_of` gives the payload position of the A row's block in column k, or -1.
+template <typename T, typename F>
+__device__ __forceinline__ void sp_pair(const T *__restrict__ a_payload, const int32_t *__restrict__ b_col_idx, const T *__restrict__ b_payload,
+                                        int lo, int hi, int NBk, int lane, F pos_of, float &acc0, float &acc1, int *status)
 {
-    const uint4 q = __ldg((const uint4 *)p);
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    const int r = lane >> 2, c = (lane & 3) * 2;
+    for (int base = lo; base < hi; base += 32) {
+        const int nb = base + lane;
+        int pa = -1;
+        if (nb < hi) {
+            const int k = b_col_idx[nb];
+            if (k >= 0 && k < NBk) pa = pos_of(k);
+            else atomicMax(status, (int)BSP_ERR_INDEX);
+        }
+        unsigned both = __ballot_sync(0xFFFFFFFFu, pa >= 0);
+        if constexpr (sizeof(T) == 2) {
+            // bfloat16 blocks: two common columns per tensor-core instruction (m16n8k16: the 8 x 8 block of C sits in
+            // rows 0-7 of the 16 x 8 result, K = the eight channels of the first column followed by those of the
+            // second).  Lane (r, c) holds exactly the words it needs: entries (r, 2c), (r, 2c + 1) of each block of A
+            // and of B, so a warp reads each 128-byte block once, four bytes per lane.
+            while (both) {
+                const int s1 = __ffs(both) - 1;
+                both &= both - 1;
+                const int s2 = both ? __ffs(both) - 1 : -1;
+                both &= both - 1;                         // (0 & -1 stays 0)
+                const int na1 = __shfl_sync(0xFFFFFFFFu, pa, s1);
+                const int na2 = __shfl_sync(0xFFFFFFFFu, pa, s2 < 0 ? s1 : s2);
+                const uint32_t *Aw = (const uint32_t *)a_payload, *Bw = (const uint32_t *)b_payload;
+                const uint32_t a0 = __ldg(Aw + (size_t)na1 * 32 + lane), b0 = __ldg(Bw + (size_t)(base + s1) * 32 + lane);
+                uint32_t a2 = 0u, b1 = 0u;
+                if (s2 >= 0) { a2 = __ldg(Aw + (size_t)na2 * 32 + lane); b1 = __ldg(Bw + (size_t)(base + s2) * 32 + lane); }
+                float d2 = 0.f, d3 = 0.f;
+                asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};\n"
+                             : "+f"(acc0), "+f"(acc1), "+f"(d2), "+f"(d3) : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
+            }
+        } else
+        while (both) {                                    // common columns, ascending
+            const int src = __ffs(both) - 1;
+            both &= both - 1;
+            const int na = __shfl_sync(0xFFFFFFFFu, pa, src);
+            const T *Ab = a_payload + ((size_t)na * kSpEdge + r) * kSpEdge;
+            const T *Bb = b_payload + ((size_t)(base + src) * kSpEdge + c) * kSpEdge;
+            float av[8], b0[8], b1[8];
+            sp_row(Ab, av); sp_row(Bb, b0); sp_row(Bb + kSpEdge, b1);
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        v[2 * t] = __uint_as_float(w[t] << 16);
-        v[2 * t + 1] = __uint_as_float(w[t] & 0xFFFF0000u);
+            for (int t = 0; t < kSpEdge; ++t) {
+                acc0 = fmaf(av[t], b0[t], acc0);
+                acc1 = fmaf(av[t], b1[t], acc1);
+            }
+        }
     }
 }
 
@@ -54,54 +98,349 @@ spgemm_kernel(const int32_t *__restrict__ a_row_ptr, const int32_t *__restrict__
     const size_t ldc = (size_t)NBb * kSpEdge;
     for (int j = blockIdx.y * (kSpThreads / 32) + warp; j < NBb; j += gridDim.y * (kSpThreads / 32)) {
         float acc0 = 0.f, acc1 = 0.f;
-        const int lo = b_row_ptr[j], hi = b_row_ptr[j + 1];
-        for (int base = lo; base < hi; base += 32) {
-            const int nb = base + lane;
-            int pa = -1;
-            if (nb < hi) {
-                const int k = b_col_idx[nb];
-                if (k >= 0 && k < NBk) pa = s_pos[k];
-                else atomicMax(status, (int)BSP_ERR_INDEX);
-            }
-            unsigned both = __ballot_sync(0xFFFFFFFFu, pa >= 0);
-            if constexpr (sizeof(T) == 2) {
-                // bfloat16 blocks: two common columns per tensor-core instruction (m16n8k16: the 8 x 8 block of C sits in
-                // rows 0-7 of the 16 x 8 result, K = the eight channels of the first column followed by those of the
-                // second).  Lane (r, c) holds exactly the words it needs: entries (r, 2c), (r, 2c + 1) of each block of A
-                // and of B, so a warp reads each 128-byte block once, four bytes per lane.
-                while (both) {
-                    const int s1 = __ffs(both) - 1;
-                    both &= both - 1;
-                    const int s2 = both ? __ffs(both) - 1 : -1;
-                    both &= both - 1;                         // (0 & -1 stays 0)
-                    const int na1 = __shfl_sync(0xFFFFFFFFu, pa, s1);
-                    const int na2 = __shfl_sync(0xFFFFFFFFu, pa, s2 < 0 ? s1 : s2);
-                    const uint32_t *Aw = (const uint32_t *)a_payload, *Bw = (const uint32_t *)b_payload;
-                    const uint32_t a0 = __ldg(Aw + (size_t)na1 * 32 + lane), b0 = __ldg(Bw + (size_t)(base + s1) * 32 + lane);
-                    uint32_t a2 = 0u, b1 = 0u;
-                    if (s2 >= 0) { a2 = __ldg(Aw + (size_t)na2 * 32 + lane); b1 = __ldg(Bw + (size_t)(base + s2) * 32 + lane); }
-                    float d2 = 0.f, d3 = 0.f;
-                    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};\n"
-                                 : "+f"(acc0), "+f"(acc1), "+f"(d2), "+f"(d3) : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
-                }
-            } else
-            while (both) {                                    // common columns, ascending
-                const int src = __ffs(both) - 1;
-                both &= both - 1;
-                const int na = __shfl_sync(0xFFFFFFFFu, pa, src);
-                const T *Ab = a_payload + ((size_t)na * kSpEdge + r) * kSpEdge;
-                const T *Bb = b_payload + ((size_t)(base + src) * kSpEdge + c) * kSpEdge;
-                float av[8], b0[8], b1[8];
-                sp_row(Ab, av); sp_row(Bb, b0); sp_row(Bb + kSpEdge, b1);
-#pragma unroll
-                for (int t = 0; t < kSpEdge; ++t) {
-                    acc0 = fmaf(av[t], b0[t], acc0);
-                    acc1 = fmaf(av[t], b1[t], acc1);
-                }
-            }
-        }
+        sp_pair<T>(a_payload, b_col_idx, b_payload, b_row_ptr[j], b_row_ptr[j + 1], NBk, lane, [&](int k) { return s_pos[k]; }, acc0, acc1, status);
         *(float2 *)(C + ((size_t)i * kSpEdge + r) * ldc + (size_t)j * kSpEdge + c) = make_float2(acc0, acc1);
     }
+}
+
+// ---- bfloat16 operands on 5th-generation tensor cores -----------------------------------------------------------------
+// A CTA owns 128 rows of A (16 block rows) x BN rows of B (BN = 64, 128 or 256), or with split reductions a share of the
+// columns of such a tile.  The payload positions of its block rows are spread into a table over the block columns in
+// shared memory; then 16 producer warps walk the columns in chunks of eight blocks (64 values, the span of the 128-byte
+// swizzle), in groups that take turns: the 8 rows of a kept block are 16 bytes each, one per lane, loaded ahead and written
+// straight into the swizzled operand layout, dropped blocks as zeros; one warp issues the four MMAs of a chunk into one
+// accumulator of BN columns.  Zeroed blocks are multiplied, but nothing is read for them.
+// A dropped block must not turn a non-finite weight into NaN (0 * inf): a piece of C whose sums are not all finite is
+// computed again by the sparse form.
+constexpr int kStProducers = 16;
+constexpr int kStThreads = (kStProducers + 1) * 32;
+constexpr int kStMaxStages = 8;
+constexpr int kStARows = kGtBM / kSpEdge;         // block rows of A per tile
+
+// Groups of producer warps by tile width: a group's chain of wait, store, fence, arrive and load is longer than the MMAs of
+// a chunk, so groups overlap theirs.  2048 x 2048 x 4096 at 50 %, us: one group 52 / 82 / 130 (256 / 128 / 64 columns), two
+// 50 / 72 / 113, four 105 with 64; 16-byte cp.async straight to shared memory instead of registers: 72 / 93 / 143.
+__host__ __device__ constexpr int st_groups(int BN) { return BN == 64 ? 4 : 2; }
+
+struct StParams {
+    const int32_t *a_row_ptr, *a_col_idx, *b_row_ptr, *b_col_idx;
+    const uint8_t *a_payload, *b_payload;
+    float *C;
+    int *status;
+    int NBa, NBb, NBk, n_chunks, stages, split;
+};
+
+template <int BN>
+__global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_constant__ StParams p)
+{
+    constexpr int kGroups = st_groups(BN), kDepth = BN == 128 ? 2 : 1;    // (chunks loaded ahead per group: what 120 registers hold)
+    constexpr int kRows = kStARows + BN / kSpEdge;            // block rows of the tile: 16 of A, then those of B
+    constexpr int kW = kStProducers / kGroups;                // warps of a group: they share a chunk
+    constexpr int kUnits = kRows * 2 / kW;                    // half block rows (four blocks of a chunk) per warp
+    constexpr uint32_t kStage = kRows * 1024u;                // a block row of a chunk: 8 rows of 128 bytes
+    extern __shared__ __align__(16) uint8_t st_smem_raw[];
+    uint8_t *smem = st_smem_raw + ((1024u - (sm32(st_smem_raw) & 1023u)) & 1023u);
+    __shared__ __align__(8) uint64_t s_full[kStMaxStages], s_empty[kStMaxStages], s_acc;
+    __shared__ uint32_t s_tmem;
+    __shared__ volatile uint32_t s_fail;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    const int S = p.stages, pitch = p.n_chunks * 8;
+    const uint32_t ring = sm32(smem);
+    int16_t *s_pos = (int16_t *)(smem + (size_t)S * kStage);  // [kRows][pitch]: position within its row's stored blocks, or -1
+    const int i0 = (int)blockIdx.y * kStARows, j0 = (int)blockIdx.x * (BN / kSpEdge);
+    // this CTA's chunks: all of them, or its share of a split reduction (the CTAs of a tile are a cluster along z)
+    const int share = (p.n_chunks + p.split - 1) / p.split;
+    const int c_lo = (int)blockIdx.z * share, c_hi = min(p.n_chunks, c_lo + share);
+
+    if (tid == 0) {
+        s_fail = 0u;
+        for (int s = 0; s < S; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_full[s])), "r"(kW) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_empty[s])), "r"(1) : "memory");
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc)), "r"(1) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == kStProducers) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(BN) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    // a block row's first and last stored block (rows past the last one are empty)
+    auto row_of = [&](int b, int &lo, int &hi) {
+        const bool is_a = b < kStARows;
+        const int g = is_a ? i0 + b : j0 + b - kStARows;
+        const int32_t *rp = is_a ? p.a_row_ptr : p.b_row_ptr;
+        const bool in = g < (is_a ? p.NBa : p.NBb);
+        lo = in ? rp[g] : 0;
+        hi = in ? rp[g + 1] : 0;
+    };
+    for (int k = tid; k < kRows * pitch / 8; k += kStThreads) ((uint4 *)s_pos)[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    __syncthreads();
+    for (int b = warp; b < kRows; b += kStProducers + 1) {
+        int lo, hi;
+        row_of(b, lo, hi);
+        const int32_t *ci = b < kStARows ? p.a_col_idx : p.b_col_idx;
+        for (int n = lo + lane; n < hi; n += 128) {
+            int k[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) k[u] = n + 32 * u < hi ? __ldg(ci + n + 32 * u) : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (n + 32 * u >= hi) continue;
+                if (k[u] >= 0 && k[u] < p.NBk) s_pos[b * pitch + k[u]] = (int16_t)(n + 32 * u - lo);
+                else atomicMax(p.status, (int)BSP_ERR_INDEX);          // a column outside the matrix: skipped
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, s_tmem, 0);
+    const uint32_t full0 = sm32(&s_full[0]), empty0 = sm32(&s_empty[0]);
+
+    if (warp < kStProducers) {
+        // ================= producers =================
+        // Group g takes every kGroups-th chunk.  Unit u of a warp: a half (four blocks) of block row b0 + (kW / 2) u;
+        // lane = row q of block j of the chunk.
+        const int grp = warp / kW, wg = warp % kW;
+        const int q = lane & 7, j = (wg & 1) * 4 + (lane >> 3), b0 = wg >> 1;
+        const uint8_t *src[kUnits];
+        const int16_t *pos = s_pos + b0 * pitch + j;
+#pragma unroll
+        for (int u = 0; u < kUnits; ++u) {
+            int lo, hi;
+            row_of(b0 + (kW / 2) * u, lo, hi);
+            src[u] = (u < 2 * kStARows / kW ? p.a_payload : p.b_payload) + (size_t)lo * 128 + q * 16;
+        }
+        const uint32_t off = (uint32_t)(b0 * 1024 + q * 128 + ((j ^ q) << 4));
+        uint4 v[kDepth][kUnits];
+        auto load = [&](int c, uint4 (&w)[kUnits]) {
+            if (c >= c_hi) return;
+#pragma unroll
+            for (int u = 0; u < kUnits; ++u) {
+                const int n = pos[(kW / 2) * u * pitch + c * 8];
+                w[u] = make_uint4(0u, 0u, 0u, 0u);
+                if (n >= 0) w[u] = __ldg((const uint4 *)(src[u] + (size_t)n * 128));
+            }
+        };
+        uint32_t slot = (uint32_t)grp, epar = 1;               // (a fresh barrier counts as released)
+        bool ok = true;
+        auto put = [&](const uint4 (&w)[kUnits]) {
+            if (!gt_wait(empty0 + slot * 8u, epar)) ok = false;
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (!ok) return;
+            const uint32_t dst = ring + slot * kStage + off;
+#pragma unroll
+            for (int u = 0; u < kUnits; ++u)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + u * (uint32_t)(kW * 512)), "r"(w[u].x), "r"(w[u].y), "r"(w[u].z), "r"(w[u].w) : "memory");
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(full0 + slot * 8u) : "memory");
+            slot += kGroups;
+            if (slot >= (uint32_t)S) { slot -= (uint32_t)S; epar ^= 1u; }
+        };
+#pragma unroll
+        for (int d = 0; d < kDepth; ++d) load(c_lo + grp + d * kGroups, v[d]);
+        for (int c = c_lo + grp; c < c_hi && ok; c += kDepth * kGroups)
+#pragma unroll
+            for (int d = 0; d < kDepth; ++d)
+                if (c + d * kGroups < c_hi && ok) {
+                    put(v[d]);
+                    load(c + (d + kDepth) * kGroups, v[d]);
+                }
+        if (!gt_wait(sm32(&s_acc), 0u)) ok = false;
+        if (!__all_sync(0xFFFFFFFFu, ok) && lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
+    } else {
+        // ================= MMA issuer =================
+        constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((128u >> 4) << 24);
+        uint32_t slot = 0, par = 0, a16 = ring >> 4;
+        bool ok = true, full_now = false;
+        for (int c = c_lo; c < c_hi; ++c) {
+            if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; break; }
+            const bool wrap = slot + 1u == (uint32_t)S;
+            const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            gt_issue_stage<BSP_BF16, false>(tmem, kGtDesc | (uint64_t)(a16 & 0x3FFFu), kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu),
+                                            idesc, empty0 + slot * 8u, c != c_lo ? 1u : 0u);
+            full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+            if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += kStage >> 4; }
+        }
+        if (ok) gt_commit_elected<false>(sm32(&s_acc));
+        else if (lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
+    }
+    __syncthreads();
+    const bool ok = (s_fail & 1u) == 0u;
+
+    // ================= epilogue =================
+    // The tile is cut into pieces of 32 x 32 sums (piece = 32-column part * 4 + quarter of the tensor-memory lanes), which go
+    // through 4 KB of the idle ring each, so that rows of C are written 128 bytes at a time.
+    constexpr int kPieces = BN / 8;
+    const bool wide = ((uintptr_t)p.C & 15u) == 0;         // (rows of C are multiples of 32 bytes)
+    const size_t ldc = (size_t)p.NBb * kSpEdge;
+    auto to_smem = [&](int piece) {
+        uint32_t w[32];
+        gt_load32(tmem + ((uint32_t)((piece & 3) * 32) << 16) + (uint32_t)(piece >> 2) * 32u, w);
+        const uint32_t buf = ring + (uint32_t)piece * 4096u + lane * 128u;
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(buf + (uint32_t)((e ^ (lane & 7)) << 4)), "r"(w[4 * e]), "r"(w[4 * e + 1]), "r"(w[4 * e + 2]), "r"(w[4 * e + 3]) : "memory");
+    };
+    // sums the shares of a piece in the order of the CTAs (`peers` of them) and writes it
+    auto to_global = [&](int piece, int peers) {
+        const int row0 = i0 * kSpEdge + (piece & 3) * 32, col = j0 * kSpEdge + (piece >> 2) * 32 + (lane & 7) * 4;
+        const uint32_t buf = ring + (uint32_t)piece * 4096u;
+        bool odd = false;                                      // a sum that is not finite
+#pragma unroll
+        for (int it = 0; it < 8; ++it) {
+            const int r = it * 4 + (lane >> 3);
+            const uint32_t at = buf + r * 128u + (uint32_t)(((lane & 7) ^ (r & 7)) << 4);
+            float4 x;
+            if (peers == 1) {
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(at) : "memory");
+            } else {
+                x = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int k = 0; k < peers; ++k) {
+                    uint32_t far;
+                    float4 y;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(far) : "r"(at), "r"(k));
+                    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w) : "r"(far) : "memory");
+                    x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+                }
+            }
+            odd |= !(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(x.w));
+            if (row0 + r < p.NBa * kSpEdge && col < p.NBb * kSpEdge) {
+                float *dst = p.C + (size_t)(row0 + r) * ldc + col;
+                if (wide) *(float4 *)dst = x;
+                else { *(float2 *)dst = make_float2(x.x, x.y); *(float2 *)(dst + 2) = make_float2(x.z, x.w); }
+            }
+        }
+        if (!__any_sync(0xFFFFFFFFu, odd)) return;
+        for (int t = 0; t < 16; ++t) {
+            const int bi = (piece & 3) * 4 + (t & 3), i = i0 + bi, jj = j0 + (piece >> 2) * 4 + (t >> 2);
+            if (i >= p.NBa || jj >= p.NBb) continue;
+            float acc0 = 0.f, acc1 = 0.f;
+            const int first = p.a_row_ptr[i];
+            const int16_t *row = s_pos + bi * pitch;
+            sp_pair<__nv_bfloat16>((const __nv_bfloat16 *)p.a_payload, p.b_col_idx, (const __nv_bfloat16 *)p.b_payload, p.b_row_ptr[jj], p.b_row_ptr[jj + 1],
+                                   p.NBk, lane, [&](int k) { const int n = row[k]; return n < 0 ? -1 : first + n; }, acc0, acc1, p.status);
+            *(float2 *)(p.C + ((size_t)i * kSpEdge + (lane >> 2)) * ldc + (size_t)jj * kSpEdge + (lane & 3) * 2) = make_float2(acc0, acc1);
+        }
+    };
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (p.split == 1) {
+        if (ok && warp < kStProducers)
+            for (int piece = warp; piece < kPieces; piece += kStProducers) { to_smem(piece); __syncwarp(); to_global(piece, 1); }
+    } else {
+        if (ok && warp < kStProducers)
+            for (int piece = warp; piece < kPieces; piece += kStProducers) to_smem(piece);
+        gt_sync_all<true>();
+        if (ok && warp < kStProducers)
+            for (int piece = (int)blockIdx.z + p.split * warp; piece < kPieces; piece += p.split * kStProducers) to_global(piece, p.split);
+        gt_sync_all<true>();                                   // (no CTA leaves while another still reads its sums)
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (!ok && tid == 0) atomicMax(p.status, (int)BSP_ERR_TIMEOUT);
+    if (warp == kStProducers) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(BN) : "memory");
+}
+
+// Stages that fit beside the position table of a tile (zero: too many block columns).
+int spgemm_tc_stages(int BN, int n_chunks)
+{
+    const long long rows = kStARows + BN / kSpEdge;
+    const long long room = (long long)kGtMaxSmem - 1024 - rows * n_chunks * 16;
+    const long long n = room / (rows * 1024);
+    return n < 0 ? 0 : (n > kStMaxStages ? kStMaxStages : (int)n);
+}
+
+// Tile width and split of the tensor-core form, or BN = 0 where the sparse form is expected to be faster.  Estimates in
+// microseconds, fitted on a B200.  Tensor-core form: a tile costs a start, a share per chunk for the table and the fill of
+// the operands (0.31 / 0.44 / 0.60 a chunk at 64 / 128 / 256 columns, bound by shared memory: stores of the fill, reads
+// of the MMAs), whatever the masks hold.  Sparse form: 28.7 per million pairs of blocks with a common column plus 3.6 per
+// million look-ups, or the chain of one warp where there are few rows.  Measured, sparse / tensor core: 2048 x 2048 x 4096
+// at 50 % 304 / 50, at 75 % 90 / 47, at 90 % 25 / 44; 512 x 512 x 4096 at 50 % 27 / 15, at 75 % 11 / 14.
+// The densities come from the host counts; a wrong count costs time only.
+struct StPlan { int BN, split; };
+// slots[k] = CTAs of clusters of 2^k that the GPU holds at once (clusters of eight do not reach every SM: 512 x 512 x 4096 on
+// 16 of them took two waves, 28.5 us, against 15.3 on 32 clusters of four).
+StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, int gy, const int (&slots)[4])
+{
+    auto density = [](long long nnz, double nb) { return nnz <= 0 ? 0.0 : (nnz >= nb ? 1.0 : nnz / nb); };
+    const double da = density(nnz_a, (double)NBa * NBk), db = density(nnz_b, (double)NBb * NBk);
+    const double common = NBk * da * db, lookups = NBk * db;
+    const double rows = (NBb + gy * (kSpThreads / 32) - 1) / (gy * (kSpThreads / 32));
+    const double pairs = (double)NBa * NBb;
+    const double bulk = pairs * (28.7e-6 * common + 3.6e-6 * lookups), chain = rows * (0.14 * common + 0.3 * (int)(lookups / 32 + 1));
+    double best = 0.95 * (2.9 + (bulk > chain ? bulk : chain));
+    StPlan plan = {0, 1};
+    const int n_chunks = (NBk + 7) / 8;
+    for (int w = 0; w < 3; ++w) {
+        const int BN = 64 << w;
+        const int stages = spgemm_tc_stages(BN, n_chunks);
+        if (stages < (BN == 256 ? 3 : st_groups(BN))) continue;        // (the ring also holds the tile's sums)
+        const double start = w == 0 ? 5.7 : (w == 1 ? 6.4 : 9.0), chunk = w == 0 ? 0.31 : (w == 1 ? 0.44 : 0.60);
+        const long long tiles = (long long)((NBa + kStARows - 1) / kStARows) * ((NBb * kSpEdge + BN - 1) / BN);
+        for (int k = 0; k < 4 && slots[k] > 0; ++k) {
+            const int split = 1 << k;
+            const int share = (n_chunks + split - 1) / split;
+            if ((split - 1) * share >= n_chunks) break;                // (every CTA of a split has at least one chunk)
+            const long long waves = (tiles * split + slots[k] - 1) / slots[k];
+            const double t = waves * (start + 0.03 * n_chunks + chunk * share) + (split > 1 ? 2.5 : 0.0);
+            if (t < best) { best = t; plan = {BN, split}; }
+        }
+    }
+    return plan;
+}
+
+void spgemm_tc_config(int split, cudaLaunchAttribute *attr, cudaLaunchConfig_t &cfg)
+{
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)split;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    cfg.blockDim = dim3(kStThreads);
+}
+
+// Per device, once: the kernels' shared-memory limit and the slots of spgemm_plan.
+bsp_status spgemm_tc_device(const int (**slots)[4])
+{
+    static int known[kGtMaxDevices][4] = {};
+    static bool done[kGtMaxDevices] = {};
+    int dev = 0;
+    BSP_CUDA_OK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
+    if (!done[dev]) {
+        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        for (int k = 0; k < 4; ++k) {
+            cudaLaunchAttribute attr[1];
+            cudaLaunchConfig_t cfg = {};
+            spgemm_tc_config(1 << k, attr, cfg);
+            cfg.gridDim = dim3(1, 1, 8);
+            cfg.dynamicSmemBytes = kGtMaxSmem;
+            int n = 0;
+            BSP_CUDA_OK(cudaOccupancyMaxActiveClusters(&n, spgemm_tc_kernel<64>, &cfg));
+            known[dev][k] = n << k;
+        }
+        done[dev] = true;
+    }
+    *slots = &known[dev];
+    return BSP_OK;
+}
+
+template <int BN>
+bsp_status launch_spgemm_tc(StParams p, cudaStream_t st)
+{
+    constexpr int kRows = kStARows + BN / kSpEdge;
+    p.stages = spgemm_tc_stages(BN, p.n_chunks);
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = {};
+    spgemm_tc_config(p.split, attr, cfg);
+    cfg.gridDim = dim3((unsigned)((p.NBb * kSpEdge + BN - 1) / BN), (unsigned)((p.NBa + kStARows - 1) / kStARows), (unsigned)p.split);
+    cfg.dynamicSmemBytes = 1024 + (size_t)kRows * p.n_chunks * 16 + (size_t)p.stages * kRows * 1024;
+    cfg.stream = st;
+    BSP_CUDA_OK(cudaLaunchKernelEx(&cfg, spgemm_tc_kernel<BN>, p));
+    return BSP_OK;
 }
 
 // One thread per row of Gamma: the first kept block keeps its column, the others store the distance to their predecessor.
@@ -163,9 +502,19 @@ bsp_status bsp_spgemm(const bsp_wdesc *wa, const bsp_bcsr *a, const bsp_wdesc *w
     if (wa->wtype == BSP_F32)
         spgemm_kernel<float><<<grid, kSpThreads, smem, st>>>(a->row_ptr, a->col_idx, (const float *)a->payload, b->row_ptr, b->col_idx,
                                                              (const float *)b->payload, NBb, NBk, C, (int *)ws);
-    else
+    else {
+        const int(*slots)[4] = nullptr;
+        rc = spgemm_tc_device(&slots);
+        if (rc != BSP_OK) return rc;
+        const StPlan plan = spgemm_plan(NBa, NBb, NBk, a->nnz, b->nnz, gy, *slots);
+        const StParams q = {a->row_ptr, a->col_idx, b->row_ptr, b->col_idx, (const uint8_t *)a->payload, (const uint8_t *)b->payload,
+                            C, (int *)ws, NBa, NBb, NBk, (NBk + 7) / 8, 0, plan.split};
+        if (plan.BN == 64) return launch_spgemm_tc<64>(q, st);
+        if (plan.BN == 128) return launch_spgemm_tc<128>(q, st);
+        if (plan.BN == 256) return launch_spgemm_tc<256>(q, st);
         spgemm_kernel<__nv_bfloat16><<<grid, kSpThreads, smem, st>>>(a->row_ptr, a->col_idx, (const __nv_bfloat16 *)a->payload, b->row_ptr,
                                                                      b->col_idx, (const __nv_bfloat16 *)b->payload, NBb, NBk, C, (int *)ws);
+    }
     BSP_CUDA_OK(cudaGetLastError());
     return BSP_OK;
 }

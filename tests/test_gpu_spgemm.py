@@ -42,6 +42,38 @@ def test_spgemm_many_rows_and_long_lists():
     run_spgemm(911, 64, 2048, 1024, "bf16", 0.5, 0.5)
 
 
+@pytest.mark.parametrize("Oa,Ob,I,fa,fb", [
+    (256, 512, 1024, 0.25, 0.25),        # 64 columns of C per CTA, reduction split over a cluster
+    (264, 456, 1032, 0.3, 0.1),          # the same with ragged tiles and a last chunk of one block column
+    (2040, 1032, 264, 0.1, 0.1),         # 128 columns, ragged, odd number of chunks
+    (2048, 1800, 776, 0.05, 0.05),       # 256 columns, ragged
+])
+def test_spgemm_tensor_core_tiles(Oa, Ob, I, fa, fb):
+    run_spgemm(931, Oa, Ob, I, "bf16", fa, fb)
+
+
+def test_spgemm_dropped_blocks_hide_non_finite_weights():
+    """An infinite weight reaches the blocks of C whose row of B keeps its column, and no other."""
+    O, I = 256, 512
+    A, B = make_case(941, O, I, 1, 1, "bf16"), make_case(942, O, I, 1, 1, "bf16")
+    ga, gb = synth.random_gamma(943, O // 8, I // 8, 200), synth.random_gamma(944, O // 8, I // 8, 200)
+    ga[3, 10], gb[:, 10] = 1, 0
+    gb[7, 10] = 1
+    A[3 * 8 + 2, 0, 0, 10 * 8 + 1] = np.inf
+    B[7 * 8:8 * 8, 0, 0, 10 * 8:11 * 8] = 1.0
+    la, lb = gpu_layer(A, ga, 8, 8, "bf16"), gpu_layer(B, gb, 8, 8, "bf16")
+    Cm = torch.empty((O, O), dtype=torch.float32, device="cuda")
+    bsp.bsp_spgemm(la.wd, la.handle(), lb.wd, lb.handle(), Cm, la.ws)
+    la.check()
+    got = Cm.cpu().numpy()
+    hit = np.zeros_like(got, dtype=bool)
+    hit[3 * 8 + 2, 7 * 8:8 * 8] = True
+    assert np.all(np.isposinf(got[hit])) and np.all(np.isfinite(got[~hit]))
+    A[3 * 8 + 2, 0, 0, 10 * 8 + 1] = 0.0
+    want = ref.spgemm(8, ref.compact(A, ga, 8, 8), ref.compact(B, gb, 8, 8))
+    assert rel_err(np.where(hit, 0.0, got), np.where(hit, 0.0, want)) <= 2e-5
+
+
 def test_spgemm_argument_errors():
     la = bsp.SparseLayer(64, 64, 1, 1, 8, 8, torch.bfloat16)
     lb = bsp.SparseLayer(64, 128, 1, 1, 8, 8, torch.bfloat16)
