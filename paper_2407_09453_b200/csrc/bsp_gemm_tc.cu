@@ -19,8 +19,8 @@
 // cores) was measured two to five times slower than these dense loads.
 //
 // Warps: 0 producer and 1 MMA issuer (each runs its loop as a whole, converged warp with warp-uniform values; one
-// elected lane issues), 2-9 epilogue in two groups of four (warp w reads the tensor-memory lanes 32 (w % 4) ..; group g
-// drains accumulator buffer g, so the epilogues of two consecutive tiles overlap).  Barriers per stage: full (one
+// elected lane issues), 2-9 epilogue in two groups of four (warp w reads the tensor-memory lanes 32 (w % 4) ..; the groups
+// take turns with the tiles and share the last one).  Barriers per stage: full (one
 // arrival that announces the bytes of both loads) and empty (tcgen05.commit); per accumulator buffer: acc_full (commit)
 // and acc_empty (4 warps).  Every wait is bounded; on expiry BSP_ERR_TIMEOUT is latched, the roles wind down, loads
 // in flight are awaited (bounded) and tensor memory is freed.
@@ -50,6 +50,19 @@ struct GtParams {
     int kbytes, a_stride;             // bytes of K per row of a stage: 128, or 64 for layers with at most 64 bytes of input channels; bytes of the activation part of a stage
 };
 
+// What follows the ring and the two staging buffers in shared memory.  (All of it is dynamic, so that the ring starts on
+// the 1024-byte boundary that the swizzled tiles need without room for rounding: four 48 KB stages, the staging buffers
+// and this fill the 227 KB of a CTA.)
+struct GtTail {
+    uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc_full[2], acc_empty[2];
+    uint32_t tmem;
+    uint32_t fail;
+    __align__(16) uint32_t bias[2][256];     // per epilogue group: bias and shift of its tile's channels
+    __align__(16) uint8_t shift[2][256];
+};
+constexpr int kGtGemmSmem = 227 * 1024;
+static_assert(4 * (kGtABytes + 256 * 128) + 8 * kGtStagingBytes + sizeof(GtTail) <= kGtGemmSmem, "four stages at 256 channels");
+
 // First output position (image, row, column) of position tile mt.
 __device__ __forceinline__ void gt_tile_origin(const GtParams &p, int mt, int &n0, int &y0, int &x0)
 {
@@ -65,15 +78,14 @@ __device__ __forceinline__ uint32_t gt_bias(const GtParams &p, int ch)
     return (p.bias != nullptr && ch < p.O) ? __ldg((const uint32_t *)p.bias + ch) : 0u;
 }
 
-template <int kWT, bool kPair>
+// kWT: operand type; kEy: bytes of an output element (4: float32 or int32, 2: bfloat16, 1: int8).
+template <int kWT, int kEy, bool kPair>
 __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_constant__ GtParams p)
 {
-    extern __shared__ __align__(16) uint8_t gt_smem_raw[];
-    uint8_t *smem = gt_smem_raw + ((1024u - (sm32(gt_smem_raw) & 1023u)) & 1023u);
-    __shared__ __align__(8) uint64_t s_full[kGtMaxStages], s_empty[kGtMaxStages];
-    __shared__ __align__(8) uint64_t s_acc_full[2], s_acc_empty[2];
-    __shared__ uint32_t s_tmem;
-    __shared__ volatile uint32_t s_fail;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    GtTail &tail = *(GtTail *)(smem + (size_t)p.stages * p.stage_bytes + 8 * kGtStagingBytes);
+    uint64_t *s_full = tail.full, *s_empty = tail.empty, *s_acc_full = tail.acc_full, *s_acc_empty = tail.acc_empty;
+    volatile uint32_t &s_fail = tail.fail;
 
     // (the warp's number, the tensor-memory base and the go-ahead below come through a shuffle, which makes them uniform to
     // the compiler: the role branches and the loops under them are then warp-uniform code.  Without it every MMA cost about
@@ -100,8 +112,10 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
         const PackedHeader *h = (const PackedHeader *)p.packed;
         const bool ok = h->magic == kPackedMagic && h->dtype == p.wtype && h->O == p.O && h->I == p.I && h->H == p.H &&
                         h->K == p.K && h->bo == p.bo && h->bi == p.bi && (h->forms & kFormDense) != 0;
-        s_fail = ok ? 0u : 2u;
+        const bool placed = (ring & 1023u) == 0u;
+        s_fail = ok && placed ? 0u : 2u;
         if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
+        else if (!placed) atomicMax(p.status, (int)BSP_ERR_CUDA);
         for (int s = 0; s < S; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_full[s])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_empty[s])), "r"(1) : "memory");
@@ -117,17 +131,17 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     }
     if (warp == 0) {
         if constexpr (kPair) {
-            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(kGtTmemCols) : "memory");
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&tail.tmem)), "r"(kGtTmemCols) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
         } else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(kGtTmemCols) : "memory");
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&tail.tmem)), "r"(kGtTmemCols) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     gt_sync_all<kPair>();                   // (a pair: both CTAs' barriers are initialised before either signals the other)
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, s_tmem, 0);
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tail.tmem, 0);
     const bool run = __shfl_sync(0xFFFFFFFFu, s_fail, 0) == 0u;
 
     if (warp == 0) {
@@ -187,7 +201,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             if (!ok && lane == 0) {
                 // winding down after a wait that ran out: the loads already issued still write into this CTA's shared
                 // memory, so the barriers of the stages in flight are awaited (bounded) before the CTA may leave
-                atomicExch((uint32_t *)&s_fail, 1u);
+                atomicExch((uint32_t *)&tail.fail, 1u);
                 // (the follower of a pair has no barrier of its own to watch: its loads announce themselves to the leader;
                 // both CTAs meet at the cluster barrier before they leave)
                 for (uint32_t back = 0; back < (uint32_t)S && back < issued && rank == 0; ++back) {
@@ -229,86 +243,62 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 }
                 if (ok) gt_commit_elected<kPair>(sm32(&s_acc_full[buf]));
             }
-            if (!ok && lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
+            if (!ok && lane == 0) atomicExch((uint32_t *)&tail.fail, 1u);
         }
     } else {
         // ================= epilogue (warps 2-9) =================
         // Two groups of four warps: group g drains accumulator buffer g, that is every second tile of the CTA, so the
-        // epilogues of two consecutive tiles run side by side.
+        // epilogues of two consecutive tiles run side by side.  The last tile of a CTA (often its only one) is shared, each
+        // group taking every second of its 128-byte rounds: 1x1 256->1024 at 14x14, batch 64, 14.1 -> 12.9 us; sharing every
+        // tile instead cost 10 % where a CTA has many small ones (8-bit 3x3 64->64 at 224x224, int32 output).
         if (run) {
             const int q = warp & 3;                              // quarter of the tensor-memory lanes this warp reaches
-            const int ew = warp - 2, grp = ew >> 2;
-            const int ey = p.ey;
-            const int cpr = 128 / ey;                            // output channels per staging round (128 bytes of a row)
+            const int grp = (warp - 2) >> 2;
+            constexpr int cpr = 128 / kEy;                       // output channels per round (128 bytes of a row)
             // the group's staging buffer: 128 rows of 128 bytes, this warp's 32 rows at its quarter
             const uint32_t sg = staging + (uint32_t)(grp * 4 * kGtStagingBytes), sb = sg + (uint32_t)(q * kGtStagingBytes);
             const bool issuer = q == 0 && lane == 0;             // one thread of the group issues its stores
-            uint32_t tile_i = (uint32_t)grp;
+            uint32_t *bias = tail.bias[grp];
+            uint8_t *shift = tail.shift[grp];
+            uint32_t tile_i = 0;
+            int have = -1;                                       // first channel of the entries in `bias` and `shift`
             bool ok = true;
-            for (int tile = t_first + grp * t_step; tile < t_count && ok; tile += 2 * t_step, tile_i += 2) {
+            for (int tile = t_first; tile < t_count && ok; tile += t_step, ++tile_i) {
+                const bool last = tile + t_step >= t_count, shared_tile = last && BN > cpr;
+                if (!shared_tile && (int)(tile_i & 1u) != grp) continue;
+                const int c_first = shared_tile ? grp * cpr : 0, c_step = shared_tile ? 2 * cpr : cpr;
                 const uint32_t buf = tile_i & 1u, use = tile_i >> 1;
                 int mt, tn;
                 gt_divmod(tile, p.n_tiles_n, p.m_ntn, mt, tn);
                 const int n0 = tn * BN;
                 int in0, y0, x0;
                 gt_tile_origin(p, kPair ? 2 * mt + (int)rank : mt, in0, y0, x0);
+                // (the entries of the tile before were last read ahead of the group barrier of its last store; a layer with one
+                // channel tile keeps them: a trip to memory per tile costs where a tile takes about a microsecond)
+                for (int c = ((warp - 2) & 3) * 32 + lane; c < BN && n0 != have; c += 128) {
+                    bias[c] = gt_bias(p, n0 + c);
+                    if constexpr (kEy == 1) shift[c] = n0 + c < p.O ? (uint8_t)((uint32_t)__ldg(p.shift + n0 + c) & 31u) : (uint8_t)0;
+                }
+                have = n0;
                 if (!gt_wait(sm32(&s_acc_full[buf]), use & 1u)) ok = false;
                 if (s_fail) ok = false;
                 ok = gt_group_all(1 + grp, ok);                // the four warps go on or give up as one (they meet at barriers below)
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + buf * 256u;
-                for (int c0 = 0; c0 < BN; c0 += cpr) {
+                for (int c0 = c_first; c0 < BN; c0 += c_step) {
                     uint32_t out[32];                            // 128 bytes of this lane's row of Y
-                    if (ey == 4) {                               // fp32 or int32 output: 32 channels
-                        uint32_t v[32];
-                        gt_load32(tbase + (uint32_t)c0, v);
-                        const uint32_t bl = gt_bias(p, n0 + c0 + lane);      // lane e holds the bias of channel c0 + e
-                        if (kWT == BSP_I8) {
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) out[e] = (uint32_t)((int)v[e] + (int)__shfl_sync(0xFFFFFFFFu, bl, e));
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 32; ++e)
-                                out[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(__shfl_sync(0xFFFFFFFFu, bl, e)));
-                        }
-                    } else if (ey == 1) {                        // int8 output: 128 channels, requantised after the bias
-#pragma unroll
-                        for (int sub = 0; sub < 4; ++sub) {
-                            // (32-channel pieces past the tile or past the last channel are not computed: their bytes are clipped by the store)
-                            if (c0 + sub * 32 >= BN || n0 + c0 + sub * 32 >= p.O) {
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) out[sub * 8 + e] = 0u;
-                                continue;
-                            }
-                            uint32_t v[32];
-                            gt_load32(tbase + (uint32_t)(c0 + sub * 32), v);
-                            const int ch = n0 + c0 + sub * 32 + lane;
-                            const uint32_t bl = gt_bias(p, ch);
-                            const uint32_t sl = ch < p.O ? (uint32_t)__ldg(p.shift + ch) & 31u : 0u;
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) {
-                                int r4[4];
-#pragma unroll
-                                for (int b = 0; b < 4; ++b)
-                                    r4[b] = gt_round_shift((int)v[4 * e + b] + (int)__shfl_sync(0xFFFFFFFFu, bl, 4 * e + b),
-                                                           __shfl_sync(0xFFFFFFFFu, sl, 4 * e + b));
-                                out[sub * 8 + e] = gt_pack_s8x4(r4[0], r4[1], r4[2], r4[3]);
-                            }
-                        }
-                    } else {                                     // bf16 output: 64 channels, rounded to nearest even after the bias
-#pragma unroll
-                        for (int sub = 0; sub < 2; ++sub) {
-                            uint32_t v[32];
-                            gt_load32(tbase + (uint32_t)(c0 + sub * 32), v);
-                            const uint32_t bl = gt_bias(p, n0 + c0 + sub * 32 + lane);
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) {
-                                const __nv_bfloat162 h = __floats2bfloat162_rn(
-                                    __uint_as_float(v[2 * e]) + __uint_as_float(__shfl_sync(0xFFFFFFFFu, bl, 2 * e)),
-                                    __uint_as_float(v[2 * e + 1]) + __uint_as_float(__shfl_sync(0xFFFFFFFFu, bl, 2 * e + 1)));
-                                out[sub * 16 + e] = *(const uint32_t *)&h;
-                            }
+                    const int left = (p.O - n0 < BN ? p.O - n0 : BN) - c0;          // channels from here on
+                    gt_epilogue_round<kWT == BSP_I8, kEy>(tbase + (uint32_t)c0, bias + c0, shift + c0, left, out);
+                    if (!last && c0 + c_step >= BN) {
+                        // the accumulator buffer has been read: hand it back to the MMA issuer
+                        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) {
+                            if constexpr (kPair)
+                                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(lead_acc_empty0 + buf * 8u) : "memory");
+                            else
+                                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&s_acc_empty[buf])) : "memory");
                         }
                     }
                     // the staging buffer was handed to a TMA store in the previous round: the issuing thread waits until it
@@ -324,24 +314,15 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                     gt_group_sync(1 + grp);
                     // one store of the tile's box: 128 bytes of every row; what lies past the last channel, column, row or image
                     // of Y is clipped (rows of the buffer beyond the box are not part of the store)
-                    if (issuer && n0 + c0 < p.O) {
+                    if (issuer && left > 0) {
                         asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n"
-                                     ::"l"(&p.tmy), "r"(sg), "r"((n0 + c0) * ey), "r"(x0), "r"(y0), "r"(in0) : "memory");
+                                     ::"l"(&p.tmy), "r"(sg), "r"((n0 + c0) * kEy), "r"(x0), "r"(y0), "r"(in0) : "memory");
                         asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
                     }
                 }
-                // the accumulator buffer has been read: hand it back to the MMA issuer
-                asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    if constexpr (kPair)
-                        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(lead_acc_empty0 + buf * 8u) : "memory");
-                    else
-                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&s_acc_empty[buf])) : "memory");
-                }
             }
-            if (issuer) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
-            if (!ok && lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
+            if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");      // (the stores have read this CTA's memory)
+            if (!ok && lane == 0) atomicExch((uint32_t *)&tail.fail, 1u);
         }
     }
 
@@ -402,21 +383,22 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     p.kbytes = (long long)wd.I * esz <= 64 ? 64 : 128;
     p.a_stride = kGtBM * p.kbytes;
     p.a_bytes = p.rows_tile * p.kbytes;
-    // kernels by operand type (in the order of bsp_dtype) and by CTA pairs
+    // kernels by operand type (in the order of bsp_dtype), width of the output (32 bits or the narrow form) and CTA pairs
     typedef void (*Kernel)(const GtParams);
-    static const Kernel kernels[3][2] = {{gemm_tc_kernel<BSP_F32, false>, gemm_tc_kernel<BSP_F32, true>},
-                                         {gemm_tc_kernel<BSP_BF16, false>, gemm_tc_kernel<BSP_BF16, true>},
-                                         {gemm_tc_kernel<BSP_I8, false>, gemm_tc_kernel<BSP_I8, true>}};
+    static const Kernel kernels[3][2][2] = {
+        {{gemm_tc_kernel<BSP_F32, 4, false>, gemm_tc_kernel<BSP_F32, 4, true>}, {gemm_tc_kernel<BSP_F32, 2, false>, gemm_tc_kernel<BSP_F32, 2, true>}},
+        {{gemm_tc_kernel<BSP_BF16, 4, false>, gemm_tc_kernel<BSP_BF16, 4, true>}, {gemm_tc_kernel<BSP_BF16, 2, false>, gemm_tc_kernel<BSP_BF16, 2, true>}},
+        {{gemm_tc_kernel<BSP_I8, 4, false>, gemm_tc_kernel<BSP_I8, 4, true>}, {gemm_tc_kernel<BSP_I8, 1, false>, gemm_tc_kernel<BSP_I8, 1, true>}}};
     static_assert(BSP_F32 == 0 && BSP_BF16 == 1 && BSP_I8 == 2, "the table is indexed by type");
+    const Kernel *kernel = kernels[wd.wtype][ey == 4 ? 0 : 1];
     static bool opted[kGtMaxDevices] = {};
     static int n_sm[kGtMaxDevices] = {};
     int dev = 0;
     BSP_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
     if (!opted[dev]) {
-        for (int t = 0; t < 3; ++t)
-            for (int q = 0; q < 2; ++q)
-                BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t][q], cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        for (int t = 0; t < 12; ++t)
+            BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 4][t / 2 % 2][t % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, kGtGemmSmem));
         BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
         opted[dev] = true;
     }
@@ -449,11 +431,11 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     p.m_ntn = gt_magic(p.n_tiles_n); p.m_tx = gt_magic(p.tiles_x); p.m_ty = gt_magic(p.tiles_y);
     p.stage_bytes = p.a_stride + (pair ? p.BN / 2 : p.BN) * p.kbytes;
     const int staging = 8 * kGtStagingBytes;
-    int stages = (kGtMaxSmem - 1024 - staging) / p.stage_bytes;
+    int stages = (kGtGemmSmem - staging - (int)sizeof(GtTail)) / p.stage_bytes;
     if (stages > kGtMaxStages) stages = kGtMaxStages;
     if (stages < 2) return BSP_ERR_SHAPE;
     p.stages = stages;
-    const size_t smem = 1024 + (size_t)stages * p.stage_bytes + staging;
+    const size_t smem = (size_t)stages * p.stage_bytes + staging + sizeof(GtTail);
 
     GtEncodeFn enc = gt_encode();
     if (!enc) return BSP_ERR_CUDA;
@@ -501,11 +483,11 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
-        BSP_CUDA_OK(cudaLaunchKernelEx(&cfg, kernels[wd.wtype][1], p));
+        BSP_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel[1], p));
         return BSP_OK;
     }
     const int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
-    kernels[wd.wtype][0]<<<grid, kGtThreads, smem, st>>>(p);
+    kernel[0]<<<grid, kGtThreads, smem, st>>>(p);
     BSP_CUDA_OK(cudaGetLastError());
     return BSP_OK;
 }

@@ -133,10 +133,9 @@ __device__ __forceinline__ void gt_divmod(int n, int d, uint32_t m, int &q, int 
 // magnitude is formed without overflow; -2^31 with s = 0 comes back as itself) ...
 __device__ __forceinline__ int gt_round_shift(int v, uint32_t s)
 {
-    const uint32_t sg = (uint32_t)(v >> 31);                              // 0 or all ones
-    const uint32_t mag = ((uint32_t)v ^ sg) - sg;                        // |v|, at most 2^31
+    const uint32_t mag = v < 0 ? 0u - (uint32_t)v : (uint32_t)v;          // |v|, at most 2^31
     const uint32_t r = (mag + ((1u << s) >> 1)) >> s;
-    return (int)((r ^ sg) - sg);
+    return (int)(v < 0 ? 0u - r : r);
 }
 // ... and four such values saturated to int8 and packed, the first in the lowest byte (cvt.pack saturates two 32-bit
 // values to bytes, its first source above its second, and shifts the third operand up by 16 bits).
@@ -158,8 +157,9 @@ __device__ __forceinline__ bool gt_group_all(int id, bool flag)
     return r != 0u;
 }
 
-// 32 consecutive accumulator columns of this thread's tensor-memory lane.
-__device__ __forceinline__ void gt_load32(uint32_t taddr, uint32_t (&v)[32])
+// 32 consecutive accumulator columns of this thread's tensor-memory lane: the load, and the wait after which the values of
+// the loads issued so far may be used (it names the registers, so that no use of them moves before it).
+__device__ __forceinline__ void gt_load32_issue(uint32_t taddr, uint32_t (&v)[32])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
                  "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
@@ -168,7 +168,82 @@ __device__ __forceinline__ void gt_load32(uint32_t taddr, uint32_t (&v)[32])
                    "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
                    "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
                  : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void gt_load32_wait(uint32_t (&v)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+                   "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+                   "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+                 :: "memory");
+}
+__device__ __forceinline__ void gt_load32(uint32_t taddr, uint32_t (&v)[32])
+{
+    gt_load32_issue(taddr, v);
+    gt_load32_wait(v);
+}
+
+// One round of an epilogue: 128 bytes of this lane's row of the output (32 channels of 4 bytes, 64 of bfloat16, 128 of
+// int8) from the accumulator columns at `taddr`, after the bias.  kEy: bytes of an output element.  `bias` (raw bits) and
+// `shift` are the channels' own entries in shared memory, read four channels at a time by all lanes at once: a shuffle per
+// channel (two for int8) had made the int8 round five times as long.  `n`: channels left; 32-channel pieces past them are
+// neither loaded nor computed (their bytes are clipped by the store).
+template <bool kInt, int kEy>
+__device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t *bias, const uint8_t *shift, int n, uint32_t (&out)[32])
+{
+    auto bias4 = [&](int c) { return *(const uint4 *)(bias + c); };
+    if constexpr (kEy == 4) {
+        gt_load32(taddr, out);
+#pragma unroll
+        for (int e = 0; e < 32; e += 4) {
+            const uint4 b = bias4(e);
+            if constexpr (kInt) { out[e] += b.x; out[e + 1] += b.y; out[e + 2] += b.z; out[e + 3] += b.w; }
+            else {
+                out[e] = __float_as_uint(__uint_as_float(out[e]) + __uint_as_float(b.x));
+                out[e + 1] = __float_as_uint(__uint_as_float(out[e + 1]) + __uint_as_float(b.y));
+                out[e + 2] = __float_as_uint(__uint_as_float(out[e + 2]) + __uint_as_float(b.z));
+                out[e + 3] = __float_as_uint(__uint_as_float(out[e + 3]) + __uint_as_float(b.w));
+            }
+        }
+    } else if constexpr (kEy == 2) {                     // rounded to nearest even after the bias
+#pragma unroll
+        for (int sub = 0; sub < 2; ++sub) {
+            if (sub * 32 >= n) {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) out[sub * 16 + e] = 0u;
+                continue;
+            }
+            uint32_t v[32];
+            gt_load32(taddr + (uint32_t)(sub * 32), v);
+#pragma unroll
+            for (int e = 0; e < 32; e += 4) {
+                const uint4 b = bias4(sub * 32 + e);
+                const __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(v[e]) + __uint_as_float(b.x), __uint_as_float(v[e + 1]) + __uint_as_float(b.y));
+                const __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(v[e + 2]) + __uint_as_float(b.z), __uint_as_float(v[e + 3]) + __uint_as_float(b.w));
+                out[sub * 16 + e / 2] = *(const uint32_t *)&h0;
+                out[sub * 16 + e / 2 + 1] = *(const uint32_t *)&h1;
+            }
+        }
+    } else {                                             // requantised after the bias
+#pragma unroll
+        for (int sub = 0; sub < 4; ++sub) {
+            if (sub * 32 >= n) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) out[sub * 8 + e] = 0u;
+                continue;
+            }
+            uint32_t v[32];
+            gt_load32(taddr + (uint32_t)(sub * 32), v);
+#pragma unroll
+            for (int e = 0; e < 32; e += 4) {
+                const uint4 b = bias4(sub * 32 + e);
+                const uint32_t s = *(const uint32_t *)(shift + sub * 32 + e);
+                out[sub * 8 + e / 4] = gt_pack_s8x4(gt_round_shift((int)(v[e] + b.x), s & 31u), gt_round_shift((int)(v[e + 1] + b.y), (s >> 8) & 31u),
+                                                    gt_round_shift((int)(v[e + 2] + b.z), (s >> 16) & 31u), gt_round_shift((int)(v[e + 3] + b.w), s >> 24));
+            }
+        }
+    }
 }
 
 typedef CUresult (*GtEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
