@@ -84,9 +84,6 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
     const int t_first = (int)blockIdx.x, t_step = (int)gridDim.x, t_count = p.n_tiles;
 
     if (tid == 0) {
-        const bool ok = ct_header_ok(p.packed1, p.wtype, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1) && ct_header_ok(p.packed2, p.wtype, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
-        s_fail = ok ? 0u : 2u;
-        if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
         for (int s = 0; s < S; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_full[s])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_empty[s])), "r"(1) : "memory");
@@ -110,6 +107,12 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(kGtTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    wait_for_previous();
+    if (tid == 0) {
+        const bool ok = ct_header_ok(p.packed1, p.wtype, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1) && ct_header_ok(p.packed2, p.wtype, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
+        s_fail = ok ? 0u : 2u;
+        if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -427,7 +430,7 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&s_acc2_empty[buf])) : "memory");
                 }
             }
-            if (issuer) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+            if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");      // (the stores have read this CTA's memory)
             if (!ok && lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
         }
     }
@@ -560,9 +563,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
             return BSP_ERR_CUDA;
     }
     const int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
-    if (wd1.wtype == BSP_I8) chain_tc_kernel<true><<<grid, kCtThreads, smem, st>>>(p);
-    else chain_tc_kernel<false><<<grid, kCtThreads, smem, st>>>(p);
-    BSP_CUDA_OK(cudaGetLastError());
+    BSP_CUDA_OK(launch_after(wd1.wtype == BSP_I8 ? chain_tc_kernel<true> : chain_tc_kernel<false>, dim3((unsigned)grid), dim3(kCtThreads), smem, st, p));
     return BSP_OK;
 }
 

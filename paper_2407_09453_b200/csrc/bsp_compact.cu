@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(kThreads, 5) compact_kernel(const CompactArgs 
 {
     __shared__ __align__(16) uint8_t s_gamma[kBig ? 16 : kSmallBlocks];
     __shared__ int s_sum[kThreads / 32];
+    wait_for_previous();
     const int n_fill = a.NBo * a.fill_parts;
     if ((int)blockIdx.x >= n_fill) {
         if ((int)blockIdx.x == n_fill && threadIdx.x == 0 && a.hdr != nullptr) *a.hdr = a.hdr_init;
@@ -371,10 +372,9 @@ bsp_status launch_compact(const bsp_wdesc &wd, const void *W, const uint8_t *gam
             a.fill_parts = (int)(p < 1 ? 1 : (p > 8 ? 8 : p));
         }
         const unsigned grid = (unsigned)(NBo * a.fill_parts + a.dense_ctas);
-        if (wd.wtype == BSP_I8) compact_kernel<uint8_t, false><<<grid, kThreads, smem, st>>>(a);
-        else if (wd.wtype == BSP_BF16) compact_kernel<uint16_t, false><<<grid, kThreads, smem, st>>>(a);
-        else compact_kernel<uint32_t, false><<<grid, kThreads, smem, st>>>(a);
-        BSP_CUDA_OK(cudaGetLastError());
+        if (wd.wtype == BSP_I8) BSP_CUDA_OK(launch_after(compact_kernel<uint8_t, false>, dim3(grid), dim3(kThreads), smem, st, a));
+        else if (wd.wtype == BSP_BF16) BSP_CUDA_OK(launch_after(compact_kernel<uint16_t, false>, dim3(grid), dim3(kThreads), smem, st, a));
+        else BSP_CUDA_OK(launch_after(compact_kernel<uint32_t, false>, dim3(grid), dim3(kThreads), smem, st, a));
         return BSP_OK;
     }
     if ((long long)NBo * NBi > 0x7FFFFFFF) return BSP_ERR_SHAPE;
@@ -383,10 +383,9 @@ bsp_status launch_compact(const bsp_wdesc &wd, const void *W, const uint8_t *gam
     if (a.fill_parts > 16) a.fill_parts = 16;
     if (a.fill_parts < 1) a.fill_parts = 1;
     const unsigned grid = (unsigned)(NBo * a.fill_parts + a.dense_ctas);
-    if (wd.wtype == BSP_I8) compact_kernel<uint8_t, true><<<grid, kThreads, smem, st>>>(a);
-    else if (wd.wtype == BSP_BF16) compact_kernel<uint16_t, true><<<grid, kThreads, smem, st>>>(a);
-    else compact_kernel<uint32_t, true><<<grid, kThreads, smem, st>>>(a);
-    BSP_CUDA_OK(cudaGetLastError());
+    if (wd.wtype == BSP_I8) BSP_CUDA_OK(launch_after(compact_kernel<uint8_t, true>, dim3(grid), dim3(kThreads), smem, st, a));
+    else if (wd.wtype == BSP_BF16) BSP_CUDA_OK(launch_after(compact_kernel<uint16_t, true>, dim3(grid), dim3(kThreads), smem, st, a));
+    else BSP_CUDA_OK(launch_after(compact_kernel<uint32_t, true>, dim3(grid), dim3(kThreads), smem, st, a));
     return BSP_OK;
 }
 

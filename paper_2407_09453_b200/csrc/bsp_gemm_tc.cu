@@ -108,14 +108,6 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     }
 
     if (tid == 0) {
-        // the packed buffer must be the one bsp_compact filled for this descriptor, with the masked dense form in it
-        const PackedHeader *h = (const PackedHeader *)p.packed;
-        const bool ok = h->magic == kPackedMagic && h->dtype == p.wtype && h->O == p.O && h->I == p.I && h->H == p.H &&
-                        h->K == p.K && h->bo == p.bo && h->bi == p.bi && (h->forms & kFormDense) != 0;
-        const bool placed = (ring & 1023u) == 0u;
-        s_fail = ok && placed ? 0u : 2u;
-        if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
-        else if (!placed) atomicMax(p.status, (int)BSP_ERR_CUDA);
         for (int s = 0; s < S; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_full[s])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_empty[s])), "r"(1) : "memory");
@@ -137,6 +129,17 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&tail.tmem)), "r"(kGtTmemCols) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
         }
+    }
+    wait_for_previous();
+    if (tid == 0) {
+        // the packed buffer must be the one bsp_compact filled for this descriptor, with the masked dense form in it
+        const PackedHeader *h = (const PackedHeader *)p.packed;
+        const bool ok = h->magic == kPackedMagic && h->dtype == p.wtype && h->O == p.O && h->I == p.I && h->H == p.H &&
+                        h->K == p.K && h->bo == p.bo && h->bi == p.bi && (h->forms & kFormDense) != 0;
+        const bool placed = (ring & 1023u) == 0u;
+        s_fail = ok && placed ? 0u : 2u;
+        if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
+        else if (!placed) atomicMax(p.status, (int)BSP_ERR_CUDA);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     gt_sync_all<kPair>();                   // (a pair: both CTAs' barriers are initialised before either signals the other)
@@ -473,22 +476,12 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     }
 
     if (pair) {
-        cudaLaunchConfig_t cfg = {};
         const int pairs = p.n_tile_pairs < n_sm[dev] / 2 ? p.n_tile_pairs : n_sm[dev] / 2;
-        cfg.gridDim = dim3((unsigned)(2 * pairs));
-        cfg.blockDim = dim3(kGtThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        BSP_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel[1], p));
+        BSP_CUDA_OK(launch_after_clusters(kernel[1], dim3((unsigned)(2 * pairs)), dim3(kGtThreads), smem, st, 2, 1, p));
         return BSP_OK;
     }
     const int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
-    kernel[0]<<<grid, kGtThreads, smem, st>>>(p);
-    BSP_CUDA_OK(cudaGetLastError());
+    BSP_CUDA_OK(launch_after(kernel[0], dim3((unsigned)grid), dim3(kGtThreads), smem, st, p));
     return BSP_OK;
 }
 

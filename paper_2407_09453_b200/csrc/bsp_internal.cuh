@@ -70,6 +70,38 @@ inline int gemm_tile_n(int O)
     return (((O + tiles - 1) / tiles) + 63) / 64 * 64;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_after() may start while the kernel before it on the stream
+// still runs, once every CTA of that one has called let_next_start() or left.  Until wait_for_previous() returns - the
+// kernel before it has then completed and its writes are visible - it touches nothing in global memory (it sets up
+// barriers, tensor memory and descriptors).  It lets its own successor start only after that, so at most two kernels of a
+// stream overlap, and no successor can hold a line in L1 that was read before the kernel in between wrote it.  (Launched
+// one after another without this, the kernels of a stream started in steps of about 2 us.)
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous()
+{
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    let_next_start();
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_after_clusters(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster_x, int cluster_z, A... args)
+{
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster_x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = (unsigned)cluster_z;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = attr; cfg.numAttrs = cluster_x * cluster_z > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    return launch_after_clusters(kernel, grid, block, smem, st, 1, 1, args...);
+}
+
 #define BSP_CUDA_OK(expr)                                            \
     do {                                                             \
         cudaError_t e_ = (expr);                                     \

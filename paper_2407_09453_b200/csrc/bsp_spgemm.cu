@@ -87,6 +87,7 @@ spgemm_kernel(const int32_t *__restrict__ a_row_ptr, const int32_t *__restrict__
     extern __shared__ int s_pos[];                 // [NBk]: payload position of row i's block in column k, or -1
     const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = threadIdx.x; k < NBk; k += kSpThreads) s_pos[k] = -1;
+    wait_for_previous();
     __syncthreads();
     for (int n = a_row_ptr[i] + threadIdx.x; n < a_row_ptr[i + 1]; n += kSpThreads) {
         const int k = a_col_idx[n];
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(BN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
+    wait_for_previous();
     // a block row's first and last stored block (rows past the last one are empty)
     auto row_of = [&](int b, int &lo, int &hi) {
         const bool is_a = b < kStARows;
@@ -392,14 +394,6 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
     return plan;
 }
 
-void spgemm_tc_config(int split, cudaLaunchAttribute *attr, cudaLaunchConfig_t &cfg)
-{
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)split;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    cfg.blockDim = dim3(kStThreads);
-}
-
 // Per device, once: the kernels' shared-memory limit and the slots of spgemm_plan.
 bsp_status spgemm_tc_device(const int (**slots)[4])
 {
@@ -415,9 +409,10 @@ bsp_status spgemm_tc_device(const int (**slots)[4])
         for (int k = 0; k < 4; ++k) {
             cudaLaunchAttribute attr[1];
             cudaLaunchConfig_t cfg = {};
-            spgemm_tc_config(1 << k, attr, cfg);
-            cfg.gridDim = dim3(1, 1, 8);
-            cfg.dynamicSmemBytes = kGtMaxSmem;
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1u << k;
+            cfg.attrs = attr; cfg.numAttrs = 1;
+            cfg.gridDim = dim3(1, 1, 8); cfg.blockDim = dim3(kStThreads); cfg.dynamicSmemBytes = kGtMaxSmem;
             int n = 0;
             BSP_CUDA_OK(cudaOccupancyMaxActiveClusters(&n, spgemm_tc_kernel<64>, &cfg));
             known[dev][k] = n << k;
@@ -433,13 +428,9 @@ bsp_status launch_spgemm_tc(StParams p, cudaStream_t st)
 {
     constexpr int kRows = kStARows + BN / kSpEdge;
     p.stages = spgemm_tc_stages(BN, p.n_chunks);
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = {};
-    spgemm_tc_config(p.split, attr, cfg);
-    cfg.gridDim = dim3((unsigned)((p.NBb * kSpEdge + BN - 1) / BN), (unsigned)((p.NBa + kStARows - 1) / kStARows), (unsigned)p.split);
-    cfg.dynamicSmemBytes = 1024 + (size_t)kRows * p.n_chunks * 16 + (size_t)p.stages * kRows * 1024;
-    cfg.stream = st;
-    BSP_CUDA_OK(cudaLaunchKernelEx(&cfg, spgemm_tc_kernel<BN>, p));
+    const dim3 grid((unsigned)((p.NBb * kSpEdge + BN - 1) / BN), (unsigned)((p.NBa + kStARows - 1) / kStARows), (unsigned)p.split);
+    const size_t smem = 1024 + (size_t)kRows * p.n_chunks * 16 + (size_t)p.stages * kRows * 1024;
+    BSP_CUDA_OK(launch_after_clusters(spgemm_tc_kernel<BN>, grid, dim3(kStThreads), smem, st, 1, p.split, p));
     return BSP_OK;
 }
 
@@ -499,10 +490,10 @@ bsp_status bsp_spgemm(const bsp_wdesc *wa, const bsp_bcsr *a, const bsp_wdesc *w
     if (gy < 1) gy = 1;
     const dim3 grid((unsigned)NBa, (unsigned)gy);
     cudaStream_t st = (cudaStream_t)stream;
-    if (wa->wtype == BSP_F32)
-        spgemm_kernel<float><<<grid, kSpThreads, smem, st>>>(a->row_ptr, a->col_idx, (const float *)a->payload, b->row_ptr, b->col_idx,
-                                                             (const float *)b->payload, NBb, NBk, C, (int *)ws);
-    else {
+    if (wa->wtype == BSP_F32) {
+        BSP_CUDA_OK(launch_after(spgemm_kernel<float>, grid, dim3(kSpThreads), smem, st, a->row_ptr, a->col_idx, (const float *)a->payload, b->row_ptr, b->col_idx,
+                                                             (const float *)b->payload, NBb, NBk, C, (int *)ws));
+    } else {
         const int(*slots)[4] = nullptr;
         rc = spgemm_tc_device(&slots);
         if (rc != BSP_OK) return rc;
@@ -512,10 +503,9 @@ bsp_status bsp_spgemm(const bsp_wdesc *wa, const bsp_bcsr *a, const bsp_wdesc *w
         if (plan.BN == 64) return launch_spgemm_tc<64>(q, st);
         if (plan.BN == 128) return launch_spgemm_tc<128>(q, st);
         if (plan.BN == 256) return launch_spgemm_tc<256>(q, st);
-        spgemm_kernel<__nv_bfloat16><<<grid, kSpThreads, smem, st>>>(a->row_ptr, a->col_idx, (const __nv_bfloat16 *)a->payload, b->row_ptr,
-                                                                     b->col_idx, (const __nv_bfloat16 *)b->payload, NBb, NBk, C, (int *)ws);
+        BSP_CUDA_OK(launch_after(spgemm_kernel<__nv_bfloat16>, grid, dim3(kSpThreads), smem, st, a->row_ptr, a->col_idx, (const __nv_bfloat16 *)a->payload, b->row_ptr,
+                                                                     b->col_idx, (const __nv_bfloat16 *)b->payload, NBb, NBk, C, (int *)ws));
     }
-    BSP_CUDA_OK(cudaGetLastError());
     return BSP_OK;
 }
 

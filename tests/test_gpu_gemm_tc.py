@@ -107,3 +107,34 @@ def test_packed_buffer_of_another_layer_is_refused():
     assert e.value.status == bsp.ERR_INDEX
     assert bool((Y == -7.0).all())
     lay.check()                                   # the latched status is cleared once read
+
+
+@pytest.mark.parametrize("P,C", [(64, 64), (1, 256), (4096, 256)])
+def test_calls_that_depend_on_each_other_back_to_back(P, C):
+    """Consecutive kernels of a stream overlap their starts: a run of calls in which each reads what the call before wrote, or
+    overwrites what it read, and new weights arrive in between, gives what the same calls give one at a time."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    Ws = [(torch.randn((C, 1, 1, C), device="cuda", generator=g) / C ** 0.5).to(torch.bfloat16) for _ in range(3)]
+    X = torch.randn((P, C), device="cuda", generator=g).to(torch.bfloat16)
+    out = []
+    for wait in (True, False, False):
+        lay = bsp.SparseLayer(C, C, 1, 1, 8, 8, torch.bfloat16)
+        a, b = X.clone(), torch.empty_like(X)
+        for k in range(12):
+            if k % 4 == 0:
+                lay.mask(Ws[k // 4], lay.NBo * lay.NBi // 2)
+                if wait:
+                    torch.cuda.synchronize()
+                lay.compact(Ws[k // 4])
+                if wait:
+                    torch.cuda.synchronize()
+            lay.gemm(a, None, b)
+            if wait:
+                torch.cuda.synchronize()
+            a, b = b, a
+        lay.check()
+        out.append((a.clone(), b.clone(), lay.payload.clone()))
+    for o in out[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(o, out[0]))
