@@ -135,6 +135,7 @@ def test_calls_that_depend_on_each_other_back_to_back(P, C):
                 torch.cuda.synchronize()
             a, b = b, a
         lay.check()
-        out.append((a.clone(), b.clone(), lay.payload.clone()))
+        out.append((a.clone(), b.clone(), lay.payload[:lay.nnz * 64].clone()))
     for o in out[1:]:
-        assert all(torch.equal(x, y) for x, y in zip(o, out[0]))
+        for what, x, y in zip(("last input", "last output", "payload"), o, out[0]):
+            assert torch.equal(x, y), what

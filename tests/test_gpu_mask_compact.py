@@ -80,6 +80,31 @@ def test_gamma_large_layer_many_select_passes():
     assert np.array_equal(g, ref.mask(want_s, want_s.size // 2))
 
 
+@pytest.mark.parametrize("rows,cols,scope", [
+    (19, 27, bsp.SCOPE_LAYER),           # 513 blocks: counted
+    (47, 45, bsp.SCOPE_LAYER),           # 2115: the one-launch kernel selects by digits
+    (64, 64, bsp.SCOPE_LAYER),           # 4096: the last
+    (33, 128, bsp.SCOPE_ROW),            # rows of 128, 256, 257 and 600 in a layer of more than 4096 blocks
+    (17, 256, bsp.SCOPE_ROW),
+    (17, 257, bsp.SCOPE_ROW),
+    (7, 600, bsp.SCOPE_ROW),
+])
+def test_select_within_one_cta(rows, cols, scope):
+    """Distinct float scores, int8 scores with long runs of equal keys, and all keys equal."""
+    seg = rows * cols if scope == bsp.SCOPE_LAYER else cols
+    for dtype in ("bf16", "i8", "equal"):
+        if dtype == "equal":
+            W = np.full((rows * 8, 1, 1, cols * 8), 3, dtype=np.int8)
+        elif dtype == "i8":
+            W = synth.uniform_int(141, (rows * 8, 1, 1, cols * 8), -1, 1).astype(np.int8)
+        else:
+            W = make_case(142, rows * 8, cols * 8, 1, 1, "bf16")
+        want = ref.scores(W, 8, 8)
+        for n_zero in (1, seg // 3, seg // 2, seg - 1):
+            g, _, _, _ = gpu_mask(W, 8, 8, "bf16" if dtype == "bf16" else "i8", n_zero, scope=scope)
+            assert np.array_equal(g, ref.mask(want, n_zero, ref.SCOPE_ROW if scope == bsp.SCOPE_ROW else ref.SCOPE_LAYER)), (dtype, n_zero)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32", "i8"])
 @pytest.mark.parametrize("bo,bi", SHAPES)
 def test_compact_bit_exact(dtype, bo, bi):
