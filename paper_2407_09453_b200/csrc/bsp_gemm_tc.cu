@@ -24,6 +24,7 @@
 // arrival that announces the bytes of both loads) and empty (tcgen05.commit); per accumulator buffer: acc_full (commit)
 // and acc_empty (4 warps).  Every wait is bounded; on expiry BSP_ERR_TIMEOUT is latched, the roles wind down, loads
 // in flight are awaited (bounded) and tensor memory is freed.
+#include <type_traits>
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -46,6 +47,9 @@ struct GtParams {
     int a_bytes;                      // bytes of one activation box
     uint8_t *Y;
     int ey;
+    int small_acc;                    // int8: the sums of products are at most 2^29
+    // kHalo: bytes of the resident weights, pitch and rows of an image's box, position tiles, planes of 32-byte rows and their pitch
+    int w_bytes, halo_w, halo_rows, n_pos, planes, plane_bytes;
     uint32_t m_ntn, m_tx, m_ty;       // floor(2^32 / d) of n_tiles_n, tiles_x, tiles_y (division by multiplication)
     int kbytes, a_stride;             // bytes of K per row of a stage: 128, or 64 for layers with at most 64 bytes of input channels; bytes of the activation part of a stage
 };
@@ -53,12 +57,14 @@ struct GtParams {
 // What follows the ring and the two staging buffers in shared memory.  (All of it is dynamic, so that the ring starts on
 // the 1024-byte boundary that the swizzled tiles need without room for rounding: four 48 KB stages, the staging buffers
 // and this fill the 227 KB of a CTA.)
+constexpr int kGtHaloTaps = 30;
 struct GtTail {
-    uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc_full[2], acc_empty[2];
+    uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc_full[2], acc_empty[2], w_full[kGtHaloTaps];
     uint32_t tmem;
     uint32_t fail;
-    __align__(16) uint32_t bias[2][256];     // per epilogue group: bias and shift of its tile's channels
-    __align__(16) uint8_t shift[2][256];
+    // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
+    __align__(16) uint32_t bias[2][128], half[2][128];
+    __align__(16) uint8_t shift[2][128];
 };
 constexpr int kGtGemmSmem = 227 * 1024;
 static_assert(4 * (kGtABytes + 256 * 128) + 8 * kGtStagingBytes + sizeof(GtTail) <= kGtGemmSmem, "four stages at 256 channels");
@@ -78,12 +84,19 @@ __device__ __forceinline__ uint32_t gt_bias(const GtParams &p, int ch)
     return (p.bias != nullptr && ch < p.O) ? __ldg((const uint32_t *)p.bias + ch) : 0u;
 }
 
-// kWT: operand type; kEy: bytes of an output element (4: float32 or int32, 2: bfloat16, 1: int8).
-template <int kWT, int kEy, bool kPair>
+// kWT: operand type; kEy: bytes of an output element (4: float32 or int32, 2: bfloat16, 1: int8); kMode: how operands are staged.
+// kTaps loads an activation box and a weight tile per K-stage.  kPairs is the same on pairs of CTAs.  kHalo is for stride-1
+// layers with taps whose input channels fit one stage and whose weights fit shared memory: the weights of the CTA's channel
+// tile are loaded once and stay, the activations of a position tile arrive in ONE load with the border that its taps reach,
+// and a tap is a view of that box shifted by whole rows (the swizzle goes by the shared-memory address).  Nine loads of
+// shifted boxes and nine weight tiles per tile had kept such layers at the pace of the TMA unit (about 1.5 cycles per row).
+constexpr int kTaps = 0, kPairs = 1, kHalo = 2;
+template <int kWT, int kEy, int kMode>
 __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_constant__ GtParams p)
 {
+    constexpr bool kPair = kMode == kPairs;
     extern __shared__ __align__(1024) uint8_t smem[];
-    GtTail &tail = *(GtTail *)(smem + (size_t)p.stages * p.stage_bytes + 8 * kGtStagingBytes);
+    GtTail &tail = *(GtTail *)(smem + (kMode == kHalo ? p.w_bytes : 0) + (size_t)p.stages * p.stage_bytes + 8 * kGtStagingBytes);
     uint64_t *s_full = tail.full, *s_empty = tail.empty, *s_acc_full = tail.acc_full, *s_acc_empty = tail.acc_empty;
     volatile uint32_t &s_fail = tail.fail;
 
@@ -92,14 +105,25 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     // 100 cycles of issue and every poll 150, against 48 / 64 / 127 for the MMA itself at 64 / 128 / 256 channels and 90.)
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const int S = p.stages, n_ks = p.n_ks, BN = p.BN;
-    const uint32_t ring = sm32(smem);
+    const uint32_t ring = sm32(smem) + (kMode == kHalo ? (uint32_t)p.w_bytes : 0u);
     const uint32_t staging = ring + (uint32_t)(S * p.stage_bytes);
     // Work items: tiles, or for CTA pairs two position tiles side by side on one channel tile (CTA r of the pair takes
     // position tile 2 mp + r; a pair past an odd count loads zeros and stores nothing).
     uint32_t rank = 0;
     if constexpr (kPair) asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
-    const int t_first = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, t_step = kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-    const int t_count = kPair ? p.n_tile_pairs : p.n_tiles;
+    // kHalo: a CTA keeps one channel tile and walks position tiles.
+    const int ntn = p.n_tiles_n;
+    const int t_first = kMode == kTaps ? (int)blockIdx.x : kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x / ntn;
+    const int t_step = kMode == kTaps ? (int)gridDim.x : kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x / ntn;
+    const int t_count = kMode == kTaps ? p.n_tiles : kPair ? p.n_tile_pairs : p.n_pos;
+    // position tile (of this CTA, in a pair) and channel tile of a work item
+    auto tile_of = [&](int tile, int &mt, int &tn) {
+        if constexpr (kMode == kHalo) { mt = tile; tn = (int)blockIdx.x - t_first * ntn; }
+        else {
+            gt_divmod(tile, ntn, p.m_ntn, mt, tn);
+            if constexpr (kPair) mt = 2 * mt + (int)rank;
+        }
+    };
     // barriers of the pair's leader (CTA 0), as shared::cluster addresses
     uint32_t lead_full0 = sm32(&s_full[0]), lead_acc_empty0 = sm32(&s_acc_empty[0]);
     if constexpr (kPair) {
@@ -116,6 +140,8 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc_full[b])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc_empty[b])), "r"(kPair ? 8 : 4) : "memory");
         }
+        if constexpr (kMode == kHalo)
+            for (int t = 0; t < p.n_ks; ++t) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.w_full[t])), "r"(1) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&p.tmx) : "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&p.tmw) : "memory");
@@ -155,17 +181,41 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             // (a pair: each CTA loads its own activation box and its half of the weight tile, all four loads announce their
             // bytes on the leader's barrier, which the leader arms with the total)
             const uint32_t stage_bytes = (uint32_t)p.stage_bytes;
-            const uint32_t tx = (uint32_t)(p.a_bytes + (BN >> (kPair ? 1 : 0)) * p.kbytes) * (kPair ? 2u : 1u);
-            const int cpt128 = p.cpt * 128, Kw = p.K, ntn = p.n_tiles_n;
+            const uint32_t tx = (uint32_t)(p.a_bytes + (kMode == kHalo ? 0 : BN >> (kPair ? 1 : 0)) * p.kbytes) * (kPair ? 2u : 1u);
+            const int cpt128 = p.cpt * 128, Kw = p.K;
             // (a fresh barrier counts as released: the wait on parity 1 of the first round returns at once)
             uint32_t slot = 0, epar = 1, issued = 0, dst = ring;
             bool ok = true, free_now = true;
             for (int tile = t_first; tile < t_count && ok; tile += t_step) {
                 int mt, tn;
-                gt_divmod(tile, ntn, p.m_ntn, mt, tn);
+                tile_of(tile, mt, tn);
                 const int ch0 = tn * BN + (kPair ? (int)rank * (BN >> 1) : 0);
                 int n0, y0, x0;
-                gt_tile_origin(p, kPair ? 2 * mt + (int)rank : mt, n0, y0, x0);
+                gt_tile_origin(p, mt, n0, y0, x0);
+                if constexpr (kMode == kHalo) {
+                    if (s_fail) { ok = false; break; }
+                    if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; break; }
+                    const bool wrap = slot + 1u == (uint32_t)S;
+                    const uint32_t next_free = gt_test(empty0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? epar ^ 1u : epar);
+                    // (the second plane's load is predicated off where one plane holds all channels, or rows are 128 bytes)
+                    asm volatile("{\n .reg .pred e, e1;\n elect.sync _|e, 0xFFFFFFFF;\n setp.ne.b32 e1, %8, 0;\n and.pred e1, e1, e;\n"
+                                 " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+                                 " @e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6, %7}], [%0];\n"
+                                 " @e1 cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%9], [%3, {%10, %5, %6, %7}], [%0];\n}\n"
+                                 ::"r"(full0 + slot * 8u), "r"(tx), "r"(dst), "l"(&p.tmx), "r"(0), "r"(x0 - p.pw), "r"(y0 - p.ph), "r"(n0),
+                                   "r"(p.planes - 1), "r"(dst + (uint32_t)p.plane_bytes), "r"(32) : "memory");
+                    ++issued;
+                    free_now = __all_sync(0xFFFFFFFFu, next_free != 0u);
+                    if (wrap) { slot = 0; epar ^= 1u; dst = ring; } else { ++slot; dst += stage_bytes; }
+                    if (tile == t_first)
+                        for (int t = 0; t < n_ks; ++t)
+                            asm volatile("{\n .reg .pred e, e1;\n elect.sync _|e, 0xFFFFFFFF;\n setp.ne.b32 e1, %7, 0;\n and.pred e1, e1, e;\n"
+                                         " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+                                         " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6}], [%0];\n"
+                                         " @e1 cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%3, {%9, %5, %6}], [%0];\n}\n"
+                                         ::"r"(sm32(&tail.w_full[t])), "r"((uint32_t)(BN * p.kbytes)), "r"(sm32(smem) + (uint32_t)(t * BN * p.kbytes)), "l"(&p.tmw), "r"(0), "r"(t), "r"(ch0),
+                                           "r"(p.planes - 1), "r"(sm32(smem) + (uint32_t)(t * BN * p.kbytes + BN * 32)), "r"(32) : "memory");
+                } else {
                 // input position of the tile's first output position at tap (0, 0); a tap is a shift of the box, positions
                 // outside the image read as zeros (the padding)
                 const int xi0 = x0 * p.sw - p.pw;
@@ -200,6 +250,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                         if (++kk == Kw) { kk = 0; kx = xi0; ++hy; }
                     }
                 }
+                }
             }
             if (!ok && lane == 0) {
                 // winding down after a wait that ran out: the loads already issued still write into this CTA's shared
@@ -207,11 +258,65 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 atomicExch((uint32_t *)&tail.fail, 1u);
                 // (the follower of a pair has no barrier of its own to watch: its loads announce themselves to the leader;
                 // both CTAs meet at the cluster barrier before they leave)
+                if (kMode == kHalo && issued > 0)
+                    for (int t = 0; t < n_ks; ++t) gt_poll(sm32(&tail.w_full[t]), 0u);
                 for (uint32_t back = 0; back < (uint32_t)S && back < issued && rank == 0; ++back) {
                     const uint32_t it = issued - 1u - back;
                     gt_poll(full0 + (it % (uint32_t)S) * 8u, (it / (uint32_t)S) & 1u);
                 }
             }
+        }
+    } else if (kMode == kHalo && warp == 1) {
+        // ================= MMA issuer of kHalo =================
+        if (run) {
+            const uint32_t dfmt = kWT == BSP_I8 ? 2u : 1u, abfmt = kWT == BSP_F32 ? 2u : 1u;
+            const uint32_t idesc = (dfmt << 4) | (abfmt << 7) | (abfmt << 10) | ((uint32_t)(BN >> 3) << 17) | ((128u >> 4) << 24);
+            const uint32_t full0 = sm32(&s_full[0]), empty0 = sm32(&s_empty[0]);
+            const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4;
+            // One tile's MMAs.  kWide: rows of 128 bytes, else planes of 32-byte rows; kFirst: the CTA's first tile, whose taps
+            // wait for their weights.  (Apart, so that the loop over the taps has no branch but its own: one on kWide inside
+            // it cost 10 %.)
+            auto issue = [&](auto wide_c, auto first_c, uint32_t d, uint32_t a_tap) -> bool {
+                constexpr bool kWide = decltype(wide_c)::value, kFirst = decltype(first_c)::value;
+                const uint32_t row16 = kWide ? 8u : 2u, w_tap16 = (uint32_t)(BN * p.kbytes) >> 4, row_step = (uint32_t)(p.halo_w - p.K) * row16;
+                const uint64_t plane_a = (uint64_t)(p.plane_bytes >> 4), plane_b = (uint64_t)(BN * 32 >> 4);
+                const uint32_t two = (uint32_t)p.planes - 1u;
+                uint64_t da = (kWide ? kGtDesc : kGtDesc32) | (uint64_t)a_tap, db = (kWide ? kGtDesc : kGtDesc32) | (uint64_t)(sm32(smem) >> 4);
+                uint32_t acc = 0u;
+                int t = 0;
+#pragma unroll 1
+                for (int h = 0; h < p.H; ++h, da += row_step)
+#pragma unroll 1
+                    for (int k = 0; k < p.K; ++k, ++t, da += row16, db += w_tap16) {
+                        if constexpr (kFirst) {
+                            if (!__all_sync(0xFFFFFFFFu, gt_poll(sm32(&tail.w_full[t]), 0u))) return false;
+                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        }
+                        if constexpr (kWide) gt_issue_tap<kWT>(d, da, db, idesc, acc);
+                        else gt_issue_planes<kWT>(d, da, db, plane_a, plane_b, two, idesc, acc);
+                        acc = 1u;
+                    }
+                return true;
+            };
+            auto run_tiles = [&](auto wide_c) -> bool {
+                uint32_t slot = 0, par = 0, tile_i = 0;
+                for (int tile = t_first; tile < t_count; tile += t_step, ++tile_i) {
+                    const uint32_t buf = tile_i & 1u, use = tile_i >> 1, d = tmem + buf * 256u;
+                    bool ok = gt_poll(sm32(&s_acc_empty[buf]), (use & 1u) ^ 1u) && gt_poll(full0 + slot * 8u, par) && s_fail == 0u;
+                    if (!__all_sync(0xFFFFFFFFu, ok)) return false;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const uint32_t a_tap = (ring >> 4) + slot * stage16;
+                    if (tile_i == 0) ok = issue(wide_c, std::true_type(), d, a_tap);
+                    else issue(wide_c, std::false_type(), d, a_tap);
+                    if (!ok) return false;
+                    gt_commit_elected<false>(empty0 + slot * 8u);
+                    gt_commit_elected<false>(sm32(&s_acc_full[buf]));
+                    if (++slot == (uint32_t)S) { slot = 0; par ^= 1u; }
+                }
+                return true;
+            };
+            const bool ok = p.kbytes == 128 ? run_tiles(std::true_type()) : run_tiles(std::false_type());
+            if (!ok && lane == 0) atomicExch((uint32_t *)&tail.fail, 1u);
         }
     } else if (warp == 1) {
         // ================= MMA issuer =================
@@ -258,13 +363,37 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             const int q = warp & 3;                              // quarter of the tensor-memory lanes this warp reaches
             const int grp = (warp - 2) >> 2;
             constexpr int cpr = 128 / kEy;                       // output channels per round (128 bytes of a row)
-            // the group's staging buffer: 128 rows of 128 bytes, this warp's 32 rows at its quarter
-            const uint32_t sg = staging + (uint32_t)(grp * 4 * kGtStagingBytes), sb = sg + (uint32_t)(q * kGtStagingBytes);
+            // the group's staging buffer: 128 rows of 128 bytes
+            const uint32_t sg = staging + (uint32_t)(grp * 4 * kGtStagingBytes);
             const bool issuer = q == 0 && lane == 0;             // one thread of the group issues its stores
-            uint32_t *bias = tail.bias[grp];
+            // this lane's row of the staging buffer: the lane's row of the tile, or in kHalo the place of its output in the box
+            int row = q * 32 + lane;
+            if constexpr (kMode == kHalo) {
+                const int per_image = p.halo_rows * p.halo_w, n = row / per_image, y = (row - n * per_image) / p.halo_w, x = row - n * per_image - y * p.halo_w;
+                row = n < p.Nt && y < p.Ht && x < p.Wt ? (n * p.Ht + y) * p.Wt + x : -1;
+            }
+            // Constants of a round's channels: the group's thread c holds channel c of the next round and puts them into shared
+            // memory once the group has read the current ones, so that the trip to memory is never waited for.
+            uint32_t *bias = tail.bias[grp], *half = tail.half[grp];
             uint8_t *shift = tail.shift[grp];
+            const int ct = ((warp - 2) & 3) * 32 + lane;
+            uint32_t next_bias = 0u, next_shift = 1u;
+            int have = -1;                                       // first channel of the round whose constants are in shared memory
+            bool small = false;
+            auto fetch = [&](int ch0) {
+                if (ct >= cpr) return;
+                next_bias = gt_bias(p, ch0 + ct);
+                if constexpr (kEy == 1) next_shift = ch0 + ct < p.O ? (uint32_t)__ldg(p.shift + ch0 + ct) & 31u : 1u;
+            };
+            auto place = [&]() {                                 // (followed by a barrier of the group)
+                if (ct >= cpr) return;
+                bias[ct] = next_bias;
+                if constexpr (kEy == 1) { half[ct] = (1u << next_shift) >> 1; shift[ct] = (uint8_t)next_shift; }
+            };
+            auto is_small = [&]() {
+                return p.small_acc != 0 && next_shift != 0u && next_shift != 31u && (int)next_bias <= (1 << 29) && (int)next_bias >= -(1 << 29);
+            };
             uint32_t tile_i = 0;
-            int have = -1;                                       // first channel of the entries in `bias` and `shift`
             bool ok = true;
             for (int tile = t_first; tile < t_count && ok; tile += t_step, ++tile_i) {
                 const bool last = tile + t_step >= t_count, shared_tile = last && BN > cpr;
@@ -272,27 +401,36 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 const int c_first = shared_tile ? grp * cpr : 0, c_step = shared_tile ? 2 * cpr : cpr;
                 const uint32_t buf = tile_i & 1u, use = tile_i >> 1;
                 int mt, tn;
-                gt_divmod(tile, p.n_tiles_n, p.m_ntn, mt, tn);
+                tile_of(tile, mt, tn);
                 const int n0 = tn * BN;
                 int in0, y0, x0;
-                gt_tile_origin(p, kPair ? 2 * mt + (int)rank : mt, in0, y0, x0);
-                // (the entries of the tile before were last read ahead of the group barrier of its last store; a layer with one
-                // channel tile keeps them: a trip to memory per tile costs where a tile takes about a microsecond)
-                for (int c = ((warp - 2) & 3) * 32 + lane; c < BN && n0 != have; c += 128) {
-                    bias[c] = gt_bias(p, n0 + c);
-                    if constexpr (kEy == 1) shift[c] = n0 + c < p.O ? (uint8_t)((uint32_t)__ldg(p.shift + n0 + c) & 31u) : (uint8_t)0;
+                gt_tile_origin(p, mt, in0, y0, x0);
+                if (have != n0 + c_first) {                      // (the first tile, or an order of rounds that was not foreseen)
+                    fetch(n0 + c_first);
+                    place();
+                    if constexpr (kEy == 1) small = gt_group_all(1 + grp, is_small());
+                    have = n0 + c_first;
                 }
-                have = n0;
                 if (!gt_wait(sm32(&s_acc_full[buf]), use & 1u)) ok = false;
                 if (s_fail) ok = false;
                 ok = gt_group_all(1 + grp, ok);                // the four warps go on or give up as one (they meet at barriers below)
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + buf * 256u;
+                // the channels of the round after the last one of this tile: those of the group's next tile
+                int after = n0 + c_first;
+                if (!last && kMode != kHalo && ntn > 1) {
+                    int m2, t2;
+                    const int next = tile + 2 * t_step < t_count ? tile + 2 * t_step : tile + t_step;
+                    gt_divmod(next, ntn, p.m_ntn, m2, t2);
+                    after = t2 * BN + (next + t_step >= t_count && BN > cpr ? grp * cpr : 0);
+                }
                 for (int c0 = c_first; c0 < BN; c0 += c_step) {
                     uint32_t out[32];                            // 128 bytes of this lane's row of Y
                     const int left = (p.O - n0 < BN ? p.O - n0 : BN) - c0;          // channels from here on
-                    gt_epilogue_round<kWT == BSP_I8, kEy>(tbase + (uint32_t)c0, bias + c0, shift + c0, left, out);
+                    const int next_ch = c0 + c_step < BN ? n0 + c0 + c_step : after;
+                    if (next_ch != have) fetch(next_ch);
+                    gt_epilogue_round<kWT == BSP_I8, kEy>(tbase + (uint32_t)c0, bias, half, shift, small, left, out);
                     if (!last && c0 + c_step >= BN) {
                         // the accumulator buffer has been read: hand it back to the MMA issuer
                         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -308,13 +446,16 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                     // has been read (the loads and the arithmetic of this round ran meanwhile), then the group may write
                     if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
                     gt_group_sync(1 + grp);
-                    const uint32_t srow = sb + (uint32_t)lane * 128u;
+                    if (next_ch != have) place();
+                    const uint32_t srow = sg + (uint32_t)row * 128u;
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
-                                     ::"r"(srow + (uint32_t)((j ^ (lane & 7)) << 4)), "r"(out[4 * j]), "r"(out[4 * j + 1]), "r"(out[4 * j + 2]), "r"(out[4 * j + 3]) : "memory");
+                        if (kMode != kHalo || row >= 0) asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
+                                     ::"r"(srow + (uint32_t)((j ^ (row & 7)) << 4)), "r"(out[4 * j]), "r"(out[4 * j + 1]), "r"(out[4 * j + 2]), "r"(out[4 * j + 3]) : "memory");
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                    gt_group_sync(1 + grp);
+                    if (kEy == 1 && next_ch != have) small = gt_group_all(1 + grp, is_small());
+                    else gt_group_sync(1 + grp);
+                    have = next_ch;
                     // one store of the tile's box: 128 bytes of every row; what lies past the last channel, column, row or image
                     // of Y is clipped (rows of the buffer beyond the box are not part of the store)
                     if (issuer && left > 0) {
@@ -373,25 +514,27 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     p.status = (int *)ws;
     p.O = wd.O; p.I = wd.I; p.H = wd.H; p.K = wd.K; p.bo = wd.bo; p.bi = wd.bi;
     p.wtype = wd.wtype; p.ytype = ytype; p.ey = ey; p.Y = (uint8_t *)Y;
+    p.small_acc = (long long)wd.I * HK * 128 * 128 <= (1 << 29) ? 1 : 0;
     p.N = xd.N; p.sh = xd.stride_h; p.sw = xd.stride_w; p.ph = xd.pad_h; p.pw = xd.pad_w;
     p.M = (xd.L + 2 * xd.pad_h - wd.H) / xd.stride_h + 1;
     p.Nw = (xd.J + 2 * xd.pad_w - wd.K) / xd.stride_w + 1;
     const long long P = (long long)xd.N * p.M * p.Nw;
     p.P = (int)P;
-    const GtTile T = gt_pick_tile(xd.N, p.M, p.Nw, p.sh, p.sw);
+    GtTile T = gt_pick_tile(xd.N, p.M, p.Nw, p.sh, p.sw);
     if (T.tiles <= 0) return BSP_ERR_SHAPE;
-    p.Wt = T.Wt; p.Ht = T.Ht; p.Nt = T.Nt; p.rows_tile = T.Wt * T.Ht * T.Nt;
-    p.tiles_x = (p.Nw + T.Wt - 1) / T.Wt; p.tiles_y = (p.M + T.Ht - 1) / T.Ht;
     // layers with at most 64 bytes of input channels per position stage 64-byte rows (64-byte swizzle, two MMAs a stage)
     p.kbytes = (long long)wd.I * esz <= 64 ? 64 : 128;
-    p.a_stride = kGtBM * p.kbytes;
-    p.a_bytes = p.rows_tile * p.kbytes;
-    // kernels by operand type (in the order of bsp_dtype), width of the output (32 bits or the narrow form) and CTA pairs
+    p.cpt = (int)(((long long)wd.I * esz + 127) / 128);
+    p.n_ks = HK * p.cpt;
+    // kernels by operand type (in the order of bsp_dtype), width of the output (32 bits or the narrow form) and mode
     typedef void (*Kernel)(const GtParams);
-    static const Kernel kernels[3][2][2] = {
-        {{gemm_tc_kernel<BSP_F32, 4, false>, gemm_tc_kernel<BSP_F32, 4, true>}, {gemm_tc_kernel<BSP_F32, 2, false>, gemm_tc_kernel<BSP_F32, 2, true>}},
-        {{gemm_tc_kernel<BSP_BF16, 4, false>, gemm_tc_kernel<BSP_BF16, 4, true>}, {gemm_tc_kernel<BSP_BF16, 2, false>, gemm_tc_kernel<BSP_BF16, 2, true>}},
-        {{gemm_tc_kernel<BSP_I8, 4, false>, gemm_tc_kernel<BSP_I8, 4, true>}, {gemm_tc_kernel<BSP_I8, 1, false>, gemm_tc_kernel<BSP_I8, 1, true>}}};
+    static const Kernel kernels[3][2][3] = {
+        {{gemm_tc_kernel<BSP_F32, 4, kTaps>, gemm_tc_kernel<BSP_F32, 4, kPairs>, gemm_tc_kernel<BSP_F32, 4, kHalo>},
+         {gemm_tc_kernel<BSP_F32, 2, kTaps>, gemm_tc_kernel<BSP_F32, 2, kPairs>, gemm_tc_kernel<BSP_F32, 2, kHalo>}},
+        {{gemm_tc_kernel<BSP_BF16, 4, kTaps>, gemm_tc_kernel<BSP_BF16, 4, kPairs>, gemm_tc_kernel<BSP_BF16, 4, kHalo>},
+         {gemm_tc_kernel<BSP_BF16, 2, kTaps>, gemm_tc_kernel<BSP_BF16, 2, kPairs>, gemm_tc_kernel<BSP_BF16, 2, kHalo>}},
+        {{gemm_tc_kernel<BSP_I8, 4, kTaps>, gemm_tc_kernel<BSP_I8, 4, kPairs>, gemm_tc_kernel<BSP_I8, 4, kHalo>},
+         {gemm_tc_kernel<BSP_I8, 1, kTaps>, gemm_tc_kernel<BSP_I8, 1, kPairs>, gemm_tc_kernel<BSP_I8, 1, kHalo>}}};
     static_assert(BSP_F32 == 0 && BSP_BF16 == 1 && BSP_I8 == 2, "the table is indexed by type");
     const Kernel *kernel = kernels[wd.wtype][ey == 4 ? 0 : 1];
     static bool opted[kGtMaxDevices] = {};
@@ -400,14 +543,26 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     BSP_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
     if (!opted[dev]) {
-        for (int t = 0; t < 12; ++t)
-            BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 4][t / 2 % 2][t % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, kGtGemmSmem));
+        for (int t = 0; t < 18; ++t)
+            BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 6][t / 3 % 2][t % 3], cudaFuncAttributeMaxDynamicSharedMemorySize, kGtGemmSmem));
         BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
         opted[dev] = true;
     }
     // Channels per tile: the widest tile keeps the tensor pipe busiest (a stage costs about 256 + 2 BN cycles of operand
     // fetch from shared memory), but a layer with few position tiles fills more SMs with narrower ones: the width with
-    // the lowest waves x stage cost wins.
+    // the lowest waves x stage cost wins.  kHalo competes where it applies, with cycles per tile for both: a K-stage costs
+    // its MMAs (32 + BN / 4 cycles of operand reads or BN / 2 of arithmetic per 32 bytes of K) or, loaded per tap, 1.5
+    // cycles per row of its two boxes; kHalo pays only the MMAs, on tiles that the border makes a few more.
+    const int staging = 8 * kGtStagingBytes, nk = p.kbytes / 32;
+    const GtTile Th = gt_pick_halo(xd.N, p.M, p.Nw, wd.H, wd.K);
+    const bool halo_ok = HK > 1 && HK <= kGtHaloTaps && p.cpt == 1 && p.sh == 1 && p.sw == 1 && Th.tiles > 0;
+    // (up to 64 bytes of channels lie in planes of 32-byte rows: MMAs on 64-byte rows took 90 cycles instead of 67 at 128
+    // channels and 72 instead of 59 at 64)
+    const int halo_kb = (long long)wd.I * esz <= 32 ? 32 : p.kbytes, planes = halo_kb == 128 ? 1 : halo_kb / 32;
+    const int plane_bytes = halo_ok ? (Th.Nt * (Th.Ht + wd.H - 1) * (Th.Wt + wd.K - 1) * (halo_kb / planes) + 1023) / 1024 * 1024 : 0;
+    const int halo_bytes = planes * plane_bytes;
+    int mode = kTaps, halo_bn = 0;
+    double taps_cycles = -1.0, halo_cycles = -1.0;
     {
         const int step = 64;
         const int widest = (gemm_tile_n(wd.O) + step - 1) / step * step;
@@ -416,30 +571,54 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
             if (bn != widest && bn != 128 && bn != 64) continue;
             // (a round of the int8 output stores 128 channels: a tile that is not a multiple of that must be the only one)
             if (ytype == BSP_I8 && bn % 128 != 0 && bn < wd.O) continue;
-            const long long tiles = T.tiles * ((wd.O + bn - 1) / bn);
-            const long long cost = ((tiles + n_sm[dev] - 1) / n_sm[dev]) * (256 + 2 * bn);
-            if (best_cost < 0 || cost < best_cost) { best_cost = cost; p.BN = bn; }
+            const long long ntn = (wd.O + bn - 1) / bn, tiles = T.tiles * ntn;
+            const long long waves = (tiles + n_sm[dev] - 1) / n_sm[dev], cost = waves * (256 + 2 * bn);
+            const double mma = nk * (bn >= 128 ? (32 + bn / 4 > bn / 2 ? 32 + bn / 4 : bn / 2) : 32 + bn / 4);
+            if (best_cost < 0 || cost < best_cost) {
+                best_cost = cost; p.BN = bn;
+                const double loads = 1.5 * (T.Wt * T.Ht * T.Nt + bn);
+                taps_cycles = waves * (p.n_ks * (mma > loads ? mma : loads) + 400.0);
+            }
+            if (halo_ok && ntn <= n_sm[dev] && HK * bn * halo_kb + 2 * halo_bytes + staging + (int)sizeof(GtTail) <= kGtGemmSmem) {
+                const long long hw = (Th.tiles + n_sm[dev] / ntn - 1) / (n_sm[dev] / ntn);
+                const double c = hw * (HK * mma * halo_kb / p.kbytes + 400.0);
+                if (halo_cycles < 0 || c < halo_cycles) { halo_cycles = c; halo_bn = bn; }
+            }
         }
     }
+    if (halo_cycles >= 0 && halo_cycles < taps_cycles) { mode = kHalo; p.BN = halo_bn; T = Th; }
+    p.Wt = T.Wt; p.Ht = T.Ht; p.Nt = T.Nt; p.rows_tile = T.Wt * T.Ht * T.Nt;
+    p.tiles_x = (p.Nw + T.Wt - 1) / T.Wt; p.tiles_y = (p.M + T.Ht - 1) / T.Ht;
     p.n_tiles_n = (wd.O + p.BN - 1) / p.BN;
     if (T.tiles * p.n_tiles_n > 0x7FFFFFFF - 4096) return BSP_ERR_SHAPE;      // (tile counters step by up to twice the grid)
     p.n_tiles = (int)(T.tiles * p.n_tiles_n);
+    p.n_pos = (int)T.tiles;
     // Large products run on CTA pairs: two position tiles side by side on one 256-channel tile, every CTA loading its
     // own activations and half of the weights (the operand fetch per SM and MMA falls from 12 KB to 8 KB).
     // (Tiles of a few K-stages are bound by their epilogue, and there the pair's cross-CTA hand-shakes only cost.)
-    p.cpt = (int)(((long long)wd.I * esz + 127) / 128);
-    p.n_ks = HK * p.cpt;
-    const bool pair = p.kbytes == 128 && p.BN == 256 && p.n_ks >= 8 && (long long)p.n_tiles >= 4LL * n_sm[dev] && n_sm[dev] >= 2;
+    if (mode == kTaps && p.kbytes == 128 && p.BN == 256 && p.n_ks >= 8 && (long long)p.n_tiles >= 4LL * n_sm[dev] && n_sm[dev] >= 2) mode = kPairs;
+    const bool pair = mode == kPairs;
     p.n_tile_pairs = (int)(((T.tiles + 1) / 2) * p.n_tiles_n);
     p.m_ntn = gt_magic(p.n_tiles_n); p.m_tx = gt_magic(p.tiles_x); p.m_ty = gt_magic(p.tiles_y);
+    p.a_stride = kGtBM * p.kbytes;
+    p.a_bytes = p.rows_tile * p.kbytes;
     p.stage_bytes = p.a_stride + (pair ? p.BN / 2 : p.BN) * p.kbytes;
-    const int staging = 8 * kGtStagingBytes;
-    int stages = (kGtGemmSmem - staging - (int)sizeof(GtTail)) / p.stage_bytes;
+    if (mode == kHalo) {
+        p.kbytes = halo_kb; p.planes = planes; p.plane_bytes = plane_bytes;
+        p.halo_w = T.Wt + wd.K - 1; p.halo_rows = T.Ht + wd.H - 1;
+        p.w_bytes = HK * p.BN * p.kbytes;
+        p.a_bytes = T.Nt * p.halo_rows * p.halo_w * p.kbytes;
+        p.stage_bytes = halo_bytes;
+    }
+    int stages = (kGtGemmSmem - staging - (int)sizeof(GtTail) - p.w_bytes) / p.stage_bytes;
     if (stages > kGtMaxStages) stages = kGtMaxStages;
     if (stages < 2) return BSP_ERR_SHAPE;
     p.stages = stages;
-    const size_t smem = (size_t)stages * p.stage_bytes + staging + sizeof(GtTail);
+    const size_t smem = (size_t)p.w_bytes + (size_t)stages * p.stage_bytes + staging + sizeof(GtTail);
 
+    // bytes of an operand row in shared memory, and its swizzle
+    const int row_bytes = mode == kHalo && p.kbytes < 128 ? 32 : p.kbytes;
+    const CUtensorMapSwizzle swizzle = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
     GtEncodeFn enc = gt_encode();
     if (!enc) return BSP_ERR_CUDA;
     {
@@ -447,20 +626,21 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
         const cuuint64_t gdim[4] = {row, (cuuint64_t)xd.J, (cuuint64_t)xd.L, (cuuint64_t)xd.N};
         const cuuint64_t gstr[3] = {row, row * xd.J, row * xd.J * xd.L};
         // a box spans Wt * s_w x Ht * s_h input positions in steps of the strides: Wt x Ht positions arrive
-        const cuuint32_t box[4] = {(cuuint32_t)p.kbytes, (cuuint32_t)(T.Wt * p.sw), (cuuint32_t)(T.Ht * p.sh), (cuuint32_t)T.Nt};
+        const cuuint32_t box[4] = {(cuuint32_t)row_bytes, (cuuint32_t)(mode == kHalo ? p.halo_w : T.Wt * p.sw),
+                                   (cuuint32_t)(mode == kHalo ? p.halo_rows : T.Ht * p.sh), (cuuint32_t)T.Nt};
         const cuuint32_t estr[4] = {1, (cuuint32_t)p.sw, (cuuint32_t)p.sh, 1};
         if (enc(&p.tmx, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(X), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                p.kbytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return BSP_ERR_CUDA;
     }
     {
         const cuuint64_t row = (cuuint64_t)wd.I * esz;
         const cuuint64_t gdim[3] = {row, (cuuint64_t)HK, (cuuint64_t)wd.O};
         const cuuint64_t gstr[2] = {row, row * HK};
-        const cuuint32_t box[3] = {(cuuint32_t)p.kbytes, 1, (cuuint32_t)(pair ? p.BN / 2 : p.BN)};
+        const cuuint32_t box[3] = {(cuuint32_t)row_bytes, 1, (cuuint32_t)(pair ? p.BN / 2 : p.BN)};
         const cuuint32_t estr[3] = {1, 1, 1};
         if (enc(&p.tmw, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t *>((const uint8_t *)packed + L.off_payload), gdim, gstr, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, p.kbytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return BSP_ERR_CUDA;
     }
@@ -477,11 +657,12 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
 
     if (pair) {
         const int pairs = p.n_tile_pairs < n_sm[dev] / 2 ? p.n_tile_pairs : n_sm[dev] / 2;
-        BSP_CUDA_OK(launch_after_clusters(kernel[1], dim3((unsigned)(2 * pairs)), dim3(kGtThreads), smem, st, 2, 1, p));
+        BSP_CUDA_OK(launch_after_clusters(kernel[kPairs], dim3((unsigned)(2 * pairs)), dim3(kGtThreads), smem, st, 2, 1, p));
         return BSP_OK;
     }
-    const int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
-    BSP_CUDA_OK(launch_after(kernel[0], dim3((unsigned)grid), dim3(kGtThreads), smem, st, p));
+    int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
+    if (mode == kHalo) grid = grid / p.n_tiles_n * p.n_tiles_n;
+    BSP_CUDA_OK(launch_after(kernel[mode], dim3((unsigned)grid), dim3(kGtThreads), smem, st, p));
     return BSP_OK;
 }
 

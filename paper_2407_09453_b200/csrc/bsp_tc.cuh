@@ -62,6 +62,9 @@ constexpr uint64_t kGtDesc = (1ull << 16) | ((uint64_t)(1024u >> 4) << 32) | (1u
 // groups 512 bytes apart, two K-steps of 32 bytes.
 constexpr uint64_t kGtDesc64 = (1ull << 16) | ((uint64_t)(512u >> 4) << 32) | (1ull << 46) | (4ull << 61);
 
+// Rows of 32 bytes under the 32-byte swizzle (one K-step): 8-row groups 256 bytes apart.
+constexpr uint64_t kGtDesc32 = (1ull << 16) | ((uint64_t)(256u >> 4) << 32) | (1ull << 46) | (6ull << 61);
+
 // The four MMAs of one stage (two when the stage holds 64 bytes of K: `nk`) and the commit that releases the stage,
 // issued by one elected lane of a converged warp.  All lanes execute this statement with the same operands; the MMA of
 // the first K-step overwrites the accumulator when `acc` is 0.
@@ -77,6 +80,40 @@ constexpr uint64_t kGtDesc64 = (1ull << 16) | ((uint64_t)(512u >> 4) << 32) | (1
                  " @e3 tcgen05.mma.cta_group::" CG ".kind::" KIND " [%0], a3, b3, %3, t;\n"                                \
                  " @e tcgen05.commit.cta_group::" CG ".mbarrier::arrive::one.shared::cluster" COMMIT_TAIL ";\n}\n"        \
                  ::"r"(d), "l"(da), "l"(db), "r"(idesc), "r"(bar_empty), "r"(acc), "h"((unsigned short)3), "r"(nk) : "memory")
+
+// The MMAs of one tap without a commit (its activations stay in place for the taps to come): four K-steps inside the span of
+// the 128-byte swizzle, or one or two (`two`) in planes of 32-byte rows, `pa` and `pb` 16-byte units apart.
+#define GT_ISSUE_TAP(KIND)                                                                                           \
+    asm volatile("{\n .reg .pred e, p, t;\n .reg .b64 a1, a2, a3, b1, b2, b3;\n"                                     \
+                 " elect.sync _|e, 0xFFFFFFFF;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, %4, %4;\n"                    \
+                 " add.u64 a1, %1, 2;\n add.u64 a2, %1, 4;\n add.u64 a3, %1, 6;\n"                                    \
+                 " add.u64 b1, %2, 2;\n add.u64 b2, %2, 4;\n add.u64 b3, %2, 6;\n"                                    \
+                 " @e tcgen05.mma.cta_group::1.kind::" KIND " [%0], %1, %2, %3, p;\n"                                   \
+                 " @e tcgen05.mma.cta_group::1.kind::" KIND " [%0], a1, b1, %3, t;\n"                                   \
+                 " @e tcgen05.mma.cta_group::1.kind::" KIND " [%0], a2, b2, %3, t;\n"                                   \
+                 " @e tcgen05.mma.cta_group::1.kind::" KIND " [%0], a3, b3, %3, t;\n}\n"                                \
+                 ::"r"(d), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory")
+#define GT_ISSUE_PLANES(KIND)                                                                                        \
+    asm volatile("{\n .reg .pred e, e1, p, t;\n .reg .b64 a1, b1;\n"                                                 \
+                 " elect.sync _|e, 0xFFFFFFFF;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, %4, %4;\n"                    \
+                 " setp.ne.b32 e1, %7, 0;\n and.pred e1, e1, e;\n add.u64 a1, %1, %5;\n add.u64 b1, %2, %6;\n"        \
+                 " @e tcgen05.mma.cta_group::1.kind::" KIND " [%0], %1, %2, %3, p;\n"                                   \
+                 " @e1 tcgen05.mma.cta_group::1.kind::" KIND " [%0], a1, b1, %3, t;\n}\n"                               \
+                 ::"r"(d), "l"(da), "l"(db), "r"(idesc), "r"(acc), "l"(pa), "l"(pb), "r"(two) : "memory")
+template <int kWT>
+__device__ __forceinline__ void gt_issue_tap(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc)
+{
+    if constexpr (kWT == BSP_BF16) GT_ISSUE_TAP("f16");
+    else if constexpr (kWT == BSP_I8) GT_ISSUE_TAP("i8");
+    else GT_ISSUE_TAP("tf32");
+}
+template <int kWT>
+__device__ __forceinline__ void gt_issue_planes(uint32_t d, uint64_t da, uint64_t db, uint64_t pa, uint64_t pb, uint32_t two, uint32_t idesc, uint32_t acc)
+{
+    if constexpr (kWT == BSP_BF16) GT_ISSUE_PLANES("f16");
+    else if constexpr (kWT == BSP_I8) GT_ISSUE_PLANES("i8");
+    else GT_ISSUE_PLANES("tf32");
+}
 
 // kPair: the MMAs span a pair of CTAs (cta_group::2, M = 256: each CTA its own 128 positions and half of the weight
 // tile); the commits then arrive on the barrier at the same shared-memory offset in both CTAs.
@@ -137,6 +174,9 @@ __device__ __forceinline__ int gt_round_shift(int v, uint32_t s)
     const uint32_t r = (mag + ((1u << s) >> 1)) >> s;
     return (int)(v < 0 ? 0u - r : r);
 }
+// The same for 1 <= s <= 30 and |v| <= 2^30, with half = 2^(s - 1): one is taken from negative values, then halves go up.
+// (Integer operations run at half rate, and ten of them per value bound the 8-bit layers with few channels.)
+__device__ __forceinline__ int gt_round_shift_small(int v, uint32_t half, uint32_t s) { return (v + (int)half + (v >> 31)) >> s; }
 // ... and four such values saturated to int8 and packed, the first in the lowest byte (cvt.pack saturates two 32-bit
 // values to bytes, its first source above its second, and shifts the third operand up by 16 bits).
 __device__ __forceinline__ uint32_t gt_pack_s8x4(int v0, int v1, int v2, int v3)
@@ -189,8 +229,10 @@ __device__ __forceinline__ void gt_load32(uint32_t taddr, uint32_t (&v)[32])
 // `shift` are the channels' own entries in shared memory, read four channels at a time by all lanes at once: a shuffle per
 // channel (two for int8) had made the int8 round five times as long.  `n`: channels left; 32-channel pieces past them are
 // neither loaded nor computed (their bytes are clipped by the store).
+// `small`: 1 <= shift <= 30 for all of them and every sum at most 2^30 (gt_round_shift_small holds, `half` has its 2^(s - 1)).
 template <bool kInt, int kEy>
-__device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t *bias, const uint8_t *shift, int n, uint32_t (&out)[32])
+__device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t *bias, const uint32_t *half, const uint8_t *shift, bool small, int n,
+                                                  uint32_t (&out)[32])
 {
     auto bias4 = [&](int c) { return *(const uint4 *)(bias + c); };
     if constexpr (kEy == 4) {
@@ -207,25 +249,24 @@ __device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t
             }
         }
     } else if constexpr (kEy == 2) {                     // rounded to nearest even after the bias
+        uint32_t v[2][32];
+        gt_load32_issue(taddr, v[0]);
+        if (n > 32) gt_load32_issue(taddr + 32u, v[1]);
+        gt_load32_wait(v[0]);
+        gt_load32_wait(v[1]);
 #pragma unroll
-        for (int sub = 0; sub < 2; ++sub) {
-            if (sub * 32 >= n) {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) out[sub * 16 + e] = 0u;
-                continue;
-            }
-            uint32_t v[32];
-            gt_load32(taddr + (uint32_t)(sub * 32), v);
+        for (int sub = 0; sub < 2; ++sub)
 #pragma unroll
             for (int e = 0; e < 32; e += 4) {
                 const uint4 b = bias4(sub * 32 + e);
-                const __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(v[e]) + __uint_as_float(b.x), __uint_as_float(v[e + 1]) + __uint_as_float(b.y));
-                const __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(v[e + 2]) + __uint_as_float(b.z), __uint_as_float(v[e + 3]) + __uint_as_float(b.w));
+                const __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(v[sub][e]) + __uint_as_float(b.x), __uint_as_float(v[sub][e + 1]) + __uint_as_float(b.y));
+                const __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(v[sub][e + 2]) + __uint_as_float(b.z), __uint_as_float(v[sub][e + 3]) + __uint_as_float(b.w));
                 out[sub * 16 + e / 2] = *(const uint32_t *)&h0;
                 out[sub * 16 + e / 2 + 1] = *(const uint32_t *)&h1;
             }
-        }
     } else {                                             // requantised after the bias
+        uint32_t v[2][32];
+        gt_load32_issue(taddr, v[0]);
 #pragma unroll
         for (int sub = 0; sub < 4; ++sub) {
             if (sub * 32 >= n) {
@@ -233,14 +274,27 @@ __device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t
                 for (int e = 0; e < 8; ++e) out[sub * 8 + e] = 0u;
                 continue;
             }
-            uint32_t v[32];
-            gt_load32(taddr + (uint32_t)(sub * 32), v);
+            uint32_t(&cur)[32] = v[sub & 1];
+            gt_load32_wait(cur);
+            if (sub < 3 && (sub + 1) * 32 < n) gt_load32_issue(taddr + (uint32_t)((sub + 1) * 32), v[(sub + 1) & 1]);
+            if (small) {
 #pragma unroll
-            for (int e = 0; e < 32; e += 4) {
-                const uint4 b = bias4(sub * 32 + e);
-                const uint32_t s = *(const uint32_t *)(shift + sub * 32 + e);
-                out[sub * 8 + e / 4] = gt_pack_s8x4(gt_round_shift((int)(v[e] + b.x), s & 31u), gt_round_shift((int)(v[e + 1] + b.y), (s >> 8) & 31u),
-                                                    gt_round_shift((int)(v[e + 2] + b.z), (s >> 16) & 31u), gt_round_shift((int)(v[e + 3] + b.w), s >> 24));
+                for (int e = 0; e < 32; e += 4) {
+                    const uint4 b = bias4(sub * 32 + e), h = *(const uint4 *)(half + sub * 32 + e);
+                    const uint32_t s = *(const uint32_t *)(shift + sub * 32 + e);
+                    out[sub * 8 + e / 4] = gt_pack_s8x4(gt_round_shift_small((int)(cur[e] + b.x), h.x, __byte_perm(s, 0u, 0x4440)),
+                                                        gt_round_shift_small((int)(cur[e + 1] + b.y), h.y, __byte_perm(s, 0u, 0x4441)),
+                                                        gt_round_shift_small((int)(cur[e + 2] + b.z), h.z, __byte_perm(s, 0u, 0x4442)),
+                                                        gt_round_shift_small((int)(cur[e + 3] + b.w), h.w, s >> 24));
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 32; e += 4) {
+                    const uint4 b = bias4(sub * 32 + e);
+                    const uint32_t s = *(const uint32_t *)(shift + sub * 32 + e);
+                    out[sub * 8 + e / 4] = gt_pack_s8x4(gt_round_shift((int)(cur[e] + b.x), s & 31u), gt_round_shift((int)(cur[e + 1] + b.y), (s >> 8) & 31u),
+                                                        gt_round_shift((int)(cur[e + 2] + b.z), (s >> 16) & 31u), gt_round_shift((int)(cur[e + 3] + b.w), s >> 24));
+                }
             }
         }
     }
@@ -300,6 +354,32 @@ GtTile gt_pick_tile(int N, int M, int Nw, int sh, int sw)
         if (best.tiles < 0 || cnt < best.tiles || (cnt == best.tiles && area < best_area)) best = {w, h, b, cnt};
         if (tx == 1) break;
         w = (Nw + tx - 2) / (tx - 1);                 // the narrowest box with one tile less across
+    }
+    return best;
+}
+
+// Position tile of a stride-1 layer whose activations are staged once per tile, with the H - 1 rows and K - 1 columns that its
+// taps reach beyond it: the rows of the MMA are the 128 consecutive positions of that box from the tap's own offset on, so
+// output (n, y, x) sits in row (n (Ht + H - 1) + y) (Wt + K - 1) + x and the rows between are not used.
+GtTile gt_pick_halo(int N, int M, int Nw, int H, int K)
+{
+    GtTile best = {0, 0, 0, -1};
+    long long best_area = 0;
+    for (int w = 1; w <= Nw && w <= kGtBM;) {
+        const int pitch = w + K - 1, tx = (Nw + w - 1) / w;
+        int h = (kGtBM - w) / pitch + 1;
+        if (h > M) h = M;
+        const int ty = (M + h - 1) / h;
+        h = (M + ty - 1) / ty;
+        int b = 1;
+        if (w == Nw && h == M) { b = (kGtBM - ((h - 1) * pitch + w)) / ((h + H - 1) * pitch) + 1; if (b > N) b = N; }
+        const long long cnt = (long long)((N + b - 1) / b) * ty * tx, area = (long long)b * (h + H - 1) * pitch;
+        if (pitch <= 256 && h + H - 1 <= 256 && (best.tiles < 0 || cnt < best.tiles || (cnt == best.tiles && area < best_area))) {
+            best = {w, h, b, cnt};
+            best_area = area;
+        }
+        if (tx == 1) break;
+        w = (Nw + tx - 2) / (tx - 1);
     }
     return best;
 }

@@ -1,0 +1,65 @@
+"""GPU parity of stride-1 layers with taps whose input channels fit one stage: the weights stay in shared memory and a tile's
+activations arrive once, with the border that its taps reach."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import ref
+from paper_2407_09453_b200 import bsp, synth
+from gpu_util import gpu_layer, make_bias, make_case, make_x
+from test_gpu_product import run_conv_case
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,I", [("bf16", 8), ("bf16", 16), ("bf16", 24), ("bf16", 32), ("bf16", 40), ("bf16", 64),
+                                     ("i8", 16), ("i8", 32), ("i8", 48), ("i8", 64), ("i8", 80), ("f32", 8), ("f32", 16), ("f32", 32)])
+def test_input_channels_by_planes_and_rows(dtype, I):
+    """One or two planes of 32-byte rows up to 64 bytes of channels, 128-byte rows above; channel tails inside a row."""
+    run_conv_case(801, 64, I, 3, 3, 8, 8, dtype, (3, 19, 21, I), (1, 1), (1, 1))
+
+
+@pytest.mark.parametrize("H,K,L,J,N,pad", [
+    (3, 3, 7, 7, 9, (1, 1)),             # several whole images in a tile
+    (3, 3, 5, 200, 2, (1, 1)),           # a row of the image in two tiles
+    (5, 5, 30, 31, 2, (2, 2)),
+    (1, 7, 17, 17, 3, (0, 3)),
+    (7, 1, 17, 17, 3, (3, 0)),
+    (2, 3, 12, 140, 1, (0, 0)),          # no padding, even taps
+    (3, 3, 1, 1, 130, (1, 1)),           # one position an image
+    (3, 3, 40, 40, 20, (2, 2)),          # more tiles than SMs, an output larger than the input
+])
+@pytest.mark.parametrize("dtype,out", [("bf16", "bf16"), ("i8", "i32")])
+def test_taps_and_images(H, K, L, J, N, pad, dtype, out):
+    run_conv_case(811, 64, 32, H, K, 8, 8, dtype, (N, L, J, 32), (1, 1), pad, out=out if dtype == "bf16" else "f32")
+
+
+@pytest.mark.parametrize("dtype,O", [("bf16", 48), ("bf16", 200), ("i8", 136), ("f32", 72)])
+def test_channel_tiles(dtype, O):
+    """A CTA keeps one channel tile: ragged last tiles, more position tiles than CTAs."""
+    run_conv_case(821, O, 32, 3, 3, 8, 8, dtype, (8, 40, 40, 32), (1, 1), (1, 1))
+
+
+@pytest.mark.parametrize("O", [64, 128])
+@pytest.mark.parametrize("case", ["plain", "shift 0", "shift 31", "bias"])
+def test_requantised_output(O, case):
+    """The short form of the rounding shift, and the cases that must leave it: a shift of 0 or 31, a bias near the rails."""
+    W = make_case(831, O, 64, 3, 3, "i8")
+    gamma = synth.random_gamma(832, O // 8, 8, O // 2)
+    X = make_x(833, (3, 33, 29, 64), "i8")
+    b = make_bias(834, O, "i8")
+    s = synth.uniform_int(835, (O,), 1, 14).astype(np.int32)
+    if case == "shift 0":
+        s[::7] = 0
+    elif case == "shift 31":
+        s[::5] = 31
+    elif case == "bias":
+        b[::3], b[1::3] = (1 << 31) - 1 - (1 << 24), -(1 << 31) + (1 << 24)
+        s[::2] = 25
+    lay = gpu_layer(W, gamma, 8, 8, "i8")
+    Y = torch.full((3, 33, 29, O), -7, dtype=torch.int8, device="cuda")
+    lay.conv2d_q8(torch.from_numpy(X).cuda(), torch.from_numpy(b).cuda(), torch.from_numpy(s).cuda(), Y, (1, 1), (1, 1))
+    lay.check()
+    rp, ci, pl = ref.compact(W, gamma, 8, 8)
+    acc = ref.conv2d(W.shape, 8, 8, rp, ci, pl, X, b, (1, 1), (1, 1))
+    assert np.array_equal(Y.cpu().numpy().reshape(-1, O), ref.requant_i8(acc, s))
