@@ -252,6 +252,10 @@ __device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t
         uint32_t v[2][32];
         gt_load32_issue(taddr, v[0]);
         if (n > 32) gt_load32_issue(taddr + 32u, v[1]);
+        else {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[1][e] = 0u;       // (channels past the last one come out as zeros)
+        }
         gt_load32_wait(v[0]);
         gt_load32_wait(v[1]);
 #pragma unroll
@@ -266,7 +270,7 @@ __device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t
             }
     } else {                                             // requantised after the bias
         uint32_t v[2][32];
-        gt_load32_issue(taddr, v[0]);
+        if (n > 0) gt_load32_issue(taddr, v[0]);             // (every load issued is waited for below)
 #pragma unroll
         for (int sub = 0; sub < 4; ++sub) {
             if (sub * 32 >= n) {

@@ -55,7 +55,7 @@ def test_gemm_q8_block_shapes_ragged(bo, bi):
     run_q8(801, 192, 256, 1, 1, (333, 256), None, None, bo, bi, gemm=True)
 
 
-@pytest.mark.parametrize("O,P", [(1008, 77), (48, 300), (16, 5), (320, 129)])
+@pytest.mark.parametrize("O,P", [(1008, 77), (48, 300), (16, 5), (320, 129), (640, 20000)])
 def test_gemm_q8_channel_tiles_off_the_grid(O, P):
     """128-channel staging rounds against channel counts that end inside one (O a multiple of 16)."""
     run_q8(811, O, 96, 1, 1, (P, 96), None, None, gemm=True)
