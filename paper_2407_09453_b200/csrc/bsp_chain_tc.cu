@@ -14,9 +14,12 @@
 //   3. the second layer: for every tile of 128 output channels, MMAs of that tensor against weight chunks that arrive
 //      through the same ring of stages, into one of two 128-column accumulators;
 //   4. its epilogue: + b2 -> convert -> global memory, overlapping the MMAs of the next 128 channels.
-// Warps: 0 producer, 1 MMA issuer (both converged, one elected lane issues), 2-9 epilogue in two groups of four: the
-// groups share the first epilogue (alternate 64-channel chunks) and each drains one of the two second accumulators.
-// Every wait is bounded.
+// Where layer one has stride 1 and taps, its input channels fit one stage and shared memory allows (kHalo), its weights stay
+// in shared memory and a tile's activations arrive once with the border that the taps reach, as in the product kernel; the
+// weights of layer two then have a ring of their own, or stay too.
+// Warps: 0 producer, 1 MMA issuer (both converged, one elected lane issues), 2-9 epilogue in two groups of four, which take
+// turns with the rounds of both epilogues: 128 bytes of T's or Y's channels each.  Every wait is bounded.
+#include <type_traits>
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -27,25 +30,41 @@ constexpr int kCtBN2 = 128;                        // channels of layer two per 
 constexpr int kCtChunk = kGtBM * 128;              // bytes of one chunk (128 bytes of channels) of the tensor between the layers
 
 struct CtParams {
-    CUtensorMap tmx;          // X as bytes: (I1 * 2, J, L, N), box 128 bytes x Wt x Ht x Nt positions
-    CUtensorMap tmw1;         // Gamma1 (.) W1 as bytes: (I1 * 2, H K, O1), box 128 bytes x 1 tap x O1p channels
-    CUtensorMap tmw2;         // Gamma2 (.) W2 as bytes: (O1 * 2, 1, O2), box 128 bytes x 1 x 128 channels
+    CUtensorMap tmx;          // X as bytes: (I1 * esz, J, L, N), box of one operand row x the tile's positions (kHalo: with their border)
+    CUtensorMap tmw1;         // Gamma1 (.) W1 as bytes: (I1 * esz, H K, O1), box of one operand row x 1 tap x O1p channels
+    CUtensorMap tmw2;         // Gamma2 (.) W2 as bytes: (O1 * esz, 1, O2), box 128 bytes x 1 x 128 channels
     CUtensorMap tmy;          // Y as bytes: (O2 * ey, N_w, M, N), box 128 bytes x Wt x Ht x Nt positions (a tile)
     const void *bias1, *bias2;        // float32, or int32 for the 8-bit chain
     const int32_t *shift1, *shift2;   // 8-bit chain: rounding shifts of T (required) and of an int8 Y
     const uint8_t *packed1, *packed2;
     int *status;
-    int O1, I1, H, K, bo1, bi1, O2, bo2, bi2, relu, wtype, ytype, ey;
+    int O1, I1, H, K, bo1, bi1, O2, bo2, bi2, relu, wtype;
     int O1p;                  // O1 rounded up to a whole chunk of T (64 or 128 channels): columns of accumulator one
     int tcc;                  // channels per chunk of T: 64 (bfloat16) or 128 (int8)
     int n_ks1, cpt1, n_c2, n_t2;      // K-stages of layer one, its channel chunks per tap; chunks of T; channel tiles of layer two
     int stages, stage_bytes, n_tiles;
-    int db;                   // O1p <= 128: accumulator one and the tensor between the layers are double-buffered
-    int N, M, Nw, Wt, Ht, Nt, tiles_x, tiles_y, rows_tile, P;
+    int ahead;                // the first epilogue runs one tile ahead of the second
+    int db, dbt;              // O1p <= 128: accumulator one is double-buffered, and without kHalo the tensor between the layers too
+    int N, M, Nw, Wt, Ht, Nt, tiles_x, tiles_y;
     int sh, sw, ph, pw, a_bytes;
     uint32_t m_tx, m_ty;
-    uint8_t *Y;
+    uint32_t off_ring, off_w2, off_t, off_staging, off_tail;         // bytes into shared memory
+    // kHalo: bytes of K per position, planes and their pitch, pitch and rows of an image's box; slots of layer two's weights
+    int kbytes, planes, plane_bytes, halo_w, halo_rows, w2_slots, w2_stay;
+    int small1, small2;       // 8-bit: sums of products of either layer at most 2^29
 };
+
+// Barriers and constants, after everything else in shared memory (all of it dynamic: the base is 1024-byte aligned).
+constexpr int kCtTaps = 30, kCtW2Slots = 8;
+struct CtTail {
+    uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc1_full[2], acc1_empty[2], t_full[2], t_empty[2], acc2_full[2], acc2_empty[2];
+    uint64_t w1_full[kCtTaps], w2_full[kCtW2Slots], w2_empty[kCtW2Slots];
+    uint32_t tmem, fail;
+    // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
+    __align__(16) uint32_t bias[2][128], half[2][128];
+    __align__(16) uint8_t shift[2][128];
+};
+constexpr int kCtSmem = 227 * 1024;
 
 __device__ __forceinline__ void ct_tile_origin(const CtParams &p, int mt, int &n0, int &y0, int &x0)
 {
@@ -62,41 +81,44 @@ __device__ __forceinline__ bool ct_header_ok(const uint8_t *packed, int wtype, i
            h->bi == bi && (h->forms & kFormDense) != 0;
 }
 
-// kI8: the 8-bit chain (compiled apart, so that neither form carries the other's epilogue code and registers).
-template <bool kI8>
+// kI8: the 8-bit chain; kEy: bytes of an element of Y (compiled apart, so that no form carries another's epilogue code).
+template <bool kI8, int kEy, bool kHalo>
 __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_constant__ CtParams p)
 {
     constexpr int kWt = kI8 ? BSP_I8 : BSP_BF16;
-    extern __shared__ __align__(16) uint8_t ct_smem_raw[];
-    uint8_t *smem = ct_smem_raw + ((1024u - (sm32(ct_smem_raw) & 1023u)) & 1023u);
-    __shared__ __align__(8) uint64_t s_full[kGtMaxStages], s_empty[kGtMaxStages];
-    __shared__ __align__(8) uint64_t s_acc1_full[2], s_acc1_empty[2], s_t_full[2], s_t_empty[2], s_acc2_full[2], s_acc2_empty[2];
-    __shared__ uint32_t s_tmem;
-    __shared__ volatile uint32_t s_fail;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    CtTail &tail = *(CtTail *)(smem + p.off_tail);
+    volatile uint32_t &s_fail = tail.fail;
 
     // (warp number, tensor-memory base and go-ahead through a shuffle: uniform to the compiler, as in the product kernel)
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const int S = p.stages;
-    const uint32_t ring = sm32(smem);
-    const uint32_t tbuf = ring + (uint32_t)(S * p.stage_bytes);          // the tensor between the layers: n_c2 chunks
+    const uint32_t base = sm32(smem), ring = base + p.off_ring;
+    const uint32_t tbuf = base + p.off_t;                                // the tensor between the layers: n_c2 chunks
     const uint32_t tbytes = (uint32_t)(p.n_c2 * kCtChunk);
-    const uint32_t staging = tbuf + (p.db ? 2u : 1u) * tbytes;
+    const uint32_t staging = base + p.off_staging;
     const int t_first = (int)blockIdx.x, t_step = (int)gridDim.x, t_count = p.n_tiles;
+    constexpr int cpr = 128 / kEy, kRpt = kCtBN2 / cpr;                  // channels of a round of Y, rounds per 128-channel tile
 
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_full[s])), "r"(1) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_empty[s])), "r"(1) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.full[s])), "r"(1) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.empty[s])), "r"(1) : "memory");
         }
         for (int b = 0; b < 2; ++b) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc1_full[b])), "r"(1) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc1_empty[b])), "r"(8) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_t_full[b])), "r"(8) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_t_empty[b])), "r"(1) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.acc1_full[b])), "r"(1) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.acc1_empty[b])), "r"(4 * p.n_c2) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.t_full[b])), "r"(4 * p.n_c2) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.t_empty[b])), "r"(1) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.acc2_full[b])), "r"(1) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.acc2_empty[b])), "r"(4 * kRpt) : "memory");
         }
-        for (int b = 0; b < 2; ++b) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc2_full[b])), "r"(1) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc2_empty[b])), "r"(4) : "memory");
+        if constexpr (kHalo) {
+            for (int t = 0; t < p.n_ks1; ++t) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.w1_full[t])), "r"(1) : "memory");
+            for (int t = 0; t < p.w2_slots; ++t) {
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.w2_full[t])), "r"(1) : "memory");
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.w2_empty[t])), "r"(1) : "memory");
+            }
         }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&p.tmx) : "memory");
@@ -105,88 +127,137 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&p.tmy) : "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(kGtTmemCols) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&tail.tmem)), "r"(kGtTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     wait_for_previous();
     if (tid == 0) {
         const bool ok = ct_header_ok(p.packed1, p.wtype, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1) && ct_header_ok(p.packed2, p.wtype, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
-        s_fail = ok ? 0u : 2u;
+        const bool placed = (base & 1023u) == 0u;
+        s_fail = ok && placed ? 0u : 2u;
         if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
+        else if (!placed) atomicMax(p.status, (int)BSP_ERR_CUDA);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, s_tmem, 0);
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tail.tmem, 0);
     const bool run = __shfl_sync(0xFFFFFFFFu, s_fail, 0) == 0u;
-    const uint32_t full0 = sm32(&s_full[0]), empty0 = sm32(&s_empty[0]);
+    const uint32_t full0 = sm32(&tail.full[0]), empty0 = sm32(&tail.empty[0]);
 
     if (warp == 0) {
         // ================= producer =================
         if (run) {
             const uint32_t stage_bytes = (uint32_t)p.stage_bytes;
-            const uint32_t tx1 = (uint32_t)(p.a_bytes + p.O1p * 128), tx2 = (uint32_t)(kCtBN2 * 128);
+            const uint32_t tx1 = (uint32_t)(p.a_bytes + (kHalo ? 0 : p.O1p * 128)), tx2 = (uint32_t)(kCtBN2 * 128);
             const int cpt128 = p.cpt1 * 128, Kw = p.K;
             uint32_t slot = 0, epar = 1, issued = 0, dst = ring;      // (a fresh barrier counts as released)
+            uint32_t slot2 = 0, epar2 = 1, issued2 = 0;
             bool ok = true, free_now = true;
-            // layer one of a tile: the activation box shifted by the tap and that tap's weights, per 128-byte chunk of channels
+            // layer one of a tile: per 128-byte chunk of channels of a tap, the activation box shifted by the tap and the tap's
+            // weights; kHalo: one box (of each plane), and with the first tile the weights of all taps
             auto load_layer_one = [&](int tile) {
                 int n0, y0, x0;
                 ct_tile_origin(p, tile, n0, y0, x0);
                 const int xi0 = x0 * p.sw - p.pw;
-                int c128 = 0, kx = xi0, hy = y0 * p.sh - p.ph, tap = 0, kk = 0;
-                for (int ks = 0; ks < p.n_ks1; ++ks) {
+                if constexpr (kHalo) {
                     if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; return; }
                     const bool wrap = slot + 1u == (uint32_t)S;
                     const uint32_t next_free = gt_test(empty0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? epar ^ 1u : epar);
-                    asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xFFFFFFFF;\n"
+                    asm volatile("{\n .reg .pred e, e1;\n elect.sync _|e, 0xFFFFFFFF;\n setp.ne.b32 e1, %8, 0;\n and.pred e1, e1, e;\n"
                                  " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
                                  " @e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6, %7}], [%0];\n"
-                                 " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%4, %10, %11}], [%0];\n}\n"
-                                 ::"r"(full0 + slot * 8u), "r"(tx1), "r"(dst), "l"(&p.tmx), "r"(c128), "r"(kx), "r"(hy), "r"(n0),
-                                   "r"(dst + (uint32_t)kGtABytes), "l"(&p.tmw1), "r"(tap), "r"(0) : "memory");
+                                 " @e1 cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%9], [%3, {%10, %5, %6, %7}], [%0];\n}\n"
+                                 ::"r"(full0 + slot * 8u), "r"(tx1), "r"(dst), "l"(&p.tmx), "r"(0), "r"(xi0), "r"(y0 * p.sh - p.ph), "r"(n0),
+                                   "r"(p.planes - 1), "r"(dst + (uint32_t)p.plane_bytes), "r"(32) : "memory");
                     ++issued;
                     free_now = __all_sync(0xFFFFFFFFu, next_free != 0u);
                     if (wrap) { slot = 0; epar ^= 1u; dst = ring; } else { ++slot; dst += stage_bytes; }
-                    c128 += 128;
-                    if (c128 == cpt128) {
-                        c128 = 0; ++tap; ++kx;
-                        if (++kk == Kw) { kk = 0; kx = xi0; ++hy; }
-                    }
-                }
-            };
-            // layer two: for every tile of 128 output channels, the weight chunk of each 64 channels of T
-            auto load_layer_two = [&]() {
-                for (int t2 = 0; t2 < p.n_t2; ++t2)
-                    for (int c2 = 0; c2 < p.n_c2; ++c2) {
+                    if (tile == t_first)
+                        for (int t = 0; t < p.n_ks1; ++t) {
+                            const uint32_t w = base + (uint32_t)(t * p.O1p * p.kbytes);
+                            asm volatile("{\n .reg .pred e, e1;\n elect.sync _|e, 0xFFFFFFFF;\n setp.ne.b32 e1, %7, 0;\n and.pred e1, e1, e;\n"
+                                         " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+                                         " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6}], [%0];\n"
+                                         " @e1 cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%3, {%9, %5, %6}], [%0];\n}\n"
+                                         ::"r"(sm32(&tail.w1_full[t])), "r"((uint32_t)(p.O1p * p.kbytes)), "r"(w), "l"(&p.tmw1), "r"(0), "r"(t), "r"(0),
+                                           "r"(p.planes - 1), "r"(w + (uint32_t)(p.O1p * 32)), "r"(32) : "memory");
+                        }
+                } else {
+                    int c128 = 0, kx = xi0, hy = y0 * p.sh - p.ph, tap = 0, kk = 0;
+                    for (int ks = 0; ks < p.n_ks1; ++ks) {
                         if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; return; }
                         const bool wrap = slot + 1u == (uint32_t)S;
                         const uint32_t next_free = gt_test(empty0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? epar ^ 1u : epar);
                         asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xFFFFFFFF;\n"
                                      " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
-                                     " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6}], [%0];\n}\n"
-                                     ::"r"(full0 + slot * 8u), "r"(tx2), "r"(dst), "l"(&p.tmw2), "r"(c2 * 128), "r"(0), "r"(t2 * kCtBN2) : "memory");
+                                     " @e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6, %7}], [%0];\n"
+                                     " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%4, %10, %11}], [%0];\n}\n"
+                                     ::"r"(full0 + slot * 8u), "r"(tx1), "r"(dst), "l"(&p.tmx), "r"(c128), "r"(kx), "r"(hy), "r"(n0),
+                                       "r"(dst + (uint32_t)kGtABytes), "l"(&p.tmw1), "r"(tap), "r"(0) : "memory");
                         ++issued;
                         free_now = __all_sync(0xFFFFFFFFu, next_free != 0u);
                         if (wrap) { slot = 0; epar ^= 1u; dst = ring; } else { ++slot; dst += stage_bytes; }
+                        c128 += 128;
+                        if (c128 == cpt128) {
+                            c128 = 0; ++tap; ++kx;
+                            if (++kk == Kw) { kk = 0; kx = xi0; ++hy; }
+                        }
+                    }
+                }
+            };
+            // layer two: for every tile of 128 output channels, the weight chunk of each 128 bytes of T's channels
+            auto load_layer_two = [&](int tile) {
+                if (kHalo && p.w2_stay && tile != t_first) return;
+                for (int t2 = 0; t2 < p.n_t2; ++t2)
+                    for (int c2 = 0; c2 < p.n_c2; ++c2) {
+                        uint32_t bar, to;
+                        if constexpr (kHalo) {
+                            if (!__all_sync(0xFFFFFFFFu, gt_poll(sm32(&tail.w2_empty[slot2]), epar2))) { ok = false; return; }
+                            bar = sm32(&tail.w2_full[slot2]);
+                            to = base + p.off_w2 + slot2 * tx2;
+                            ++issued2;
+                            if (++slot2 == (uint32_t)p.w2_slots) { slot2 = 0; epar2 ^= 1u; }
+                        } else {
+                            if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; return; }
+                            const bool wrap = slot + 1u == (uint32_t)S;
+                            const uint32_t next_free = gt_test(empty0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? epar ^ 1u : epar);
+                            bar = full0 + slot * 8u;
+                            to = dst;
+                            ++issued;
+                            free_now = __all_sync(0xFFFFFFFFu, next_free != 0u);
+                            if (wrap) { slot = 0; epar ^= 1u; dst = ring; } else { ++slot; dst += stage_bytes; }
+                        }
+                        asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xFFFFFFFF;\n"
+                                     " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+                                     " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6}], [%0];\n}\n"
+                                     ::"r"(bar), "r"(tx2), "r"(to), "l"(&p.tmw2), "r"(c2 * 128), "r"(0), "r"(t2 * kCtBN2) : "memory");
                     }
             };
-            // the stages follow the order in which the MMA warp consumes them: with double buffers, layer one of the next
+            // the loads follow the order in which the MMA warp consumes them: with double buffers, layer one of the next
             // tile goes before layer two of this one
             if (p.db && t_first < t_count) load_layer_one(t_first);
             for (int tile = t_first; tile < t_count && ok; tile += t_step) {
                 if (s_fail) { ok = false; break; }
                 if (p.db) { if (tile + t_step < t_count) load_layer_one(tile + t_step); }
                 else load_layer_one(tile);
-                if (ok) load_layer_two();
+                if (ok) load_layer_two(tile);
             }
             if (!ok && lane == 0) {
                 // winding down after a wait that ran out: the loads already issued still write into this CTA's shared
                 // memory, so the barriers of the stages in flight are awaited (bounded) before the CTA may leave
-                atomicExch((uint32_t *)&s_fail, 1u);
+                atomicExch((uint32_t *)&tail.fail, 1u);
                 for (uint32_t back = 0; back < (uint32_t)S && back < issued; ++back) {
                     const uint32_t it = issued - 1u - back;
                     gt_poll(full0 + (it % (uint32_t)S) * 8u, (it / (uint32_t)S) & 1u);
+                }
+                if constexpr (kHalo) {
+                    if (issued > 0)
+                        for (int t = 0; t < p.n_ks1; ++t) gt_poll(sm32(&tail.w1_full[t]), 0u);
+                    for (uint32_t back = 0; back < (uint32_t)p.w2_slots && back < issued2; ++back) {
+                        const uint32_t it = issued2 - 1u - back;
+                        gt_poll(sm32(&tail.w2_full[it % (uint32_t)p.w2_slots]), (it / (uint32_t)p.w2_slots) & 1u);
+                    }
                 }
             }
         }
@@ -198,58 +269,100 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
             const uint32_t idesc1 = (dfmt << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.O1p >> 3) << 17) | ((128u >> 4) << 24);
             const uint32_t idesc2 = (dfmt << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kCtBN2 >> 3) << 17) | ((128u >> 4) << 24);
             const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4;
-            uint32_t slot = 0, par = 0, a16 = ring >> 4, tile_i = 0, u2 = 0;
+            uint32_t slot = 0, par = 0, a16 = ring >> 4, tile_i = 0, u2 = 0, slot2 = 0, par2 = 0;
             bool ok = true, full_now = false;
+            // the taps of a kHalo tile (see the product kernel)
+            auto taps = [&](auto wide_c, auto first_c, uint32_t d) -> bool {
+                constexpr bool kWide = decltype(wide_c)::value, kFirst = decltype(first_c)::value;
+                const uint32_t row16 = kWide ? 8u : 2u, w_tap16 = (uint32_t)(p.O1p * p.kbytes) >> 4, row_step = (uint32_t)(p.halo_w - p.K) * row16;
+                const uint64_t plane_a = (uint64_t)(p.plane_bytes >> 4), plane_b = (uint64_t)(p.O1p * 32 >> 4);
+                const uint32_t two = (uint32_t)p.planes - 1u;
+                uint64_t da = (kWide ? kGtDesc : kGtDesc32) | (uint64_t)a16, db = (kWide ? kGtDesc : kGtDesc32) | (uint64_t)(base >> 4);
+                uint32_t acc = 0u;
+                int t = 0;
+#pragma unroll 1
+                for (int h = 0; h < p.H; ++h, da += row_step)
+#pragma unroll 1
+                    for (int k = 0; k < p.K; ++k, ++t, da += row16, db += w_tap16) {
+                        if constexpr (kFirst) {
+                            if (!__all_sync(0xFFFFFFFFu, gt_poll(sm32(&tail.w1_full[t]), 0u))) return false;
+                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        }
+                        if constexpr (kWide) gt_issue_tap<kWt>(d, da, db, idesc1, acc);
+                        else gt_issue_planes<kWt>(d, da, db, plane_a, plane_b, two, idesc1, acc);
+                        acc = 1u;
+                    }
+                return true;
+            };
             // layer one of the CTA's i-th tile into accumulator one (buffer b, used for the u-th time)
             auto layer_one = [&](uint32_t i) {
                 const uint32_t b = p.db ? (i & 1u) : 0u, u = p.db ? (i >> 1) : i;
                 // the buffer is free once the first epilogue of its previous tile has read it
-                if (!gt_poll(sm32(&s_acc1_empty[b]), (u & 1u) ^ 1u) || s_fail != 0u) ok = false;
+                if (!gt_poll(sm32(&tail.acc1_empty[b]), (u & 1u) ^ 1u) || s_fail != 0u) ok = false;
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) return;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t d = tmem + b * 128u;
-                for (int ks = 0; ks < p.n_ks1; ++ks) {
-                    if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
-                    const bool wrap = slot + 1u == (uint32_t)S;
-                    const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
+                if constexpr (kHalo) {
+                    if (!__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint64_t da = kGtDesc | (uint64_t)(a16 & 0x3FFFu), db = kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu);
-                    gt_issue_stage<kWt, false>(d, da, db, idesc1, empty0 + slot * 8u, ks != 0 ? 1u : 0u);
-                    full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
-                    if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
+                    if (p.kbytes == 128) { if (i == 0u) ok = taps(std::true_type(), std::true_type(), d); else taps(std::true_type(), std::false_type(), d); }
+                    else { if (i == 0u) ok = taps(std::false_type(), std::true_type(), d); else taps(std::false_type(), std::false_type(), d); }
+                    if (!ok) return;
+                    gt_commit_elected<false>(empty0 + slot * 8u);
+                    if (++slot == (uint32_t)S) { slot = 0; par ^= 1u; a16 = ring >> 4; } else a16 += stage16;
+                } else {
+                    for (int ks = 0; ks < p.n_ks1; ++ks) {
+                        if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
+                        const bool wrap = slot + 1u == (uint32_t)S;
+                        const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        const uint64_t da = kGtDesc | (uint64_t)(a16 & 0x3FFFu), db = kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu);
+                        gt_issue_stage<kWt, false>(d, da, db, idesc1, empty0 + slot * 8u, ks != 0 ? 1u : 0u);
+                        full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+                        if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
+                    }
                 }
-                gt_commit_elected<false>(sm32(&s_acc1_full[b]));
+                gt_commit_elected<false>(sm32(&tail.acc1_full[b]));
             };
             // layer two of the i-th tile: the tensor between the layers is in shared memory once the first epilogue has written it
             auto layer_two = [&](uint32_t i) {
-                const uint32_t b = p.db ? (i & 1u) : 0u, u = p.db ? (i >> 1) : i;
-                if (!gt_poll(sm32(&s_t_full[b]), u & 1u)) ok = false;
+                const uint32_t b = p.dbt ? (i & 1u) : 0u, u = p.dbt ? (i >> 1) : i;
+                if (!gt_poll(sm32(&tail.t_full[b]), u & 1u)) ok = false;
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) return;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                if (kHalo && p.w2_stay) { slot2 = 0; par2 = 0; }
                 for (int t2 = 0; t2 < p.n_t2 && ok; ++t2, ++u2) {
                     const uint32_t buf = u2 & 1u, use = u2 >> 1;
-                    if (!gt_poll(sm32(&s_acc2_empty[buf]), (use & 1u) ^ 1u)) ok = false;
+                    if (!gt_poll(sm32(&tail.acc2_empty[buf]), (use & 1u) ^ 1u)) ok = false;
                     ok = __all_sync(0xFFFFFFFFu, ok);
                     if (!ok) return;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint32_t d = tmem + 256u + buf * (uint32_t)kCtBN2;
                     for (int c2 = 0; c2 < p.n_c2; ++c2) {
-                        if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
-                        const bool wrap = slot + 1u == (uint32_t)S;
-                        const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
-                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                         const uint64_t da = kGtDesc | (uint64_t)(((tbuf + b * tbytes + (uint32_t)(c2 * kCtChunk)) >> 4) & 0x3FFFu);
-                        const uint64_t db = kGtDesc | (uint64_t)(a16 & 0x3FFFu);
-                        gt_issue_stage<kWt, false>(d, da, db, idesc2, empty0 + slot * 8u, c2 != 0 ? 1u : 0u);
-                        full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
-                        if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
+                        if constexpr (kHalo) {
+                            if (!__all_sync(0xFFFFFFFFu, gt_poll(sm32(&tail.w2_full[slot2]), par2))) { ok = false; return; }
+                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                            const uint64_t db = kGtDesc | (uint64_t)((base + p.off_w2 + slot2 * (uint32_t)(kCtBN2 * 128)) >> 4);
+                            // (weights that stay are never handed back: the arrivals on their barriers go unread)
+                            gt_issue_stage<kWt, false>(d, da, db, idesc2, sm32(&tail.w2_empty[slot2]), c2 != 0 ? 1u : 0u);
+                            if (++slot2 == (uint32_t)p.w2_slots) { slot2 = 0; par2 ^= 1u; }
+                        } else {
+                            if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
+                            const bool wrap = slot + 1u == (uint32_t)S;
+                            const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
+                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                            gt_issue_stage<kWt, false>(d, da, kGtDesc | (uint64_t)(a16 & 0x3FFFu), idesc2, empty0 + slot * 8u, c2 != 0 ? 1u : 0u);
+                            full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+                            if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
+                        }
                     }
-                    gt_commit_elected<false>(sm32(&s_acc2_full[buf]));
+                    gt_commit_elected<false>(sm32(&tail.acc2_full[buf]));
                 }
                 // all MMAs that read the tensor have been issued: their completion frees its buffer
-                gt_commit_elected<false>(sm32(&s_t_empty[b]));
+                gt_commit_elected<false>(sm32(&tail.t_empty[b]));
             };
             if (p.db && t_first < t_count) layer_one(0u);
             for (int tile = t_first; tile < t_count && ok; tile += t_step, ++tile_i) {
@@ -257,181 +370,145 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
                 else layer_one(tile_i);
                 if (ok) layer_two(tile_i);
             }
-            if (!ok && lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
+            if (!ok && lane == 0) atomicExch((uint32_t *)&tail.fail, 1u);
         }
     } else {
         // ================= epilogues (warps 2-9) =================
+        // The work goes in steps: the n_c2 chunks of T of tile s + ahead, then the 128-byte rounds of Y of tile s; the two groups
+        // take turns with these rounds, across steps too.  With ahead = 1 the MMA warp finds the next T ready when it is
+        // done with this tile (else layer two of a tile waited for both of the previous tile's epilogues).
         if (run) {
             const int q = warp & 3;                              // quarter of the tensor-memory lanes this warp reaches
             const int grp = (warp - 2) >> 2;
-            const int ey = p.ey;
-            const int cpr = 128 / ey;                            // output channels per staging round (128 bytes of a row)
-            // the group's staging buffer: 128 rows of 128 bytes, this warp's 32 rows at its quarter
-            const uint32_t sg = staging + (uint32_t)(grp * 4 * kGtStagingBytes), sb = sg + (uint32_t)(q * kGtStagingBytes);
+            // the group's staging buffer: 128 rows of 128 bytes
+            const uint32_t sg = staging + (uint32_t)(grp * 4 * kGtStagingBytes);
             const bool issuer = q == 0 && lane == 0;             // one thread of the group issues its stores
-            uint32_t tile_i = 0, u2 = 0;
-            bool ok = true;
             const int r = q * 32 + lane;                         // this lane's row of a tile
-            const uint32_t trow = tbuf + (uint32_t)r * 128u;     // this lane's row of a chunk of T (first buffer)
-            for (int tile = t_first; tile < t_count && ok; tile += t_step, ++tile_i) {
-                int in0, y0, x0;
-                ct_tile_origin(p, tile, in0, y0, x0);
-                // ---- first epilogue: accumulator one -> + b1 -> activation -> bfloat16 -> T in shared memory ----
-                // (T may be overwritten once the MMAs of the previous tile's second layer have read it)
+            int row = r;                                         // its row of the staging buffer (kHalo: the place in the box, or none)
+            if constexpr (kHalo) {
+                const int per_image = p.halo_rows * p.halo_w, n = r / per_image, y = (r - n * per_image) / p.halo_w, x = r - n * per_image - y * p.halo_w;
+                row = n < p.Nt && y < p.Ht && x < p.Wt ? (n * p.Ht + y) * p.Wt + x : -1;
+            }
+            // constants of a round's channels, fetched one round ahead (thread c holds channel c)
+            uint32_t *bias = tail.bias[grp], *half = tail.half[grp];
+            uint8_t *shift = tail.shift[grp];
+            const int ct = ((warp - 2) & 3) * 32 + lane;
+            uint32_t next_bias = 0u, next_shift = 1u;
+            bool small = false;
+            const int n_rounds = p.n_c2 + p.n_t2 * kRpt;
+            auto fetch = [&](int rnd) {
+                const bool one = rnd < p.n_c2;
+                const int ch = (one ? rnd * p.tcc : (rnd - p.n_c2) * cpr) + ct, O = one ? p.O1 : p.O2;
+                const uint32_t *b = (const uint32_t *)(one ? p.bias1 : p.bias2);
+                const int32_t *s = one ? p.shift1 : p.shift2;
+                const bool in = ct < (one ? p.tcc : cpr) && ch < O;
+                next_bias = in && b != nullptr ? __ldg(b + ch) : 0u;
+                if constexpr (kI8) next_shift = in && s != nullptr ? (uint32_t)__ldg(s + ch) & 31u : 1u;
+            };
+            bool mine_small = false, fresh = true;
+            auto place = [&](int rnd) {                          // (between two barriers of the group)
+                fresh = true;
+                if constexpr (kI8)
+                    mine_small = (rnd < p.n_c2 ? p.small1 : p.small2) != 0 && next_shift != 0u && next_shift != 31u && (int)next_bias <= (1 << 29) && (int)next_bias >= -(1 << 29);
+                bias[ct] = next_bias;
+                if constexpr (kI8) { half[ct] = (1u << next_shift) >> 1; shift[ct] = (uint8_t)next_shift; }
+            };
+            const int n_local = t_first < t_count ? (t_count - t_first + t_step - 1) / t_step : 0;       // tiles of this CTA
+            int step = -p.ahead, rnd = grp;
+            bool ok = true;
+            while (rnd >= n_rounds) { rnd -= n_rounds; ++step; }
+            if (step < n_local) { fetch(rnd); place(rnd); }
+            gt_group_sync(1 + grp);
+            while (step < n_local) {
+                int next = rnd + 2, next_step = step;
+                while (next >= n_rounds) { next -= n_rounds; ++next_step; }
+                const bool change = next != rnd;
+                if (change) fetch(next);
+                const bool one = rnd < p.n_c2;
+                const int idx = one ? step + p.ahead : step;     // which of the CTA's tiles
+                const uint32_t tile_i = (uint32_t)idx;
+                if (idx < 0 || idx >= n_local) {                 // (before the first Y, after the last T)
+                    if (change) { gt_group_sync(1 + grp); place(next); gt_group_sync(1 + grp); }
+                    rnd = next; step = next_step;
+                    continue;
+                }
+                // what the round waits for: accumulator one and a free T (the MMAs of the second layer that read it have
+                // completed), or accumulator two (int8: and a staging buffer that its last store has read)
+                const int t2 = one ? 0 : (rnd - p.n_c2) / kRpt, c0 = one ? 0 : (rnd - p.n_c2) % kRpt * cpr, n0 = t2 * kCtBN2;
                 const uint32_t b1 = p.db ? (tile_i & 1u) : 0u, u1 = p.db ? (tile_i >> 1) : tile_i;
-                if (!gt_wait(sm32(&s_acc1_full[b1]), u1 & 1u) || !gt_wait(sm32(&s_t_empty[b1]), (u1 & 1u) ^ 1u)) ok = false;
+                const uint32_t bt = p.dbt ? (tile_i & 1u) : 0u, ut = p.dbt ? (tile_i >> 1) : tile_i;
+                const uint32_t u2 = tile_i * (uint32_t)p.n_t2 + (uint32_t)t2, buf = u2 & 1u, use = u2 >> 1;
+                // A wait that ran out is latched below; the group goes on (its warps meet at barriers) and waits no more.
                 if (s_fail) ok = false;
-                ok = gt_group_all(1 + grp, ok);                  // the four warps of a group go on or give up as one
-                if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t t1 = tmem + ((uint32_t)(q * 32) << 16);
-                const uint32_t a1 = t1 + b1 * 128u;                  // this tile's accumulator one
-                for (int c2 = grp; c2 < p.n_c2; c2 += 2) {
-                    uint32_t out[32];                            // one chunk (128 bytes of channels) of this lane's row of T
-                    if constexpr (kI8) {                         // 128 channels: + b1, rounding shift, activation, int8
-#pragma unroll
-                        for (int sub = 0; sub < 4; ++sub) {
-                            if (c2 * 128 + sub * 32 >= p.O1) {       // (past the last channel of T: zeros, as the weights of layer two there)
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) out[sub * 8 + e] = 0u;
-                                continue;
-                            }
-                            uint32_t v[32];
-                            gt_load32(a1 + (uint32_t)(c2 * 128 + sub * 32), v);
-                            const int ch = c2 * 128 + sub * 32 + lane;
-                            const int bl = (p.bias1 != nullptr && ch < p.O1) ? __ldg((const int *)p.bias1 + ch) : 0;   // lane e: channel .. + e
-                            const uint32_t sl = ch < p.O1 ? (uint32_t)__ldg(p.shift1 + ch) & 31u : 0u;
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) {
-                                int r4[4];
-#pragma unroll
-                                for (int b = 0; b < 4; ++b)
-                                    r4[b] = gt_round_shift((int)v[4 * e + b] + __shfl_sync(0xFFFFFFFFu, bl, 4 * e + b),
-                                                           __shfl_sync(0xFFFFFFFFu, sl, 4 * e + b));
-                                uint32_t w = gt_pack_s8x4(r4[0], r4[1], r4[2], r4[3]);
-                                if (p.relu) w = __vmaxs4(w, 0u);
-                                out[sub * 8 + e] = w;
-                            }
-                        }
-                    } else {
-#pragma unroll
-                    for (int sub = 0; sub < 2; ++sub) {
-                        uint32_t v[32];
-                        gt_load32(a1 + (uint32_t)(c2 * 64 + sub * 32), v);
-                        const int ch = c2 * 64 + sub * 32 + lane;
-                        const float bl = (p.bias1 != nullptr && ch < p.O1) ? __ldg((const float *)p.bias1 + ch) : 0.f;     // lane e: bias of channel .. + e
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            float a = __uint_as_float(v[2 * e]) + __shfl_sync(0xFFFFFFFFu, bl, 2 * e);
-                            float b = __uint_as_float(v[2 * e + 1]) + __shfl_sync(0xFFFFFFFFu, bl, 2 * e + 1);
-                            if (p.relu) { a = fmaxf(a, 0.f); b = fmaxf(b, 0.f); }
-                            const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-                            out[sub * 16 + e] = *(const uint32_t *)&h;
-                        }
-                    }
-                    }
-                    // K-major rows of 128 bytes under the 128-byte swizzle: the 16-byte piece j of row r sits at piece j ^ (r % 8)
-                    const uint32_t dst = trow + b1 * tbytes + (uint32_t)(c2 * kCtChunk);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
-                                     ::"r"(dst + (uint32_t)((j ^ (lane & 7)) << 4)), "r"(out[4 * j]), "r"(out[4 * j + 1]), "r"(out[4 * j + 2]), "r"(out[4 * j + 3]) : "memory");
-                }
-                // the MMAs read T through the asynchronous proxy
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&s_acc1_empty[b1])) : "memory");
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&s_t_full[b1])) : "memory");
-                }
-                // ---- second epilogue, per tile of 128 output channels: + b2 -> convert -> Y ----
-                for (int t2 = 0; t2 < p.n_t2 && ok; ++t2, ++u2) {
-                    const uint32_t buf = u2 & 1u, use = u2 >> 1;
-                    if ((int)buf != grp) continue;               // (the other group drains this accumulator)
-                    const int n0 = t2 * kCtBN2;
-                    if (!gt_wait(sm32(&s_acc2_full[buf]), use & 1u)) ok = false;
-                    if (s_fail) ok = false;
-                    ok = gt_group_all(1 + grp, ok);              // the four warps go on or give up as one (they meet at barriers below)
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t t2base = t1 + 256u + buf * (uint32_t)kCtBN2;
-                    for (int c0 = 0; c0 < kCtBN2; c0 += cpr) {
-                        uint32_t out[32];                        // 128 bytes of this lane's row of Y
-                        if (ey == 4) {                           // float32 or int32 output: 32 channels
-                            uint32_t v[32];
-                            gt_load32(t2base + (uint32_t)c0, v);
-                            const int ch = n0 + c0 + lane;
-                            const uint32_t bl = (p.bias2 != nullptr && ch < p.O2) ? __ldg((const uint32_t *)p.bias2 + ch) : 0u;
-                            if constexpr (kI8) {
-#pragma unroll
-                                for (int e = 0; e < 32; ++e) out[e] = (uint32_t)((int)v[e] + (int)__shfl_sync(0xFFFFFFFFu, bl, e));
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 32; ++e) out[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(__shfl_sync(0xFFFFFFFFu, bl, e)));
-                            }
-                        } else if (kI8 && ey == 1) {             // int8 output: 128 channels, requantised after the bias
-#pragma unroll
-                            for (int sub = 0; sub < 4; ++sub) {
-                                if (n0 + c0 + sub * 32 >= p.O2) {    // (past the last channel: clipped by the store)
-#pragma unroll
-                                    for (int e = 0; e < 8; ++e) out[sub * 8 + e] = 0u;
-                                    continue;
-                                }
-                                uint32_t v[32];
-                                gt_load32(t2base + (uint32_t)(c0 + sub * 32), v);
-                                const int ch = n0 + c0 + sub * 32 + lane;
-                                const int bl = (p.bias2 != nullptr && ch < p.O2) ? __ldg((const int *)p.bias2 + ch) : 0;
-                                const uint32_t sl = ch < p.O2 ? (uint32_t)__ldg(p.shift2 + ch) & 31u : 0u;
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    int r4[4];
-#pragma unroll
-                                    for (int b = 0; b < 4; ++b)
-                                        r4[b] = gt_round_shift((int)v[4 * e + b] + __shfl_sync(0xFFFFFFFFu, bl, 4 * e + b), __shfl_sync(0xFFFFFFFFu, sl, 4 * e + b));
-                                    const uint32_t w = gt_pack_s8x4(r4[0], r4[1], r4[2], r4[3]);
-                                    out[sub * 8 + e] = w;
-                                }
-                            }
-                        } else {                                 // bfloat16 output: 64 channels
-#pragma unroll
-                            for (int sub = 0; sub < 2; ++sub) {
-                                uint32_t v[32];
-                                gt_load32(t2base + (uint32_t)(c0 + sub * 32), v);
-                                const int ch = n0 + c0 + sub * 32 + lane;
-                                const float bl = (p.bias2 != nullptr && ch < p.O2) ? __ldg((const float *)p.bias2 + ch) : 0.f;
-#pragma unroll
-                                for (int e = 0; e < 16; ++e) {
-                                    const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[2 * e]) + __shfl_sync(0xFFFFFFFFu, bl, 2 * e),
-                                                                                   __uint_as_float(v[2 * e + 1]) + __shfl_sync(0xFFFFFFFFu, bl, 2 * e + 1));
-                                    out[sub * 16 + e] = *(const uint32_t *)&h;
-                                }
-                            }
-                        }
-                        // staged under the 128-byte swizzle and stored as the tile's box of positions by one TMA store; what lies
-                        // past the last channel, column, row or image of Y is clipped
+                if (one) {
+                    if (ok && (!gt_wait(sm32(&tail.acc1_full[b1]), u1 & 1u) || !gt_wait(sm32(&tail.t_empty[bt]), (ut & 1u) ^ 1u))) ok = false;
+                } else {
+                    if (ok && !gt_wait(sm32(&tail.acc2_full[buf]), use & 1u)) ok = false;
+                    if (kEy == 1) {
                         if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
-                        gt_group_sync(1 + grp);
-                        const uint32_t srow = sb + (uint32_t)lane * 128u;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
-                                         ::"r"(srow + (uint32_t)((j ^ (lane & 7)) << 4)), "r"(out[4 * j]), "r"(out[4 * j + 1]), "r"(out[4 * j + 2]), "r"(out[4 * j + 3]) : "memory");
-                        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                        gt_group_sync(1 + grp);
-                        if (issuer && n0 + c0 < p.O2) {
-                            asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n"
-                                         ::"l"(&p.tmy), "r"(sg), "r"((n0 + c0) * ey), "r"(x0), "r"(y0), "r"(in0) : "memory");
-                            asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-                        }
+                        if (!fresh) gt_group_sync(1 + grp);
                     }
+                }
+                if (kI8 && fresh) small = gt_group_all(1 + grp, mine_small);
+                fresh = false;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
+                const uint32_t sw = (uint32_t)(one ? lane : row) & 7u;
+                // (an accumulator is handed back as soon as it has been read)
+                auto hand_back = [&](uint64_t *bar) {
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&s_acc2_empty[buf])) : "memory");
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(bar)) : "memory");
+                };
+                if (one) {
+                    // ---- first epilogue: accumulator one -> + b1 -> activation -> T in shared memory, K-major rows of 128 bytes ----
+                    const uint32_t tcol = lanes + b1 * 128u + (uint32_t)(rnd * p.tcc), trow = tbuf + bt * tbytes + (uint32_t)(rnd * kCtChunk + r * 128);
+                    if constexpr (kI8) {
+                        gt_epilogue_int8<true>(tcol, bias, half, shift, small, p.O1 - rnd * p.tcc, p.relu, trow, sw, true);
+                        hand_back(&tail.acc1_empty[b1]);
+                    } else {
+                        uint32_t out[32];
+                        gt_epilogue_round<false, 2, true>(tcol, bias, p.O1 - rnd * p.tcc, p.relu, out);
+                        hand_back(&tail.acc1_empty[b1]);
+                        gt_store_round(trow, sw, true, out);
+                    }
+                    // the MMAs read T through the asynchronous proxy
+                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&tail.t_full[bt])) : "memory");
+                    if (change) { gt_group_sync(1 + grp); place(next); gt_group_sync(1 + grp); }
+                } else {
+                    // ---- second epilogue: + b2 -> convert -> staging -> the tile's box of Y by one TMA store; what lies past the
+                    // last channel, column, row or image of Y is clipped ----
+                    const uint32_t tcol = lanes + 256u + buf * (uint32_t)kCtBN2 + (uint32_t)c0, srow = sg + (uint32_t)row * 128u;
+                    if constexpr (kEy == 1) {
+                        gt_epilogue_int8<false>(tcol, bias, half, shift, small, p.O2 - n0 - c0, 0, srow, sw, row >= 0);
+                        hand_back(&tail.acc2_empty[buf]);
+                    } else {
+                        uint32_t out[32];
+                        gt_epilogue_round<kI8, kEy, false>(tcol, bias, p.O2 - n0 - c0, 0, out);
+                        hand_back(&tail.acc2_empty[buf]);
+                        // (loads and arithmetic run while the last store reads the staging buffer)
+                        if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+                        gt_group_sync(1 + grp);
+                        if (change) place(next);
+                        gt_store_round(srow, sw, row >= 0, out);
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                    gt_group_sync(1 + grp);
+                    if (kEy == 1 && change) place(next);
+                    if (issuer && n0 + c0 < p.O2) {
+                        int in0, y0, x0;
+                        ct_tile_origin(p, t_first + idx * t_step, in0, y0, x0);
+                        asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n"
+                                     ::"l"(&p.tmy), "r"(sg), "r"((n0 + c0) * kEy), "r"(x0), "r"(y0), "r"(in0) : "memory");
+                        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+                    }
                 }
+                rnd = next; step = next_step;
             }
             if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");      // (the stores have read this CTA's memory)
-            if (!ok && lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
+            if (!ok && lane == 0) atomicExch((uint32_t *)&tail.fail, 1u);
         }
     }
 
@@ -479,65 +556,116 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.bias1 = bias1; p.bias2 = bias2; p.shift1 = shift1; p.shift2 = shift2; p.wtype = wd1.wtype; p.packed1 = (const uint8_t *)packed1; p.packed2 = (const uint8_t *)packed2;
     p.status = (int *)ws;
     p.O1 = wd1.O; p.I1 = wd1.I; p.H = wd1.H; p.K = wd1.K; p.bo1 = wd1.bo; p.bi1 = wd1.bi;
-    p.O2 = wd2.O; p.bo2 = wd2.bo; p.bi2 = wd2.bi; p.relu = relu ? 1 : 0; p.ytype = ytype; p.ey = ey; p.Y = (uint8_t *)Y;
+    p.O2 = wd2.O; p.bo2 = wd2.bo; p.bi2 = wd2.bi; p.relu = relu ? 1 : 0;
     p.tcc = 128 / esz;
     p.O1p = (wd1.O + p.tcc - 1) / p.tcc * p.tcc;
     p.N = xd.N; p.sh = xd.stride_h; p.sw = xd.stride_w; p.ph = xd.pad_h; p.pw = xd.pad_w;
     p.M = (xd.L + 2 * xd.pad_h - wd1.H) / xd.stride_h + 1;
     p.Nw = (xd.J + 2 * xd.pad_w - wd1.K) / xd.stride_w + 1;
-    const long long P = (long long)xd.N * p.M * p.Nw;
-    p.P = (int)P;
-    const GtTile T = gt_pick_tile(xd.N, p.M, p.Nw, p.sh, p.sw);
+    GtTile T = gt_pick_tile(xd.N, p.M, p.Nw, p.sh, p.sw);
     if (T.tiles <= 0 || T.tiles > 0x7FFFFFFF - 4096) return BSP_ERR_SHAPE;
-    p.Wt = T.Wt; p.Ht = T.Ht; p.Nt = T.Nt; p.rows_tile = T.Wt * T.Ht * T.Nt;
-    p.tiles_x = (p.Nw + T.Wt - 1) / T.Wt; p.tiles_y = (p.M + T.Ht - 1) / T.Ht;
-    p.m_tx = gt_magic(p.tiles_x); p.m_ty = gt_magic(p.tiles_y);
-    p.a_bytes = p.rows_tile * 128;
-    p.n_tiles = (int)T.tiles;
-    p.cpt1 = (wd1.I * esz + 127) / 128;
-    p.n_ks1 = wd1.H * wd1.K * p.cpt1;
+    const int HK = wd1.H * wd1.K, row1 = wd1.I * esz;
+    p.cpt1 = (row1 + 127) / 128;
+    p.n_ks1 = HK * p.cpt1;
     p.n_c2 = p.O1p / p.tcc;
     p.n_t2 = (wd2.O + kCtBN2 - 1) / kCtBN2;
-    p.stage_bytes = kGtABytes + p.O1p * 128;
     p.db = p.O1p <= 128 ? 1 : 0;
-    const int fixed = 1024 + (p.db ? 2 : 1) * p.n_c2 * kCtChunk + 8 * kGtStagingBytes;
-    int stages = (kGtMaxSmem - fixed) / p.stage_bytes;
-    if (stages > kGtMaxStages) stages = kGtMaxStages;
-    if (stages < 2) return BSP_ERR_SHAPE;
-    p.stages = stages;
-    const size_t smem = (size_t)fixed + (size_t)stages * p.stage_bytes;
+    p.dbt = p.db;
+    p.kbytes = 128; p.planes = 1;
+    p.small1 = (long long)row1 * HK * 128 * 128 <= (1 << 29) ? 1 : 0;
+    p.small2 = (long long)wd1.O * 128 * 128 <= (1 << 29) ? 1 : 0;
+    const int staging = 8 * kGtStagingBytes, fixed = staging + (int)sizeof(CtTail);
+    // kHalo: where two boxes of activations, the weights of layer one and at least two chunks of layer two's fit, and the
+    // tiles with their border are not many more.  3x3 64->64 then 64->256 at 56x56, batch 64: 44.5 us loaded tap by tap.
+    bool halo = false;
+    int w2_slots = 0;
+    const GtTile Th = gt_pick_halo(xd.N, p.M, p.Nw, wd1.H, wd1.K);
+    if (HK > 1 && HK <= kCtTaps && p.cpt1 == 1 && p.sh == 1 && p.sw == 1 && p.db && Th.tiles > 0 && Th.tiles * 4 <= T.tiles * 5) {
+        const int kb = row1 <= 32 ? 32 : (row1 <= 64 ? 64 : 128), planes = kb == 128 ? 1 : kb / 32;
+        const int plane = (Th.Nt * (Th.Ht + wd1.H - 1) * (Th.Wt + wd1.K - 1) * (kb / planes) + 1023) / 1024 * 1024;
+        const int room = kCtSmem - fixed - p.n_c2 * kCtChunk - HK * p.O1p * kb - 2 * planes * plane;
+        const int room2 = room - p.n_c2 * kCtChunk;          // with two buffers for T
+        int want = p.n_t2 * p.n_c2;
+        if (want > kCtW2Slots) want = kCtW2Slots;
+        const int one_t = room / (kCtBN2 * 128), two_t = room2 / (kCtBN2 * 128);
+        // (a second buffer for T before the weights of layer two stay, where the tile does not fit both accumulators)
+        const bool second = two_t >= want || (p.n_t2 > 2 && two_t >= 2);
+        w2_slots = second ? two_t : one_t;
+        if (w2_slots > want) w2_slots = want;
+        if (w2_slots >= 2 || w2_slots == p.n_t2 * p.n_c2) {
+            halo = true;
+            T = Th;
+            p.kbytes = kb; p.planes = planes; p.plane_bytes = plane;
+            p.dbt = second ? 1 : 0;
+            p.w2_slots = w2_slots; p.w2_stay = w2_slots == p.n_t2 * p.n_c2 ? 1 : 0;
+            p.halo_w = T.Wt + wd1.K - 1; p.halo_rows = T.Ht + wd1.H - 1;
+        }
+    }
+    p.Wt = T.Wt; p.Ht = T.Ht; p.Nt = T.Nt;
+    p.tiles_x = (p.Nw + T.Wt - 1) / T.Wt; p.tiles_y = (p.M + T.Ht - 1) / T.Ht;
+    p.m_tx = gt_magic(p.tiles_x); p.m_ty = gt_magic(p.tiles_y);
+    p.n_tiles = (int)T.tiles;
+    size_t at = 0;                          // shared memory: (weights of layer one) ring (weights of layer two) T staging tail
+    if (halo) {
+        p.a_bytes = T.Nt * p.halo_rows * p.halo_w * p.kbytes;
+        p.stage_bytes = p.planes * p.plane_bytes;
+        at = (size_t)HK * p.O1p * p.kbytes;
+        int stages = (kCtSmem - fixed - (p.dbt ? 2 : 1) * p.n_c2 * kCtChunk - (int)at - w2_slots * kCtBN2 * 128) / p.stage_bytes;
+        p.stages = stages > 4 ? 4 : stages;
+    } else {
+        p.a_bytes = T.Wt * T.Ht * T.Nt * 128;
+        p.stage_bytes = kGtABytes + p.O1p * 128;
+        int stages = (kCtSmem - fixed - (p.dbt ? 2 : 1) * p.n_c2 * kCtChunk) / p.stage_bytes;
+        p.stages = stages > kGtMaxStages ? kGtMaxStages : stages;
+    }
+    if (p.stages < 2) return BSP_ERR_SHAPE;
+    // (T of the next tile before Y of this one: with one buffer for T, layer two must be able to finish without the second
+    // epilogue, that is both its accumulators must hold the whole tile)
+    p.ahead = p.db && (p.dbt || p.n_t2 <= 2) ? 1 : 0;
+    p.off_ring = (uint32_t)at; at += (size_t)p.stages * p.stage_bytes;
+    p.off_w2 = (uint32_t)at; at += (size_t)p.w2_slots * kCtBN2 * 128;
+    p.off_t = (uint32_t)at; at += (size_t)(p.dbt ? 2 : 1) * p.n_c2 * kCtChunk;
+    p.off_staging = (uint32_t)at; at += staging;
+    p.off_tail = (uint32_t)at;
+    const size_t smem = at + sizeof(CtTail);
 
+    // kernels by type of the pair, width of Y (32 bits or the narrow form) and kHalo
+    typedef void (*Kernel)(const CtParams);
+    static const Kernel kernels[2][2][2] = {{{chain_tc_kernel<false, 4, false>, chain_tc_kernel<false, 4, true>}, {chain_tc_kernel<false, 2, false>, chain_tc_kernel<false, 2, true>}},
+                                            {{chain_tc_kernel<true, 4, false>, chain_tc_kernel<true, 4, true>}, {chain_tc_kernel<true, 1, false>, chain_tc_kernel<true, 1, true>}}};
     static bool opted[kGtMaxDevices] = {};
     static int n_sm[kGtMaxDevices] = {};
     int dev = 0;
     BSP_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
     if (!opted[dev]) {
-        BSP_CUDA_OK(cudaFuncSetAttribute(chain_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
-        BSP_CUDA_OK(cudaFuncSetAttribute(chain_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        for (int t = 0; t < 8; ++t) BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 4][t / 2 % 2][t % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, kCtSmem));
         BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
         opted[dev] = true;
     }
+    // bytes of an operand row of layer one in shared memory, and its swizzle
+    const int row_bytes = halo && p.kbytes < 128 ? 32 : 128;
+    const CUtensorMapSwizzle swizzle = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_32B;
     GtEncodeFn enc = gt_encode();
     if (!enc) return BSP_ERR_CUDA;
     {
         const cuuint64_t row = (cuuint64_t)wd1.I * esz;
         const cuuint64_t gdim[4] = {row, (cuuint64_t)xd.J, (cuuint64_t)xd.L, (cuuint64_t)xd.N};
         const cuuint64_t gstr[3] = {row, row * xd.J, row * xd.J * xd.L};
-        const cuuint32_t box[4] = {128, (cuuint32_t)(T.Wt * p.sw), (cuuint32_t)(T.Ht * p.sh), (cuuint32_t)T.Nt};
+        const cuuint32_t box[4] = {(cuuint32_t)row_bytes, (cuuint32_t)(halo ? p.halo_w : T.Wt * p.sw), (cuuint32_t)(halo ? p.halo_rows : T.Ht * p.sh), (cuuint32_t)T.Nt};
         const cuuint32_t estr[4] = {1, (cuuint32_t)p.sw, (cuuint32_t)p.sh, 1};
         if (enc(&p.tmx, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(X), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return BSP_ERR_CUDA;
     }
     {
         const cuuint64_t row = (cuuint64_t)wd1.I * esz;
         const cuuint64_t gdim[3] = {row, (cuuint64_t)(wd1.H * wd1.K), (cuuint64_t)wd1.O};
         const cuuint64_t gstr[2] = {row, row * wd1.H * wd1.K};
-        const cuuint32_t box[3] = {128, 1, (cuuint32_t)p.O1p};
+        const cuuint32_t box[3] = {(cuuint32_t)row_bytes, 1, (cuuint32_t)p.O1p};
         const cuuint32_t estr[3] = {1, 1, 1};
         if (enc(&p.tmw1, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t *>((const uint8_t *)packed1 + L1.off_payload), gdim, gstr, box,
-                estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return BSP_ERR_CUDA;
     }
@@ -563,7 +691,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
             return BSP_ERR_CUDA;
     }
     const int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
-    BSP_CUDA_OK(launch_after(wd1.wtype == BSP_I8 ? chain_tc_kernel<true> : chain_tc_kernel<false>, dim3((unsigned)grid), dim3(kCtThreads), smem, st, p));
+    BSP_CUDA_OK(launch_after(kernels[wd1.wtype == BSP_I8 ? 1 : 0][ey == 4 ? 0 : 1][halo ? 1 : 0], dim3((unsigned)grid), dim3(kCtThreads), smem, st, p));
     return BSP_OK;
 }
 

@@ -379,23 +379,24 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             const int ct = ((warp - 2) & 3) * 32 + lane;
             uint32_t next_bias = 0u, next_shift = 1u;
             int have = -1;                                       // first channel of the round whose constants are in shared memory
-            bool small = false;
+            bool small = false, mine_small = false, fresh = false;
             auto fetch = [&](int ch0) {
                 if (ct >= cpr) return;
                 next_bias = gt_bias(p, ch0 + ct);
                 if constexpr (kEy == 1) next_shift = ch0 + ct < p.O ? (uint32_t)__ldg(p.shift + ch0 + ct) & 31u : 1u;
             };
-            auto place = [&]() {                                 // (followed by a barrier of the group)
+            auto place = [&](int ch0) {                          // (between two barriers of the group)
+                have = ch0;
+                fresh = true;
+                if constexpr (kEy == 1)
+                    mine_small = p.small_acc != 0 && next_shift != 0u && next_shift != 31u && (int)next_bias <= (1 << 29) && (int)next_bias >= -(1 << 29);
                 if (ct >= cpr) return;
                 bias[ct] = next_bias;
                 if constexpr (kEy == 1) { half[ct] = (1u << next_shift) >> 1; shift[ct] = (uint8_t)next_shift; }
             };
-            auto is_small = [&]() {
-                return p.small_acc != 0 && next_shift != 0u && next_shift != 31u && (int)next_bias <= (1 << 29) && (int)next_bias >= -(1 << 29);
-            };
             uint32_t tile_i = 0;
             bool ok = true;
-            for (int tile = t_first; tile < t_count && ok; tile += t_step, ++tile_i) {
+            for (int tile = t_first; tile < t_count; tile += t_step, ++tile_i) {
                 const bool last = tile + t_step >= t_count, shared_tile = last && BN > cpr;
                 if (!shared_tile && (int)(tile_i & 1u) != grp) continue;
                 const int c_first = shared_tile ? grp * cpr : 0, c_step = shared_tile ? 2 * cpr : cpr;
@@ -405,16 +406,15 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 const int n0 = tn * BN;
                 int in0, y0, x0;
                 gt_tile_origin(p, mt, in0, y0, x0);
-                if (have != n0 + c_first) {                      // (the first tile, or an order of rounds that was not foreseen)
-                    fetch(n0 + c_first);
-                    place();
-                    if constexpr (kEy == 1) small = gt_group_all(1 + grp, is_small());
-                    have = n0 + c_first;
-                }
-                if (!gt_wait(sm32(&s_acc_full[buf]), use & 1u)) ok = false;
+                // (here every thread of the group is past the barrier of its last round: its constants may be replaced)
+                const bool replace = have != n0 + c_first;       // the first tile, or an order of rounds that was not foreseen
+                if (replace) { fetch(n0 + c_first); place(n0 + c_first); }
+                // A wait that ran out is latched below; the group goes on (its warps meet at barriers) and waits no more.
                 if (s_fail) ok = false;
-                ok = gt_group_all(1 + grp, ok);                // the four warps go on or give up as one (they meet at barriers below)
-                if (!ok) break;
+                if (ok && !gt_wait(sm32(&s_acc_full[buf]), use & 1u)) ok = false;
+                // int8: the staging buffer was handed to a TMA store; the issuing thread waits until it has been read
+                if (kEy == 1 && issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+                if (kEy == 1 ? !fresh : replace) gt_group_sync(1 + grp);
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + buf * 256u;
                 // the channels of the round after the last one of this tile: those of the group's next tile
@@ -425,37 +425,45 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                     gt_divmod(next, ntn, p.m_ntn, m2, t2);
                     after = t2 * BN + (next + t_step >= t_count && BN > cpr ? grp * cpr : 0);
                 }
+                // the accumulator buffer has been read: hand it back to the MMA issuer (before the round is staged, where that can be)
+                auto hand_back = [&]() {
+                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        if constexpr (kPair)
+                            asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(lead_acc_empty0 + buf * 8u) : "memory");
+                        else
+                            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&s_acc_empty[buf])) : "memory");
+                    }
+                };
                 for (int c0 = c_first; c0 < BN; c0 += c_step) {
-                    uint32_t out[32];                            // 128 bytes of this lane's row of Y
+                    const bool hand = !last && c0 + c_step >= BN;
                     const int left = (p.O - n0 < BN ? p.O - n0 : BN) - c0;          // channels from here on
                     const int next_ch = c0 + c_step < BN ? n0 + c0 + c_step : after;
                     if (next_ch != have) fetch(next_ch);
-                    gt_epilogue_round<kWT == BSP_I8, kEy>(tbase + (uint32_t)c0, bias, half, shift, small, left, out);
-                    if (!last && c0 + c_step >= BN) {
-                        // the accumulator buffer has been read: hand it back to the MMA issuer
-                        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) {
-                            if constexpr (kPair)
-                                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(lead_acc_empty0 + buf * 8u) : "memory");
-                            else
-                                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(&s_acc_empty[buf])) : "memory");
+                    const uint32_t tcol = tbase + (uint32_t)c0, srow = sg + (uint32_t)row * 128u, sw = (uint32_t)row & 7u;
+                    if constexpr (kEy == 1) {
+                        if (c0 != c_first) {
+                            if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+                            if (!fresh) gt_group_sync(1 + grp);
                         }
+                        if (fresh) small = gt_group_all(1 + grp, mine_small);
+                        fresh = false;
+                        gt_epilogue_int8<false>(tcol, bias, half, shift, small, left, 0, srow, sw, row >= 0);
+                        if (hand) hand_back();
+                    } else {
+                        // (loads and arithmetic run while the last store reads the staging buffer)
+                        uint32_t out[32];
+                        gt_epilogue_round<kWT == BSP_I8, kEy, false>(tcol, bias, left, 0, out);
+                        if (hand) hand_back();
+                        if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+                        gt_group_sync(1 + grp);
+                        if (next_ch != have) place(next_ch);
+                        gt_store_round(srow, sw, row >= 0, out);
                     }
-                    // the staging buffer was handed to a TMA store in the previous round: the issuing thread waits until it
-                    // has been read (the loads and the arithmetic of this round ran meanwhile), then the group may write
-                    if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
-                    gt_group_sync(1 + grp);
-                    if (next_ch != have) place();
-                    const uint32_t srow = sg + (uint32_t)row * 128u;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if (kMode != kHalo || row >= 0) asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
-                                     ::"r"(srow + (uint32_t)((j ^ (row & 7)) << 4)), "r"(out[4 * j]), "r"(out[4 * j + 1]), "r"(out[4 * j + 2]), "r"(out[4 * j + 3]) : "memory");
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                    if (kEy == 1 && next_ch != have) small = gt_group_all(1 + grp, is_small());
-                    else gt_group_sync(1 + grp);
-                    have = next_ch;
+                    gt_group_sync(1 + grp);
+                    if (kEy == 1 && next_ch != have) place(next_ch);
                     // one store of the tile's box: 128 bytes of every row; what lies past the last channel, column, row or image
                     // of Y is clipped (rows of the buffer beyond the box are not part of the store)
                     if (issuer && left > 0) {

@@ -225,21 +225,19 @@ __device__ __forceinline__ void gt_load32(uint32_t taddr, uint32_t (&v)[32])
 }
 
 // One round of an epilogue: 128 bytes of this lane's row of the output (32 channels of 4 bytes, 64 of bfloat16, 128 of
-// int8) from the accumulator columns at `taddr`, after the bias.  kEy: bytes of an output element.  `bias` (raw bits) and
-// `shift` are the channels' own entries in shared memory, read four channels at a time by all lanes at once: a shuffle per
-// channel (two for int8) had made the int8 round five times as long.  `n`: channels left; 32-channel pieces past them are
-// neither loaded nor computed (their bytes are clipped by the store).
-// `small`: 1 <= shift <= 30 for all of them and every sum at most 2^30 (gt_round_shift_small holds, `half` has its 2^(s - 1)).
-template <bool kInt, int kEy>
-__device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t *bias, const uint32_t *half, const uint8_t *shift, bool small, int n,
-                                                  uint32_t (&out)[32])
+// int8) from the accumulator columns at `taddr`, after the bias.  kEy: bytes of an output element.  `bias` (raw bits), `half`
+// and `shift` are the channels' own entries in shared memory, read four channels at a time by all lanes at once.  `n`:
+// channels left; zeros past them (in steps of 32).  kRelu: max(., 0) if `relu`.
+//
+// 4-byte and bfloat16 output: into registers.
+template <bool kInt, int kEy, bool kRelu>
+__device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t *bias, int n, int relu, uint32_t (&out)[32])
 {
-    auto bias4 = [&](int c) { return *(const uint4 *)(bias + c); };
     if constexpr (kEy == 4) {
         gt_load32(taddr, out);
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
-            const uint4 b = bias4(e);
+            const uint4 b = *(const uint4 *)(bias + e);
             if constexpr (kInt) { out[e] += b.x; out[e + 1] += b.y; out[e + 2] += b.z; out[e + 3] += b.w; }
             else {
                 out[e] = __float_as_uint(__uint_as_float(out[e]) + __uint_as_float(b.x));
@@ -248,13 +246,13 @@ __device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t
                 out[e + 3] = __float_as_uint(__uint_as_float(out[e + 3]) + __uint_as_float(b.w));
             }
         }
-    } else if constexpr (kEy == 2) {                     // rounded to nearest even after the bias
+    } else {                                             // rounded to nearest even after the bias
         uint32_t v[2][32];
         gt_load32_issue(taddr, v[0]);
         if (n > 32) gt_load32_issue(taddr + 32u, v[1]);
         else {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) v[1][e] = 0u;       // (channels past the last one come out as zeros)
+            for (int e = 0; e < 32; ++e) v[1][e] = 0u;
         }
         gt_load32_wait(v[0]);
         gt_load32_wait(v[1]);
@@ -262,44 +260,72 @@ __device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t
         for (int sub = 0; sub < 2; ++sub)
 #pragma unroll
             for (int e = 0; e < 32; e += 4) {
-                const uint4 b = bias4(sub * 32 + e);
-                const __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(v[sub][e]) + __uint_as_float(b.x), __uint_as_float(v[sub][e + 1]) + __uint_as_float(b.y));
-                const __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(v[sub][e + 2]) + __uint_as_float(b.z), __uint_as_float(v[sub][e + 3]) + __uint_as_float(b.w));
+                const uint4 b = *(const uint4 *)(bias + sub * 32 + e);
+                __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(v[sub][e]) + __uint_as_float(b.x), __uint_as_float(v[sub][e + 1]) + __uint_as_float(b.y));
+                __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(v[sub][e + 2]) + __uint_as_float(b.z), __uint_as_float(v[sub][e + 3]) + __uint_as_float(b.w));
+                if (kRelu && relu) { h0 = __hmax2(h0, __float2bfloat162_rn(0.f)); h1 = __hmax2(h1, __float2bfloat162_rn(0.f)); }
                 out[sub * 16 + e / 2] = *(const uint32_t *)&h0;
                 out[sub * 16 + e / 2 + 1] = *(const uint32_t *)&h1;
             }
-    } else {                                             // requantised after the bias
-        uint32_t v[2][32];
-        if (n > 0) gt_load32_issue(taddr, v[0]);             // (every load issued is waited for below)
+    }
+}
+// ... and from there to the row at `srow` of a tile in shared memory under the 128-byte swizzle (`sw`: the row modulo 8;
+// `live`: the lane has a row).
+__device__ __forceinline__ void gt_store_round(uint32_t srow, uint32_t sw, bool live, const uint32_t (&out)[32])
+{
+    if (live) {
 #pragma unroll
-        for (int sub = 0; sub < 4; ++sub) {
-            if (sub * 32 >= n) {
+        for (uint32_t j = 0; j < 8u; ++j)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
+                         ::"r"(srow + ((j ^ sw) << 4)), "r"(out[4 * j]), "r"(out[4 * j + 1]), "r"(out[4 * j + 2]), "r"(out[4 * j + 3]) : "memory");
+    }
+}
+// int8 output: requantised after the bias and written piece by piece, 32 channels at a time in a loop that stays a loop.
+// (Unrolled, a round is a thousand instructions that eight warps fetch in eight places: 4800 cycles a round in the pair
+// 64->64->256 at 56x56, which took 89 us and 47 us like this.)  `small`: 1 <= shift <= 30 for all channels and every sum at
+// most 2^30 (gt_round_shift_small holds, `half` has its 2^(s - 1)).
+template <bool kRelu>
+__device__ __forceinline__ void gt_epilogue_int8(uint32_t taddr, const uint32_t *bias, const uint32_t *half, const uint8_t *shift, bool small, int n, int relu,
+                                                 uint32_t srow, uint32_t sw, bool live)
+{
+#pragma unroll 1
+    for (int sub = 0; sub < 4; ++sub, n -= 32, taddr += 32u, bias += 32, half += 32, shift += 32) {
+        uint32_t out[8];
+        if (n <= 0) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) out[sub * 8 + e] = 0u;
-                continue;
-            }
-            uint32_t(&cur)[32] = v[sub & 1];
-            gt_load32_wait(cur);
-            if (sub < 3 && (sub + 1) * 32 < n) gt_load32_issue(taddr + (uint32_t)((sub + 1) * 32), v[(sub + 1) & 1]);
+            for (int e = 0; e < 8; ++e) out[e] = 0u;
+        } else {
+            uint32_t v[32];
+            gt_load32(taddr, v);
             if (small) {
 #pragma unroll
                 for (int e = 0; e < 32; e += 4) {
-                    const uint4 b = bias4(sub * 32 + e), h = *(const uint4 *)(half + sub * 32 + e);
-                    const uint32_t s = *(const uint32_t *)(shift + sub * 32 + e);
-                    out[sub * 8 + e / 4] = gt_pack_s8x4(gt_round_shift_small((int)(cur[e] + b.x), h.x, __byte_perm(s, 0u, 0x4440)),
-                                                        gt_round_shift_small((int)(cur[e + 1] + b.y), h.y, __byte_perm(s, 0u, 0x4441)),
-                                                        gt_round_shift_small((int)(cur[e + 2] + b.z), h.z, __byte_perm(s, 0u, 0x4442)),
-                                                        gt_round_shift_small((int)(cur[e + 3] + b.w), h.w, s >> 24));
+                    const uint4 b = *(const uint4 *)(bias + e), h = *(const uint4 *)(half + e);
+                    const uint32_t s = *(const uint32_t *)(shift + e);
+                    out[e / 4] = gt_pack_s8x4(gt_round_shift_small((int)(v[e] + b.x), h.x, __byte_perm(s, 0u, 0x4440)),
+                                              gt_round_shift_small((int)(v[e + 1] + b.y), h.y, __byte_perm(s, 0u, 0x4441)),
+                                              gt_round_shift_small((int)(v[e + 2] + b.z), h.z, __byte_perm(s, 0u, 0x4442)),
+                                              gt_round_shift_small((int)(v[e + 3] + b.w), h.w, s >> 24));
                 }
             } else {
 #pragma unroll
                 for (int e = 0; e < 32; e += 4) {
-                    const uint4 b = bias4(sub * 32 + e);
-                    const uint32_t s = *(const uint32_t *)(shift + sub * 32 + e);
-                    out[sub * 8 + e / 4] = gt_pack_s8x4(gt_round_shift((int)(cur[e] + b.x), s & 31u), gt_round_shift((int)(cur[e + 1] + b.y), (s >> 8) & 31u),
-                                                        gt_round_shift((int)(cur[e + 2] + b.z), (s >> 16) & 31u), gt_round_shift((int)(cur[e + 3] + b.w), s >> 24));
+                    const uint4 b = *(const uint4 *)(bias + e);
+                    const uint32_t s = *(const uint32_t *)(shift + e);
+                    out[e / 4] = gt_pack_s8x4(gt_round_shift((int)(v[e] + b.x), s & 31u), gt_round_shift((int)(v[e + 1] + b.y), (s >> 8) & 31u),
+                                              gt_round_shift((int)(v[e + 2] + b.z), (s >> 16) & 31u), gt_round_shift((int)(v[e + 3] + b.w), s >> 24));
                 }
             }
+            if (kRelu && relu) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) out[e] = __vmaxs4(out[e], 0u);
+            }
+        }
+        if (live) {
+#pragma unroll
+            for (uint32_t j = 0; j < 2u; ++j)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
+                             ::"r"(srow + ((((uint32_t)sub * 2u + j) ^ sw) << 4)), "r"(out[4 * j]), "r"(out[4 * j + 1]), "r"(out[4 * j + 2]), "r"(out[4 * j + 3]) : "memory");
         }
     }
 }

@@ -63,3 +63,56 @@ def test_requantised_output(O, case):
     rp, ci, pl = ref.compact(W, gamma, 8, 8)
     acc = ref.conv2d(W.shape, 8, 8, rp, ci, pl, X, b, (1, 1), (1, 1))
     assert np.array_equal(Y.cpu().numpy().reshape(-1, O), ref.requant_i8(acc, s))
+
+
+@pytest.mark.parametrize("N,L,J,I,O1,O2,H,K,relu", [
+    (6, 56, 56, 64, 64, 256, 3, 3, 1),   # the weights of layer two stay in shared memory, several tiles a CTA
+    (6, 40, 40, 32, 64, 1024, 3, 3, 0),  # ... and stream through their ring
+    (9, 7, 7, 16, 128, 200, 3, 3, 1),    # several images a tile, one plane of 32-byte rows, clipped channels
+    (2, 17, 33, 40, 72, 64, 1, 7, 1),    # two chunks of T with a tail
+    (1, 1, 300, 64, 48, 48, 1, 3, 0),    # T and Y narrower than a chunk
+])
+def test_pair_equals_the_two_calls(N, L, J, I, O1, O2, H, K, relu):
+    for dtype in ("bf16", "i8"):
+        W1, W2 = make_case(841, O1, I, H, K, dtype), make_case(842, O2, O1, 1, 1, dtype)
+        ls = []
+        for k, W in enumerate((W1, W2)):
+            nb = (W.shape[0] // 8) * (W.shape[3] // 8)
+            ls.append(gpu_layer(W, synth.random_gamma(843 + k, W.shape[0] // 8, W.shape[3] // 8, nb // 2), 8, 8, dtype))
+        l1, l2 = ls
+        X = torch.from_numpy(make_x(845, (N, L, J, I), dtype)).cuda()
+        b1, b2 = (torch.from_numpy(make_bias(846 + k, O, dtype)).cuda() for k, O in enumerate((O1, O2)))
+        pad, P = (H // 2, K // 2), (N, L, J)
+        xd = bsp.XDesc(N, L, J, 1, 1, pad[0], pad[1])
+        if dtype == "bf16":
+            X = X.to(torch.bfloat16)
+            T = torch.empty(P + (O1,), dtype=torch.bfloat16, device="cuda")
+            l1.conv2d(X, b1, T, (1, 1), pad)
+            if relu:
+                T.clamp_(min=0)
+            for ydt in (torch.bfloat16, torch.float32):
+                Ya, Yb = (torch.full(P + (O2,), -7.0, dtype=ydt, device="cuda") for _ in range(2))
+                l2.conv2d(T, b2, Ya)
+                bsp.bsp_conv2d_chain(l1.wd, l1.handle(), l2.wd, l2.handle(), xd, X, b1, relu, b2, Yb, bsp.dtype_code(ydt), l1.ws)
+                l1.check()
+                assert torch.equal(Ya, Yb), (dtype, ydt)
+            continue
+        if I % 16 or O1 % 16 or O2 % 16:
+            continue
+        s1, s2 = (torch.from_numpy(synth.uniform_int(848 + k, (O,), 8, 13).astype(np.int32)).cuda() for k, O in enumerate((O1, O2)))
+        for slow in (False, True):
+            if slow:
+                s1[0], s2[1] = 0, 31
+            T = torch.empty(P + (O1,), dtype=torch.int8, device="cuda")
+            l1.conv2d_q8(X, b1, s1, T, (1, 1), pad)
+            if relu:
+                T.clamp_(min=0)
+            Ya, Yb = (torch.full(P + (O2,), -7, dtype=torch.int8, device="cuda") for _ in range(2))
+            l2.conv2d_q8(T, b2, s2, Ya)
+            bsp.bsp_conv2d_chain_q8(l1.wd, l1.handle(), l2.wd, l2.handle(), xd, X, b1, s1, relu, b2, s2, Yb, l1.ws)
+            assert torch.equal(Ya, Yb), (dtype, slow)
+            Za, Zb = (torch.full(P + (O2,), -7, dtype=torch.int32, device="cuda") for _ in range(2))
+            l2.conv2d(T, b2, Za)
+            bsp.bsp_conv2d_chain_q8(l1.wd, l1.handle(), l2.wd, l2.handle(), xd, X, b1, s1, relu, b2, None, Zb, l1.ws)
+            l1.check()
+            assert torch.equal(Za, Zb), (dtype, slow)
