@@ -17,15 +17,17 @@
 // Where layer one has stride 1 and taps, its input channels fit one stage and shared memory allows (kHalo), its weights stay
 // in shared memory and a tile's activations arrive once with the border that the taps reach, as in the product kernel; the
 // weights of layer two then have a ring of their own, or stay too.
-// Warps: 0 producer, 1 MMA issuer (both converged, one elected lane issues), 2-9 epilogue in two groups of four, which take
-// turns with the rounds of both epilogues: 128 bytes of T's or Y's channels each.  Every wait is bounded.
+// Warps: 0 producer, 1 MMA issuer (both converged, one elected lane issues), 2.. epilogue in two or three groups of four, which
+// take turns with the rounds of both epilogues: 128 bytes of T's or Y's channels each.  Every wait is bounded.
 #include <type_traits>
 #include "bsp_tc.cuh"
 
 namespace bsp {
 namespace {
 
-constexpr int kCtThreads = 320;                    // producer warp, MMA warp, two groups of four epilogue warps
+// Epilogue groups of four warps: three where the tap-by-tap loads are gone and the epilogues bound the tile, else two (their
+// staging buffers cost ring stages).
+__host__ __device__ constexpr int ct_groups(bool halo) { return halo ? 3 : 2; }
 constexpr int kCtBN2 = 128;                        // channels of layer two per accumulator buffer
 constexpr int kCtChunk = kGtBM * 128;              // bytes of one chunk (128 bytes of channels) of the tensor between the layers
 
@@ -49,6 +51,7 @@ struct CtParams {
     int sh, sw, ph, pw, a_bytes;
     uint32_t m_tx, m_ty;
     uint32_t off_ring, off_w2, off_t, off_staging, off_tail;         // bytes into shared memory
+    uint32_t staging_bytes;           // a group's staging buffer: 128 bytes of every position of the tile
     // kHalo: bytes of K per position, planes and their pitch, pitch and rows of an image's box; slots of layer two's weights
     int kbytes, planes, plane_bytes, halo_w, halo_rows, w2_slots, w2_stay;
     int small1, small2;       // 8-bit: sums of products of either layer at most 2^29
@@ -56,13 +59,14 @@ struct CtParams {
 
 // Barriers and constants, after everything else in shared memory (all of it dynamic: the base is 1024-byte aligned).
 constexpr int kCtTaps = 30, kCtW2Slots = 8;
+template <int kGroups>
 struct CtTail {
     uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc1_full[2], acc1_empty[2], t_full[2], t_empty[2], acc2_full[2], acc2_empty[2];
     uint64_t w1_full[kCtTaps], w2_full[kCtW2Slots], w2_empty[kCtW2Slots];
     uint32_t tmem, fail;
     // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
-    __align__(16) uint32_t bias[2][128], half[2][128];
-    __align__(16) uint8_t shift[2][128];
+    __align__(16) uint32_t bias[kGroups][128], half[kGroups][128];
+    __align__(16) uint8_t shift[kGroups][128];
 };
 constexpr int kCtSmem = 227 * 1024;
 
@@ -83,11 +87,12 @@ __device__ __forceinline__ bool ct_header_ok(const uint8_t *packed, int wtype, i
 
 // kI8: the 8-bit chain; kEy: bytes of an element of Y (compiled apart, so that no form carries another's epilogue code).
 template <bool kI8, int kEy, bool kHalo>
-__global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_constant__ CtParams p)
+__global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kernel(const __grid_constant__ CtParams p)
 {
     constexpr int kWt = kI8 ? BSP_I8 : BSP_BF16;
     extern __shared__ __align__(1024) uint8_t smem[];
-    CtTail &tail = *(CtTail *)(smem + p.off_tail);
+    constexpr int kGroups = ct_groups(kHalo);
+    CtTail<kGroups> &tail = *(CtTail<kGroups> *)(smem + p.off_tail);
     volatile uint32_t &s_fail = tail.fail;
 
     // (warp number, tensor-memory base and go-ahead through a shuffle: uniform to the compiler, as in the product kernel)
@@ -374,14 +379,14 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
         }
     } else {
         // ================= epilogues (warps 2-9) =================
-        // The work goes in steps: the n_c2 chunks of T of tile s + ahead, then the 128-byte rounds of Y of tile s; the two groups
-        // take turns with these rounds, across steps too.  With ahead = 1 the MMA warp finds the next T ready when it is
+        // The work goes in steps: the n_c2 chunks of T of tile s + ahead, then the 128-byte rounds of Y of tile s; the groups take
+        // turns with these rounds, across steps too.  With ahead = 1 the MMA warp finds the next T ready when it is
         // done with this tile (else layer two of a tile waited for both of the previous tile's epilogues).
         if (run) {
             const int q = warp & 3;                              // quarter of the tensor-memory lanes this warp reaches
             const int grp = (warp - 2) >> 2;
             // the group's staging buffer: 128 rows of 128 bytes
-            const uint32_t sg = staging + (uint32_t)(grp * 4 * kGtStagingBytes);
+            const uint32_t sg = staging + (uint32_t)grp * p.staging_bytes;
             const bool issuer = q == 0 && lane == 0;             // one thread of the group issues its stores
             const int r = q * 32 + lane;                         // this lane's row of a tile
             int row = r;                                         // its row of the staging buffer (kHalo: the place in the box, or none)
@@ -396,6 +401,9 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
             uint32_t next_bias = 0u, next_shift = 1u;
             bool small = false;
             const int n_rounds = p.n_c2 + p.n_t2 * kRpt;
+            // (A barrier tells a phase from the one two before only.  A group sees enough of them when it has a round in every
+            // step, or, of two groups, always the same ones: steps of two rounds take two groups.)
+            const int groups = n_rounds < kGroups ? 2 : kGroups;
             auto fetch = [&](int rnd) {
                 const bool one = rnd < p.n_c2;
                 const int ch = (one ? rnd * p.tcc : (rnd - p.n_c2) * cpr) + ct, O = one ? p.O1 : p.O2;
@@ -414,13 +422,13 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
                 if constexpr (kI8) { half[ct] = (1u << next_shift) >> 1; shift[ct] = (uint8_t)next_shift; }
             };
             const int n_local = t_first < t_count ? (t_count - t_first + t_step - 1) / t_step : 0;       // tiles of this CTA
-            int step = -p.ahead, rnd = grp;
+            int step = grp < groups ? -p.ahead : n_local, rnd = grp;
             bool ok = true;
             while (rnd >= n_rounds) { rnd -= n_rounds; ++step; }
             if (step < n_local) { fetch(rnd); place(rnd); }
             gt_group_sync(1 + grp);
             while (step < n_local) {
-                int next = rnd + 2, next_step = step;
+                int next = rnd + groups, next_step = step;
                 while (next >= n_rounds) { next -= n_rounds; ++next_step; }
                 const bool change = next != rnd;
                 if (change) fetch(next);
@@ -443,6 +451,9 @@ __global__ void __launch_bounds__(kCtThreads, 1) chain_tc_kernel(const __grid_co
                 if (one) {
                     if (ok && (!gt_wait(sm32(&tail.acc1_full[b1]), u1 & 1u) || !gt_wait(sm32(&tail.t_empty[bt]), (ut & 1u) ^ 1u))) ok = false;
                 } else {
+                    // (With one round per tile of layer two, a group of three sees every third of these phases, and a barrier
+                    // tells a phase from the one two before only: the phase before, on the other barrier, comes first.)
+                    if (kGroups > 2 * kRpt && u2 > 0u && ok && !gt_wait(sm32(&tail.acc2_full[buf ^ 1u]), ((u2 - 1u) >> 1) & 1u)) ok = false;
                     if (ok && !gt_wait(sm32(&tail.acc2_full[buf]), use & 1u)) ok = false;
                     if (kEy == 1) {
                         if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
@@ -574,7 +585,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.kbytes = 128; p.planes = 1;
     p.small1 = (long long)row1 * HK * 128 * 128 <= (1 << 29) ? 1 : 0;
     p.small2 = (long long)wd1.O * 128 * 128 <= (1 << 29) ? 1 : 0;
-    const int staging = 8 * kGtStagingBytes, fixed = staging + (int)sizeof(CtTail);
+    const int fixed = ct_groups(false) * 4 * kGtStagingBytes + (int)sizeof(CtTail<2>);
     // kHalo: where two boxes of activations, the weights of layer one and at least two chunks of layer two's fit, and the
     // tiles with their border are not many more.  3x3 64->64 then 64->256 at 56x56, batch 64: 44.5 us loaded tap by tap.
     bool halo = false;
@@ -583,7 +594,9 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     if (HK > 1 && HK <= kCtTaps && p.cpt1 == 1 && p.sh == 1 && p.sw == 1 && p.db && Th.tiles > 0 && Th.tiles * 4 <= T.tiles * 5) {
         const int kb = row1 <= 32 ? 32 : (row1 <= 64 ? 64 : 128), planes = kb == 128 ? 1 : kb / 32;
         const int plane = (Th.Nt * (Th.Ht + wd1.H - 1) * (Th.Wt + wd1.K - 1) * (kb / planes) + 1023) / 1024 * 1024;
-        const int room = kCtSmem - fixed - p.n_c2 * kCtChunk - HK * p.O1p * kb - 2 * planes * plane;
+        p.staging_bytes = (uint32_t)(Th.Wt * Th.Ht * Th.Nt * 128 + 1023) / 1024 * 1024;
+        const int fixed_h = ct_groups(true) * (int)p.staging_bytes + (int)sizeof(CtTail<3>);
+        const int room = kCtSmem - fixed_h - p.n_c2 * kCtChunk - HK * p.O1p * kb - 2 * planes * plane;
         const int room2 = room - p.n_c2 * kCtChunk;          // with two buffers for T
         int want = p.n_t2 * p.n_c2;
         if (want > kCtW2Slots) want = kCtW2Slots;
@@ -610,9 +623,10 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
         p.a_bytes = T.Nt * p.halo_rows * p.halo_w * p.kbytes;
         p.stage_bytes = p.planes * p.plane_bytes;
         at = (size_t)HK * p.O1p * p.kbytes;
-        int stages = (kCtSmem - fixed - (p.dbt ? 2 : 1) * p.n_c2 * kCtChunk - (int)at - w2_slots * kCtBN2 * 128) / p.stage_bytes;
+        int stages = (kCtSmem - ct_groups(true) * (int)p.staging_bytes - (int)sizeof(CtTail<3>) - (p.dbt ? 2 : 1) * p.n_c2 * kCtChunk - (int)at - w2_slots * kCtBN2 * 128) / p.stage_bytes;
         p.stages = stages > 4 ? 4 : stages;
     } else {
+        p.staging_bytes = 4 * kGtStagingBytes;
         p.a_bytes = T.Wt * T.Ht * T.Nt * 128;
         p.stage_bytes = kGtABytes + p.O1p * 128;
         int stages = (kCtSmem - fixed - (p.dbt ? 2 : 1) * p.n_c2 * kCtChunk) / p.stage_bytes;
@@ -625,9 +639,9 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.off_ring = (uint32_t)at; at += (size_t)p.stages * p.stage_bytes;
     p.off_w2 = (uint32_t)at; at += (size_t)p.w2_slots * kCtBN2 * 128;
     p.off_t = (uint32_t)at; at += (size_t)(p.dbt ? 2 : 1) * p.n_c2 * kCtChunk;
-    p.off_staging = (uint32_t)at; at += staging;
+    p.off_staging = (uint32_t)at; at += (size_t)ct_groups(halo) * p.staging_bytes;
     p.off_tail = (uint32_t)at;
-    const size_t smem = at + sizeof(CtTail);
+    const size_t smem = at + (halo ? sizeof(CtTail<3>) : sizeof(CtTail<2>));
 
     // kernels by type of the pair, width of Y (32 bits or the narrow form) and kHalo
     typedef void (*Kernel)(const CtParams);
@@ -691,7 +705,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
             return BSP_ERR_CUDA;
     }
     const int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
-    BSP_CUDA_OK(launch_after(kernels[wd1.wtype == BSP_I8 ? 1 : 0][ey == 4 ? 0 : 1][halo ? 1 : 0], dim3((unsigned)grid), dim3(kCtThreads), smem, st, p));
+    BSP_CUDA_OK(launch_after(kernels[wd1.wtype == BSP_I8 ? 1 : 0][ey == 4 ? 0 : 1][halo ? 1 : 0], dim3((unsigned)grid), dim3(64u + 128u * ct_groups(halo)), smem, st, p));
     return BSP_OK;
 }
 

@@ -71,6 +71,7 @@ def test_requantised_output(O, case):
     (9, 7, 7, 16, 128, 200, 3, 3, 1),    # several images a tile, one plane of 32-byte rows, clipped channels
     (2, 17, 33, 40, 72, 64, 1, 7, 1),    # two chunks of T with a tail
     (1, 1, 300, 64, 48, 48, 1, 3, 0),    # T and Y narrower than a chunk
+    (12, 56, 56, 48, 64, 112, 3, 3, 1),  # two rounds a tile in the 8-bit form, many tiles a CTA
 ])
 def test_pair_equals_the_two_calls(N, L, J, I, O1, O2, H, K, relu):
     for dtype in ("bf16", "i8"):
