@@ -126,40 +126,6 @@ __device__ __forceinline__ int csr_fill_body(int l, int part, int parts, const T
     return cnt;
 }
 
-// Sixteen bytes of W[o][tap][ch0 ..] (16 / esz consecutive input channels of esz bytes each), with the channels of
-// zeroed blocks cleared; rows past O and taps past HK read as zero.  Needs 16-byte aligned rows of W.
-template <int esz>
-__device__ __forceinline__ uint4 w_chunk(const void *__restrict__ W, const uint8_t *gamma, int o, int tap, int ch0,
-                                         int O, int I, int HK, int bo, int bi, int NBi)
-{
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (o >= O || tap >= HK) return v;
-    const uint8_t *grow = gamma + (size_t)(o >> lg(bo)) * NBi;
-    constexpr int cpc = 16 / esz;
-    const int b0 = ch0 >> lg(bi);
-    if (bi >= cpc) {
-        if (grow[b0] == 0) return v;
-        return __ldg((const uint4 *)((const uint8_t *)W + (((size_t)o * HK + tap) * I + ch0) * esz));
-    }
-    const uint4 *src = (const uint4 *)((const uint8_t *)W + (((size_t)o * HK + tap) * I + ch0) * esz);
-    if (cpc == 8 || cpc / bi == 2) {                       // two blocks per chunk (always, for 8-channel chunks and b_i = 4)
-        const bool k0 = grow[b0] != 0, k1 = grow[b0 + 1] != 0;
-        if (!k0 && !k1) return v;
-        v = __ldg(src);
-        if (!k0) v.x = v.y = 0u;
-        if (!k1) v.z = v.w = 0u;
-        return v;
-    }
-    const bool k0 = grow[b0] != 0, k1 = grow[b0 + 1] != 0, k2 = grow[b0 + 2] != 0, k3 = grow[b0 + 3] != 0;   // four
-    if (!k0 && !k1 && !k2 && !k3) return v;
-    v = __ldg(src);
-    if (!k0) v.x = 0u;
-    if (!k1) v.y = 0u;
-    if (!k2) v.z = 0u;
-    if (!k3) v.w = 0u;
-    return v;
-}
-
 // Sum of v over the CTA's threads; every thread of the CTA must call it.
 __device__ __forceinline__ int block_sum(int v, int *warp_sums)
 {
@@ -210,46 +176,118 @@ __device__ __forceinline__ int ones_share_global(const uint8_t *__restrict__ g, 
     return c;
 }
 
-// The packed form: Gamma (.) W in the layout of W, [O][H][K][I], the channels of zeroed blocks cleared.  CTA `idx` of
-// `n_ctas` takes every n_ctas-th stretch of 16-byte chunks, one chunk of input channels per thread and step, four loads
-// in flight per thread.  A "row" below is one (o, tap).
+// The packed form: Gamma (.) W in the layout of W, [O][H][K][I], the channels of zeroed blocks cleared.  The b_o H K rows
+// (o, tap) of a row of Gamma share its entries, so a thread takes one 16-byte chunk of input channels of up to eight of
+// these rows: Gamma is read once, then the rows that are needed are loaded together.  (One chunk at a time, each behind its
+// own look at Gamma, took 16.9 us for 4096 x 4096 bf16; see compact_kernel for the figure now.)
+constexpr int kDenseRows = 8;
 template <int esz>
-__device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *__restrict__ W, const uint8_t *gamma, int O, int I,
-                                           int HK, int bo, int bi, int NBi, uint8_t *__restrict__ out)
+__device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *__restrict__ W, const uint8_t *__restrict__ gamma, int I, int HK, int bo, int bi,
+                                           int NBo, int NBi, uint8_t *__restrict__ out)
 {
     const bool aligned = (((uintptr_t)W) & 15u) == 0;
-    const int cpr = I * esz / 16;                     // chunks per row
-    constexpr int cpc = 16 / esz;
-    const long long total = (long long)O * HK * cpr, stride = (long long)n_ctas * kThreads;
+    constexpr int cpc = 16 / esz;                     // channels per chunk
+    const int cpr = I / cpc;                          // chunks per row
+    const int rows = bo * HK, groups = (rows + kDenseRows - 1) / kDenseRows;
+    const long long total = (long long)NBo * groups * cpr, stride = (long long)n_ctas * kThreads;
     const bool small = total < (1ll << 31);
-    for (long long e0 = (long long)idx * kThreads + threadIdx.x; e0 < total; e0 += 4 * stride) {
-        uint4 v[4];
+    for (long long e = (long long)idx * kThreads + threadIdx.x; e < total; e += stride) {
+        // (a 64-bit division costs an order of magnitude more than a 32-bit one: taken only by layers that need it)
+        const int lg_ = small ? (int)((unsigned)e / (unsigned)cpr) : (int)(e / cpr);
+        const int c = (int)(e - (long long)lg_ * cpr);
+        const int l = lg_ / groups, r0 = (lg_ - l * groups) * kDenseRows, n = min(kDenseRows, rows - r0);
+        // which 4-byte words of the chunk are kept (a word's channels lie in one block: b_i is a multiple of 4)
+        const uint8_t *g = gamma + (size_t)l * NBi + ((c * cpc) >> lg(bi));
+        uint32_t keep[4];
+        if (bi >= cpc) {
+            keep[0] = keep[1] = keep[2] = keep[3] = g[0] ? 0xFFFFFFFFu : 0u;
+        } else if (cpc / bi == 2) {
+            keep[0] = keep[1] = g[0] ? 0xFFFFFFFFu : 0u;
+            keep[2] = keep[3] = g[1] ? 0xFFFFFFFFu : 0u;
+        } else {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const long long e = e0 + u * stride;
-            if (e >= total) continue;
-            // (a 64-bit division costs an order of magnitude more than a 32-bit one: taken only by layers that need it)
-            const int ot = small ? (int)((unsigned)e / (unsigned)cpr) : (int)(e / cpr);
-            const int c = (int)(e - (long long)ot * cpr);
-            const int o = ot / HK, tap = ot - o * HK;
-            if (aligned) {
-                v[u] = w_chunk<esz>(W, gamma, o, tap, c * cpc, O, I, HK, bo, bi, NBi);
-            } else {
-                // W only 4-byte aligned: word by word (the channels of a word lie in one block: b_i is a multiple of 4)
-                uint32_t w[4];
-                for (int q = 0; q < 4; ++q) {
-                    const int ch = c * cpc + q * (4 / esz);
-                    const bool on = gamma[(size_t)(o >> lg(bo)) * NBi + (ch >> lg(bi))] != 0;
-                    w[q] = on ? *(const uint32_t *)((const uint8_t *)W + ((size_t)ot * I + ch) * esz) : 0u;
+            for (int q = 0; q < 4; ++q) keep[q] = g[q] ? 0xFFFFFFFFu : 0u;
+        }
+        const bool any = (keep[0] | keep[1] | keep[2] | keep[3]) != 0u;
+        const size_t pitch = (size_t)cpr * 16, at = ((size_t)l * rows + r0) * pitch + (size_t)c * 16;
+        const uint8_t *src = (const uint8_t *)W + at;
+        uint4 v[kDenseRows];
+#pragma unroll
+        for (int u = 0; u < kDenseRows; ++u) {
+            v[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (u < n && any) {
+                if (aligned) v[u] = __ldg((const uint4 *)(src + u * pitch));
+                else {                                // W only 4-byte aligned: word by word
+                    const uint32_t *s4 = (const uint32_t *)(src + u * pitch);
+                    v[u] = make_uint4(__ldg(s4), __ldg(s4 + 1), __ldg(s4 + 2), __ldg(s4 + 3));
                 }
-                v[u] = make_uint4(w[0], w[1], w[2], w[3]);
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const long long e = e0 + u * stride;
-            if (e < total) *(uint4 *)(out + e * 16) = v[u];
+        for (int u = 0; u < kDenseRows; ++u)
+            if (u < n) *(uint4 *)(out + at + u * pitch) = make_uint4(v[u].x & keep[0], v[u].y & keep[1], v[u].z & keep[2], v[u].w & keep[3]);
+    }
+}
+
+// Column indices and row pointers of kIndexRows rows of Gamma without a payload, one row per warp: the CTA counts the stored
+// blocks of all rows before its first one together (one count for eight rows instead of one for each: with 512 rows of 512
+// the counts read 67 MB and took 13 us), then every warp counts and lists its own row, 16 entries per lane and step.
+constexpr int kIndexRows = kThreads / 32;
+__device__ __forceinline__ void index_rows(int cta, const uint8_t *__restrict__ gamma, int NBo, int NBi, int32_t *__restrict__ row_ptr,
+                                           int32_t *__restrict__ col_idx, long long capacity_blocks, int *s_sum, int *status)
+{
+    __shared__ int s_cnt[kIndexRows];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l0 = cta * kIndexRows, l = l0 + warp;
+    const uint8_t *g = gamma + (size_t)l * NBi;
+    const bool wide = NBi % 16 == 0 && (((uintptr_t)gamma) & 15u) == 0;
+    // bit q of the result: entry i + q of the row is kept (i = 16 entries of this lane)
+    auto bits_of = [&](int i) -> unsigned {
+        unsigned m = 0u;
+        if (wide) {
+            if (i < NBi) {
+                const uint4 w = __ldg((const uint4 *)(g + i));
+                const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t one = __vsetne4(x[k], 0u);       // 1 in every non-zero byte
+                    m |= ((one | (one >> 7) | (one >> 14) | (one >> 21)) & 15u) << (4 * k);
+                }
+            }
+        } else {
+            for (int q = 0; q < 16 && i + q < NBi; ++q) m |= g[i + q] ? 1u << q : 0u;
         }
+        return m;
+    };
+    int cnt = 0;
+    if (l < NBo)
+        for (int i = lane * 16; i < NBi; i += 512) cnt += __popc(bits_of(i));
+    for (int d = 16; d > 0; d >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, d);
+    if (lane == 0) s_cnt[warp] = cnt;
+    int first = block_sum(ones_share_global(gamma, l0 * NBi), s_sum);      // (its barriers publish s_cnt too)
+    for (int w = 0; w < warp; ++w) first += s_cnt[w];
+    if (l >= NBo) return;
+    if (lane == 0) {
+        row_ptr[l] = first;
+        if (l == NBo - 1) {
+            row_ptr[NBo] = first + cnt;
+            if ((long long)(first + cnt) > capacity_blocks) atomicMax(status, (int)BSP_ERR_CAPACITY);
+        }
+    }
+    int at = first;
+    for (int base = 0; base < NBi; base += 512) {
+        const int i = base + lane * 16;
+        unsigned m = i < NBi ? bits_of(i) : 0u;
+        int inc = __popc(m);
+        const int mine = inc;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += o;
+        }
+        int n = at + inc - mine;
+        for (; m; m &= m - 1, ++n)
+            if ((long long)n < capacity_blocks) col_idx[n] = i + __ffs(m) - 1;
+        at += __shfl_sync(0xFFFFFFFFu, inc, 31);
     }
 }
 
@@ -257,12 +295,12 @@ struct CompactArgs {
     const void *W;
     const uint8_t *gamma;
     int O, I, HK, bo, bi, NBo, NBi;
-    const int32_t *row_ptr;           // multi-launch path: written by the scan launch
-    int32_t *row_ptr_out;             // single-launch path
+    int32_t *row_ptr_out;
     int32_t *col_idx;
     void *payload;
     long long capacity_blocks;
     int fill_parts;                   // CTAs per row of Gamma in the first part of the grid
+    int n_fill;                       // CTAs of the first part
     uint8_t *dense;                   // packed form (NULL: none)
     int dense_ctas;                   // CTAs of the second part of the grid
     PackedHeader *hdr;
@@ -283,13 +321,18 @@ __global__ void __launch_bounds__(kThreads, 5) compact_kernel(const CompactArgs 
     __shared__ __align__(16) uint8_t s_gamma[kBig ? 16 : kSmallBlocks];
     __shared__ int s_sum[kThreads / 32];
     wait_for_previous();
-    const int n_fill = a.NBo * a.fill_parts;
+    const int n_fill = a.n_fill;
     if ((int)blockIdx.x >= n_fill) {
         if ((int)blockIdx.x == n_fill && threadIdx.x == 0 && a.hdr != nullptr) *a.hdr = a.hdr_init;
         if (a.dense != nullptr)
-            dense_body<(int)sizeof(T)>((int)blockIdx.x - n_fill, a.dense_ctas, a.W, a.gamma, a.O, a.I, a.HK, a.bo, a.bi, a.NBi, a.dense);
+            dense_body<(int)sizeof(T)>((int)blockIdx.x - n_fill, a.dense_ctas, a.W, a.gamma, a.I, a.HK, a.bo, a.bi, a.NBo, a.NBi, a.dense);
         return;
     }
+    if constexpr (kBig)
+        if (a.payload == nullptr) {
+            index_rows((int)blockIdx.x, a.gamma, a.NBo, a.NBi, a.row_ptr_out, a.col_idx, a.capacity_blocks, s_sum, a.status);
+            return;
+        }
     const int l = (int)blockIdx.x / a.fill_parts, part = (int)blockIdx.x % a.fill_parts;
     int first;
     if constexpr (kBig) {
@@ -350,15 +393,15 @@ bsp_status launch_compact(const bsp_wdesc &wd, const void *W, const uint8_t *gam
 
     CompactArgs a = {};
     a.W = W; a.gamma = gamma; a.O = wd.O; a.I = wd.I; a.HK = HK; a.bo = wd.bo; a.bi = wd.bi; a.NBo = NBo; a.NBi = NBi;
-    a.row_ptr = row_ptr; a.row_ptr_out = row_ptr; a.col_idx = col_idx; a.payload = payload; a.capacity_blocks = capacity_blocks;
+    a.row_ptr_out = row_ptr; a.col_idx = col_idx; a.payload = payload; a.capacity_blocks = capacity_blocks;
     a.dense = dense_on ? pk + L.off_payload : nullptr;
     a.hdr = (PackedHeader *)pk; a.status = status;
     PackedHeader &h = a.hdr_init;
     h.magic = kPackedMagic; h.dtype = wd.wtype; h.O = wd.O; h.I = wd.I; h.H = wd.H; h.K = wd.K; h.bo = wd.bo; h.bi = wd.bi;
     h.forms = dense_on ? kFormDense : 0; h.off_payload = (int64_t)L.off_payload;
-    // packed form: four 16-byte chunks per thread and pass, at most 16 CTAs per SM's worth of CTAs
-    const long long chunks = dense_on ? (long long)wd.O * HK * wd.I * esz / 16 : 0;
-    long long dg = (chunks + 4LL * kThreads - 1) / (4LL * kThreads);
+    // packed form: a chunk of up to eight rows per thread and pass, at most 16 CTAs per SM's worth of CTAs
+    const long long units = dense_on ? (long long)NBo * ((wd.bo * HK + kDenseRows - 1) / kDenseRows) * (wd.I * esz / 16) : 0;
+    long long dg = (units + kThreads - 1) / kThreads;
     if (dg > 2368) dg = 2368;
     a.dense_ctas = dense_on ? (int)(dg < 1 ? 1 : dg) : (pk ? 1 : 0);      // (a packed buffer without the form still gets its header)
     const size_t smem = (size_t)NBi * sizeof(int);
@@ -371,7 +414,8 @@ bsp_status launch_compact(const bsp_wdesc &wd, const void *W, const uint8_t *gam
             const long long p = (row_pieces / 2 + 4LL * kThreads - 1) / (4LL * kThreads);
             a.fill_parts = (int)(p < 1 ? 1 : (p > 8 ? 8 : p));
         }
-        const unsigned grid = (unsigned)(NBo * a.fill_parts + a.dense_ctas);
+        a.n_fill = NBo * a.fill_parts;
+        const unsigned grid = (unsigned)(a.n_fill + a.dense_ctas);
         if (wd.wtype == BSP_I8) BSP_CUDA_OK(launch_after(compact_kernel<uint8_t, false>, dim3(grid), dim3(kThreads), smem, st, a));
         else if (wd.wtype == BSP_BF16) BSP_CUDA_OK(launch_after(compact_kernel<uint16_t, false>, dim3(grid), dim3(kThreads), smem, st, a));
         else BSP_CUDA_OK(launch_after(compact_kernel<uint32_t, false>, dim3(grid), dim3(kThreads), smem, st, a));
@@ -382,7 +426,8 @@ bsp_status launch_compact(const bsp_wdesc &wd, const void *W, const uint8_t *gam
     a.fill_parts = payload ? (296 + NBo - 1) / NBo : 1;
     if (a.fill_parts > 16) a.fill_parts = 16;
     if (a.fill_parts < 1) a.fill_parts = 1;
-    const unsigned grid = (unsigned)(NBo * a.fill_parts + a.dense_ctas);
+    a.n_fill = payload ? NBo * a.fill_parts : (NBo + kIndexRows - 1) / kIndexRows;
+    const unsigned grid = (unsigned)(a.n_fill + a.dense_ctas);
     if (wd.wtype == BSP_I8) BSP_CUDA_OK(launch_after(compact_kernel<uint8_t, true>, dim3(grid), dim3(kThreads), smem, st, a));
     else if (wd.wtype == BSP_BF16) BSP_CUDA_OK(launch_after(compact_kernel<uint16_t, true>, dim3(grid), dim3(kThreads), smem, st, a));
     else BSP_CUDA_OK(launch_after(compact_kernel<uint32_t, true>, dim3(grid), dim3(kThreads), smem, st, a));
