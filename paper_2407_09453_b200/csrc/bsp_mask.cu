@@ -381,49 +381,55 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync)
     return s_bar_ok != 0;
 }
 
-// The digit d of a 256-bin histogram with cum(d - 1) < need <= cum(d), found by the first warp: each lane sums eight
-// bins, a warp scan finds the lane, the lane walks its bins.  Writes the remaining count, the extended prefix and the
-// number of keys in the chosen bin; the caller synchronises the CTA afterwards.
-__device__ __forceinline__ void select_digit(const unsigned *hist, int tid, unsigned long long prefix, long long *s_k,
+// The digit d of a histogram of kBins bins with cum(d - 1) < need <= cum(d), by a CTA of kT threads: each sums kBins / kT
+// neighbouring bins, a scan over the CTA finds the thread that holds it.  Writes the remaining count, the extended prefix and
+// the number of keys in the chosen bin, and synchronises the CTA.
+template <int kT, int kBins>
+__device__ __forceinline__ void select_digit(const unsigned *hist, unsigned *warp_sums, unsigned long long prefix, long long *s_k,
                                              unsigned long long *s_prefix, unsigned *s_left, int width)
 {
-    if (tid >= 32) return;
+    constexpr int kPer = kBins / kT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long need = *s_k;
-    long long mine = 0;
+    unsigned h[kPer], mine = 0u;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) mine += hist[tid * 8 + q];
-    long long inc = mine;
+    for (int q = 0; q < kPer; ++q) { h[q] = hist[tid * kPer + q]; mine += h[q]; }
+    unsigned inc = mine;
 #pragma unroll
-    for (int dd = 1; dd < 32; dd <<= 1) {
-        const long long n = __shfl_up_sync(0xFFFFFFFFu, inc, dd);
-        if (tid >= dd) inc += n;
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned n = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+        if (lane >= d) inc += n;
     }
-    const unsigned reach = __ballot_sync(0xFFFFFFFFu, inc >= need);
-    const int owner = reach ? __ffs(reach) - 1 : 31;        // need <= total, so some lane reaches it
-    if (tid == owner) {
-        long long cum = inc - mine;
-        int d = tid * 8;
-        for (; d < tid * 8 + 7; ++d) {
-            if (cum + (long long)hist[d] >= need) break;
-            cum += hist[d];
+    if (lane == 31) warp_sums[warp] = inc;
+    __syncthreads();
+    long long cum = (long long)inc - mine;
+    for (int w = 0; w < warp; ++w) cum += warp_sums[w];
+    if (cum < need && need <= cum + mine) {                // (need <= the sum of all bins: one thread)
+        int q = 0;
+        for (; q < kPer - 1; ++q) {
+            if (cum + h[q] >= need) break;
+            cum += h[q];
         }
         *s_k = need - cum;
-        *s_prefix = (prefix << width) | (unsigned long long)d;
-        *s_left = hist[d];
+        *s_prefix = (prefix << width) | (unsigned long long)(tid * kPer + q);
+        *s_left = h[q];
     }
+    __syncthreads();
 }
 
 // The radix select of select_kernel for one large segment (the whole layer), spread over a cooperative grid:
-// CTA c owns a contiguous slice of the keys.  Each of the eight passes adds the CTAs' digit histograms into
-// ghist[pass][256] (zeroed by the host before the launch), the CTAs meet at the grid barrier, and every CTA
+// CTA c owns a contiguous slice of the keys.  Each pass adds the CTAs' digit histograms into
+// ghist[pass][kCoopBins] (zeroed by the host before the launch), the CTAs meet at the grid barrier, and every CTA
 // derives the digit for itself.  Keys equal to the threshold T are zeroed lowest index first: the CTAs publish
 // how many such keys their slices hold (geq[c]), meet again, and each counts those in the slices before its own.
 constexpr int kCoopThreads = 512;
+constexpr int kCoopWidth = 10, kCoopBins = 1 << kCoopWidth;      // digit of a grid-wide pass
+static_assert(7 * kCoopBins == kSelectHist, "a histogram for each digit of a 64-bit key");
 constexpr int kLocalMax = 8192;          // candidates that the CTAs finish on their own, in (dynamic) shared memory
 
 // The select starts at the highest bit in which any two keys differ (the score kernel leaves the OR of all keys in
 // gcount[2..3] and the OR of their complements in gcount[4..5]: the bits above it are the same in every key, e.g. the
-// sign and most of the exponent of float scores, or the leading zero bytes of integer ones) and takes digits of eight
+// sign and most of the exponent of float scores, or the leading zero bytes of integer ones) and takes digits of ten
 // bits downwards.  Passes run grid-wide (global histograms, a grid barrier
 // each) only while more than kLocalMax keys still match the prefix; then the CTAs append their matching keys to one
 // list (`cand`, counted in gcount[0], zeroed by the host with the histograms), meet
@@ -435,7 +441,7 @@ __global__ void __launch_bounds__(kCoopThreads)
 select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long long n_zero, uint8_t *__restrict__ gamma,
                    unsigned *ghist, unsigned *gcount, unsigned long long *cand, unsigned *geq, unsigned *sync, int *status)
 {
-    __shared__ unsigned hist[256];
+    __shared__ unsigned hist[kCoopBins], warp_sums[kCoopThreads / 32];
     extern __shared__ unsigned long long s_dyn[];
     unsigned long long *s_cand = s_dyn;                  // [kLocalMax]
     unsigned long long *s_keys = s_dyn + kLocalMax;      // [kSliceMax]
@@ -463,23 +469,23 @@ select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long
     if (tid == 0) { s_prefix = top >= 63 ? 0ull : (k0 >> (top + 1)); s_k = n_zero; s_left = n > 0xFFFFFFFFll ? 0xFFFFFFFFu : (unsigned)n; }
     int pi = 0;
     while (top >= 0) {
-        if (tid < 256) hist[tid] = 0u;
+        for (int q = tid; q < kCoopBins; q += kCoopThreads) hist[q] = 0u;
         __syncthreads();
         if (s_left <= (unsigned)kLocalMax) break;          // few enough candidates: the rest is local
         const unsigned long long prefix = s_prefix;
-        const int width = min(8, top + 1), shift = top + 1 - width;
+        const int width = min(kCoopWidth, top + 1), shift = top + 1 - width;
         const unsigned dmask = (1u << width) - 1u;
         for (int i = tid; i < len; i += kCoopThreads) {
             const unsigned long long v = ks[i];
             if (top >= 63 || ((v >> (top + 1)) == prefix)) atomicAdd(&hist[(unsigned)(v >> shift) & dmask], 1u);
         }
         __syncthreads();
-        if (tid < 256 && hist[tid]) atomicAdd(&ghist[pi * 256 + tid], hist[tid]);
+        for (int q = tid; q < kCoopBins; q += kCoopThreads)
+            if (hist[q]) atomicAdd(&ghist[pi * kCoopBins + q], hist[q]);
         if (!grid_barrier(sync)) { if (tid == 0) atomicMax(status, (int)BSP_ERR_TIMEOUT); return; }
-        if (tid < 256) hist[tid] = __ldcg(&ghist[pi * 256 + tid]);
+        for (int q = tid; q < kCoopBins; q += kCoopThreads) hist[q] = __ldcg(&ghist[pi * kCoopBins + q]);
         __syncthreads();
-        select_digit(hist, tid, prefix, &s_k, &s_prefix, &s_left, width);
-        __syncthreads();
+        select_digit<kCoopThreads, kCoopBins>(hist, warp_sums, prefix, &s_k, &s_prefix, &s_left, width);
         top -= width;
         ++pi;
     }
@@ -503,10 +509,10 @@ select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long
         __syncthreads();
         constexpr int kMine = kLocalMax / kCoopThreads;    // candidates per thread
         while (top >= 0 && cnt > (unsigned)kCoopThreads) {
-            if (tid < 256) hist[tid] = 0u;
+            for (int q = tid; q < kCoopBins; q += kCoopThreads) hist[q] = 0u;
             if (tid == 0) s_n = 0u;
             __syncthreads();
-            const int width = min(8, top + 1), shift = top + 1 - width;
+            const int width = min(kCoopWidth, top + 1), shift = top + 1 - width;
             const unsigned dmask = (1u << width) - 1u;
             // every candidate matches the prefix so far (the list is thinned after each digit)
             unsigned long long mine[kMine];
@@ -517,8 +523,7 @@ select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long
                 if (i < cnt) atomicAdd(&hist[(unsigned)(mine[u] >> shift) & dmask], 1u);
             }
             __syncthreads();
-            select_digit(hist, tid, s_prefix, &s_k, &s_prefix, &s_left, width);
-            __syncthreads();
+            select_digit<kCoopThreads, kCoopBins>(hist, warp_sums, s_prefix, &s_k, &s_prefix, &s_left, width);
             top -= width;
             // keep the candidates of the chosen digit (all were read into registers above)
             const unsigned long long pre = s_prefix;
@@ -600,30 +605,32 @@ select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long
     }
 }
 
-// Select within one CTA of 256 threads, for segments of up to kRankMax keys: key u * 256 + t of the segment is v[u] of thread
-// t.  Most-significant-digit radix passes in shared memory from the highest bit in which two keys differ, until at most
+// Select within one CTA, for segments of up to 16 keys a thread: key u * kT + t of the segment is v[u] of thread t.  Most-significant-digit radix passes in shared memory from the highest bit in which two keys differ, until at most
 // kFew keys match the prefix; those are ranked directly.  `T` is the threshold key, `ties` how many keys equal to it are
 // still to be zeroed (lowest index first), `same` how many there are.  0 < n_zero < n; every thread must call it.
 // (Counting the smaller keys of every key instead, 4096 of them, took 10 us of the 15.5 of a 512x512 3x3 layer.)
 constexpr int kRankMax = 4096;
 constexpr int kKeysPerThread = kRankMax / kScoreThreads;
 constexpr int kFew = 128;
+template <int kT>
 struct SmallSelect {
-    unsigned hist[256];
+    static constexpr int kBins = 4 * kT, kWidth = kT == 256 ? 10 : 12;     // digits wide enough that one pass usually leaves a few keys
+    unsigned hist[kBins], warp_sums[kT / 32];
     unsigned long long cand[kFew];
     unsigned long long prefix;
     long long k;
     unsigned left, n;
-    unsigned bits[4][kScoreThreads / 32];
+    unsigned bits[4][kT / 32];
 };
-__device__ __forceinline__ void select_small(const unsigned long long (&v)[kKeysPerThread], int n, long long n_zero, SmallSelect &sh,
+template <int kT>
+__device__ __forceinline__ void select_small(const unsigned long long (&v)[kKeysPerThread], int n, long long n_zero, SmallSelect<kT> &sh,
                                              unsigned long long &T, long long &ties, unsigned &same)
 {
     const int tid = threadIdx.x;
     unsigned long long or1 = 0ull, or0 = 0ull;
 #pragma unroll
     for (int u = 0; u < kKeysPerThread; ++u)
-        if (u * kScoreThreads + tid < n) { or1 |= v[u]; or0 |= ~v[u]; }
+        if (u * kT + tid < n) { or1 |= v[u]; or0 |= ~v[u]; }
     const unsigned w[4] = {(unsigned)or1, (unsigned)(or1 >> 32), (unsigned)or0, (unsigned)(or0 >> 32)};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -636,7 +643,7 @@ __device__ __forceinline__ void select_small(const unsigned long long (&v)[kKeys
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int o = 0; o < kScoreThreads / 32; ++o) m[q] |= sh.bits[q][o];
+        for (int o = 0; o < kT / 32; ++o) m[q] |= sh.bits[q][o];
     const unsigned long long ones = ((unsigned long long)m[1] << 32) | m[0], diff = ones & (((unsigned long long)m[3] << 32) | m[2]);
     int top = diff ? 63 - __clzll((long long)diff) : -1;
     // (bits above `top` are common to all keys: those of the OR)
@@ -644,16 +651,16 @@ __device__ __forceinline__ void select_small(const unsigned long long (&v)[kKeys
     unsigned left = (unsigned)n;
     if (top < 0 && tid == 0) sh.prefix = prefix;
     while (top >= 0 && left > (unsigned)kFew) {
-        sh.hist[tid] = 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sh.hist[q * kT + tid] = 0u;
         __syncthreads();
-        const int width = min(8, top + 1), shift = top + 1 - width;
+        const int width = min(SmallSelect<kT>::kWidth, top + 1), shift = top + 1 - width;
         const unsigned dmask = (1u << width) - 1u;
 #pragma unroll
         for (int u = 0; u < kKeysPerThread; ++u)
-            if (u * kScoreThreads + tid < n && (top >= 63 || (v[u] >> (top + 1)) == prefix)) atomicAdd(&sh.hist[(unsigned)(v[u] >> shift) & dmask], 1u);
+            if (u * kT + tid < n && (top >= 63 || (v[u] >> (top + 1)) == prefix)) atomicAdd(&sh.hist[(unsigned)(v[u] >> shift) & dmask], 1u);
         __syncthreads();
-        select_digit(sh.hist, tid, prefix, &sh.k, &sh.prefix, &sh.left, width);
-        __syncthreads();
+        select_digit<kT, SmallSelect<kT>::kBins>(sh.hist, sh.warp_sums, prefix, &sh.k, &sh.prefix, &sh.left, width);
         prefix = sh.prefix;
         left = sh.left;
         top -= width;
@@ -661,7 +668,7 @@ __device__ __forceinline__ void select_small(const unsigned long long (&v)[kKeys
     if (top >= 0) {
 #pragma unroll
         for (int u = 0; u < kKeysPerThread; ++u)
-            if (u * kScoreThreads + tid < n && (top >= 63 || (v[u] >> (top + 1)) == prefix)) sh.cand[atomicAdd(&sh.n, 1u)] = v[u];
+            if (u * kT + tid < n && (top >= 63 || (v[u] >> (top + 1)) == prefix)) sh.cand[atomicAdd(&sh.n, 1u)] = v[u];
         __syncthreads();
         const unsigned cnt = sh.n;
         const long long need = sh.k;
@@ -685,12 +692,12 @@ __device__ __forceinline__ void select_small(const unsigned long long (&v)[kKeys
 }
 
 // Loads the keys of a segment into registers (all loads are issued before the first is used, so they share one trip to memory).
-template <bool kThroughL2>
+template <bool kThroughL2, int kT = kScoreThreads>
 __device__ __forceinline__ void load_keys(const unsigned long long *k, int n, unsigned long long (&v)[kKeysPerThread])
 {
 #pragma unroll
     for (int u = 0; u < kKeysPerThread; ++u) {
-        const int i = u * kScoreThreads + threadIdx.x;
+        const int i = u * kT + threadIdx.x;
         v[u] = i < n ? (kThroughL2 ? __ldcg(k + i) : __ldg(k + i)) : 0ull;
     }
 }
@@ -700,7 +707,7 @@ __device__ __forceinline__ void load_keys(const unsigned long long *k, int n, un
 __global__ void __launch_bounds__(kScoreThreads)
 segment_kernel(const unsigned long long *__restrict__ key, int n, long long n_zero, uint8_t *__restrict__ gamma)
 {
-    __shared__ SmallSelect sh;
+    __shared__ SmallSelect<kScoreThreads> sh;
     __shared__ unsigned long long s_key[kScoreThreads];
     const unsigned long long *k = key + (size_t)blockIdx.x * n;
     uint8_t *g = gamma + (size_t)blockIdx.x * n;
@@ -748,6 +755,41 @@ segment_kernel(const unsigned long long *__restrict__ key, int n, long long n_ze
     }
 }
 
+// One segment of up to kMidMax keys: every CTA finds the threshold for itself, on all keys, and writes 1024 entries of Gamma.
+// (16384 keys on the cooperative kernel below, with its three grid barriers: 12.3 us.)
+constexpr int kMidThreads = 1024;
+constexpr int kMidMax = kMidThreads * kKeysPerThread;
+__global__ void __launch_bounds__(kMidThreads)
+select_mid_kernel(const unsigned long long *__restrict__ key, int n, long long n_zero, uint8_t *__restrict__ gamma)
+{
+    __shared__ SmallSelect<kMidThreads> sh;
+    const int tid = threadIdx.x, i = blockIdx.x * kMidThreads + tid;
+    if (n_zero <= 0 || n_zero >= n) {
+        if (i < n) gamma[i] = n_zero <= 0 ? 1 : 0;
+        return;
+    }
+    unsigned long long v[kKeysPerThread], T;
+    long long ties;
+    unsigned same;
+    load_keys<false, kMidThreads>(key, n, v);
+    const unsigned long long mine = i < n ? __ldg(key + i) : ~0ull;
+    select_small(v, n, n_zero, sh, T, ties, same);
+    long long rank = 0;                                    // keys equal to T before this one
+    const bool eq = i < n && mine == T;
+    if ((long long)same != ties) {                         // (else every key equal to T is zeroed)
+        unsigned before = 0u;
+#pragma unroll
+        for (int u = 0; u < kKeysPerThread; ++u) before += u < (int)blockIdx.x && u * kMidThreads + tid < n && v[u] == T ? 1u : 0u;
+        before = __reduce_add_sync(0xFFFFFFFFu, before);
+        const unsigned ball = __ballot_sync(0xFFFFFFFFu, eq);
+        if ((tid & 31) == 0) { sh.hist[tid >> 5] = before; sh.hist[32 + (tid >> 5)] = (unsigned)__popc(ball); }
+        __syncthreads();
+        rank = __popc(ball & ((1u << (tid & 31)) - 1u));
+        for (int w = 0; w < kMidThreads / 32; ++w) rank += sh.hist[w] + (w < (tid >> 5) ? sh.hist[32 + w] : 0u);
+    }
+    if (i < n) gamma[i] = (mine < T || (eq && rank < ties)) ? 0 : 1;
+}
+
 // Layers of up to kRankMax blocks: scores and Gamma in ONE cooperative launch.  Every CTA scores its blocks, the CTAs meet at
 // a grid-wide barrier, then every CTA decides its own blocks: by the select above (each CTA for itself, on all keys) for a
 // layer-wide scope, by counting the smaller keys of the segment for short segments.  The barrier is two words: arrivals
@@ -764,7 +806,7 @@ mask_small_kernel(const uint32_t *__restrict__ W, int I, int HK, int bo, int bi,
     using acc_t = typename Acc<DT>::type;
     __shared__ acc_t part[kScoreThreads];
     __shared__ unsigned long long s_key[kRankMax];
-    __shared__ SmallSelect sh;
+    __shared__ SmallSelect<kScoreThreads> sh;
     const int NB = NBo * NBi;
     // BC blocks per CTA: b_o threads score one block, then 256 / BC lanes rank one key
     {
@@ -924,16 +966,18 @@ bsp_status launch_mask(const bsp_wdesc &wd, const void *W, bsp_norm norm, bsp_sc
     const unsigned nseg = (scope == BSP_SCOPE_LAYER) ? 1u : (unsigned)NBo;
     // one large segment: the select runs on a cooperative grid; its histograms, counter and the span of the keys (filled
     // by the score kernel) are zeroed first
-    const bool coop = ws != nullptr && nseg == 1 && seg > kRankMax && n_zero > 0 && n_zero < seg;
+    const bool coop = ws != nullptr && nseg == 1 && seg > kMidMax && n_zero > 0 && n_zero < seg;
     unsigned *ghist = coop ? (unsigned *)((char *)ws + kWsHeader + align_up((size_t)NB * 8, 256)) : nullptr;
-    unsigned *gcount = coop ? ghist + 8 * 256 : nullptr;     // [0] candidate counter, [2..3] OR of the keys, [4..5] OR of their complements
-    if (coop) BSP_CUDA_OK(cudaMemsetAsync(ghist, 0, (8 * 256 + 8) * sizeof(unsigned), st));
+    unsigned *gcount = coop ? ghist + kSelectHist : nullptr;     // [0] candidate counter, [2..3] OR of the keys, [4..5] OR of their complements
+    if (coop) BSP_CUDA_OK(cudaMemsetAsync(ghist, 0, (kSelectHist + 8) * sizeof(unsigned), st));
     unsigned long long *span = coop ? (unsigned long long *)(gcount + 2) : nullptr;
     if (wd.wtype == BSP_F32) rc = run_scores<BSP_F32>(wd, W, norm, scores, span, st);
     else if (wd.wtype == BSP_BF16) rc = run_scores<BSP_BF16>(wd, W, norm, scores, span, st);
     else rc = run_scores<BSP_I8>(wd, W, norm, scores, span, st);
     if (rc != BSP_OK) return rc;
-    if (seg <= kRankMax)
+    if (nseg == 1 && seg > kRankMax && seg <= kMidMax)
+        select_mid_kernel<<<(unsigned)((seg + kMidThreads - 1) / kMidThreads), kMidThreads, 0, st>>>((const unsigned long long *)scores, (int)seg, n_zero, gamma);
+    else if (seg <= kRankMax)
         segment_kernel<<<nseg, kScoreThreads, 0, st>>>((const unsigned long long *)scores, (int)seg, n_zero, gamma);
     else if (coop) {
         // at most one CTA per SM
