@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libbsp.so: same names as the C ABI (include/bsp.h), argument marshalling only.
+"""Thin binding of libbsp.so: same names as the C ABI (include/bsp.h), argument marshalling only.  The calls that a
+program repeats are marshalled by csrc/bsp_call.cpp, the others by ctypes.
 
 Every function takes torch CUDA tensors (device memory and streams are PyTorch's), passes raw device
 pointers to the library and raises ``BspError`` on a non-zero status.  All arithmetic runs in the CUDA
@@ -47,13 +48,15 @@ class Bcsr(C.Structure):
 
 
 # Argument types of the calls that return a status, one letter per argument: p pointer, i int, l int64.  Declared types let
-# the calls below pass plain Python integers and None, which costs a fraction of building a ctypes object per argument
-# (a product call of a few microseconds on the GPU was bound by that).
+# the calls below pass plain Python integers and None, which costs a fraction of building a ctypes object per argument.
 _ARG = {"p": C.c_void_p, "i": C.c_int, "l": C.c_int64}
 _ARGS = {"bsp_mask": "ppiilpppp", "bsp_mask_static": "ppiilpp", "bsp_compact_nnz": "ppppp", "bsp_compact": "pppppppl" "pp",
          "bsp_gemm": "ppplppipp", "bsp_conv2d": "ppppppipp", "bsp_gemm_q8": "ppplppppp", "bsp_conv2d_q8": "ppppppppp",
          "bsp_conv2d_chain": "ppppppp" "ippipp", "bsp_conv2d_chain_q8": "pppppppp" "ippppp", "bsp_spgemm": "ppppppp",
          "bsp_index_to_relative": "ipppp", "bsp_index_from_relative": "ipppp", "bsp_check": "pp"}
+# The functions that csrc/bsp_call.cpp calls, in the order in which it takes their addresses.
+_BOUND = ["bsp_mask", "bsp_compact", "bsp_gemm", "bsp_conv2d", "bsp_gemm_q8", "bsp_conv2d_q8", "bsp_conv2d_chain",
+          "bsp_conv2d_chain_q8", "bsp_spgemm"]
 
 _lib = None
 
@@ -76,6 +79,24 @@ def lib():
             getattr(L, n).argtypes = [_ARG[c] for c in a]
         _lib = L
     return _lib
+
+
+_calls = None
+
+
+def _native():
+    """The compiled marshalling (csrc/bsp_call.cpp), bound to the functions of the loaded library; no fallback if absent."""
+    global _calls
+    if _calls is None:
+        L = lib()
+        try:
+            from . import _bspcall
+        except ImportError as e:
+            raise RuntimeError("_bspcall.so is missing or of another PyTorch: run `python -m paper_2407_09453_b200.build` "
+                               f"(or __graft_entry__.build()): {e}") from e
+        _bspcall.bind(*[C.cast(getattr(L, n), C.c_void_p).value for n in _BOUND])
+        _calls = _bspcall
+    return _calls
 
 
 def status_string(status: int) -> str:
@@ -126,8 +147,7 @@ def bsp_mask_workspace_bytes(wd: WDesc) -> int:
 
 
 def bsp_mask(wd: WDesc, W, norm, scope, n_zero, gamma, scores_opt, ws, stream=None):
-    _raise(lib().bsp_mask(C.byref(wd), _ptr(W), norm, scope, n_zero, _ptr(gamma),
-                          _ptr(scores_opt), _ptr(ws), _stream(stream)), "bsp_mask")
+    _raise(_native().mask(wd, W, norm, scope, n_zero, gamma, scores_opt, ws, stream), "bsp_mask")
 
 
 def bsp_packed_bytes(wd: WDesc, nnz: int) -> int:
@@ -146,12 +166,13 @@ def bsp_compact_nnz(wd: WDesc, gamma, ws, stream=None) -> int:
 
 
 def bsp_compact(wd: WDesc, W, gamma, row_ptr, col_idx, payload, packed, capacity_blocks, ws, stream=None):
-    _raise(lib().bsp_compact(C.byref(wd), _ptr(W), _ptr(gamma), _ptr(row_ptr), _ptr(col_idx), _ptr(payload),
-                             _ptr(packed), capacity_blocks, _ptr(ws), _stream(stream)), "bsp_compact")
+    _raise(_native().compact(wd, W, gamma, row_ptr, col_idx, payload, packed, capacity_blocks, ws, stream), "bsp_compact")
 
 
 def bcsr(row_ptr, col_idx, payload, packed, nnz) -> Bcsr:
-    return Bcsr(_ptr(row_ptr), _ptr(col_idx), _ptr(payload), _ptr(packed), int(nnz))
+    w = Bcsr()
+    _native().fill_handle(w, row_ptr, col_idx, payload, packed, int(nnz))
+    return w
 
 
 def bsp_conv_workspace_bytes(wd: WDesc, xd: XDesc) -> int:
@@ -159,39 +180,32 @@ def bsp_conv_workspace_bytes(wd: WDesc, xd: XDesc) -> int:
 
 
 def bsp_gemm(wd: WDesc, w: Bcsr, X, P, bias, Y, ytype, ws, stream=None):
-    _raise(lib().bsp_gemm(C.byref(wd), C.byref(w), _ptr(X), P, _ptr(bias), _ptr(Y), ytype,
-                          _ptr(ws), _stream(stream)), "bsp_gemm")
+    _raise(_native().gemm(wd, w, X, P, bias, Y, ytype, ws, stream), "bsp_gemm")
 
 
 def bsp_conv2d(wd: WDesc, w: Bcsr, xd: XDesc, X, bias, Y, ytype, ws, stream=None):
-    _raise(lib().bsp_conv2d(C.byref(wd), C.byref(w), C.byref(xd), _ptr(X), _ptr(bias), _ptr(Y), ytype,
-                            _ptr(ws), _stream(stream)), "bsp_conv2d")
+    _raise(_native().conv2d(wd, w, xd, X, bias, Y, ytype, ws, stream), "bsp_conv2d")
 
 
 def bsp_conv2d_q8(wd: WDesc, w: Bcsr, xd: XDesc, X, bias, shift, Y, ws, stream=None):
-    _raise(lib().bsp_conv2d_q8(C.byref(wd), C.byref(w), C.byref(xd), _ptr(X), _ptr(bias), _ptr(shift), _ptr(Y), _ptr(ws),
-                               _stream(stream)), "bsp_conv2d_q8")
+    _raise(_native().conv2d_q8(wd, w, xd, X, bias, shift, Y, ws, stream), "bsp_conv2d_q8")
 
 
 def bsp_gemm_q8(wd: WDesc, w: Bcsr, X, P, bias, shift, Y, ws, stream=None):
-    _raise(lib().bsp_gemm_q8(C.byref(wd), C.byref(w), _ptr(X), P, _ptr(bias), _ptr(shift), _ptr(Y), _ptr(ws),
-                             _stream(stream)), "bsp_gemm_q8")
+    _raise(_native().gemm_q8(wd, w, X, P, bias, shift, Y, ws, stream), "bsp_gemm_q8")
 
 
 def bsp_conv2d_chain(wd1: WDesc, w1: Bcsr, wd2: WDesc, w2: Bcsr, xd: XDesc, X, bias1, relu, bias2, Y, ytype, ws, stream=None):
-    _raise(lib().bsp_conv2d_chain(C.byref(wd1), C.byref(w1), C.byref(wd2), C.byref(w2), C.byref(xd), _ptr(X), _ptr(bias1),
-                                  1 if relu else 0, _ptr(bias2), _ptr(Y), ytype, _ptr(ws), _stream(stream)),
-           "bsp_conv2d_chain")
+    _raise(_native().conv2d_chain(wd1, w1, wd2, w2, xd, X, bias1, 1 if relu else 0, bias2, Y, ytype, ws, stream), "bsp_conv2d_chain")
 
 
 def bsp_conv2d_chain_q8(wd1: WDesc, w1: Bcsr, wd2: WDesc, w2: Bcsr, xd: XDesc, X, bias1, shift1, relu, bias2, shift2, Y, ws, stream=None):
-    _raise(lib().bsp_conv2d_chain_q8(C.byref(wd1), C.byref(w1), C.byref(wd2), C.byref(w2), C.byref(xd), _ptr(X), _ptr(bias1),
-                                     _ptr(shift1), 1 if relu else 0, _ptr(bias2), _ptr(shift2), _ptr(Y), _ptr(ws),
-                                     _stream(stream)), "bsp_conv2d_chain_q8")
+    _raise(_native().conv2d_chain_q8(wd1, w1, wd2, w2, xd, X, bias1, shift1, 1 if relu else 0, bias2, shift2, Y, ws, stream),
+           "bsp_conv2d_chain_q8")
 
 
 def bsp_spgemm(wa: WDesc, a: Bcsr, wb: WDesc, b: Bcsr, Cm, ws, stream=None):
-    _raise(lib().bsp_spgemm(C.byref(wa), C.byref(a), C.byref(wb), C.byref(b), _ptr(Cm), _ptr(ws), _stream(stream)), "bsp_spgemm")
+    _raise(_native().spgemm(wa, a, wb, b, Cm, ws, stream), "bsp_spgemm")
 
 
 def bsp_index_to_relative(NBo, row_ptr, col_idx, rel, stream=None):
@@ -261,20 +275,20 @@ class SparseLayer:
         return bcsr(self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity))
 
     def conv2d(self, X, bias, Y, stride=(1, 1), pad=(0, 0), stream=None):
-        N, L, J, _ = X.shape
-        xd = XDesc(N, L, J, stride[0], stride[1], pad[0], pad[1])
-        bsp_conv2d(self.wd, self.handle(), xd, X, bias, Y, dtype_code(Y.dtype), self.ws, stream)
+        _raise(_native().layer_conv2d(False, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
+                                      X, bias, None, Y, stride[0], stride[1], pad[0], pad[1], self.ws, stream), "bsp_conv2d")
 
     def gemm(self, X, bias, Y, stream=None):
-        bsp_gemm(self.wd, self.handle(), X, X.shape[0], bias, Y, dtype_code(Y.dtype), self.ws, stream)
+        _raise(_native().layer_gemm(False, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
+                                    X, bias, None, Y, self.ws, stream), "bsp_gemm")
 
     def conv2d_q8(self, X, bias, shift, Y, stride=(1, 1), pad=(0, 0), stream=None):
-        N, L, J, _ = X.shape
-        xd = XDesc(N, L, J, stride[0], stride[1], pad[0], pad[1])
-        bsp_conv2d_q8(self.wd, self.handle(), xd, X, bias, shift, Y, self.ws, stream)
+        _raise(_native().layer_conv2d(True, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
+                                      X, bias, shift, Y, stride[0], stride[1], pad[0], pad[1], self.ws, stream), "bsp_conv2d_q8")
 
     def gemm_q8(self, X, bias, shift, Y, stream=None):
-        bsp_gemm_q8(self.wd, self.handle(), X, X.shape[0], bias, shift, Y, self.ws, stream)
+        _raise(_native().layer_gemm(True, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
+                                    X, bias, shift, Y, self.ws, stream), "bsp_gemm_q8")
 
     def check(self, stream=None):
         bsp_check(self.ws, stream)

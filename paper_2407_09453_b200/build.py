@@ -1,7 +1,8 @@
 """Builds libbsp.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
 
 Every .cu under csrc/ is compiled to an object of its own (in parallel, rebuilt only when it or a header is
-newer) under _build/, then the objects are linked into paper_2407_09453_b200/libbsp.so.
+newer) under _build/, then the objects are linked into paper_2407_09453_b200/libbsp.so.  The marshalling of the Python
+calls, csrc/bsp_call.cpp, is compiled by the host compiler into paper_2407_09453_b200/_bspcall.so.
 """
 from __future__ import annotations
 
@@ -9,6 +10,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -16,6 +18,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libbsp.so")
+CALL_SOURCE = os.path.join(CSRC, "bsp_call.cpp")
+CALL = os.path.join(HERE, "_bspcall.so")
 
 
 def sources():
@@ -45,8 +49,25 @@ def _flags(verbose: bool):
     return f
 
 
+def build_call(force: bool = False) -> str:
+    """Compile the marshalling of the Python calls against the installed Python and PyTorch; returns its path."""
+    if not force and not _newer([CALL_SOURCE] + _headers(), CALL):
+        return CALL
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    include = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(root, "include"), os.path.join(cuda, "include")]
+    tmp = CALL + ".tmp%d" % os.getpid()
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi())] + ["-I" + d for d in include] +
+                          [CALL_SOURCE, "-o", tmp, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-lc10", "-lc10_cuda"])
+    os.replace(tmp, CALL)
+    return CALL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ and link them into one shared library; returns its path."""
+    """Compile every .cu under csrc/ and link them into one shared library; returns its path.  Builds the marshalling too."""
+    build_call(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

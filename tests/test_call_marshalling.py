@@ -1,0 +1,65 @@
+"""The compiled marshalling of the Python calls (csrc/bsp_call.cpp): every argument arrives as the C ABI declares it, wrong
+kinds raise, and refused calls give the library's own status.  No call here reaches a launch."""
+import pytest
+import torch
+
+from paper_2407_09453_b200 import bsp, build
+
+
+class Stream:
+    cuda_stream = 0
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    build.build()
+
+
+def buffers():
+    return torch.zeros(64, dtype=torch.int32), torch.zeros(64, dtype=torch.bfloat16)
+
+
+@pytest.mark.parametrize("nnz", [0, 1, 2 ** 31 + 5])
+def test_handle_fields(nnz):
+    i, p = buffers()
+    h = bsp.bcsr(i, i[1:], None, torch.nn.Parameter(p), nnz)
+    assert (h.row_ptr, h.col_idx, h.payload, h.packed, h.nnz) == (i.data_ptr(), i.data_ptr() + 4, None, p.data_ptr(), nnz)
+
+
+def test_refused_calls_give_the_status_of_the_library():
+    i, p = buffers()
+    wd, h, xd = bsp.wdesc(64, 64, 1, 1, 8, 8, bsp.BF16), bsp.bcsr(i, i, p, p, 8), bsp.XDesc(1, 1, 1, 1, 1, 0, 0)
+    x, s = torch.zeros(4, 64, dtype=torch.bfloat16), Stream()
+    lay = bsp.SparseLayer(64, 64, 1, 1, 8, 8, torch.bfloat16, device="cpu")
+    y = torch.zeros(4, 64)
+    calls = [(bsp.ERR_NULL, lambda: bsp.bsp_gemm(wd, h, None, 4, None, y, bsp.F32, p, s)),
+             (bsp.ERR_DTYPE, lambda: bsp.bsp_gemm(wd, h, x, 4, None, y, bsp.I32, p, s)),
+             (bsp.ERR_DTYPE, lambda: bsp.bsp_conv2d(wd, h, xd, x, None, y, bsp.I32, p, s)),
+             (bsp.ERR_NULL, lambda: bsp.bsp_mask(wd, None, 0, 0, 1, i, None, p, s)),
+             (bsp.ERR_CAPACITY, lambda: bsp.bsp_mask(wd, x, 0, 0, 65, i, None, p, s)),
+             (bsp.ERR_NULL, lambda: lay.gemm_q8(x, None, None, y.to(torch.int8), s)),
+             (bsp.ERR_DTYPE, lambda: lay.gemm(x, None, y.to(torch.int32), s)),
+             (bsp.ERR_SHAPE, lambda: lay.conv2d(x.view(4, 1, 1, 64), None, y, (0, 1), (0, 0), s)),
+             (bsp.ERR_SHAPE, lambda: lay.conv2d(x.view(4, 1, 1, 64), None, y, (1, 1), (0, -1), s))]
+    for want, call in calls:
+        with pytest.raises(bsp.BspError) as e:
+            call()
+        assert e.value.status == want
+
+
+@pytest.mark.parametrize("call", [lambda n, a: n.gemm(*a), lambda n, a: n.gemm(a[1], *a[1:]), lambda n, a: n.gemm(*a[:-1]),
+                                  lambda n, a: n.gemm(*a[:3], 1.5, *a[4:]), lambda n, a: n.gemm(*a[:2], object(), *a[3:])])
+def test_wrong_kinds_raise(call):
+    i, p = buffers()
+    args = [bsp.wdesc(64, 64, 1, 1, 8, 8, bsp.BF16), bsp.bcsr(i, i, p, p, 8), p, 4, None, p, bsp.F32, p, object()]
+    with pytest.raises((TypeError, AttributeError)):
+        call(bsp._native(), args)
+
+
+def test_input_shape_and_output_type():
+    lay = bsp.SparseLayer(64, 64, 1, 1, 8, 8, torch.bfloat16, device="cpu")
+    x = torch.zeros(4, 64, dtype=torch.bfloat16)
+    with pytest.raises(ValueError):
+        lay.conv2d(x, None, x, stream=Stream())
+    with pytest.raises(KeyError):
+        lay.gemm(x, None, x.double(), stream=Stream())
