@@ -47,6 +47,7 @@ struct GtParams {
     int a_bytes;                      // bytes of one activation box
     uint8_t *Y;
     int ey;
+    int half_rows;                    // kTaps: tiles of at most 64 positions, multiplied with M = 64
     int small_acc;                    // int8: the sums of products are at most 2^29
     // kHalo: bytes of the resident weights, pitch and rows of an image's box, position tiles, planes of 32-byte rows and their pitch
     int w_bytes, halo_w, halo_rows, n_pos, planes, plane_bytes;
@@ -323,9 +324,10 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
         // The whole warp runs the loop (so that its address arithmetic stays warp-uniform); one elected lane issues.
         if (run && rank == 0) {               // (of a pair, the leader issues for both CTAs)
             // instruction descriptor: D fp32 (int32 for int8), A and B bf16 / signed int8 / tf32, K-major both, M = 128
-            // (256 over a pair), N = BN
+            // (256 over a pair, 64 for low tiles), N = BN
             const uint32_t dfmt = kWT == BSP_I8 ? 2u : 1u, abfmt = kWT == BSP_F32 ? 2u : 1u;
-            const uint32_t idesc = (dfmt << 4) | (abfmt << 7) | (abfmt << 10) | ((uint32_t)(BN >> 3) << 17) | (((kPair ? 256u : 128u) >> 4) << 24);
+            const uint32_t idesc = (dfmt << 4) | (abfmt << 7) | (abfmt << 10) | ((uint32_t)(BN >> 3) << 17) |
+                                   (((kPair ? 256u : kMode == kTaps && p.half_rows ? 64u : 128u) >> 4) << 24);
             const uint32_t full0 = sm32(&s_full[0]), empty0 = sm32(&s_empty[0]);
             const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, astride16 = (uint32_t)p.a_stride >> 4;
             const uint64_t desc0 = p.kbytes == 64 ? kGtDesc64 : kGtDesc;
@@ -368,6 +370,8 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             const bool issuer = q == 0 && lane == 0;             // one thread of the group issues its stores
             // this lane's row of the staging buffer: the lane's row of the tile, or in kHalo the place of its output in the box
             int row = q * 32 + lane;
+            if constexpr (kMode == kTaps)                        // (with M = 64, 16 rows in the first half of each quarter)
+                if (p.half_rows) row = lane < 16 ? q * 16 + lane : -1;
             if constexpr (kMode == kHalo) {
                 const int per_image = p.halo_rows * p.halo_w, n = row / per_image, y = (row - n * per_image) / p.halo_w, x = row - n * per_image - y * p.halo_w;
                 row = n < p.Nt && y < p.Ht && x < p.Wt ? (n * p.Ht + y) * p.Wt + x : -1;
@@ -594,7 +598,23 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
             }
         }
     }
+    // A layer that leaves most SMs idle takes lower position tiles, for as long as its tiles stay on SMs of their own: what it
+    // waits for is the pace of one SM, 1.5 cycles a row of its two boxes and, in tiles of up to 64 positions, MMAs with M = 64
+    // that read half as much of the activations.  (Measured: 3x3 176->64 at 27x27 9.2 -> 6.3 us, of which M = 64 is 1.0;
+    // 3x3 128->128 at 28x28 5.8 -> 5.4; a product of 64 positions, K = 2048, 7.4 -> 6.9.  Sharing the K-stages of a tile over a
+    // cluster of CTAs instead took 9.9 us for that one: a kernel on all SMs cannot start before the one ahead of it ends.)
+    for (int rows = kGtBM / 2; rows >= 32; rows /= 2) {
+        const GtTile low = gt_pick_tile(xd.N, p.M, p.Nw, p.sh, p.sw, rows);
+        const long long ntn = (wd.O + p.BN - 1) / p.BN;
+        if (low.tiles <= 0 || low.tiles * ntn > n_sm[dev]) break;
+        const double mma = nk * (16 + p.BN / 4 > p.BN / 2 ? 16 + p.BN / 4 : p.BN / 2), loads = 1.5 * (low.Wt * low.Ht * low.Nt + p.BN);
+        const double cycles = p.n_ks * (mma > loads ? mma : loads) + 400.0;
+        if (cycles >= taps_cycles) break;
+        T = low;
+        taps_cycles = cycles;
+    }
     if (halo_cycles >= 0 && halo_cycles < taps_cycles) { mode = kHalo; p.BN = halo_bn; T = Th; }
+    p.half_rows = mode == kTaps && T.Wt * T.Ht * T.Nt <= 64 ? 1 : 0;
     p.Wt = T.Wt; p.Ht = T.Ht; p.Nt = T.Nt; p.rows_tile = T.Wt * T.Ht * T.Nt;
     p.tiles_x = (p.Nw + T.Wt - 1) / T.Wt; p.tiles_y = (p.M + T.Ht - 1) / T.Ht;
     p.n_tiles_n = (wd.O + p.BN - 1) / p.BN;

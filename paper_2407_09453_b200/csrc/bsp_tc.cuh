@@ -368,17 +368,17 @@ uint32_t gt_magic(int d) { return d <= 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32)
 // For every width the tallest box that fits has the fewest tiles, and of the heights with that many tiles the lowest has
 // the smallest area; the same holds for the widths with the same number of tiles across, so only the distinct tile
 // counts in x are looked at, each with one height (about 2 sqrt(N_w) of them instead of every width and height).
-GtTile gt_pick_tile(int N, int M, int Nw, int sh, int sw)
+GtTile gt_pick_tile(int N, int M, int Nw, int sh, int sw, int rows = kGtBM)
 {
     GtTile best = {0, 0, 0, -1};
     if (sh > 256 || sw > 256) return best;
-    for (int w = 1; w <= Nw && w <= kGtBM && w * sw <= 256;) {
-        int hmax = kGtBM / w;
+    for (int w = 1; w <= Nw && w <= rows && w * sw <= 256;) {
+        int hmax = rows / w;
         if (hmax > M) hmax = M;
         if (hmax * sh > 256) hmax = 256 / sh;
         const int ty = (M + hmax - 1) / hmax, h = (M + ty - 1) / ty, tx = (Nw + w - 1) / w;
         int b = 1;
-        if (w == Nw && h == M) { b = kGtBM / (w * h); if (b > N) b = N; if (b > 256) b = 256; if (b < 1) b = 1; }
+        if (w == Nw && h == M) { b = rows / (w * h); if (b > N) b = N; if (b > 256) b = 256; if (b < 1) b = 1; }
         const long long cnt = (long long)((N + b - 1) / b) * ty * tx;
         const long long area = (long long)b * h * w, best_area = (long long)best.Wt * best.Ht * best.Nt;
         if (best.tiles < 0 || cnt < best.tiles || (cnt == best.tiles && area < best_area)) best = {w, h, b, cnt};
