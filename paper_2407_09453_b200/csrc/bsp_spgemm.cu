@@ -118,9 +118,10 @@ constexpr int kStThreads = (kStProducers + 1) * 32;
 constexpr int kStMaxStages = 8;
 constexpr int kStARows = kGtBM / kSpEdge;         // block rows of A per tile
 
-// Groups of producer warps by tile width: a group's chain of wait, store, fence, arrive and load is longer than the MMAs of
+// Groups of producer warps by tile width: a group's chain of wait, store, arrive and load is longer than the MMAs of
 // a chunk, so groups overlap theirs.  2048 x 2048 x 4096 at 50 %, us: one group 52 / 82 / 130 (256 / 128 / 64 columns), two
-// 50 / 72 / 113, four 105 with 64; 16-byte cp.async straight to shared memory instead of registers: 72 / 93 / 143.
+// 50 / 72 / 113, four 105 with 64; 16-byte cp.async straight to shared memory instead of registers: 72 / 93 / 143.  (These with
+// a proxy fence in the producers.)  Pairs of CTAs that fill half of B each: 48.3, against 46.0 for 256 columns alone.
 __host__ __device__ constexpr int st_groups(int BN) { return BN == 64 ? 4 : 2; }
 
 struct StParams {
@@ -235,7 +236,6 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
 #pragma unroll
             for (int u = 0; u < kUnits; ++u)
                 asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + u * (uint32_t)(kW * 512)), "r"(w[u].x), "r"(w[u].y), "r"(w[u].z), "r"(w[u].w) : "memory");
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(full0 + slot * 8u) : "memory");
             slot += kGroups;
@@ -261,6 +261,9 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
             if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; break; }
             const bool wrap = slot + 1u == (uint32_t)S;
             const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
+            // (the stage's stores come before this thread through its barrier, and before the MMAs by this one fence: a fence in
+            // every producer also waited for the loads it had in flight; 2048 x 2048 x 4096 at 50 % 48.9 -> 46.0 us)
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             gt_issue_stage<BSP_BF16, false>(tmem, kGtDesc | (uint64_t)(a16 & 0x3FFFu), kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu),
                                             idesc, empty0 + slot * 8u, c != c_lo ? 1u : 0u);
@@ -357,10 +360,10 @@ int spgemm_tc_stages(int BN, int n_chunks)
 
 // Tile width and split of the tensor-core form, or BN = 0 where the sparse form is expected to be faster.  Estimates in
 // microseconds, fitted on a B200.  Tensor-core form: a tile costs a start, a share per chunk for the table and the fill of
-// the operands (0.31 / 0.44 / 0.60 a chunk at 64 / 128 / 256 columns, bound by shared memory: stores of the fill, reads
+// the operands (0.30 / 0.42 / 0.57 a chunk at 64 / 128 / 256 columns, bound by shared memory: stores of the fill, reads
 // of the MMAs), whatever the masks hold.  Sparse form: 28.7 per million pairs of blocks with a common column plus 3.6 per
 // million look-ups, or the chain of one warp where there are few rows.  Measured, sparse / tensor core: 2048 x 2048 x 4096
-// at 50 % 304 / 50, at 75 % 90 / 47, at 90 % 25 / 44; 512 x 512 x 4096 at 50 % 27 / 15, at 75 % 11 / 14.
+// at 50 % 304 / 46, at 75 % 90 / 43, at 90 % 25 / 41; 512 x 512 x 4096 at 50 % 27 / 14, at 75 % 11 / 13.
 // The densities come from the host counts; a wrong count costs time only.
 struct StPlan { int BN, split; };
 // slots[k] = CTAs of clusters of 2^k that the GPU holds at once (clusters of eight do not reach every SM: 512 x 512 x 4096 on
@@ -380,7 +383,7 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
         const int BN = 64 << w;
         const int stages = spgemm_tc_stages(BN, n_chunks);
         if (stages < (BN == 256 ? 3 : st_groups(BN))) continue;        // (the ring also holds the tile's sums)
-        const double start = w == 0 ? 5.7 : (w == 1 ? 6.4 : 9.0), chunk = w == 0 ? 0.31 : (w == 1 ? 0.44 : 0.60);
+        const double start = w == 0 ? 5.7 : (w == 1 ? 6.4 : 9.0), chunk = w == 0 ? 0.30 : (w == 1 ? 0.42 : 0.57);
         const long long tiles = (long long)((NBa + kStARows - 1) / kStARows) * ((NBb * kSpEdge + BN - 1) / BN);
         for (int k = 0; k < 4 && slots[k] > 0; ++k) {
             const int split = 1 << k;
