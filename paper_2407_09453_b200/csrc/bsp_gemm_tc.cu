@@ -534,6 +534,12 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     p.P = (int)P;
     GtTile T = gt_pick_tile(xd.N, p.M, p.Nw, p.sh, p.sw);
     if (T.tiles <= 0) return BSP_ERR_SHAPE;
+    static int n_sm[kGtMaxDevices] = {};
+    int dev = 0;
+    BSP_CUDA_OK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
+    if (n_sm[dev] == 0) BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
+    if (T.tiles * ((wd.O + 255) / 256) > n_sm[dev]) T = gt_pick_packed(T, xd.N, p.M, p.Nw, p.sh, p.sw);
     // layers with at most 64 bytes of input channels per position stage 64-byte rows (64-byte swizzle, two MMAs a stage)
     p.kbytes = (long long)wd.I * esz <= 64 ? 64 : 128;
     p.cpt = (int)(((long long)wd.I * esz + 127) / 128);
@@ -550,14 +556,9 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     static_assert(BSP_F32 == 0 && BSP_BF16 == 1 && BSP_I8 == 2, "the table is indexed by type");
     const Kernel *kernel = kernels[wd.wtype][ey == 4 ? 0 : 1];
     static bool opted[kGtMaxDevices] = {};
-    static int n_sm[kGtMaxDevices] = {};
-    int dev = 0;
-    BSP_CUDA_OK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
     if (!opted[dev]) {
         for (int t = 0; t < 18; ++t)
             BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 6][t / 3 % 2][t % 3], cudaFuncAttributeMaxDynamicSharedMemorySize, kGtGemmSmem));
-        BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
         opted[dev] = true;
     }
     // Channels per tile: the widest tile keeps the tensor pipe busiest (a stage costs about 256 + 2 BN cycles of operand

@@ -1,5 +1,6 @@
-"""GPU parity of layers with so few tiles that most SMs would idle: lower position tiles, up to 64 of them by MMAs with M = 64
-(16 rows in each quarter of the tensor-memory lanes)."""
+"""GPU parity of the position tiles at both ends of the range.  Layers with so few tiles that most SMs would idle: lower
+tiles, up to 64 positions by MMAs with M = 64 (16 rows in each quarter of the tensor-memory lanes).  Layers of several waves:
+tiles of parts of several images."""
 import numpy as np
 import pytest
 import torch
@@ -28,6 +29,16 @@ def test_rows_and_channels(P, dtype, out):
 @pytest.mark.parametrize("dtype", ["bf16", "i8", "f32"])
 def test_taps_and_images(O, I, H, K, L, J, N, stride, pad, dtype):
     run_conv_case(911, O, I, H, K, 8, 8, dtype, (N, L, J, I), stride, pad)
+
+
+@pytest.mark.parametrize("dtype,O,I,H,K,L,J,N,stride", [
+    ("bf16", 64, 176, 3, 3, 28, 28, 60, (1, 1)),     # 4 x 4 positions of 8 images, a last tile of 4 images
+    ("i8", 320, 144, 3, 3, 17, 17, 52, (1, 1)),      # 2 x 2 positions with clipped columns and rows
+    ("f32", 264, 40, 3, 3, 7, 7, 150, (1, 1)),       # a row of 18 images
+    ("bf16", 520, 72, 1, 1, 57, 57, 12, (2, 2)),     # strides
+])
+def test_tiles_of_parts_of_several_images(dtype, O, I, H, K, L, J, N, stride):
+    run_conv_case(941, O, I, H, K, 8, 8, dtype, (N, L, J, I), stride, (H // 2, K // 2))
 
 
 @pytest.mark.parametrize("P,O,I", [(64, 1008, 512), (200, 64, 1024), (5, 80, 640)])
