@@ -64,6 +64,7 @@ struct CtTail {
     uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc1_full[2], acc1_empty[2], t_full[2], t_empty[2], acc2_full[2], acc2_empty[2];
     uint64_t w1_full[kCtTaps], w2_full[kCtW2Slots], w2_empty[kCtW2Slots];
     uint32_t tmem, fail;
+    uint32_t y_read[2];               // warps that have read accumulator two, counted over all tiles (kGroups > 2 kRpt)
     // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
     __align__(16) uint32_t bias[kGroups][128], half[kGroups][128];
     __align__(16) uint8_t shift[kGroups][128];
@@ -83,6 +84,16 @@ __device__ __forceinline__ bool ct_header_ok(const uint8_t *packed, int wtype, i
     const PackedHeader *h = (const PackedHeader *)packed;
     return h->magic == kPackedMagic && h->dtype == wtype && h->O == O && h->I == I && h->H == H && h->K == K && h->bo == bo &&
            h->bi == bi && (h->forms & kFormDense) != 0;
+}
+
+// Waits (bounded) until a count in shared memory that only grows has reached n.
+__device__ __forceinline__ bool ct_wait_count(const volatile uint32_t *count, uint32_t n)
+{
+    for (uint32_t spin = 0; spin < (kGtSpin >> 2); ++spin) {
+        if (*count >= n) return true;
+        __nanosleep(32);
+    }
+    return false;
 }
 
 // kI8: the 8-bit chain; kEy: bytes of an element of Y (compiled apart, so that no form carries another's epilogue code).
@@ -106,6 +117,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
     constexpr int cpr = 128 / kEy, kRpt = kCtBN2 / cpr;                  // channels of a round of Y, rounds per 128-channel tile
 
     if (tid == 0) {
+        tail.y_read[0] = tail.y_read[1] = 0u;
         for (int s = 0; s < S; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.full[s])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.empty[s])), "r"(1) : "memory");
@@ -451,9 +463,11 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 if (one) {
                     if (ok && (!gt_wait(sm32(&tail.acc1_full[b1]), u1 & 1u) || !gt_wait(sm32(&tail.t_empty[bt]), (ut & 1u) ^ 1u))) ok = false;
                 } else {
-                    // (With one round per tile of layer two, a group of three sees every third of these phases, and a barrier
-                    // tells a phase from the one two before only: the phase before, on the other barrier, comes first.)
-                    if (kGroups > 2 * kRpt && u2 > 0u && ok && !gt_wait(sm32(&tail.acc2_full[buf ^ 1u]), ((u2 - 1u) >> 1) & 1u)) ok = false;
+                    // (With one round per tile of layer two, a group of three may come to this phase while the barrier is still
+                    // two before it, which the parity cannot tell from done.  So first the previous use of the buffer is seen
+                    // to have been read, by a count: layer two waits for that anyway.  The parity of the other buffer's barrier
+                    // would not do, as that one may have moved on by two phases already.)
+                    if (kGroups > 2 * kRpt && ok && !ct_wait_count(&tail.y_read[buf], use * (uint32_t)(4 * kRpt))) ok = false;
                     if (ok && !gt_wait(sm32(&tail.acc2_full[buf]), use & 1u)) ok = false;
                     if (kEy == 1) {
                         if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
@@ -469,6 +483,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 auto hand_back = [&](uint64_t *bar) {
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
+                    if (kGroups > 2 * kRpt && !one && lane == 0) atomicAdd(&tail.y_read[buf], 1u);
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(bar)) : "memory");
                 };
                 if (one) {

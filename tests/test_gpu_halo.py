@@ -72,6 +72,9 @@ def test_requantised_output(O, case):
     (2, 17, 33, 40, 72, 64, 1, 7, 1),    # two chunks of T with a tail
     (1, 1, 300, 64, 48, 48, 1, 3, 0),    # T and Y narrower than a chunk
     (12, 56, 56, 48, 64, 112, 3, 3, 1),  # two rounds a tile in the 8-bit form, many tiles a CTA
+    (20, 101, 101, 48, 96, 96, 7, 1, 1), # ... whose second epilogue is late: two phases of layer two pass before it looks
+    (20, 56, 56, 48, 96, 256, 3, 3, 0),  # ... three and four rounds a tile
+    (20, 56, 56, 48, 96, 384, 3, 3, 0),
 ])
 def test_pair_equals_the_two_calls(N, L, J, I, O1, O2, H, K, relu):
     for dtype in ("bf16", "i8"):
