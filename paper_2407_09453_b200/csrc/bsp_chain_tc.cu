@@ -43,7 +43,8 @@ struct CtParams {
     int O1, I1, H, K, bo1, bi1, O2, bo2, bi2, relu, wtype;
     int O1p;                  // O1 rounded up to a whole chunk of T (64 or 128 channels): columns of accumulator one
     int tcc;                  // channels per chunk of T: 64 (bfloat16) or 128 (int8)
-    int n_ks1, cpt1, n_c2, n_t2;      // K-stages of layer one, its channel chunks per tap; chunks of T; channel tiles of layer two
+    int n_ks1, cpt1, n_c2, n_t2;      // K-stages of layer one, its channel chunks per tap; chunks of T; channel tiles of layer two (of a CTA)
+    int parts;                        // CTAs that share a position tile: each computes T and n_t2 channel tiles of layer two
     int stages, stage_bytes, n_tiles;
     int ahead;                // the first epilogue runs one tile ahead of the second
     int db, dbt;              // O1p <= 128: accumulator one is double-buffered, and without kHalo the tensor between the layers too
@@ -113,7 +114,8 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
     const uint32_t tbuf = base + p.off_t;                                // the tensor between the layers: n_c2 chunks
     const uint32_t tbytes = (uint32_t)(p.n_c2 * kCtChunk);
     const uint32_t staging = base + p.off_staging;
-    const int t_first = (int)blockIdx.x, t_step = (int)gridDim.x, t_count = p.n_tiles;
+    const int t_first = (int)blockIdx.x / p.parts, t_step = (int)gridDim.x / p.parts, t_count = p.n_tiles;
+    const int o2 = ((int)blockIdx.x - t_first * p.parts) * p.n_t2 * kCtBN2;      // this CTA's first channel of layer two
     constexpr int cpr = 128 / kEy, kRpt = kCtBN2 / cpr;                  // channels of a round of Y, rounds per 128-channel tile
 
     if (tid == 0) {
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                         asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xFFFFFFFF;\n"
                                      " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
                                      " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6}], [%0];\n}\n"
-                                     ::"r"(bar), "r"(tx2), "r"(to), "l"(&p.tmw2), "r"(c2 * 128), "r"(0), "r"(t2 * kCtBN2) : "memory");
+                                     ::"r"(bar), "r"(tx2), "r"(to), "l"(&p.tmw2), "r"(c2 * 128), "r"(0), "r"(o2 + t2 * kCtBN2) : "memory");
                     }
             };
             // the loads follow the order in which the MMA warp consumes them: with double buffers, layer one of the next
@@ -418,7 +420,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             const int groups = n_rounds < kGroups ? 2 : kGroups;
             auto fetch = [&](int rnd) {
                 const bool one = rnd < p.n_c2;
-                const int ch = (one ? rnd * p.tcc : (rnd - p.n_c2) * cpr) + ct, O = one ? p.O1 : p.O2;
+                const int ch = (one ? rnd * p.tcc : o2 + (rnd - p.n_c2) * cpr) + ct, O = one ? p.O1 : p.O2;
                 const uint32_t *b = (const uint32_t *)(one ? p.bias1 : p.bias2);
                 const int32_t *s = one ? p.shift1 : p.shift2;
                 const bool in = ct < (one ? p.tcc : cpr) && ch < O;
@@ -454,7 +456,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 }
                 // what the round waits for: accumulator one and a free T (the MMAs of the second layer that read it have
                 // completed), or accumulator two (int8: and a staging buffer that its last store has read)
-                const int t2 = one ? 0 : (rnd - p.n_c2) / kRpt, c0 = one ? 0 : (rnd - p.n_c2) % kRpt * cpr, n0 = t2 * kCtBN2;
+                const int t2 = one ? 0 : (rnd - p.n_c2) / kRpt, c0 = one ? 0 : (rnd - p.n_c2) % kRpt * cpr, n0 = o2 + t2 * kCtBN2;
                 const uint32_t b1 = p.db ? (tile_i & 1u) : 0u, u1 = p.db ? (tile_i >> 1) : tile_i;
                 const uint32_t bt = p.dbt ? (tile_i & 1u) : 0u, ut = p.dbt ? (tile_i >> 1) : tile_i;
                 const uint32_t u2 = tile_i * (uint32_t)p.n_t2 + (uint32_t)t2, buf = u2 & 1u, use = u2 >> 1;
@@ -595,6 +597,22 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.n_ks1 = HK * p.cpt1;
     p.n_c2 = p.O1p / p.tcc;
     p.n_t2 = (wd2.O + kCtBN2 - 1) / kCtBN2;
+    p.parts = 1;
+    static int n_sm[kGtMaxDevices] = {};
+    int dev = 0;
+    BSP_CUDA_OK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
+    if (n_sm[dev] == 0) BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
+    const GtTile Th = gt_pick_halo(xd.N, p.M, p.Nw, wd1.H, wd1.K);
+    // Where the position tiles fill less than half of the SMs, several CTAs take one: each computes T for itself and its share of
+    // layer two's channels.  (Two 128-channel tiles of Y take about 1.2 us one after the other: 7x1 128->64->928 at 11x11 13.0 -> 6.6 us,
+    // 3x3 64->80->768 at 22x22 12.3 -> 7.4, 1x1 96->128->592 at 34x34, batch 8, 14.9 -> 11.6.)
+    const long long most = Th.tiles > T.tiles ? Th.tiles : T.tiles;
+    if (most * 2 <= n_sm[dev] && p.n_t2 > 1) {
+        const int parts = (int)(n_sm[dev] / most);
+        p.n_t2 = (p.n_t2 + parts - 1) / parts;
+        p.parts = (wd2.O + kCtBN2 * p.n_t2 - 1) / (kCtBN2 * p.n_t2);
+    }
     p.db = p.O1p <= 128 ? 1 : 0;
     p.dbt = p.db;
     p.kbytes = 128; p.planes = 1;
@@ -602,10 +620,10 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.small2 = (long long)wd1.O * 128 * 128 <= (1 << 29) ? 1 : 0;
     const int fixed = ct_groups(false) * 4 * kGtStagingBytes + (int)sizeof(CtTail<2>);
     // kHalo: where two boxes of activations, the weights of layer one and at least two chunks of layer two's fit, and the
-    // tiles with their border are not many more.  3x3 64->64 then 64->256 at 56x56, batch 64: 44.5 us loaded tap by tap.
+    // tiles with their border are not many more.  3x3 64->64 then 64->256 at 56x56, batch 64: 44.5 us loaded tap by tap,
+    // 33.8 like this.
     bool halo = false;
     int w2_slots = 0;
-    const GtTile Th = gt_pick_halo(xd.N, p.M, p.Nw, wd1.H, wd1.K);
     if (HK > 1 && HK <= kCtTaps && p.cpt1 == 1 && p.sh == 1 && p.sw == 1 && p.db && Th.tiles > 0 && Th.tiles * 4 <= T.tiles * 5) {
         const int kb = row1 <= 32 ? 32 : (row1 <= 64 ? 64 : 128), planes = kb == 128 ? 1 : kb / 32;
         const int plane = (Th.Nt * (Th.Ht + wd1.H - 1) * (Th.Wt + wd1.K - 1) * (kb / planes) + 1023) / 1024 * 1024;
@@ -629,6 +647,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
             p.halo_w = T.Wt + wd1.K - 1; p.halo_rows = T.Ht + wd1.H - 1;
         }
     }
+    if (!halo && T.tiles > n_sm[dev]) T = gt_pick_packed(T, xd.N, p.M, p.Nw, p.sh, p.sw);
     p.Wt = T.Wt; p.Ht = T.Ht; p.Nt = T.Nt;
     p.tiles_x = (p.Nw + T.Wt - 1) / T.Wt; p.tiles_y = (p.M + T.Ht - 1) / T.Ht;
     p.m_tx = gt_magic(p.tiles_x); p.m_ty = gt_magic(p.tiles_y);
@@ -663,13 +682,8 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     static const Kernel kernels[2][2][2] = {{{chain_tc_kernel<false, 4, false>, chain_tc_kernel<false, 4, true>}, {chain_tc_kernel<false, 2, false>, chain_tc_kernel<false, 2, true>}},
                                             {{chain_tc_kernel<true, 4, false>, chain_tc_kernel<true, 4, true>}, {chain_tc_kernel<true, 1, false>, chain_tc_kernel<true, 1, true>}}};
     static bool opted[kGtMaxDevices] = {};
-    static int n_sm[kGtMaxDevices] = {};
-    int dev = 0;
-    BSP_CUDA_OK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
     if (!opted[dev]) {
         for (int t = 0; t < 8; ++t) BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 4][t / 2 % 2][t % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, kCtSmem));
-        BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
         opted[dev] = true;
     }
     // bytes of an operand row of layer one in shared memory, and its swizzle
@@ -719,7 +733,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return BSP_ERR_CUDA;
     }
-    const int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
+    const int grid = p.n_tiles * p.parts < n_sm[dev] ? p.n_tiles * p.parts : n_sm[dev];      // (several parts: one wave)
     BSP_CUDA_OK(launch_after(kernels[wd1.wtype == BSP_I8 ? 1 : 0][ey == 4 ? 0 : 1][halo ? 1 : 0], dim3((unsigned)grid), dim3(64u + 128u * ct_groups(halo)), smem, st, p));
     return BSP_OK;
 }

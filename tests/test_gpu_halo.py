@@ -75,6 +75,10 @@ def test_requantised_output(O, case):
     (20, 101, 101, 48, 96, 96, 7, 1, 1), # ... whose second epilogue is late: two phases of layer two pass before it looks
     (20, 56, 56, 48, 96, 256, 3, 3, 0),  # ... three and four rounds a tile
     (20, 56, 56, 48, 96, 384, 3, 3, 0),
+    (1, 11, 11, 64, 64, 928, 7, 1, 1),   # few tiles: a CTA for each 128 channels of layer two, the last of them clipped
+    (24, 14, 14, 32, 64, 1024, 3, 3, 0), # ... for every three of eight, the last with one past the end
+    (2, 22, 22, 192, 80, 176, 3, 3, 1),  # ... with layer one loaded tap by tap
+    (60, 17, 17, 192, 64, 160, 3, 3, 0), # tiles of parts of several images
 ])
 def test_pair_equals_the_two_calls(N, L, J, I, O1, O2, H, K, relu):
     for dtype in ("bf16", "i8"):
