@@ -179,7 +179,7 @@ __device__ __forceinline__ int ones_share_global(const uint8_t *__restrict__ g, 
 // The packed form: Gamma (.) W in the layout of W, [O][H][K][I], the channels of zeroed blocks cleared.  The b_o H K rows
 // (o, tap) of a row of Gamma share its entries, so a thread takes one 16-byte chunk of input channels of up to eight of
 // these rows: Gamma is read once, then the rows that are needed are loaded together.  (One chunk at a time, each behind its
-// own look at Gamma, took 16.9 us for 4096 x 4096 bf16; see compact_kernel for the figure now.)
+// own look at Gamma, took 16.9 us for 4096 x 4096 bf16, and 20.9 with the index part beside it, which is 15.5 like this.)
 constexpr int kDenseRows = 8;
 template <int esz>
 __device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *__restrict__ W, const uint8_t *__restrict__ gamma, int I, int HK, int bo, int bi,

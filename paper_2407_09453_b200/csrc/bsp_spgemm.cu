@@ -366,7 +366,8 @@ int spgemm_tc_stages(int BN, int n_chunks)
 // the operands (0.30 / 0.42 / 0.57 a chunk at 64 / 128 / 256 columns, bound by shared memory: stores of the fill, reads
 // of the MMAs), whatever the masks hold.  Sparse form: 28.7 per million pairs of blocks with a common column plus 3.6 per
 // million look-ups, or the chain of one warp where there are few rows.  Measured, sparse / tensor core: 2048 x 2048 x 4096
-// at 50 % 304 / 46, at 75 % 90 / 43, at 90 % 25 / 41; 512 x 512 x 4096 at 50 % 27 / 14, at 75 % 11 / 13.
+// at 50 % 304 / 46, at 75 % 90 / 43, 512 x 512 x 4096 at 50 % 27 / 14; with the fence in the
+// producers 25 / 44 at 90 %, and 11 / 14 for the smaller one at 75 %.
 // The densities come from the host counts; a wrong count costs time only.
 struct StPlan { int BN, split; };
 // slots[k] = CTAs of clusters of 2^k that the GPU holds at once (clusters of eight do not reach every SM: 512 x 512 x 4096 on
