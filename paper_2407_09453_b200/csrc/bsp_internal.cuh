@@ -78,7 +78,7 @@ inline int gemm_tile_n(int O)
 // stream overlap, and no successor can hold a line in L1 that was read before the kernel in between wrote it.  (Launched
 // one after another without this, the kernels of a stream started in steps of about 2 us.)
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-// kLetNext = false: the kernel calls let_next_start() itself, later.
+// kLetNext = false: the next kernel starts when this one has ended (still without the gap between launches).
 template <bool kLetNext = true>
 __device__ __forceinline__ void wait_for_previous()
 {

@@ -87,6 +87,10 @@ spgemm_kernel(const int32_t *__restrict__ a_row_ptr, const int32_t *__restrict__
     extern __shared__ int s_pos[];                 // [NBk]: payload position of row i's block in column k, or -1
     const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = threadIdx.x; k < NBk; k += kSpThreads) s_pos[k] = -1;
+    // (The next kernel is not let in before this one has ended: its CTAs, several per SM, would be placed where slots happen to be
+    // free and stay uneven.  A stream of 1768 x 208 x 992 bfloat16 products at 50 % takes 10.0 us a call like this, 13.4 with the
+    // next one let in at once, 12.2 without programmatic launches; 232 x 2264 x 632 fp32 at 25 % 62.0, 78.1 let in at the end of
+    // each CTA, 64.3.)
     wait_for_previous<false>();
     __syncthreads();
     for (int n = a_row_ptr[i] + threadIdx.x; n < a_row_ptr[i + 1]; n += kSpThreads) {
@@ -102,9 +106,6 @@ spgemm_kernel(const int32_t *__restrict__ a_row_ptr, const int32_t *__restrict__
         sp_pair<T>(a_payload, b_col_idx, b_payload, b_row_ptr[j], b_row_ptr[j + 1], NBk, lane, [&](int k) { return s_pos[k]; }, acc0, acc1, status);
         *(float2 *)(C + ((size_t)i * kSpEdge + r) * ldc + (size_t)j * kSpEdge + c) = make_float2(acc0, acc1);
     }
-    // (Only now: a successor of several CTAs per SM that starts while this kernel's CTAs still hold most slots is placed where
-    // slots are free and stays uneven.  A stream of 1768 x 208 x 992 at 50 % took 13.1 us a call instead of 10.5.)
-    let_next_start();
 }
 
 // ---- bfloat16 operands on 5th-generation tensor cores -----------------------------------------------------------------
