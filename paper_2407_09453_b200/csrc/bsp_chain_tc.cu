@@ -65,7 +65,7 @@ struct CtTail {
     uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc1_full[2], acc1_empty[2], t_full[2], t_empty[2], acc2_full[2], acc2_empty[2];
     uint64_t w1_full[kCtTaps], w2_full[kCtW2Slots], w2_empty[kCtW2Slots];
     uint32_t tmem, fail;
-    uint32_t y_read[2];               // warps that have read accumulator two, counted over all tiles (kGroups > 2 kRpt)
+    uint32_t y_read[2];               // warps that have read accumulator two, counted over all tiles
     // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
     __align__(16) uint32_t bias[kGroups][128], half[kGroups][128];
     __align__(16) uint8_t shift[kGroups][128];
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             if (!ok && lane == 0) atomicExch((uint32_t *)&tail.fail, 1u);
         }
     } else {
-        // ================= epilogues (warps 2-9) =================
+        // ================= epilogues (warps 2-9, kHalo 2-13) =================
         // The work goes in steps: the n_c2 chunks of T of tile s + ahead, then the 128-byte rounds of Y of tile s; the groups take
         // turns with these rounds, across steps too.  With ahead = 1 the MMA warp finds the next T ready when it is
         // done with this tile (else layer two of a tile waited for both of the previous tile's epilogues).
@@ -415,8 +415,15 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             uint32_t next_bias = 0u, next_shift = 1u;
             bool small = false;
             const int n_rounds = p.n_c2 + p.n_t2 * kRpt;
-            // (A barrier tells a phase from the one two before only.  A group sees enough of them when it has a round in every
-            // step, or, of two groups, always the same ones: steps of two rounds take two groups.)
+            // A barrier's parity tells a phase from the next one only, so a group may look at a phase when it knows that the one
+            // before it has completed.  What tells it, for each barrier (all rest on the commits of the MMA warp completing in the
+            // order of its loop):
+            //   acc2_full   the count of the reads of the buffer's previous use (below).
+            //   acc1_full   of tile i: its previous phase is that of tile i - 2 (two accumulators) or i - 1 (one).  The group had a
+            //               round in step i - 1 - ahead, as a step has at least as many rounds as there are groups (hence two
+            //               groups for steps of two): T of tile i - 1, or Y of tile i - 1 - ahead, which came after it.
+            //   t_empty     of the tile before in the same buffer: acc1_full of tile i, which the group has waited for just
+            //               before, comes after layer two of tile i - 2 (i - 1 with one accumulator).
             const int groups = n_rounds < kGroups ? 2 : kGroups;
             auto fetch = [&](int rnd) {
                 const bool one = rnd < p.n_c2;
@@ -465,11 +472,11 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 if (one) {
                     if (ok && (!gt_wait(sm32(&tail.acc1_full[b1]), u1 & 1u) || !gt_wait(sm32(&tail.t_empty[bt]), (ut & 1u) ^ 1u))) ok = false;
                 } else {
-                    // (With one round per tile of layer two, a group of three may come to this phase while the barrier is still
-                    // two before it, which the parity cannot tell from done.  So first the previous use of the buffer is seen
-                    // to have been read, by a count: layer two waits for that anyway.  The parity of the other buffer's barrier
-                    // would not do, as that one may have moved on by two phases already.)
-                    if (kGroups > 2 * kRpt && ok && !ct_wait_count(&tail.y_read[buf], use * (uint32_t)(4 * kRpt))) ok = false;
+                    // First the previous use of the buffer is seen to have been read, by a count: layer two waits for that
+                    // anyway.  (The group's own last look does not tell: with one round per tile of layer two and three groups
+                    // it may be two phases back, and in the last tile, whose step has no T left, it is a whole step back.  The
+                    // parity of the other buffer's barrier would not do either, as that one may have moved on by two phases.)
+                    if (ok && !ct_wait_count(&tail.y_read[buf], use * (uint32_t)(4 * kRpt))) ok = false;
                     if (ok && !gt_wait(sm32(&tail.acc2_full[buf]), use & 1u)) ok = false;
                     if (kEy == 1) {
                         if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
@@ -485,7 +492,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 auto hand_back = [&](uint64_t *bar) {
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
-                    if (kGroups > 2 * kRpt && !one && lane == 0) atomicAdd(&tail.y_read[buf], 1u);
+                    if (!one && lane == 0) atomicAdd(&tail.y_read[buf], 1u);
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(bar)) : "memory");
                 };
                 if (one) {

@@ -155,6 +155,50 @@ def test_int8_chain_many_tiles_strides_and_taps():
     run_chain_q8(1127, 4, 28, 28, 256, 64, 256, 1, 1, (1, 1), (0, 0), 1, True)
 
 
+@pytest.mark.parametrize("dtype,O1,O2,taps,N,L", [
+    ("i8", 48, 192, 1, 38, 83),          # two rounds of Y a tile and two groups: every second use of an accumulator is looked at
+    ("i8", 48, 288, 1, 9, 60),           # three
+    ("i8", 64, 256, 3, 6, 56),           # the same with weights on chip and three groups
+    ("bf16", 64, 256, 3, 8, 56),         # four rounds of Y
+    ("bf16", 64, 512, 3, 4, 40),         # eight
+])
+def test_last_tile_of_many_calls(dtype, O1, O2, taps, N, L):
+    """The last tile of a CTA has no further tensor between the layers to make, so a group's looks at the second accumulators lie
+    further apart there: many calls in a row, each checked (status and all outputs), against the two separate calls."""
+    i8 = dtype == "i8"
+    W1, W2 = make_case(1061, O1, 32 if i8 else 64, taps, taps, dtype), make_case(1062, O2, O1, 1, 1, dtype)
+    I = W1.shape[3]
+    g1 = synth.random_gamma(1063, O1 // 8, I // 8, (O1 // 8) * (I // 8) // 2)
+    g2 = synth.random_gamma(1064, O2 // 8, O1 // 8, (O2 // 8) * (O1 // 8) // 2)
+    l1, l2 = gpu_layer(W1, g1, 8, 8, dtype), gpu_layer(W2, g2, 8, 8, dtype)
+    X = to_dev(make_x(1065, (N, L, L, I), dtype), dtype)
+    b1, b2 = torch.from_numpy(make_bias(1066, O1, dtype)).cuda(), torch.from_numpy(make_bias(1067, O2, dtype)).cuda()
+    pad = taps // 2
+    xd = bsp.XDesc(N, L, L, 1, 1, pad, pad)
+    dt = torch.int8 if i8 else torch.bfloat16
+    T, Ya = torch.empty((N, L, L, O1), dtype=dt, device="cuda"), torch.empty((N, L, L, O2), dtype=dt, device="cuda")
+    if i8:
+        s1, s2 = torch.full((O1,), 10, dtype=torch.int32, device="cuda"), torch.full((O2,), 9, dtype=torch.int32, device="cuda")
+        l1.conv2d_q8(X, b1, s1, T, (1, 1), (pad, pad))
+        l2.conv2d_q8(T, b2, s2, Ya)
+    else:
+        l1.conv2d(X, b1, T, (1, 1), (pad, pad))
+        l2.conv2d(T, b2, Ya)
+    l1.check(), l2.check()
+    Yb = [torch.full_like(Ya, -7) for _ in range(8)]
+    for _ in range(5):
+        for y in Yb:
+            y.fill_(-7)
+        for y in Yb:
+            if i8:
+                bsp.bsp_conv2d_chain_q8(l1.wd, l1.handle(), l2.wd, l2.handle(), xd, X, b1, s1, 0, b2, s2, y, l1.ws)
+            else:
+                bsp.bsp_conv2d_chain(l1.wd, l1.handle(), l2.wd, l2.handle(), xd, X, b1, 0, b2, y, bsp.BF16, l1.ws)
+        l1.check()
+        for y in Yb:
+            assert torch.equal(Ya, y)
+
+
 def test_argument_errors():
     l1 = bsp.SparseLayer(64, 64, 3, 3, 8, 8, torch.bfloat16)
     l3 = bsp.SparseLayer(128, 64, 3, 3, 8, 8, torch.bfloat16)          # not 1x1
