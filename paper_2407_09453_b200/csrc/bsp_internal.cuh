@@ -77,8 +77,12 @@ inline int gemm_tile_n(int O)
 // barriers, tensor memory and descriptors).  It lets its own successor start only after that, so at most two kernels of a
 // stream overlap, and no successor can hold a line in L1 that was read before the kernel in between wrote it.  (Launched
 // one after another without this, the kernels of a stream started in steps of about 2 us.)
+// A kernel that owns tensor memory lets its successor start behind the CTA barrier that follows its allocation.  The first
+// thread of a CTA to signal speaks for the whole CTA: while another of its warps still waits for columns, a CTA of the
+// successor on the same SM could take them and hold them until this kernel ends, and neither would move.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-// kLetNext = false: the next kernel starts when this one has ended (still without the gap between launches).
+// kLetNext = false: the next kernel starts when this one has ended (still without the gap between launches), or calls
+// let_next_start() later.
 template <bool kLetNext = true>
 __device__ __forceinline__ void wait_for_previous()
 {

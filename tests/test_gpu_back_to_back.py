@@ -1,0 +1,113 @@
+"""Consecutive kernels of a stream overlap their starts.  Runs of calls in which each reads what the call before wrote, or
+overwrites what it read, give what the same calls give one at a time, bit for bit."""
+import pytest
+import torch
+
+from paper_2407_09453_b200 import bsp
+
+pytestmark = pytest.mark.gpu
+
+
+def randn(seed, shape, scale=1.0):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return torch.randn(shape, device="cuda", generator=g) * scale
+
+
+def randi8(seed, shape):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return torch.randint(-127, 128, shape, device="cuda", generator=g, dtype=torch.int8)
+
+
+def compare(program, runs=4):
+    """program(wait) -> tensors; `wait` is called between the calls and synchronises in the first run only.  The other runs
+    queue up behind a kernel of some milliseconds, so that the GPU never waits for the host."""
+    want = [t.clone() for t in program(torch.cuda.synchronize)]
+    for _ in range(runs):
+        torch.cuda._sleep(10_000_000)
+        got = program(lambda: None)
+        torch.cuda.synchronize()
+        for k, (x, y) in enumerate(zip(got, want)):
+            assert torch.equal(x, y), k
+
+
+@pytest.mark.parametrize("N,L,C", [(1, 7, 16), (3, 14, 32), (2, 28, 64), (16, 56, 16)])
+def test_small_int8_layers(N, L, C):
+    """3x3 layers whose weights stay on chip: their CTAs are small enough to share an SM with those of the next call."""
+    lay = bsp.SparseLayer(C, C, 3, 3, 8, 8, torch.int8)
+    W = randi8(1, (C, 3, 3, C))
+    lay.mask(W, lay.NBo * lay.NBi // 2)
+    lay.compact(W)
+    shift = torch.full((C,), 7 + (C * 9).bit_length() // 2, dtype=torch.int32, device="cuda")
+    X = randi8(2, (N, L, L, C))
+
+    def program(wait):
+        a, b = X.clone(), torch.empty_like(X)
+        for _ in range(40):
+            lay.conv2d_q8(a, None, shift, b, (1, 1), (1, 1))
+            wait()
+            a, b = b, a
+        lay.check()
+        return a, b
+    compare(program)
+
+
+@pytest.mark.parametrize("dtype,N,L,C,mid,taps", [("i8", 2, 14, 32, 48, 3), ("i8", 4, 30, 192, 48, 1), ("bf16", 2, 28, 64, 64, 3), ("bf16", 3, 9, 24, 136, 3)])
+def test_pairs(dtype, N, L, C, mid, taps):
+    i8 = dtype == "i8"
+    dt = torch.int8 if i8 else torch.bfloat16
+    l1, l2 = bsp.SparseLayer(mid, C, taps, taps, 8, 8, dt), bsp.SparseLayer(C, mid, 1, 1, 8, 8, dt)
+    W1 = randi8(3, (mid, taps, taps, C)) if i8 else randn(3, (mid, taps, taps, C), 1.4 / taps / C ** 0.5).to(dt)
+    W2 = randi8(4, (C, 1, 1, mid)) if i8 else randn(4, (C, 1, 1, mid), 1.4 / mid ** 0.5).to(dt)
+    for lay, W in ((l1, W1), (l2, W2)):
+        lay.mask(W, lay.NBo * lay.NBi // 2)
+        lay.compact(W)
+    s1 = torch.full((mid,), 7 + (C * taps * taps).bit_length() // 2, dtype=torch.int32, device="cuda")
+    s2 = torch.full((C,), 7 + mid.bit_length() // 2, dtype=torch.int32, device="cuda")
+    X = randi8(5, (N, L, L, C)) if i8 else randn(5, (N, L, L, C)).to(dt)
+    xd = bsp.XDesc(N, L, L, 1, 1, taps // 2, taps // 2)
+    h1, h2 = l1.handle(), l2.handle()
+
+    def program(wait):
+        a, b = X.clone(), torch.empty_like(X)
+        for _ in range(24):
+            if i8:
+                bsp.bsp_conv2d_chain_q8(l1.wd, h1, l2.wd, h2, xd, a, None, s1, 0, None, s2, b, l1.ws)
+            else:
+                bsp.bsp_conv2d_chain(l1.wd, h1, l2.wd, h2, xd, a, None, 0, None, b, bsp.BF16, l1.ws)
+            wait()
+            a, b = b, a
+        l1.check()
+        return a, b
+    compare(program)
+
+
+def test_products_of_different_kinds_take_turns():
+    """A product, a pair and a sparse x sparse product by turns: each kernel's tensor memory is free when the next one takes it."""
+    C = 64
+    lay, l2 = bsp.SparseLayer(C, C, 3, 3, 8, 8, torch.bfloat16), bsp.SparseLayer(C, C, 1, 1, 8, 8, torch.bfloat16)
+    for s, q in ((6, lay), (7, l2)):
+        W = randn(s, (C, q.wd.H, q.wd.K, C), 1.4 / q.wd.H / C ** 0.5).to(torch.bfloat16)
+        q.mask(W, q.NBo * q.NBi // 2)
+        q.compact(W)
+    sa, sb = bsp.SparseLayer(256, 1024, 1, 1, 8, 8, torch.bfloat16), bsp.SparseLayer(512, 1024, 1, 1, 8, 8, torch.bfloat16)
+    for s, q in ((8, sa), (9, sb)):
+        W = randn(s, (q.wd.O, 1, 1, 1024)).to(torch.bfloat16)
+        q.mask(W, q.NBo * q.NBi // 4)
+        q.compact(W)
+    X = randn(10, (2, 14, 14, C)).to(torch.bfloat16)
+    xd = bsp.XDesc(2, 14, 14, 1, 1, 1, 1)
+
+    def program(wait):
+        a, b, Cm = X.clone(), torch.empty_like(X), torch.empty((256, 512), device="cuda")
+        for _ in range(12):
+            lay.conv2d(a, None, b, (1, 1), (1, 1))
+            wait()
+            bsp.bsp_spgemm(sa.wd, sa.handle(), sb.wd, sb.handle(), Cm, sa.ws)
+            wait()
+            bsp.bsp_conv2d_chain(lay.wd, lay.handle(), l2.wd, l2.handle(), xd, b, None, 1, None, a, bsp.BF16, lay.ws)
+            wait()
+        lay.check(), sa.check()
+        return a, b, Cm
+    compare(program)
