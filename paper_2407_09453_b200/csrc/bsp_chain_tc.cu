@@ -432,8 +432,8 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 const uint32_t *b = (const uint32_t *)(one ? p.bias1 : p.bias2);
                 const int32_t *s = one ? p.shift1 : p.shift2;
                 const bool in = ct < (one ? p.tcc : cpr) && ch < O;
-                next_bias = in && b != nullptr ? __ldg(b + ch) : 0u;
-                if constexpr (kI8) next_shift = in && s != nullptr ? (uint32_t)__ldg(s + ch) & 31u : 1u;
+                next_bias = in && b != nullptr ? b[ch] : 0u;
+                if constexpr (kI8) next_shift = in && s != nullptr ? (uint32_t)s[ch] & 31u : 1u;
             };
             bool mine_small = false, fresh = true;
             auto place = [&](int rnd) {                          // (between two barriers of the group)

@@ -50,7 +50,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_sums, int &
 // several elements; a block row of b_i elements is contiguous in W and in the payload).  Each thread loads four
 // pieces before it stores them.
 template <typename T, typename V>
-__device__ __forceinline__ void fill_copy(int l, int part, int parts, const T *__restrict__ W, int I, int HK, int bo, int bi,
+__device__ __forceinline__ void fill_copy(int l, int part, int parts, const T *W, int I, int HK, int bo, int bi,
                                           int first, int cnt, const int *s_cols, T *__restrict__ payload,
                                           long long capacity_blocks)
 {
@@ -86,8 +86,8 @@ __device__ __forceinline__ void fill_copy(int l, int part, int parts, const T *_
 // payload[n][r][h][k][c] = W[l b_o + r][h][k][iota b_i + c].  `first` = stored blocks in the rows above; returns
 // the number of stored blocks of row l.
 template <typename T>
-__device__ __forceinline__ int csr_fill_body(int l, int part, int parts, const T *__restrict__ W,
-                                              const uint8_t *__restrict__ gamma, int NBi, int I, int HK, int bo, int bi,
+__device__ __forceinline__ int csr_fill_body(int l, int part, int parts, const T *W,
+                                              const uint8_t *gamma, int NBi, int I, int HK, int bo, int bi,
                                               int first, int32_t *__restrict__ col_idx,
                                               T *__restrict__ payload, long long capacity_blocks)
 {
@@ -152,7 +152,7 @@ __device__ __forceinline__ int ones_share(const uint8_t *g, int n)
 
 // The same count over the first n bytes of Gamma in global memory (layers whose Gamma does not fit shared memory): 16-byte
 // loads, eight in flight per thread, when the addresses allow.
-__device__ __forceinline__ int ones_share_global(const uint8_t *__restrict__ g, int n)
+__device__ __forceinline__ int ones_share_global(const uint8_t *g, int n)
 {
     int c = 0;
     if ((((uintptr_t)g) & 15u) == 0) {
@@ -163,7 +163,7 @@ __device__ __forceinline__ int ones_share_global(const uint8_t *__restrict__ g, 
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int i = i0 + u * kThreads;
-                q[u] = i < n4 ? __ldg(g4 + i) : make_uint4(0u, 0u, 0u, 0u);
+                q[u] = i < n4 ? g4[i] : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u)
@@ -182,7 +182,7 @@ __device__ __forceinline__ int ones_share_global(const uint8_t *__restrict__ g, 
 // own look at Gamma, took 16.9 us for 4096 x 4096 bf16, and 20.9 with the index part beside it, which is 15.5 like this.)
 constexpr int kDenseRows = 8;
 template <int esz>
-__device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *__restrict__ W, const uint8_t *__restrict__ gamma, int I, int HK, int bo, int bi,
+__device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *W, const uint8_t *gamma, int I, int HK, int bo, int bi,
                                            int NBo, int NBi, uint8_t *__restrict__ out)
 {
     const bool aligned = (((uintptr_t)W) & 15u) == 0;
@@ -216,10 +216,10 @@ __device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *__re
         for (int u = 0; u < kDenseRows; ++u) {
             v[u] = make_uint4(0u, 0u, 0u, 0u);
             if (u < n && any) {
-                if (aligned) v[u] = __ldg((const uint4 *)(src + u * pitch));
+                if (aligned) v[u] = *(const uint4 *)(src + u * pitch);
                 else {                                // W only 4-byte aligned: word by word
                     const uint32_t *s4 = (const uint32_t *)(src + u * pitch);
-                    v[u] = make_uint4(__ldg(s4), __ldg(s4 + 1), __ldg(s4 + 2), __ldg(s4 + 3));
+                    v[u] = make_uint4(*s4, s4[1], s4[2], s4[3]);
                 }
             }
         }
@@ -233,7 +233,7 @@ __device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *__re
 // blocks of all rows before its first one together (one count for eight rows instead of one for each: with 512 rows of 512
 // the counts read 67 MB and took 13 us), then every warp counts and lists its own row, 16 entries per lane and step.
 constexpr int kIndexRows = kThreads / 32;
-__device__ __forceinline__ void index_rows(int cta, const uint8_t *__restrict__ gamma, int NBo, int NBi, int32_t *__restrict__ row_ptr,
+__device__ __forceinline__ void index_rows(int cta, const uint8_t *gamma, int NBo, int NBi, int32_t *__restrict__ row_ptr,
                                            int32_t *__restrict__ col_idx, long long capacity_blocks, int *s_sum, int *status)
 {
     __shared__ int s_cnt[kIndexRows];
@@ -245,7 +245,7 @@ __device__ __forceinline__ void index_rows(int cta, const uint8_t *__restrict__ 
         unsigned m = 0u;
         if (wide) {
             if (i < NBi) {
-                const uint4 w = __ldg((const uint4 *)(g + i));
+                const uint4 w = *(const uint4 *)(g + i);
                 const uint32_t x[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {

@@ -82,7 +82,7 @@ __device__ __forceinline__ void gt_tile_origin(const GtParams &p, int mt, int &n
 // Bias of output channel ch as raw bits (float32 or int32), zero without a bias or past the last channel.
 __device__ __forceinline__ uint32_t gt_bias(const GtParams &p, int ch)
 {
-    return (p.bias != nullptr && ch < p.O) ? __ldg((const uint32_t *)p.bias + ch) : 0u;
+    return (p.bias != nullptr && ch < p.O) ? ((const uint32_t *)p.bias)[ch] : 0u;
 }
 
 // kWT: operand type; kEy: bytes of an output element (4: float32 or int32, 2: bfloat16, 1: int8); kMode: how operands are staged.
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             auto fetch = [&](int ch0) {
                 if (ct >= cpr) return;
                 next_bias = gt_bias(p, ch0 + ct);
-                if constexpr (kEy == 1) next_shift = ch0 + ct < p.O ? (uint32_t)__ldg(p.shift + ch0 + ct) & 31u : 1u;
+                if constexpr (kEy == 1) next_shift = ch0 + ct < p.O ? (uint32_t)p.shift[ch0 + ct] & 31u : 1u;
             };
             auto place = [&](int ch0) {                          // (between two barriers of the group)
                 have = ch0;

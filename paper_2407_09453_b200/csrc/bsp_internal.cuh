@@ -77,6 +77,8 @@ inline int gemm_tile_n(int O)
 // barriers, tensor memory and descriptors).  It lets its own successor start only after that, so at most two kernels of a
 // stream overlap, and no successor can hold a line in L1 that was read before the kernel in between wrote it.  (Launched
 // one after another without this, the kernels of a stream started in steps of about 2 us.)
+// What an earlier kernel may have written is read by plain loads or __ldcg, through pointers without __restrict__: __ldg and
+// const __restrict__ promise data that nobody writes while the kernel runs, and it runs before wait_for_previous() returns.
 // A kernel that owns tensor memory lets its successor start behind the CTA barrier that follows its allocation.  The first
 // thread of a CTA to signal speaks for the whole CTA: while another of its warps still waits for columns, a CTA of the
 // successor on the same SM could take them and hold them until this kernel ends, and neither would move.

@@ -692,20 +692,20 @@ __device__ __forceinline__ void select_small(const unsigned long long (&v)[kKeys
 }
 
 // Loads the keys of a segment into registers (all loads are issued before the first is used, so they share one trip to memory).
-template <bool kThroughL2, int kT = kScoreThreads>
+template <int kT = kScoreThreads>
 __device__ __forceinline__ void load_keys(const unsigned long long *k, int n, unsigned long long (&v)[kKeysPerThread])
 {
 #pragma unroll
     for (int u = 0; u < kKeysPerThread; ++u) {
         const int i = u * kT + threadIdx.x;
-        v[u] = i < n ? (kThroughL2 ? __ldcg(k + i) : __ldg(k + i)) : 0ull;
+        v[u] = i < n ? __ldcg(k + i) : 0ull;
     }
 }
 
 // Segments of up to kRankMax keys, one CTA each (the rows of Gamma; a small layer without a workspace).  Up to 256 keys are
 // ranked directly, a thread per key.
 __global__ void __launch_bounds__(kScoreThreads)
-segment_kernel(const unsigned long long *__restrict__ key, int n, long long n_zero, uint8_t *__restrict__ gamma)
+segment_kernel(const unsigned long long *key, int n, long long n_zero, uint8_t *__restrict__ gamma)
 {
     __shared__ SmallSelect<kScoreThreads> sh;
     __shared__ unsigned long long s_key[kScoreThreads];
@@ -718,7 +718,7 @@ segment_kernel(const unsigned long long *__restrict__ key, int n, long long n_ze
         return;
     }
     if (n <= kScoreThreads) {
-        const unsigned long long mine = tid < n ? __ldg(k + tid) : ~0ull;
+        const unsigned long long mine = tid < n ? __ldcg(k + tid) : ~0ull;
         s_key[tid] = mine;
         __syncthreads();
         int rank = 0;
@@ -732,7 +732,7 @@ segment_kernel(const unsigned long long *__restrict__ key, int n, long long n_ze
     unsigned long long v[kKeysPerThread], T;
     long long ties;
     unsigned same;
-    load_keys<false>(k, n, v);
+    load_keys(k, n, v);
     select_small(v, n, n_zero, sh, T, ties, same);
     long long before = 0;                                  // keys equal to T in the stretches of 256 before this one
 #pragma unroll
@@ -761,7 +761,7 @@ segment_kernel(const unsigned long long *__restrict__ key, int n, long long n_ze
 constexpr int kMidThreads = 1024;
 constexpr int kMidMax = kMidThreads * kKeysPerThread;
 __global__ void __launch_bounds__(kMidThreads)
-select_mid_kernel(const unsigned long long *__restrict__ key, int n, long long n_zero, uint8_t *__restrict__ gamma)
+select_mid_kernel(const unsigned long long *key, int n, long long n_zero, uint8_t *__restrict__ gamma)
 {
     __shared__ SmallSelect<kMidThreads> sh;
     const int tid = threadIdx.x, i = blockIdx.x * kMidThreads + tid;
@@ -773,8 +773,8 @@ select_mid_kernel(const unsigned long long *__restrict__ key, int n, long long n
     unsigned long long v[kKeysPerThread], T;
     long long ties;
     unsigned same;
-    load_keys<false, kMidThreads>(key, n, v);
-    const unsigned long long mine = i < n ? __ldg(key + i) : ~0ull;
+    load_keys<kMidThreads>(key, n, v);
+    const unsigned long long mine = i < n ? __ldcg(key + i) : ~0ull;
     select_small(v, n, n_zero, sh, T, ties, same);
     long long rank = 0;                                    // keys equal to T before this one
     const bool eq = i < n && mine == T;
@@ -824,7 +824,7 @@ mask_small_kernel(const uint32_t *__restrict__ W, int I, int HK, int bo, int bi,
     }
     // every key of the layer (written by other CTAs of this launch: read through L2)
     unsigned long long v[kKeysPerThread];
-    load_keys<true>((const unsigned long long *)score, NB, v);
+    load_keys((const unsigned long long *)score, NB, v);
     const int first = blockIdx.x * BC;                         // this CTA's first block
     if (seg_len == NB && NB > kCountMax) {
         const int i = first + (int)threadIdx.x;

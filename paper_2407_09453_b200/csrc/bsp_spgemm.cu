@@ -21,13 +21,13 @@ constexpr int kSpEdge = 8;
 // One row of an 8 x 8 block (8 consecutive values) as floats: two 16-byte loads for fp32, one for bf16.
 __device__ __forceinline__ void sp_row(const float *p, float (&v)[8])
 {
-    const float4 a = __ldg((const float4 *)p), b = __ldg((const float4 *)p + 1);
+    const float4 a = *(const float4 *)p, b = *((const float4 *)p + 1);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 // The 8 x 8 block of C of one row of A and one row of B: acc0, acc1 are this lane's entries (r, 2c), (r, 2c + 1) with
 // r = lane / 4, c = lane % 4.  `pos_of` gives the payload position of the A row's block in column k, or -1.
 template <typename T, typename F>
-__device__ __forceinline__ void sp_pair(const T *__restrict__ a_payload, const int32_t *__restrict__ b_col_idx, const T *__restrict__ b_payload,
+__device__ __forceinline__ void sp_pair(const T *a_payload, const int32_t *b_col_idx, const T *b_payload,
                                         int lo, int hi, int NBk, int lane, F pos_of, float &acc0, float &acc1, int *status)
 {
     const int r = lane >> 2, c = (lane & 3) * 2;
@@ -53,9 +53,9 @@ __device__ __forceinline__ void sp_pair(const T *__restrict__ a_payload, const i
                 const int na1 = __shfl_sync(0xFFFFFFFFu, pa, s1);
                 const int na2 = __shfl_sync(0xFFFFFFFFu, pa, s2 < 0 ? s1 : s2);
                 const uint32_t *Aw = (const uint32_t *)a_payload, *Bw = (const uint32_t *)b_payload;
-                const uint32_t a0 = __ldg(Aw + (size_t)na1 * 32 + lane), b0 = __ldg(Bw + (size_t)(base + s1) * 32 + lane);
+                const uint32_t a0 = Aw[(size_t)na1 * 32 + lane], b0 = Bw[(size_t)(base + s1) * 32 + lane];
                 uint32_t a2 = 0u, b1 = 0u;
-                if (s2 >= 0) { a2 = __ldg(Aw + (size_t)na2 * 32 + lane); b1 = __ldg(Bw + (size_t)(base + s2) * 32 + lane); }
+                if (s2 >= 0) { a2 = Aw[(size_t)na2 * 32 + lane]; b1 = Bw[(size_t)(base + s2) * 32 + lane]; }
                 float d2 = 0.f, d3 = 0.f;
                 asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};\n"
                              : "+f"(acc0), "+f"(acc1), "+f"(d2), "+f"(d3) : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
@@ -80,9 +80,9 @@ __device__ __forceinline__ void sp_pair(const T *__restrict__ a_payload, const i
 
 template <typename T>
 __global__ void __launch_bounds__(kSpThreads)
-spgemm_kernel(const int32_t *__restrict__ a_row_ptr, const int32_t *__restrict__ a_col_idx, const T *__restrict__ a_payload,
-              const int32_t *__restrict__ b_row_ptr, const int32_t *__restrict__ b_col_idx, const T *__restrict__ b_payload,
-              int NBb, int NBk, float *__restrict__ C, int *status)
+spgemm_kernel(const int32_t *a_row_ptr, const int32_t *a_col_idx, const T *a_payload,
+              const int32_t *b_row_ptr, const int32_t *b_col_idx, const T *b_payload,
+              int NBb, int NBk, float *C, int *status)
 {
     extern __shared__ int s_pos[];                 // [NBk]: payload position of row i's block in column k, or -1
     const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -93,7 +93,8 @@ spgemm_kernel(const int32_t *__restrict__ a_row_ptr, const int32_t *__restrict__
     // each CTA, 64.3.)
     wait_for_previous<false>();
     __syncthreads();
-    for (int n = a_row_ptr[i] + threadIdx.x; n < a_row_ptr[i + 1]; n += kSpThreads) {
+    const int a_end = a_row_ptr[i + 1];
+    for (int n = a_row_ptr[i] + threadIdx.x; n < a_end; n += kSpThreads) {
         const int k = a_col_idx[n];
         if (k >= 0 && k < NBk) s_pos[k] = n;
         else atomicMax(status, (int)BSP_ERR_INDEX);          // a column outside the matrix: skipped
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
         for (int n = lo + lane; n < hi; n += 128) {
             int k[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) k[u] = n + 32 * u < hi ? __ldg(ci + n + 32 * u) : 0;
+            for (int u = 0; u < 4; ++u) k[u] = n + 32 * u < hi ? ci[n + 32 * u] : 0;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (n + 32 * u >= hi) continue;
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
             for (int u = 0; u < kUnits; ++u) {
                 const int n = pos[(kW / 2) * u * pitch + c * 8];
                 w[u] = make_uint4(0u, 0u, 0u, 0u);
-                if (n >= 0) w[u] = __ldg((const uint4 *)(src[u] + (size_t)n * 128));
+                if (n >= 0) w[u] = *(const uint4 *)(src[u] + (size_t)n * 128);
             }
         };
         uint32_t slot = (uint32_t)grp, epar = 1;               // (a fresh barrier counts as released)

@@ -111,3 +111,68 @@ def test_products_of_different_kinds_take_turns():
         lay.check(), sa.check()
         return a, b, Cm
     compare(program)
+
+
+@pytest.mark.parametrize("scope", [bsp.SCOPE_LAYER, bsp.SCOPE_ROW])
+@pytest.mark.parametrize("C,canonical", [(256, True), (1024, True), (1024, False), (1088, False)])
+def test_set_up_of_weights_that_the_product_before_wrote(C, canonical, scope):
+    """Mask, compaction and product by turns, the output of each product being the weights of the next layer: layers of 1024, 16384
+    and 18496 blocks, ranked as a whole and by rows, with and without the canonical payload."""
+    lay = bsp.SparseLayer(C, C, 1, 1, 8, 8, torch.bfloat16, canonical=canonical)
+    W0, X = randn(11, (C, C), C ** -0.5).to(torch.bfloat16), randn(12, (C, C), C ** -0.5).to(torch.bfloat16)
+    n_zero = lay.NBo * lay.NBi // 4 if scope == bsp.SCOPE_LAYER else lay.NBi // 4
+
+    def program(wait):
+        a, b = W0.clone(), torch.empty_like(W0)
+        for _ in range(8):
+            lay.mask(a, n_zero, scope=scope)
+            wait()
+            lay.compact(a)
+            wait()
+            lay.gemm(X, None, b)
+            wait()
+            a, b = b, a
+        lay.check()
+        return (a, b, lay.gamma, lay.row_ptr, lay.col_idx[:lay.nnz]) + ((lay.payload[:lay.nnz * 64],) if canonical else ())
+    compare(program)
+
+
+def test_sparse_operands_that_the_call_before_wrote():
+    """fp32: a sparse x sparse product is masked, compacted and multiplied by itself again.  bfloat16: operands pruned again
+    between the products, in the tensor-core form and the sparse form."""
+    C = 256
+    lay = bsp.SparseLayer(C, C, 1, 1, 8, 8, torch.float32)
+    W0 = randn(13, (C, C), 0.5 * C ** -0.5)
+
+    def square(wait):
+        a, b = W0.clone(), torch.empty_like(W0)
+        for _ in range(4):
+            lay.mask(a, lay.NBo * lay.NBi // 2)
+            wait()
+            lay.compact(a)
+            wait()
+            bsp.bsp_spgemm(lay.wd, lay.handle(), lay.wd, lay.handle(), b, lay.ws)
+            wait()
+            a, b = b, a
+        lay.check()
+        return a, b
+    compare(square)
+
+    sa, sb = bsp.SparseLayer(512, 1024, 1, 1, 8, 8, torch.bfloat16), bsp.SparseLayer(256, 1024, 1, 1, 8, 8, torch.bfloat16)
+    Ws = [(randn(20 + k, (512, 1024)).to(torch.bfloat16), randn(30 + k, (256, 1024)).to(torch.bfloat16)) for k in range(4)]
+
+    def prune(wait):
+        out = []
+        for quarters in (1, 3):
+            for A, B in Ws:
+                for q, W in ((sa, A), (sb, B)):
+                    q.mask(W, q.NBo * q.NBi * quarters // 4)
+                    wait()
+                    q.compact(W)
+                    wait()
+                out.append(torch.empty((512, 256), device="cuda"))
+                bsp.bsp_spgemm(sa.wd, sa.handle(), sb.wd, sb.handle(), out[-1], sa.ws)
+                wait()
+        sa.check(), sb.check()
+        return out
+    compare(prune)
