@@ -386,6 +386,8 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
     double best = 0.95 * (2.9 + (bulk > chain ? bulk : chain));
     StPlan plan = {0, 1};
     const int n_chunks = (NBk + 7) / 8;
+    // (the row tiles of A are the grid's y extent, which ends at 65535; the sparse form has a row of A per CTA along x)
+    if ((NBa + kStARows - 1) / kStARows > 65535) return plan;
     for (int w = 0; w < 3; ++w) {
         const int BN = 64 << w;
         const int stages = spgemm_tc_stages(BN, n_chunks);

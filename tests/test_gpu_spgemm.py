@@ -52,6 +52,34 @@ def test_spgemm_tensor_core_tiles(Oa, Ob, I, fa, fb):
     run_spgemm(931, Oa, Ob, I, "bf16", fa, fb)
 
 
+def test_spgemm_more_rows_than_a_grid_is_high():
+    """1048577 block rows of A, one more than 65535 row tiles hold.  Few of them have blocks; the count in the handle says that all
+    do, as for a mask that keeps everything (it chooses the kernel)."""
+    NBa, NBb, NBk = 16 * 65535 + 1, 8, 64
+    rows, cols = [0, 7, 524288, NBa - 1], [0, 5, 63]
+    n = len(rows) * len(cols)
+    row_ptr = torch.zeros(NBa + 1, dtype=torch.int32, device="cuda")
+    for r in rows:
+        row_ptr[r + 1:] += len(cols)
+    col_idx = torch.tensor(cols * len(rows), dtype=torch.int32, device="cuda")
+    payload = torch.randn((n, 8, 8), device="cuda").to(torch.bfloat16)
+    lb = bsp.SparseLayer(NBb * 8, NBk * 8, 1, 1, 8, 8, torch.bfloat16)
+    B = torch.randn((NBb * 8, NBk * 8), device="cuda").to(torch.bfloat16)
+    lb.mask(B, 0)
+    lb.compact(B)
+    wa = bsp.wdesc(NBa * 8, NBk * 8, 1, 1, 8, 8, bsp.BF16)
+    Cm = torch.full((NBa * 8, NBb * 8), -7.0, device="cuda")
+    bsp.bsp_spgemm(wa, bsp.bcsr(row_ptr, col_idx, payload, None, NBa * NBk), lb.wd, lb.handle(), Cm, lb.ws)
+    lb.check()
+    for k, r in enumerate(rows):
+        A = torch.zeros((8, NBk, 8), dtype=torch.float64, device="cuda")
+        A[:, cols] = payload[k * len(cols):(k + 1) * len(cols)].double().permute(1, 0, 2)
+        want = A.reshape(8, -1) @ B.double().T
+        assert rel_err(Cm[r * 8:r * 8 + 8].cpu().numpy(), want.cpu().numpy()) <= 2e-5
+        Cm[r * 8:r * 8 + 8] = 0.0
+    assert not bool(Cm.any())
+
+
 def test_spgemm_dropped_blocks_hide_non_finite_weights():
     """An infinite weight reaches the blocks of C whose row of B keeps its column, and no other."""
     O, I = 256, 512
