@@ -58,6 +58,8 @@ _ARGS = {"bsp_mask": "ppiilpppp", "bsp_mask_static": "ppiilpp", "bsp_compact_nnz
 _BOUND = ["bsp_mask", "bsp_compact", "bsp_gemm", "bsp_conv2d", "bsp_gemm_q8", "bsp_conv2d_q8", "bsp_conv2d_chain",
           "bsp_conv2d_chain_q8", "bsp_spgemm"]
 
+_C_DATA = C.Structure.__mro__[-2]                      # the base of all ctypes objects
+
 _lib = None
 
 
@@ -94,7 +96,7 @@ def _native():
         except ImportError as e:
             raise RuntimeError("_bspcall.so is missing or of another PyTorch: run `python -m paper_2407_09453_b200.build` "
                                f"(or __graft_entry__.build()): {e}") from e
-        _bspcall.bind(*[C.cast(getattr(L, n), C.c_void_p).value for n in _BOUND])
+        _bspcall.bind(_C_DATA, *[C.cast(getattr(L, n), C.c_void_p).value for n in _BOUND])
         _calls = _bspcall
     return _calls
 

@@ -34,15 +34,31 @@ void *pointer(PyObject *o)
 {
     if (o == Py_None) return nullptr;
     if (THPVariable_CheckExact(o)) return THPVariable_Unpack(o).data_ptr();
-    if (PyLong_Check(o)) return address(Py_NewRef(o));
     return address(PyObject_CallMethod(o, "data_ptr", nullptr));
 }
 
+// An int, as ctypes takes it: nothing that only converts to one.
 long long integer(PyObject *o)
 {
+    if (!PyLong_Check(o)) {
+        PyErr_Format(PyExc_TypeError, "int expected instead of %.200s instance", Py_TYPE(o)->tp_name);
+        throw Failed();
+    }
     const unsigned long long v = PyLong_AsUnsignedLongLongMask(o);
     if (PyErr_Occurred()) throw Failed();
     return (long long)v;
+}
+
+// A layer's number of blocks, which may be any object that int() takes (a mask's sum).
+long long count(PyObject *o)
+{
+    if (PyLong_Check(o)) return integer(o);
+    PyObject *v = PyNumber_Long(o);
+    if (v == nullptr) throw Failed();
+    const unsigned long long n = PyLong_AsUnsignedLongLongMask(v);
+    Py_DECREF(v);
+    if (PyErr_Occurred()) throw Failed();
+    return (long long)n;
 }
 
 void *stream(PyObject *o)
@@ -52,9 +68,14 @@ void *stream(PyObject *o)
 }
 
 // A ctypes structure: its own memory, which the caller's reference keeps for the call.
+PyTypeObject *c_data;                                          // the base of all ctypes objects, set by bind()
 template <class T>
 T *structure(PyObject *o)
 {
+    if (!PyObject_TypeCheck(o, c_data)) {
+        PyErr_Format(PyExc_TypeError, "a ctypes structure expected instead of %.200s instance", Py_TYPE(o)->tp_name);
+        throw Failed();
+    }
     Py_buffer view;
     if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw Failed();
     void *p = view.buf;
@@ -159,7 +180,7 @@ bsp_bcsr handle_of(PyObject *const *a)                         // row_ptr, col_i
     w.col_idx = (const int32_t *)pointer(a[1]);
     w.payload = pointer(a[2]);
     w.packed = pointer(a[3]);
-    w.nnz = integer(a[4]);
+    w.nnz = count(a[4]);
     return w;
 }
 
@@ -243,20 +264,27 @@ PyObject *layer_conv2d(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
-// bind(mask, compact, gemm, conv2d, gemm_q8, conv2d_q8, chain, chain_q8, spgemm): the addresses of the loaded library's functions
+// bind(c_data, mask, compact, gemm, conv2d, gemm_q8, conv2d_q8, chain, chain_q8, spgemm): the base of ctypes objects and the addresses
+// of the loaded library's functions
 PyObject *bind(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
-    if (!count_is(n, 9)) return nullptr;
+    if (!count_is(n, 10)) return nullptr;
     return guarded([&] {
-        f_mask = (decltype(f_mask))pointer(a[0]);
-        f_compact = (decltype(f_compact))pointer(a[1]);
-        f_gemm = (decltype(f_gemm))pointer(a[2]);
-        f_conv2d = (decltype(f_conv2d))pointer(a[3]);
-        f_gemm_q8 = (decltype(f_gemm_q8))pointer(a[4]);
-        f_conv2d_q8 = (decltype(f_conv2d_q8))pointer(a[5]);
-        f_chain = (decltype(f_chain))pointer(a[6]);
-        f_chain_q8 = (decltype(f_chain_q8))pointer(a[7]);
-        f_spgemm = (decltype(f_spgemm))pointer(a[8]);
+        if (!PyType_Check(a[0])) {
+            PyErr_SetString(PyExc_TypeError, "not a type");
+            throw Failed();
+        }
+        Py_INCREF(a[0]);                                       // (kept as long as the module is)
+        c_data = (PyTypeObject *)a[0];
+        f_mask = (decltype(f_mask))integer(a[1]);
+        f_compact = (decltype(f_compact))integer(a[2]);
+        f_gemm = (decltype(f_gemm))integer(a[3]);
+        f_conv2d = (decltype(f_conv2d))integer(a[4]);
+        f_gemm_q8 = (decltype(f_gemm_q8))integer(a[5]);
+        f_conv2d_q8 = (decltype(f_conv2d_q8))integer(a[6]);
+        f_chain = (decltype(f_chain))integer(a[7]);
+        f_chain_q8 = (decltype(f_chain_q8))integer(a[8]);
+        f_spgemm = (decltype(f_spgemm))integer(a[9]);
         return 0;
     });
 }

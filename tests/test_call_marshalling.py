@@ -1,5 +1,6 @@
 """The compiled marshalling of the Python calls (csrc/bsp_call.cpp): every argument arrives as the C ABI declares it, wrong
 kinds raise, and refused calls give the library's own status.  No call here reaches a launch."""
+import numpy as np
 import pytest
 import torch
 
@@ -54,6 +55,30 @@ def test_wrong_kinds_raise(call):
     args = [bsp.wdesc(64, 64, 1, 1, 8, 8, bsp.BF16), bsp.bcsr(i, i, p, p, 8), p, 4, None, p, bsp.F32, p, object()]
     with pytest.raises((TypeError, AttributeError)):
         call(bsp._native(), args)
+
+
+@pytest.mark.parametrize("k,other", [(0, bytes(28)), (0, np.zeros(7, np.int32)), (1, bytes(40)), (2, 4096), (7, 4096), (3, np.int64(4)), (3, torch.tensor(4)),
+                                     (6, np.int32(0))], ids=["bytes-wd", "array-wd", "bytes-handle", "address-x", "address-ws", "numpy-P", "tensor-P", "numpy-type"])
+def test_only_the_declared_kinds_are_taken(k, other):
+    """A descriptor is a ctypes structure, a buffer is an object with data_ptr() and no address, a count is an int: what merely
+    has the bytes or converts is refused, as ctypes refuses it."""
+    i, p = buffers()
+    args = [bsp.wdesc(64, 64, 1, 1, 8, 8, bsp.BF16), bsp.bcsr(i, i, p, p, 8), p, 4, None, p, bsp.F32, p, Stream()]
+    args[5] = p[1:]                              # (a misaligned output: a call that got through would be refused by the library)
+    with pytest.raises(bsp.BspError):
+        bsp.bsp_gemm(*args)
+    args[k] = other
+    with pytest.raises((TypeError, AttributeError)):
+        bsp.bsp_gemm(*args)
+
+
+@pytest.mark.parametrize("nnz", [np.int64(8), torch.tensor(8), 8.0])
+def test_a_layer_takes_any_count(nnz):
+    lay, x = bsp.SparseLayer(64, 64, 1, 1, 8, 8, torch.bfloat16, device="cpu"), torch.zeros(4, 64, dtype=torch.bfloat16)
+    lay.nnz = nnz
+    assert lay.handle().nnz == 8
+    with pytest.raises(bsp.BspError):
+        lay.gemm(x, None, torch.zeros(4, 64, dtype=torch.int32), Stream())
 
 
 def test_input_shape_and_output_type():
