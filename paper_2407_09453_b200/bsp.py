@@ -276,21 +276,37 @@ class SparseLayer:
     def handle(self) -> Bcsr:
         return bcsr(self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity))
 
+    # (The compiled calls answer None to what is not a plain tensor of the usual rank and type.)
     def conv2d(self, X, bias, Y, stride=(1, 1), pad=(0, 0), stream=None):
-        _raise(_native().layer_conv2d(False, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
-                                      X, bias, None, Y, stride[0], stride[1], pad[0], pad[1], self.ws, stream), "bsp_conv2d")
+        rc = _native().layer_conv2d(False, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
+                                    X, bias, None, Y, stride[0], stride[1], pad[0], pad[1], self.ws, stream)
+        if rc is None:
+            N, L, J, _ = X.shape
+            return bsp_conv2d(self.wd, self.handle(), XDesc(N, L, J, stride[0], stride[1], pad[0], pad[1]), X, bias, Y, dtype_code(Y.dtype),
+                              self.ws, stream)
+        _raise(rc, "bsp_conv2d")
 
     def gemm(self, X, bias, Y, stream=None):
-        _raise(_native().layer_gemm(False, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
-                                    X, bias, None, Y, self.ws, stream), "bsp_gemm")
+        rc = _native().layer_gemm(False, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
+                                  X, bias, None, Y, self.ws, stream)
+        if rc is None:
+            return bsp_gemm(self.wd, self.handle(), X, X.shape[0], bias, Y, dtype_code(Y.dtype), self.ws, stream)
+        _raise(rc, "bsp_gemm")
 
     def conv2d_q8(self, X, bias, shift, Y, stride=(1, 1), pad=(0, 0), stream=None):
-        _raise(_native().layer_conv2d(True, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
-                                      X, bias, shift, Y, stride[0], stride[1], pad[0], pad[1], self.ws, stream), "bsp_conv2d_q8")
+        rc = _native().layer_conv2d(True, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
+                                    X, bias, shift, Y, stride[0], stride[1], pad[0], pad[1], self.ws, stream)
+        if rc is None:
+            N, L, J, _ = X.shape
+            return bsp_conv2d_q8(self.wd, self.handle(), XDesc(N, L, J, stride[0], stride[1], pad[0], pad[1]), X, bias, shift, Y, self.ws, stream)
+        _raise(rc, "bsp_conv2d_q8")
 
     def gemm_q8(self, X, bias, shift, Y, stream=None):
-        _raise(_native().layer_gemm(True, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
-                                    X, bias, shift, Y, self.ws, stream), "bsp_gemm_q8")
+        rc = _native().layer_gemm(True, self.wd, self.row_ptr, self.col_idx, self.payload, self.packed, min(self.nnz, self.capacity),
+                                  X, bias, shift, Y, self.ws, stream)
+        if rc is None:
+            return bsp_gemm_q8(self.wd, self.handle(), X, X.shape[0], bias, shift, Y, self.ws, stream)
+        _raise(rc, "bsp_gemm_q8")
 
     def check(self, stream=None):
         bsp_check(self.ws, stream)

@@ -172,6 +172,8 @@ BSP_CALL(spgemm, f_spgemm)
 #undef BSP_CALL
 
 // ---- the calls of SparseLayer: the handle, the input's shape and the output's type are read here ----
+// What is not a plain tensor of the expected rank and type gets None for an answer and is read in Python, as every object with a
+// shape, a type and data_ptr() was, with the errors that come from there.
 
 bsp_bcsr handle_of(PyObject *const *a)                         // row_ptr, col_idx, payload, packed, nnz
 {
@@ -184,25 +186,20 @@ bsp_bcsr handle_of(PyObject *const *a)                         // row_ptr, col_i
     return w;
 }
 
-const at::Tensor &tensor(PyObject *o)
+bool plain_input(PyObject *x, int64_t dims)
 {
-    if (!THPVariable_Check(o)) {
-        PyErr_SetString(PyExc_TypeError, "not a tensor");
-        throw Failed();
-    }
-    return THPVariable_Unpack(o);
+    return THPVariable_CheckExact(x) && THPVariable_Unpack(x).dim() == dims;
 }
 
-bsp_dtype type_of(const at::Tensor &t)
+bool type_of(PyObject *y, bsp_dtype &t)
 {
-    switch (t.scalar_type()) {
-    case at::kFloat: return BSP_F32;
-    case at::kBFloat16: return BSP_BF16;
-    case at::kChar: return BSP_I8;
-    case at::kInt: return BSP_I32;
-    default:
-        PyErr_SetString(PyExc_KeyError, c10::toString(t.scalar_type()));
-        throw Failed();
+    if (!THPVariable_CheckExact(y)) return false;
+    switch (THPVariable_Unpack(y).scalar_type()) {
+    case at::kFloat: t = BSP_F32; return true;
+    case at::kBFloat16: t = BSP_BF16; return true;
+    case at::kChar: t = BSP_I8; return true;
+    case at::kInt: t = BSP_I32; return true;
+    default: return false;
     }
 }
 
@@ -221,15 +218,16 @@ PyObject *layer_gemm(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     if (!count_is(n, 13)) return nullptr;
     const bool q8 = *a++ == Py_True;
+    bsp_dtype yt = BSP_I8;
+    if (!plain_input(a[6], 2) || (!q8 && !type_of(a[9], yt))) Py_RETURN_NONE;
     return guarded([&] {
         const bsp_wdesc *wd = structure<bsp_wdesc>(a[0]);
         const bsp_bcsr w = handle_of(a + 1);
-        const int64_t P = tensor(a[6]).size(0);
+        const int64_t P = THPVariable_Unpack(a[6]).size(0);
         const void *X = pointer(a[6]), *bias = pointer(a[7]);
         void *Y = pointer(a[9]), *ws = pointer(a[10]);
         if (q8)
             return enqueue(f_gemm_q8, wd, &w, X, P, (const int32_t *)bias, (const int32_t *)pointer(a[8]), (int8_t *)Y, ws, stream(a[11]));
-        const bsp_dtype yt = type_of(tensor(a[9]));
         return enqueue(f_gemm, wd, &w, X, P, bias, Y, yt, ws, stream(a[11]));
     });
 }
@@ -239,14 +237,12 @@ PyObject *layer_conv2d(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     if (!count_is(n, 17)) return nullptr;
     const bool q8 = *a++ == Py_True;
+    bsp_dtype yt = BSP_I8;
+    if (!plain_input(a[6], 4) || (!q8 && !type_of(a[9], yt))) Py_RETURN_NONE;
     return guarded([&] {
         const bsp_wdesc *wd = structure<bsp_wdesc>(a[0]);
         const bsp_bcsr w = handle_of(a + 1);
-        const at::Tensor &x = tensor(a[6]);
-        if (x.dim() != 4) {
-            PyErr_SetString(PyExc_ValueError, "the input of a convolution has four dimensions: N, L, J, I");
-            throw Failed();
-        }
+        const at::Tensor &x = THPVariable_Unpack(a[6]);
         bsp_xdesc xd;
         xd.N = (int)x.size(0);
         xd.L = (int)x.size(1);
@@ -259,7 +255,6 @@ PyObject *layer_conv2d(PyObject *, PyObject *const *a, Py_ssize_t n)
         void *Y = pointer(a[9]), *ws = pointer(a[14]);
         if (q8)
             return enqueue(f_conv2d_q8, wd, &w, &xd, X, (const int32_t *)bias, (const int32_t *)pointer(a[8]), (int8_t *)Y, ws, stream(a[15]));
-        const bsp_dtype yt = type_of(tensor(a[9]));
         return enqueue(f_conv2d, wd, &w, &xd, X, bias, Y, yt, ws, stream(a[15]));
     });
 }

@@ -88,3 +88,42 @@ def test_input_shape_and_output_type():
         lay.conv2d(x, None, x, stream=Stream())
     with pytest.raises(KeyError):
         lay.gemm(x, None, x.double(), stream=Stream())
+
+
+class Buffer:
+    """What a layer's calls read of a buffer: a shape, a type and an address."""
+
+    def __init__(self, t):
+        self.t, self.shape, self.dtype = t, t.shape, t.dtype
+
+    def data_ptr(self):
+        return self.t.data_ptr()
+
+
+def test_a_layer_takes_any_buffer_with_a_shape_and_a_type():
+    lay, s = bsp.SparseLayer(64, 64, 1, 1, 8, 8, torch.bfloat16, device="cpu"), Stream()
+    x, y = torch.zeros(4, 1, 1, 64, dtype=torch.bfloat16), torch.zeros(4, 64)
+    x2 = x.view(4, 64)
+    class Sub(torch.Tensor):
+        pass
+    for X in (Buffer(x), x.as_subclass(Sub)):
+        for Y, want in ((Buffer(y[:0]), bsp.ERR_NULL), (Buffer(y.to(torch.int32)), bsp.ERR_DTYPE)):      # (an empty tensor has no address)
+            with pytest.raises(bsp.BspError) as e:
+                lay.conv2d(X, None, Y, stream=s)
+            assert e.value.status == want
+    for X in (Buffer(x2), x2.as_subclass(Sub)):
+        with pytest.raises(bsp.BspError) as e:
+            lay.gemm(X, None, Buffer(y.to(torch.int32)), s)
+        assert e.value.status == bsp.ERR_DTYPE
+    for X in (Buffer(x), x):
+        with pytest.raises(bsp.BspError) as e:
+            lay.conv2d_q8(X, None, None, Buffer(y.to(torch.int8)), stream=s)
+        assert e.value.status == bsp.ERR_NULL
+    for X in (x2[0].view(64), x.view(2, 2, 64)):                           # any rank: the first extent counts
+        with pytest.raises(bsp.BspError) as e:
+            lay.gemm_q8(X, None, None, y.to(torch.int8), s)
+        assert e.value.status == bsp.ERR_NULL
+    with pytest.raises(IndexError):
+        lay.gemm(x.sum(), None, y, s)
+    with pytest.raises(AttributeError):
+        lay.gemm(None, None, y, s)
