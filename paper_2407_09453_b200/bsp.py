@@ -91,11 +91,11 @@ def _native():
     global _calls
     if _calls is None:
         L = lib()
-        try:
-            from . import _bspcall
-        except ImportError as e:
-            raise RuntimeError("_bspcall.so is missing or of another PyTorch: run `python -m paper_2407_09453_b200.build` "
-                               f"(or __graft_entry__.build()): {e}") from e
+        from . import build
+        if not build.call_is_current():
+            raise RuntimeError("_bspcall.so is missing or of another PyTorch or Python: run `python -m paper_2407_09453_b200.build` "
+                               "(or __graft_entry__.build())")
+        from . import _bspcall
         _bspcall.bind(_C_DATA, *[C.cast(getattr(L, n), C.c_void_p).value for n in _BOUND])
         _calls = _bspcall
     return _calls

@@ -49,9 +49,27 @@ def _flags(verbose: bool):
     return f
 
 
+def call_stamp() -> str:
+    """What the marshalling is compiled against: it reads tensors in place, so another PyTorch or Python needs another build."""
+    import torch
+    return "%s %s %d" % (torch.__version__, sysconfig.get_config_var("SOABI"), int(torch.compiled_with_cxx11_abi()))
+
+
+def call_is_current() -> bool:
+    """Whether the built marshalling is one for the Python and PyTorch that run: the stamp stands behind the file's own contents."""
+    stamp = call_stamp().encode()
+    try:
+        with open(CALL, "rb") as f:
+            f.seek(0, os.SEEK_END)
+            f.seek(max(0, f.tell() - len(stamp) - 1))
+            return f.read() == b"\n" + stamp
+    except OSError:
+        return False
+
+
 def build_call(force: bool = False) -> str:
     """Compile the marshalling of the Python calls against the installed Python and PyTorch; returns its path."""
-    if not force and not _newer([CALL_SOURCE] + _headers(), CALL):
+    if not force and call_is_current() and not _newer([CALL_SOURCE] + _headers(), CALL):
         return CALL
     import torch
     root = os.path.dirname(os.path.abspath(torch.__file__))
@@ -61,6 +79,8 @@ def build_call(force: bool = False) -> str:
     subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
                            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi())] + ["-I" + d for d in include] +
                           [CALL_SOURCE, "-o", tmp, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-lc10", "-lc10_cuda"])
+    with open(tmp, "ab") as f:
+        f.write(b"\n" + call_stamp().encode())
     os.replace(tmp, CALL)
     return CALL
 

@@ -127,3 +127,25 @@ def test_a_layer_takes_any_buffer_with_a_shape_and_a_type():
         lay.gemm(x.sum(), None, y, s)
     with pytest.raises(AttributeError):
         lay.gemm(None, None, y, s)
+
+
+def test_a_marshalling_of_another_pytorch_is_built_again_and_not_loaded(monkeypatch, tmp_path):
+    """It reads tensors in place: what was compiled against other headers must not be loaded, and a build replaces it whatever
+    the times of the files say."""
+    so = tmp_path / "_bspcall.so"
+    so.write_bytes(b"")
+    monkeypatch.setattr(build, "CALL", str(so))
+    runs = []
+    monkeypatch.setattr(build.subprocess, "check_call", lambda cmd: (runs.append(cmd), open(cmd[cmd.index("-o") + 1], "wb").close()))
+    monkeypatch.setattr(bsp, "_calls", None)
+    with pytest.raises(RuntimeError, match="build"):
+        bsp._native()
+    build.build_call()
+    assert len(runs) == 1 and build.call_is_current()
+    build.build_call()
+    assert len(runs) == 1
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    with pytest.raises(RuntimeError, match="build"):
+        bsp._native()
+    build.build_call()
+    assert len(runs) == 2 and build.call_is_current()
