@@ -21,11 +21,12 @@ constexpr int kSpEdge = 8;
 // One row of an 8 x 8 block (8 consecutive values) as floats: two 16-byte loads for fp32, one for bf16.
 __device__ __forceinline__ void sp_row(const float *p, float (&v)[8])
 {
-    const float4 a = *(const float4 *)p, b = *((const float4 *)p + 1);
+    const float4 a = load_free((const float4 *)p), b = load_free((const float4 *)p + 1);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 // The 8 x 8 block of C of one row of A and one row of B: acc0, acc1 are this lane's entries (r, 2c), (r, 2c + 1) with
-// r = lane / 4, c = lane % 4.  `pos_of` gives the payload position of the A row's block in column k, or -1.
+// r = lane / 4, c = lane % 4.  `pos_of` gives the payload position of the A row's block in column k, or -1.  The pointers come
+// through from_here().
 template <typename T, typename F>
 __device__ __forceinline__ void sp_pair(const T *a_payload, const int32_t *b_col_idx, const T *b_payload,
                                         int lo, int hi, int NBk, int lane, F pos_of, float &acc0, float &acc1, int *status)
@@ -35,7 +36,7 @@ __device__ __forceinline__ void sp_pair(const T *a_payload, const int32_t *b_col
         const int nb = base + lane;
         int pa = -1;
         if (nb < hi) {
-            const int k = b_col_idx[nb];
+            const int k = load_free(b_col_idx + nb);
             if (k >= 0 && k < NBk) pa = pos_of(k);
             else atomicMax(status, (int)BSP_ERR_INDEX);
         }
@@ -53,9 +54,9 @@ __device__ __forceinline__ void sp_pair(const T *a_payload, const int32_t *b_col
                 const int na1 = __shfl_sync(0xFFFFFFFFu, pa, s1);
                 const int na2 = __shfl_sync(0xFFFFFFFFu, pa, s2 < 0 ? s1 : s2);
                 const uint32_t *Aw = (const uint32_t *)a_payload, *Bw = (const uint32_t *)b_payload;
-                const uint32_t a0 = Aw[(size_t)na1 * 32 + lane], b0 = Bw[(size_t)(base + s1) * 32 + lane];
+                const uint32_t a0 = load_free(Aw + (size_t)na1 * 32 + lane), b0 = load_free(Bw + (size_t)(base + s1) * 32 + lane);
                 uint32_t a2 = 0u, b1 = 0u;
-                if (s2 >= 0) { a2 = Aw[(size_t)na2 * 32 + lane]; b1 = Bw[(size_t)(base + s2) * 32 + lane]; }
+                if (s2 >= 0) { a2 = load_free(Aw + (size_t)na2 * 32 + lane); b1 = load_free(Bw + (size_t)(base + s2) * 32 + lane); }
                 float d2 = 0.f, d3 = 0.f;
                 asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};\n"
                              : "+f"(acc0), "+f"(acc1), "+f"(d2), "+f"(d3) : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
@@ -92,6 +93,8 @@ spgemm_kernel(const int32_t *a_row_ptr, const int32_t *a_col_idx, const T *a_pay
     // next one let in at once, 12.2 without programmatic launches; 232 x 2264 x 632 fp32 at 25 % 62.0, 78.1 let in at the end of
     // each CTA, 64.3.)
     wait_for_previous<false>();
+    a_payload = from_here(a_payload); b_payload = from_here(b_payload);
+    b_col_idx = from_here(b_col_idx); b_row_ptr = from_here(b_row_ptr);
     __syncthreads();
     const int a_end = a_row_ptr[i + 1];
     for (int n = a_row_ptr[i] + threadIdx.x; n < a_end; n += kSpThreads) {
@@ -104,7 +107,7 @@ spgemm_kernel(const int32_t *a_row_ptr, const int32_t *a_col_idx, const T *a_pay
     const size_t ldc = (size_t)NBb * kSpEdge;
     for (int j = blockIdx.y * (kSpThreads / 32) + warp; j < NBb; j += gridDim.y * (kSpThreads / 32)) {
         float acc0 = 0.f, acc1 = 0.f;
-        sp_pair<T>(a_payload, b_col_idx, b_payload, b_row_ptr[j], b_row_ptr[j + 1], NBk, lane, [&](int k) { return s_pos[k]; }, acc0, acc1, status);
+        sp_pair<T>(a_payload, b_col_idx, b_payload, load_free(b_row_ptr + j), load_free(b_row_ptr + j + 1), NBk, lane, [&](int k) { return s_pos[k]; }, acc0, acc1, status);
         *(float2 *)(C + ((size_t)i * kSpEdge + r) * ldc + (size_t)j * kSpEdge + c) = make_float2(acc0, acc1);
     }
 }
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
             float acc0 = 0.f, acc1 = 0.f;
             const int first = p.a_row_ptr[i];
             const int16_t *row = s_pos + bi * pitch;
-            sp_pair<__nv_bfloat16>((const __nv_bfloat16 *)p.a_payload, p.b_col_idx, (const __nv_bfloat16 *)p.b_payload, p.b_row_ptr[jj], p.b_row_ptr[jj + 1],
+            sp_pair<__nv_bfloat16>(from_here((const __nv_bfloat16 *)p.a_payload), from_here(p.b_col_idx), from_here((const __nv_bfloat16 *)p.b_payload), p.b_row_ptr[jj], p.b_row_ptr[jj + 1],
                                    p.NBk, lane, [&](int k) { const int n = row[k]; return n < 0 ? -1 : first + n; }, acc0, acc1, p.status);
             *(float2 *)(p.C + ((size_t)i * kSpEdge + (lane >> 2)) * ldc + (size_t)jj * kSpEdge + (lane & 3) * 2) = make_float2(acc0, acc1);
         }
