@@ -57,6 +57,13 @@ def test_channel_counts(O1, O2):
     run_chain(1011, 2, 9, 11, 32, O1, O2, 3, 3, (1, 1), (1, 1), 1)
 
 
+@pytest.mark.parametrize("N,L,taps,O2", [(5, 40, 3, 336), (1, 40, 3, 1000), (1, 60, 3, 1024), (2, 44, 1, 520)])
+def test_rows_that_straddle_lines_and_few_tiles(N, L, taps, O2):
+    """216 channels in: the tiles of layer two stay with one CTA, are shared by two, by four, and (one tap) by as many as fit."""
+    run_chain(1015, N, L, L, 216, 88, O2, taps, taps, (1, 1), (taps // 2, taps // 2), 1, frac=0.7)
+    run_chain_q8(1016, N, L, L, 208, 64, O2 // 16 * 16, taps, taps, (1, 1), (taps // 2, taps // 2), 1, True)
+
+
 @pytest.mark.parametrize("H,K,stride,pad", [(1, 1, (1, 1), (0, 0)), (3, 3, (2, 2), (1, 1)), (1, 7, (1, 1), (0, 3)), (5, 5, (1, 1), (0, 0))])
 def test_first_layer_taps_strides_padding(H, K, stride, pad):
     run_chain(1021, 2, 17, 17, 48, 64, 128, H, K, stride, pad, 1)
