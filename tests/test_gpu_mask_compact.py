@@ -57,8 +57,8 @@ def test_gamma_ties_broken_by_index():
 
 
 def test_gamma_ties_in_a_layer_of_many_blocks():
-    """8192 blocks with few distinct int8 scores: the multi-CTA select must zero equal keys lowest index first,
-    across the slices of different CTAs."""
+    """8192 blocks with few distinct int8 scores: every CTA selects on all keys and counts the equal ones before its share of
+    Gamma; equal keys are zeroed lowest index first."""
     bo = bi = 8
     W = synth.uniform_int(131, (512, 1, 1, 1024), -3, 3).astype(np.int8)
     want_s = ref.scores(W, bo, bi)
@@ -105,6 +105,59 @@ def test_select_within_one_cta(rows, cols, scope):
             assert np.array_equal(g, ref.mask(want, n_zero, ref.SCOPE_ROW if scope == bsp.SCOPE_ROW else ref.SCOPE_LAYER)), (dtype, n_zero)
 
 
+@pytest.mark.parametrize("rows,cols", [
+    (17, 241),                           # 4097 blocks, the fewest that every CTA selects on for itself
+    (128, 128),                          # 16384, the most
+    (145, 113),                          # 16385, the fewest of the cooperative select
+    (129, 128),
+    (256, 256),
+])
+def test_ties_across_the_ctas_of_a_select(rows, cols):
+    """Layers whose threshold key is held by many blocks, in the shares of many CTAs: few distinct int8 scores, and one score for
+    all blocks; the number to zero falls inside a run of equal keys, at its ends and one beside them."""
+    NB = rows * cols
+    for W in (synth.uniform_int(151, (rows * 8, 1, 1, cols * 8), -1, 1).astype(np.int8), np.full((rows * 8, 1, 1, cols * 8), -2, dtype=np.int8)):
+        want = ref.scores(W, 8, 8)
+        keys, counts = np.unique(want, return_counts=True)
+        run = int(np.argmax(counts))
+        below = int(counts[:run].sum())
+        assert counts[run] > 100
+        for n_zero in sorted({below + 1, below + int(counts[run]) // 2, below + int(counts[run]) - 1, below + int(counts[run]), 1, NB // 3, NB - 1} - {0, NB}):
+            g, s, _, _ = gpu_mask(W, 8, 8, "i8", n_zero)
+            assert np.array_equal(s, want)
+            assert np.array_equal(g, ref.mask(want, n_zero)), n_zero
+
+
+@pytest.mark.parametrize("NBo,NBi", [(9, 512), (17, 496), (16, 513), (8, 600), (40, 1024), (1030, 4), (7, 1040)])
+def test_index_without_a_payload(NBo, NBi):
+    """row_ptr and col_idx of layers of more than 4096 blocks that keep the packed form only: rows of one and several passes of 512
+    entries, of a multiple of 16 and not, numbers of rows that are no multiple of eight, empty and full rows, Gamma at an odd
+    address, and a capacity that ends inside a row."""
+    W = make_case(153, NBo * 8, NBi * 8, 1, 1, "i8")
+    gamma = synth.random_gamma(154, NBo, NBi, NBo * NBi // 2)
+    gamma[NBo // 2], gamma[NBo - 1, :], gamma[0, NBi // 3:] = 0, 1, 0
+    Wd = to_dev(W, "i8")
+    for g in (gamma, np.zeros_like(gamma), np.ones_like(gamma)):
+        rp, ci, _ = ref.compact(W, g, 8, 8)
+        for capacity, offset in ((NBo * NBi, 0), (NBo * NBi, 1), (max(1, len(ci) - 3), 0)):
+            lay = bsp.SparseLayer(NBo * 8, NBi * 8, 1, 1, 8, 8, torch.int8, capacity_blocks=capacity, canonical=False)
+            big = torch.zeros(NBo * NBi + 16, dtype=torch.uint8, device="cuda")
+            lay.gamma = big[offset:offset + NBo * NBi]
+            col_idx = torch.full((NBo * NBi + 1,), -5, dtype=torch.int32, device="cuda")
+            lay.col_idx = col_idx
+            lay.row_ptr.fill_(-5)
+            lay.compact(Wd, torch.from_numpy(np.ascontiguousarray(g)).cuda())
+            if len(ci) > capacity:
+                with pytest.raises(bsp.BspError) as e:
+                    lay.check()
+                assert e.value.status == bsp.ERR_CAPACITY
+            else:
+                lay.check()
+            kept = min(len(ci), capacity)
+            assert np.array_equal(from_dev(lay.row_ptr), rp)
+            assert np.array_equal(from_dev(col_idx)[:kept], ci[:kept]) and bool((col_idx[kept:] == -5).all())
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32", "i8"])
 @pytest.mark.parametrize("bo,bi", SHAPES)
 def test_compact_bit_exact(dtype, bo, bi):
@@ -126,7 +179,7 @@ def test_compact_bit_exact(dtype, bo, bi):
 @pytest.mark.parametrize("dtype", ["bf16", "i8"])
 @pytest.mark.parametrize("bo,bi", SHAPES)
 def test_compact_more_blocks_than_the_single_launch_path_takes(dtype, bo, bi):
-    """8192 blocks: the count / scan / fill launches instead of the one-launch kernel of small layers."""
+    """8192 blocks: Gamma is counted through L2 instead of from shared memory."""
     O, I, H, K = 512, 1024, 1, 1
     W = make_case(123, O, I, H, K, dtype)
     NBo, NBi = O // bo, I // bi
