@@ -10,6 +10,8 @@
 // fused multiply-adds; bfloat16 blocks: one m16n8k16 tensor-core instruction per two common columns).  Work and
 // traffic follow the kept blocks only: nothing is read or multiplied where either mask has a zero.  bfloat16 operands whose
 // masks leave enough common columns take the dense form on tcgen05 below.
+#include <atomic>
+#include <mutex>
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -409,15 +411,18 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
     return plan;
 }
 
-// Per device, once: the kernels' shared-memory limit and the slots of spgemm_plan.
+// Per device, once: the kernels' shared-memory limit and the slots of spgemm_plan.  Calls come from any thread: who finds the
+// flag set finds the slots, too.
 bsp_status spgemm_tc_device(const int (**slots)[4])
 {
     static int known[kGtMaxDevices][4] = {};
-    static bool done[kGtMaxDevices] = {};
+    static std::atomic<bool> done[kGtMaxDevices] = {};
+    static std::mutex once;
     int dev = 0;
     BSP_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
-    if (!done[dev]) {
+    if (!done[dev].load(std::memory_order_acquire)) {
+        const std::lock_guard<std::mutex> lock(once);
         BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
         BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
         BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
@@ -432,7 +437,7 @@ bsp_status spgemm_tc_device(const int (**slots)[4])
             BSP_CUDA_OK(cudaOccupancyMaxActiveClusters(&n, spgemm_tc_kernel<64>, &cfg));
             known[dev][k] = n << k;
         }
-        done[dev] = true;
+        done[dev].store(true, std::memory_order_release);
     }
     *slots = &known[dev];
     return BSP_OK;

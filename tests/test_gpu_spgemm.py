@@ -1,5 +1,9 @@
 """GPU parity of the block-sparse x block-sparse product and of the relative column index against the oracle, through the
 C ABI: the product within the fp32-accumulation tolerance (bf16 or fp32 blocks), the index bit for bit."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -100,6 +104,41 @@ def test_spgemm_dropped_blocks_hide_non_finite_weights():
     A[3 * 8 + 2, 0, 0, 10 * 8 + 1] = 0.0
     want = ref.spgemm(8, ref.compact(A, ga, 8, 8), ref.compact(B, gb, 8, 8))
     assert rel_err(np.where(hit, 0.0, got), np.where(hit, 0.0, want)) <= 2e-5
+
+
+def test_spgemm_first_calls_from_several_threads():
+    """The first calls of a process, at once and each on a stream of its own: every thread finds the device's limits in place."""
+    code = """
+import threading, torch
+from paper_2407_09453_b200 import bsp
+def layer(O, seed):
+    torch.manual_seed(seed)
+    lay = bsp.SparseLayer(O, 512, 1, 1, 8, 8, torch.bfloat16)
+    W = torch.randn((O, 1, 1, 512), device="cuda").to(torch.bfloat16)
+    lay.mask(W, lay.NBo * lay.NBi // 4)
+    lay.compact(W)
+    lay.check()
+    return lay
+jobs = [(layer(256, k), layer(256, k + 100), torch.empty((256, 256), device="cuda"), torch.cuda.Stream(), bsp.new_workspace(256)) for k in range(8)]
+torch.cuda.synchronize()
+gate, errors = threading.Barrier(8), []
+def run(a, b, C, s, ws):
+    gate.wait()
+    try:
+        bsp.bsp_spgemm(a.wd, a.handle(), b.wd, b.handle(), C, ws, s)
+        bsp.bsp_check(ws, s)
+    except Exception as e:
+        errors.append(e)
+ts = [threading.Thread(target=run, args=j) for j in jobs]
+[t.start() for t in ts], [t.join() for t in ts]
+assert not errors, errors
+for a, b, C, s, ws in jobs:
+    D = torch.empty_like(C)
+    bsp.bsp_spgemm(a.wd, a.handle(), b.wd, b.handle(), D, ws)
+    bsp.bsp_check(ws)
+    assert torch.equal(C, D)
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=300, cwd=os.path.dirname(os.path.dirname(os.path.abspath(bsp.__file__))))
 
 
 def test_spgemm_argument_errors():
