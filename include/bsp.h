@@ -228,8 +228,10 @@ bsp_status bsp_conv2d_chain_q8(const bsp_wdesc *wd1, const bsp_bcsr *w1, const b
  *             col_idx and the canonical payload are read; `packed` is not).  C is dense float32 [wa->O][wb->O], 8-byte
  *             aligned (the two payloads 16-byte aligned), written in full (blocks without a common column are zero).  Products are accumulated in float32
  *             in ascending order of k (bfloat16 operands with enough common columns run as a dense product over masked
- *             blocks: sums of 16 products inside the tensor core, and of up to eight column ranges).  A column index outside
- *             the matrix is skipped and latches BSP_ERR_INDEX.
+ *             blocks: sums of 16 products inside the tensor core, and of up to eight column ranges).  Which form and how many
+ *             ranges is decided from the sizes, from `nnz` of both handles and from the GPU, so the last bits of C may differ
+ *             between handles of the same matrices that state another `nnz`, and between GPUs.  A column index outside the
+ *             matrix is skipped and latches BSP_ERR_INDEX.
  *             ws: any workspace of at least 256 bytes (status word only).
  * bsp_index_to_relative / bsp_index_from_relative: within each row of Gamma the first kept block keeps its column, every
  *             further one stores its distance (>= 1) to the previous kept block of the row; and back.  int32 in, int32

@@ -637,8 +637,8 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.small2 = (long long)wd1.O * 128 * 128 <= (1 << 29) ? 1 : 0;
     const int fixed = ct_groups(false) * 4 * kGtStagingBytes + (int)sizeof(CtTail<2>);
     // kHalo: where two boxes of activations, the weights of layer one and at least two chunks of layer two's fit, and the
-    // tiles with their border are not many more.  3x3 64->64 then 64->256 at 56x56, batch 64: 44.5 us loaded tap by tap,
-    // 33.8 like this.
+    // tiles with their border are not many more.  3x3 64->64 then 64->256 at 56x56, batch 64, in a short burst: 44.5 us loaded
+    // tap by tap, 33.8 like this (36 in a stream of calls).
     bool halo = false;
     int w2_slots = 0;
     if (HK > 1 && HK <= kCtTaps && p.cpt1 == 1 && p.sh == 1 && p.sw == 1 && p.db && Th.tiles > 0 && Th.tiles * 4 <= T.tiles * 5) {

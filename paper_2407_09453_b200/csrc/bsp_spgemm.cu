@@ -131,7 +131,8 @@ constexpr int kStARows = kGtBM / kSpEdge;         // block rows of A per tile
 // Groups of producer warps by tile width: a group's chain of wait, store, arrive and load is longer than the MMAs of
 // a chunk, so groups overlap theirs.  2048 x 2048 x 4096 at 50 %, us: one group 52 / 82 / 130 (256 / 128 / 64 columns), two
 // 50 / 72 / 113, four 105 with 64; 16-byte cp.async straight to shared memory instead of registers: 72 / 93 / 143.  (These with
-// a proxy fence in the producers.)  Pairs of CTAs that fill half of B each: 48.3, against 46.0 for 256 columns alone.
+// a proxy fence in the producers.)  Pairs of CTAs that fill half of B each: 48.3, against 46.0 for 256 columns alone.  (All in
+// short bursts with the same operands; a call in a stream with operands that change takes 51.)
 __host__ __device__ constexpr int st_groups(int BN) { return BN == 64 ? 4 : 2; }
 
 struct StParams {
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
             const bool wrap = slot + 1u == (uint32_t)S;
             const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
             // (the stage's stores come before this thread through its barrier, and before the MMAs by this one fence: a fence in
-            // every producer also waited for the loads it had in flight; 2048 x 2048 x 4096 at 50 % 48.9 -> 46.0 us)
+            // every producer also waited for the loads it had in flight; 2048 x 2048 x 4096 at 50 % 48.9 -> 46.0 us in a burst)
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             gt_issue_stage<BSP_BF16, false>(tmem, kGtDesc | (uint64_t)(a16 & 0x3FFFu), kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu),
@@ -373,7 +374,7 @@ int spgemm_tc_stages(int BN, int n_chunks)
 // microseconds, fitted on a B200.  Tensor-core form: a tile costs a start, a share per chunk for the table and the fill of
 // the operands (0.30 / 0.42 / 0.57 a chunk at 64 / 128 / 256 columns, bound by shared memory: stores of the fill, reads
 // of the MMAs), whatever the masks hold.  Sparse form: 28.7 per million pairs of blocks with a common column plus 3.6 per
-// million look-ups, or the chain of one warp where there are few rows.  Measured, sparse / tensor core: 2048 x 2048 x 4096
+// million look-ups, or the chain of one warp where there are few rows.  Measured in bursts, sparse / tensor core: 2048 x 2048 x 4096
 // at 50 % 304 / 46, at 75 % 90 / 43, 512 x 512 x 4096 at 50 % 27 / 14; with the fence in the
 // producers 25 / 44 at 90 %, and 11 / 14 for the smaller one at 75 %.
 // The densities come from the host counts; a wrong count costs time only.

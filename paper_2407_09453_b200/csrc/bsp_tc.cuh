@@ -390,7 +390,8 @@ GtTile gt_pick_tile(int N, int M, int Nw, int sh, int sw, int rows = kGtBM)
 
 // Position tile of a layer that takes several waves: parts of several images, so that the 128 rows of a tile are filled where no
 // box of one image fills them (56 x 56: 112 of 128 rows, but 8 x 8 positions of two images all of them; 7 x 7: 98, but a row
-// of 18 images 126): int8 3x3 256->256 at 56x56, batch 32, 48.9 -> 45.0 us, TF32 3x3 464->432 at 17x17, batch 52, 141 -> 101 us.
+// of 18 images 126): int8 3x3 256->256 at 56x56, batch 32, 48.9 -> 45.0 us in a short burst (52 to 53 in a stream of calls, under
+// the power cap), TF32 3x3 464->432 at 17x17, batch 52, 141 -> 101 us.
 // (The search takes 1 to 3 us of the host, hidden behind the waves of such a layer; a layer of one wave has no use for it.)  Looks at the distinct tile counts in x and y only, each with its smallest box.
 GtTile gt_pick_packed(GtTile best, int N, int M, int Nw, int sh, int sw)
 {
