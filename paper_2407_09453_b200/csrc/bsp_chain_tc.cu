@@ -64,8 +64,9 @@ template <int kGroups>
 struct CtTail {
     uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc1_full[2], acc1_empty[2], t_full[2], t_empty[2], acc2_full[2], acc2_empty[2];
     uint64_t w1_full[kCtTaps], w2_full[kCtW2Slots], w2_empty[kCtW2Slots];
+    uint64_t before_last;             // layer two of the last tile but one is done (used once)
     uint32_t tmem, fail;
-    uint32_t y_read[2];               // warps that have read accumulator two, counted over all tiles
+    uint32_t y_read[2];               // warps that have read accumulator two, counted over all tiles (kGroups > 2 kRpt)
     // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
     __align__(16) uint32_t bias[kGroups][128], half[kGroups][128];
     __align__(16) uint8_t shift[kGroups][128];
@@ -132,6 +133,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.acc2_full[b])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.acc2_empty[b])), "r"(4 * kRpt) : "memory");
         }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.before_last)), "r"(1) : "memory");
         if constexpr (kHalo) {
             for (int t = 0; t < p.n_ks1; ++t) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.w1_full[t])), "r"(1) : "memory");
             for (int t = 0; t < p.w2_slots; ++t) {
@@ -389,6 +391,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 if (p.db) { if (tile + t_step < t_count) layer_one(tile_i + 1u); }
                 else layer_one(tile_i);
                 if (ok) layer_two(tile_i);
+                if (ok && tile + t_step < t_count && tile + 2 * t_step >= t_count) gt_commit_elected<false>(sm32(&tail.before_last));
             }
             if (!ok && lane == 0) atomicExch((uint32_t *)&tail.fail, 1u);
         }
@@ -419,7 +422,12 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             // A barrier's parity tells a phase from the next one only, so a group may look at a phase when it knows that the one
             // before it has completed.  What tells it, for each barrier (all rest on the commits of the MMA warp completing in the
             // order of its loop):
-            //   acc2_full   the count of the reads of the buffer's previous use (below).
+            //   acc2_full   of tile s: the group had its last look no further back than T of tile s + 1, if T runs ahead, or
+            //               than the use of the other accumulator before the phase in question, and either comes after the
+            //               buffer's previous use.  In the last tile, which has no such T, before_last stands in for it.
+            //               With one round per tile of layer two and three groups this does not hold, and the reads of the
+            //               previous use are counted (below).  (Checked over all orders in which the barriers can complete, for
+            //               up to six tiles and five tiles of layer two, in every form.)
             //   acc1_full   of tile i: its previous phase is that of tile i - 2 (two accumulators) or i - 1 (one).  The group had a
             //               round in step i - 1 - ahead, as a step has at least as many rounds as there are groups (hence two
             //               groups for steps of two): T of tile i - 1, or Y of tile i - 1 - ahead, which came after it.
@@ -458,6 +466,8 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 const int idx = one ? step + p.ahead : step;     // which of the CTA's tiles
                 const uint32_t tile_i = (uint32_t)idx;
                 if (idx < 0 || idx >= n_local) {                 // (before the first Y, after the last T)
+                    if (s_fail) ok = false;
+                    if (idx >= n_local && n_local > 1 && ok && !gt_wait(sm32(&tail.before_last), 0u)) ok = false;
                     if (change) { gt_group_sync(1 + grp); place(next); gt_group_sync(1 + grp); }
                     rnd = next; step = next_step;
                     continue;
@@ -473,11 +483,11 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 if (one) {
                     if (ok && (!gt_wait(sm32(&tail.acc1_full[b1]), u1 & 1u) || !gt_wait(sm32(&tail.t_empty[bt]), (ut & 1u) ^ 1u))) ok = false;
                 } else {
-                    // First the previous use of the buffer is seen to have been read, by a count: layer two waits for that
-                    // anyway.  (The group's own last look does not tell: with one round per tile of layer two and three groups
-                    // it may be two phases back, and in the last tile, whose step has no T left, it is a whole step back.  The
-                    // parity of the other buffer's barrier would not do either, as that one may have moved on by two phases.)
-                    if (ok && !ct_wait_count(&tail.y_read[buf], use * (uint32_t)(4 * kRpt))) ok = false;
+                    // (With one round per tile of layer two, a group of three may come to this phase while the barrier is still
+                    // two before it, which the parity cannot tell from done.  So first the previous use of the buffer is seen
+                    // to have been read, by a count: layer two waits for that anyway.  The parity of the other buffer's barrier
+                    // would not do, as that one may have moved on by two phases already.)
+                    if (kGroups > 2 * kRpt && ok && !ct_wait_count(&tail.y_read[buf], use * (uint32_t)(4 * kRpt))) ok = false;
                     if (ok && !gt_wait(sm32(&tail.acc2_full[buf]), use & 1u)) ok = false;
                     if (kEy == 1) {
                         if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
@@ -493,7 +503,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                 auto hand_back = [&](uint64_t *bar) {
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
-                    if (!one && lane == 0) atomicAdd(&tail.y_read[buf], 1u);
+                    if (kGroups > 2 * kRpt && !one && lane == 0) atomicAdd(&tail.y_read[buf], 1u);
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm32(bar)) : "memory");
                 };
                 if (one) {
