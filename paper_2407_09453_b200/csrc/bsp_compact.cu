@@ -99,7 +99,7 @@ __device__ __forceinline__ int csr_fill_body(int l, int part, int parts, const T
     __syncthreads();
     for (int base = 0; base < NBi; base += kThreads) {
         const int i = base + threadIdx.x;
-        const int v = (i < NBi && g[i]) ? 1 : 0;
+        const int v = (i < NBi && load_free(g + i)) ? 1 : 0;
         int tot;
         const int before = block_exclusive_scan(v, warp_sums, tot);
         if (v) {
@@ -163,15 +163,15 @@ __device__ __forceinline__ int ones_share_global(const uint8_t *g, int n)
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int i = i0 + u * kThreads;
-                q[u] = i < n4 ? g4[i] : make_uint4(0u, 0u, 0u, 0u);
+                q[u] = i < n4 ? load_free(g4 + i) : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u)
                 c += __popc(__vsetne4(q[u].x, 0u)) + __popc(__vsetne4(q[u].y, 0u)) + __popc(__vsetne4(q[u].z, 0u)) + __popc(__vsetne4(q[u].w, 0u));
         }
-        for (int i = (n4 << 4) + threadIdx.x; i < n; i += kThreads) c += g[i] ? 1 : 0;
+        for (int i = (n4 << 4) + threadIdx.x; i < n; i += kThreads) c += load_free(g + i) ? 1 : 0;
     } else {
-        for (int i = threadIdx.x; i < n; i += kThreads) c += g[i] ? 1 : 0;
+        for (int i = threadIdx.x; i < n; i += kThreads) c += load_free(g + i) ? 1 : 0;
     }
     return c;
 }
@@ -200,13 +200,13 @@ __device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *W, c
         const uint8_t *g = gamma + (size_t)l * NBi + ((c * cpc) >> lg(bi));
         uint32_t keep[4];
         if (bi >= cpc) {
-            keep[0] = keep[1] = keep[2] = keep[3] = g[0] ? 0xFFFFFFFFu : 0u;
+            keep[0] = keep[1] = keep[2] = keep[3] = load_free(g) ? 0xFFFFFFFFu : 0u;
         } else if (cpc / bi == 2) {
-            keep[0] = keep[1] = g[0] ? 0xFFFFFFFFu : 0u;
-            keep[2] = keep[3] = g[1] ? 0xFFFFFFFFu : 0u;
+            keep[0] = keep[1] = load_free(g) ? 0xFFFFFFFFu : 0u;
+            keep[2] = keep[3] = load_free(g + 1) ? 0xFFFFFFFFu : 0u;
         } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) keep[q] = g[q] ? 0xFFFFFFFFu : 0u;
+            for (int q = 0; q < 4; ++q) keep[q] = load_free(g + q) ? 0xFFFFFFFFu : 0u;
         }
         const bool any = (keep[0] | keep[1] | keep[2] | keep[3]) != 0u;
         const size_t pitch = (size_t)cpr * 16, at = ((size_t)l * rows + r0) * pitch + (size_t)c * 16;
@@ -216,10 +216,10 @@ __device__ __forceinline__ void dense_body(int idx, int n_ctas, const void *W, c
         for (int u = 0; u < kDenseRows; ++u) {
             v[u] = make_uint4(0u, 0u, 0u, 0u);
             if (u < n && any) {
-                if (aligned) v[u] = *(const uint4 *)(src + u * pitch);
+                if (aligned) v[u] = load_free((const uint4 *)(src + u * pitch));
                 else {                                // W only 4-byte aligned: word by word
                     const uint32_t *s4 = (const uint32_t *)(src + u * pitch);
-                    v[u] = make_uint4(*s4, s4[1], s4[2], s4[3]);
+                    v[u] = make_uint4(load_free(s4), load_free(s4 + 1), load_free(s4 + 2), load_free(s4 + 3));
                 }
             }
         }
@@ -245,7 +245,7 @@ __device__ __forceinline__ void index_rows(int cta, const uint8_t *gamma, int NB
         unsigned m = 0u;
         if (wide) {
             if (i < NBi) {
-                const uint4 w = *(const uint4 *)(g + i);
+                const uint4 w = load_free((const uint4 *)(g + i));
                 const uint32_t x[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -254,7 +254,7 @@ __device__ __forceinline__ void index_rows(int cta, const uint8_t *gamma, int NB
                 }
             }
         } else {
-            for (int q = 0; q < 16 && i + q < NBi; ++q) m |= g[i + q] ? 1u << q : 0u;
+            for (int q = 0; q < 16 && i + q < NBi; ++q) m |= load_free(g + i + q) ? 1u << q : 0u;
         }
         return m;
     };
@@ -316,11 +316,14 @@ struct CompactArgs {
 constexpr int kSmallBlocks = 4096;
 
 template <typename T, bool kBig>
-__global__ void __launch_bounds__(kThreads, 5) compact_kernel(const CompactArgs a)
+__global__ void __launch_bounds__(kThreads, 5) compact_kernel(const CompactArgs args)
 {
     __shared__ __align__(16) uint8_t s_gamma[kBig ? 16 : kSmallBlocks];
     __shared__ int s_sum[kThreads / 32];
     wait_for_previous();
+    CompactArgs a = args;
+    a.W = from_here((const uint8_t *)args.W);
+    a.gamma = from_here(args.gamma);
     const int n_fill = a.n_fill;
     if ((int)blockIdx.x >= n_fill) {
         if ((int)blockIdx.x == n_fill && threadIdx.x == 0 && a.hdr != nullptr) *a.hdr = a.hdr_init;
@@ -341,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 5) compact_kernel(const CompactArgs 
         const int NB = a.NBo * a.NBi;
         const bool word_ok = (((uintptr_t)a.gamma) & 3u) == 0;
         for (int i = threadIdx.x * 4; i < NB; i += kThreads * 4) {
-            if (i + 4 <= NB && word_ok) *(uint32_t *)(s_gamma + i) = *(const uint32_t *)(a.gamma + i);
+            if (i + 4 <= NB && word_ok) *(uint32_t *)(s_gamma + i) = load_free((const uint32_t *)(a.gamma + i));
             else for (int q = i; q < min(NB, i + 4); ++q) s_gamma[q] = a.gamma[q];
         }
         __syncthreads();

@@ -103,10 +103,18 @@ __device__ __forceinline__ const T *from_here(const T *p)
 }
 __device__ __forceinline__ uint32_t load_free(const uint32_t *p) { uint32_t v; asm("ld.global.b32 %0, [%1];\n" : "=r"(v) : "l"(p)); return v; }
 __device__ __forceinline__ int32_t load_free(const int32_t *p) { return (int32_t)load_free((const uint32_t *)p); }
+__device__ __forceinline__ uint32_t load_free(const uint8_t *p) { uint32_t v; asm("ld.global.u8 %0, [%1];\n" : "=r"(v) : "l"(p)); return v; }
+__device__ __forceinline__ uint4 load_free(const uint4 *p)
+{
+    uint4 v;
+    asm("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+template <int kBytes = 0>                                 // (kBytes past p: part of the instruction)
 __device__ __forceinline__ float4 load_free(const float4 *p)
 {
     float4 v;
-    asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4 + %5];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "n"(kBytes));
     return v;
 }
 

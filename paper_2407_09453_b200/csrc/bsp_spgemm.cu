@@ -20,10 +20,11 @@ namespace {
 constexpr int kSpThreads = 256;
 constexpr int kSpEdge = 8;
 
-// One row of an 8 x 8 block (8 consecutive values) as floats: two 16-byte loads for fp32, one for bf16.
+// Row kRow (from p on) of an 8 x 8 fp32 block.
+template <int kRow>
 __device__ __forceinline__ void sp_row(const float *p, float (&v)[8])
 {
-    const float4 a = load_free((const float4 *)p), b = load_free((const float4 *)p + 1);
+    const float4 a = load_free<kRow * 32>((const float4 *)p), b = load_free<kRow * 32 + 16>((const float4 *)p);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 // The 8 x 8 block of C of one row of A and one row of B: acc0, acc1 are this lane's entries (r, 2c), (r, 2c + 1) with
@@ -71,7 +72,7 @@ __device__ __forceinline__ void sp_pair(const T *a_payload, const int32_t *b_col
             const T *Ab = a_payload + ((size_t)na * kSpEdge + r) * kSpEdge;
             const T *Bb = b_payload + ((size_t)(base + src) * kSpEdge + c) * kSpEdge;
             float av[8], b0[8], b1[8];
-            sp_row(Ab, av); sp_row(Bb, b0); sp_row(Bb + kSpEdge, b1);
+            sp_row<0>(Ab, av); sp_row<0>(Bb, b0); sp_row<1>(Bb, b1);
 #pragma unroll
             for (int t = 0; t < kSpEdge; ++t) {
                 acc0 = fmaf(av[t], b0[t], acc0);
@@ -95,12 +96,12 @@ spgemm_kernel(const int32_t *a_row_ptr, const int32_t *a_col_idx, const T *a_pay
     // next one let in at once, 12.2 without programmatic launches; 232 x 2264 x 632 fp32 at 25 % 62.0, 78.1 let in at the end of
     // each CTA, 64.3.)
     wait_for_previous<false>();
-    a_payload = from_here(a_payload); b_payload = from_here(b_payload);
-    b_col_idx = from_here(b_col_idx); b_row_ptr = from_here(b_row_ptr);
+    a_payload = from_here(a_payload); a_col_idx = from_here(a_col_idx); a_row_ptr = from_here(a_row_ptr);
+    b_payload = from_here(b_payload); b_col_idx = from_here(b_col_idx); b_row_ptr = from_here(b_row_ptr);
     __syncthreads();
-    const int a_end = a_row_ptr[i + 1];
-    for (int n = a_row_ptr[i] + threadIdx.x; n < a_end; n += kSpThreads) {
-        const int k = a_col_idx[n];
+    const int a_end = load_free(a_row_ptr + i + 1);
+    for (int n = load_free(a_row_ptr + i) + threadIdx.x; n < a_end; n += kSpThreads) {
+        const int k = load_free(a_col_idx + n);
         if (k >= 0 && k < NBk) s_pos[k] = n;
         else atomicMax(status, (int)BSP_ERR_INDEX);          // a column outside the matrix: skipped
     }
