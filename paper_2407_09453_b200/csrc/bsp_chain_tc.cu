@@ -626,17 +626,21 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     // layer two's channels.  (Two 128-channel tiles of Y take about 1.2 us one after the other: 7x1 128->64->928 at 11x11 13.0 -> 6.6 us,
     // 3x3 64->80->768 at 22x22 12.3 -> 7.4, 1x1 96->128->592 at 34x34, batch 8, 14.9 -> 11.6.)
     const long long most = Th.tiles > T.tiles ? Th.tiles : T.tiles;
-    // As many as fit, but where layer one's rows straddle the 128-byte lines of L2 (more than one chunk of channels, not whole
-    // lines).  Such a row costs two lines, 3 cycles of a CTA, and all of layer one 1.4 times as much on more than half of the SMs,
-    // whatever their number: those layers take the CTAs with the lowest estimate, a tile of Y being 1.2 us.  3x3 216->88, 1x1
-    // 88->336 at 40x40, batch 5, 20.8 us a call on 63 CTAs and 25.0 on 126; 8 bits 3x3 208->64, 1x1 64->336 14.8 and 20.1.
+    // As many as fit, but where layer one's rows are not whole 32-byte sectors of L2.  Such rows cost twice the time of a CTA, and
+    // 1.4 times that on more than half of the SMs, whatever their number: those layers take the CTAs with the lowest estimate, a
+    // tile of Y being 1.2 us (4-byte output 1.8).  3x3 216->88, 1x1 88->336 at 40x40, batch 5, 20.8 us a call on 63 CTAs and 25.0 on
+    // 126; 8 bits 3x3 208->64, 1x1 64->336 14.8 and 20.1.  (Over 1056 pairs with such rows 6 % faster than as many as fit; over
+    // 2376 with rows of whole sectors half of the SMs were 7 % slower.)
+    const bool stays = HK > 1 && HK <= kCtTaps && p.cpt1 == 1 && p.sh == 1 && p.sw == 1 && p.O1p <= 128 && Th.tiles > 0 && Th.tiles * 4 <= T.tiles * 5;
     if (most * 2 <= n_sm[dev] && p.n_t2 > 1) {
-        const double rows = row1 > 128 && row1 % 128 != 0 ? 2.0 * p.n_ks1 * (kGtBM + p.O1p) : 0.0;
+        const int planes = row1 <= 32 || row1 > 64 ? 1 : 2;
+        const double rows = row1 % 32 == 0 ? 0.0 : stays ? HK * planes * p.O1p : p.n_ks1 * (kGtBM + p.O1p);
+        const long long tiles = stays ? Th.tiles : T.tiles;
         const int n_all = p.n_t2;
         double best = -1.0;
         for (int parts = 1; parts <= n_sm[dev] / most && parts <= n_all; ++parts) {
             const int n = (n_all + parts - 1) / parts, used = (wd2.O + kCtBN2 * n - 1) / (kCtBN2 * n);
-            const double t = rows * 1.5 / 1900.0 * (used * T.tiles * 2 <= n_sm[dev] ? 1.0 : 1.4) + 1.2 * n;
+            const double t = rows * 3.0 / 1900.0 * (used * tiles * 2 <= n_sm[dev] ? 1.0 : 1.4) + (ey == 4 ? 1.8 : 1.2) * n;
             if (best < 0 || t < best) { best = t; p.n_t2 = n; p.parts = used; }
         }
     }
@@ -651,7 +655,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     // tap by tap, 33.8 like this (36 in a stream of calls).
     bool halo = false;
     int w2_slots = 0;
-    if (HK > 1 && HK <= kCtTaps && p.cpt1 == 1 && p.sh == 1 && p.sw == 1 && p.db && Th.tiles > 0 && Th.tiles * 4 <= T.tiles * 5) {
+    if (stays) {
         const int kb = row1 <= 32 ? 32 : (row1 <= 64 ? 64 : 128), planes = kb == 128 ? 1 : kb / 32;
         const int plane = (Th.Nt * (Th.Ht + wd1.H - 1) * (Th.Wt + wd1.K - 1) * (kb / planes) + 1023) / 1024 * 1024;
         p.staging_bytes = (uint32_t)(Th.Wt * Th.Ht * Th.Nt * 128 + 1023) / 1024 * 1024;

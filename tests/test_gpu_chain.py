@@ -58,7 +58,7 @@ def test_channel_counts(O1, O2):
 
 
 @pytest.mark.parametrize("N,L,taps,O2", [(5, 40, 3, 336), (1, 40, 3, 1000), (1, 60, 3, 1024), (2, 44, 1, 520)])
-def test_rows_that_straddle_lines_and_few_tiles(N, L, taps, O2):
+def test_rows_of_parts_of_sectors_and_few_tiles(N, L, taps, O2):
     """216 channels in: the tiles of layer two stay with one CTA, are shared by two, by four, and (one tap) by as many as fit."""
     run_chain(1015, N, L, L, 216, 88, O2, taps, taps, (1, 1), (taps // 2, taps // 2), 1, frac=0.7)
     run_chain_q8(1016, N, L, L, 208, 64, O2 // 16 * 16, taps, taps, (1, 1), (taps // 2, taps // 2), 1, True)
