@@ -417,19 +417,55 @@ __device__ __forceinline__ void select_digit(const unsigned *hist, unsigned *war
     __syncthreads();
 }
 
+// The same for 256 bins, by the first warp: each lane sums eight, a scan over the warp finds the lane that holds the digit.
+__device__ __forceinline__ void select_digit_256(const unsigned *hist, unsigned long long prefix, long long *s_k, unsigned long long *s_prefix,
+                                                 unsigned *s_left, int width)
+{
+    const int tid = threadIdx.x;
+    if (tid < 32) {
+        const long long need = *s_k;
+        unsigned mine = 0u;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) mine += hist[tid * 8 + q];
+        unsigned inc = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned n = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (tid >= d) inc += n;
+        }
+        long long cum = (long long)inc - mine;
+        __syncwarp();
+        if (cum < need && need <= cum + mine) {            // (need <= the sum of all bins: one lane)
+            int q = tid * 8;
+            for (; q < tid * 8 + 7; ++q) {
+                if (cum + hist[q] >= need) break;
+                cum += hist[q];
+            }
+            *s_k = need - cum;
+            *s_prefix = (prefix << width) | (unsigned long long)q;
+            *s_left = hist[q];
+        }
+    }
+    __syncthreads();
+}
+
 // The radix select of select_kernel for one large segment (the whole layer), spread over a cooperative grid:
 // CTA c owns a contiguous slice of the keys.  Each pass adds the CTAs' digit histograms into
-// ghist[pass][kCoopBins] (zeroed by the host before the launch), the CTAs meet at the grid barrier, and every CTA
+// ghist[pass][bins] (zeroed by the host before the launch), the CTAs meet at the grid barrier, and every CTA
 // derives the digit for itself.  Keys equal to the threshold T are zeroed lowest index first: the CTAs publish
 // how many such keys their slices hold (geq[c]), meet again, and each counts those in the slices before its own.
 constexpr int kCoopThreads = 512;
-constexpr int kCoopWidth = 10, kCoopBins = 1 << kCoopWidth;      // digit of a grid-wide pass
-static_assert(7 * kCoopBins == kSelectHist, "a histogram for each digit of a 64-bit key");
+// Ten bits a digit save passes where there are many keys, or few of few values; else the 1024 bins cost more than they save.
+// Gamma with eight and with ten bits, us: fp32 1536 x 1536 (36864 blocks) 20.9 and 24.6 to 28.4, bfloat16 2896 x 2096 (94844) 22.6
+// and 26 to 29, int8 the same 24.7 and 26.3; int8 1200 x 1024 (19200) 26.6 and 19.9; 4096 x 2048 (131072) bfloat16 23.8 and 23.5, int8
+// 27.6 and 25.9; 4096 x 4096 33.8 and 31.9; int8 8192 x 8192 61.5 and 51.8.
+inline bool coop_wide(long long keys, bool int8) { return keys > 131072 || (int8 && (keys == 131072 || keys <= 24576)); }
+static_assert(8 * 256 <= kSelectHist && 7 * 1024 <= kSelectHist, "a histogram for each digit of a 64-bit key");
 constexpr int kLocalMax = 8192;          // candidates that the CTAs finish on their own, in (dynamic) shared memory
 
 // The select starts at the highest bit in which any two keys differ (the score kernel leaves the OR of all keys in
 // gcount[2..3] and the OR of their complements in gcount[4..5]: the bits above it are the same in every key, e.g. the
-// sign and most of the exponent of float scores, or the leading zero bytes of integer ones) and takes digits of ten
+// sign and most of the exponent of float scores, or the leading zero bytes of integer ones) and takes digits of kWidth
 // bits downwards.  Passes run grid-wide (global histograms, a grid barrier
 // each) only while more than kLocalMax keys still match the prefix; then the CTAs append their matching keys to one
 // list (`cand`, counted in gcount[0], zeroed by the host with the histograms), meet
@@ -437,11 +473,17 @@ constexpr int kLocalMax = 8192;          // candidates that the CTAs finish on t
 constexpr int kSliceMax = 4096;          // keys of a CTA's slice that are kept in shared memory for all phases
 constexpr size_t kCoopSmem = (size_t)(kLocalMax + kSliceMax) * sizeof(unsigned long long);
 
+template <int kWidth>
 __global__ void __launch_bounds__(kCoopThreads)
 select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long long n_zero, uint8_t *__restrict__ gamma,
                    unsigned *ghist, unsigned *gcount, unsigned long long *cand, unsigned *geq, unsigned *sync, int *status)
 {
-    __shared__ unsigned hist[kCoopBins], warp_sums[kCoopThreads / 32];
+    constexpr int kBins = 1 << kWidth;
+    __shared__ unsigned hist[kBins], warp_sums[kCoopThreads / 32];
+    auto digit = [&](unsigned long long prefix, long long *k, unsigned long long *pre, unsigned *left, int width) {
+        if constexpr (kBins == 256) select_digit_256(hist, prefix, k, pre, left, width);
+        else select_digit<kCoopThreads, kBins>(hist, warp_sums, prefix, k, pre, left, width);
+    };
     extern __shared__ unsigned long long s_dyn[];
     unsigned long long *s_cand = s_dyn;                  // [kLocalMax]
     unsigned long long *s_keys = s_dyn + kLocalMax;      // [kSliceMax]
@@ -469,23 +511,23 @@ select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long
     if (tid == 0) { s_prefix = top >= 63 ? 0ull : (k0 >> (top + 1)); s_k = n_zero; s_left = n > 0xFFFFFFFFll ? 0xFFFFFFFFu : (unsigned)n; }
     int pi = 0;
     while (top >= 0) {
-        for (int q = tid; q < kCoopBins; q += kCoopThreads) hist[q] = 0u;
+        for (int q = tid; q < kBins; q += kCoopThreads) hist[q] = 0u;
         __syncthreads();
         if (s_left <= (unsigned)kLocalMax) break;          // few enough candidates: the rest is local
         const unsigned long long prefix = s_prefix;
-        const int width = min(kCoopWidth, top + 1), shift = top + 1 - width;
+        const int width = min(kWidth, top + 1), shift = top + 1 - width;
         const unsigned dmask = (1u << width) - 1u;
         for (int i = tid; i < len; i += kCoopThreads) {
             const unsigned long long v = ks[i];
             if (top >= 63 || ((v >> (top + 1)) == prefix)) atomicAdd(&hist[(unsigned)(v >> shift) & dmask], 1u);
         }
         __syncthreads();
-        for (int q = tid; q < kCoopBins; q += kCoopThreads)
-            if (hist[q]) atomicAdd(&ghist[pi * kCoopBins + q], hist[q]);
+        for (int q = tid; q < kBins; q += kCoopThreads)
+            if (hist[q]) atomicAdd(&ghist[pi * kBins + q], hist[q]);
         if (!grid_barrier(sync)) { if (tid == 0) atomicMax(status, (int)BSP_ERR_TIMEOUT); return; }
-        for (int q = tid; q < kCoopBins; q += kCoopThreads) hist[q] = __ldcg(&ghist[pi * kCoopBins + q]);
+        for (int q = tid; q < kBins; q += kCoopThreads) hist[q] = __ldcg(&ghist[pi * kBins + q]);
         __syncthreads();
-        select_digit<kCoopThreads, kCoopBins>(hist, warp_sums, prefix, &s_k, &s_prefix, &s_left, width);
+        digit(prefix, &s_k, &s_prefix, &s_left, width);
         top -= width;
         ++pi;
     }
@@ -509,10 +551,10 @@ select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long
         __syncthreads();
         constexpr int kMine = kLocalMax / kCoopThreads;    // candidates per thread
         while (top >= 0 && cnt > (unsigned)kCoopThreads) {
-            for (int q = tid; q < kCoopBins; q += kCoopThreads) hist[q] = 0u;
+            for (int q = tid; q < kBins; q += kCoopThreads) hist[q] = 0u;
             if (tid == 0) s_n = 0u;
             __syncthreads();
-            const int width = min(kCoopWidth, top + 1), shift = top + 1 - width;
+            const int width = min(kWidth, top + 1), shift = top + 1 - width;
             const unsigned dmask = (1u << width) - 1u;
             // every candidate matches the prefix so far (the list is thinned after each digit)
             unsigned long long mine[kMine];
@@ -523,7 +565,7 @@ select_coop_kernel(const unsigned long long *__restrict__ key, long long n, long
                 if (i < cnt) atomicAdd(&hist[(unsigned)(mine[u] >> shift) & dmask], 1u);
             }
             __syncthreads();
-            select_digit<kCoopThreads, kCoopBins>(hist, warp_sums, s_prefix, &s_k, &s_prefix, &s_left, width);
+            digit(s_prefix, &s_k, &s_prefix, &s_left, width);
             top -= width;
             // keep the candidates of the chosen digit (all were read into registers above)
             const unsigned long long pre = s_prefix;
@@ -991,7 +1033,8 @@ bsp_status launch_mask(const bsp_wdesc &wd, const void *W, bsp_norm norm, bsp_sc
         BSP_CUDA_OK(cudaGetDevice(&dev));
         if (dev < 0 || dev >= 64) return BSP_ERR_CUDA;
         if (sm_count[dev] == 0) {
-            BSP_CUDA_OK(cudaFuncSetAttribute(select_coop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoopSmem));
+            BSP_CUDA_OK(cudaFuncSetAttribute(select_coop_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoopSmem));
+            BSP_CUDA_OK(cudaFuncSetAttribute(select_coop_kernel<10>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoopSmem));
             BSP_CUDA_OK(cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev));
         }
         long long grid = (seg + 2 * kCoopThreads - 1) / (2 * kCoopThreads);
@@ -1004,7 +1047,7 @@ bsp_status launch_mask(const bsp_wdesc &wd, const void *W, bsp_norm norm, bsp_sc
         unsigned *sync = (unsigned *)ws + kWsSyncWord;
         int *status = (int *)ws;
         void *args[] = {&keys, &n, &nz, &gamma, &ghist, &gcount, &cand, &geq, &sync, &status};
-        const cudaError_t e = cudaLaunchCooperativeKernel((const void *)select_coop_kernel, dim3((unsigned)grid), dim3(kCoopThreads), args, kCoopSmem, st);
+        const cudaError_t e = cudaLaunchCooperativeKernel(coop_wide(seg, wd.wtype == BSP_I8) ? (const void *)select_coop_kernel<10> : (const void *)select_coop_kernel<8>, dim3((unsigned)grid), dim3(kCoopThreads), args, kCoopSmem, st);
         if (e == cudaErrorCooperativeLaunchTooLarge) {
             (void)cudaGetLastError();
             select_kernel<<<nseg, kSelectThreads, 0, st>>>((const unsigned long long *)scores, seg, n_zero, gamma);

@@ -110,7 +110,9 @@ def test_select_within_one_cta(rows, cols, scope):
     (128, 128),                          # 16384, the most
     (145, 113),                          # 16385, the fewest of the cooperative select
     (129, 128),
+    (157, 157),                          # 24649, the first of int8 with digits of eight bits
     (256, 256),
+    (256, 512),                          # 131072, where digits of ten bits begin
 ])
 def test_ties_across_the_ctas_of_a_select(rows, cols):
     """Layers whose threshold key is held by many blocks, in the shares of many CTAs: few distinct int8 scores, and one score for
