@@ -416,6 +416,8 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             uint32_t *bias = tail.bias[grp], *half = tail.half[grp];
             uint8_t *shift = tail.shift[grp];
             const int ct = ((warp - 2) & 3) * 32 + lane;
+            const uint32_t *bias1 = from_here((const uint32_t *)p.bias1), *bias2 = from_here((const uint32_t *)p.bias2);
+            const int32_t *shift1 = from_here(p.shift1), *shift2 = from_here(p.shift2);
             uint32_t next_bias = 0u, next_shift = 1u;
             bool small = false;
             const int n_rounds = p.n_c2 + p.n_t2 * kRpt;
@@ -437,11 +439,11 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             auto fetch = [&](int rnd) {
                 const bool one = rnd < p.n_c2;
                 const int ch = (one ? rnd * p.tcc : o2 + (rnd - p.n_c2) * cpr) + ct, O = one ? p.O1 : p.O2;
-                const uint32_t *b = (const uint32_t *)(one ? p.bias1 : p.bias2);
-                const int32_t *s = one ? p.shift1 : p.shift2;
+                const uint32_t *b = one ? bias1 : bias2;
+                const int32_t *s = one ? shift1 : shift2;
                 const bool in = ct < (one ? p.tcc : cpr) && ch < O;
-                next_bias = in && b != nullptr ? b[ch] : 0u;
-                if constexpr (kI8) next_shift = in && s != nullptr ? (uint32_t)s[ch] & 31u : 1u;
+                next_bias = in && b != nullptr ? load_free(b + ch) : 0u;
+                if constexpr (kI8) next_shift = in && s != nullptr ? (uint32_t)load_free(s + ch) & 31u : 1u;
             };
             bool mine_small = false, fresh = true;
             auto place = [&](int rnd) {                          // (between two barriers of the group)

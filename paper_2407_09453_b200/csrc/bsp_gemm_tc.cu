@@ -82,12 +82,6 @@ __device__ __forceinline__ void gt_tile_origin(const GtParams &p, int mt, int &n
     x0 = tx * p.Wt; y0 = ty * p.Ht; n0 = ni * p.Nt;
 }
 
-// Bias of output channel ch as raw bits (float32 or int32), zero without a bias or past the last channel.
-__device__ __forceinline__ uint32_t gt_bias(const GtParams &p, int ch)
-{
-    return (p.bias != nullptr && ch < p.O) ? ((const uint32_t *)p.bias)[ch] : 0u;
-}
-
 // kWT: operand type; kEy: bytes of an output element (4: float32 or int32, 2: bfloat16, 1: int8); kMode: how operands are staged.
 // kTaps loads an activation box and a weight tile per K-stage.  kPairs is the same on pairs of CTAs.  kHalo is for stride-1
 // layers with taps whose input channels fit one stage and whose weights fit shared memory: the weights of the CTA's channel
@@ -385,13 +379,15 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             uint32_t *bias = tail.bias[grp], *half = tail.half[grp];
             uint8_t *shift = tail.shift[grp];
             const int ct = ((warp - 2) & 3) * 32 + lane;
+            const uint32_t *bias_of = from_here((const uint32_t *)p.bias);       // raw bits: float32 or int32
+            const int32_t *shift_of = from_here(p.shift);
             uint32_t next_bias = 0u, next_shift = 1u;
             int have = -1;                                       // first channel of the round whose constants are in shared memory
             bool small = false, mine_small = false, fresh = false;
             auto fetch = [&](int ch0) {
                 if (ct >= cpr) return;
-                next_bias = gt_bias(p, ch0 + ct);
-                if constexpr (kEy == 1) next_shift = ch0 + ct < p.O ? (uint32_t)p.shift[ch0 + ct] & 31u : 1u;
+                next_bias = bias_of != nullptr && ch0 + ct < p.O ? load_free(bias_of + ch0 + ct) : 0u;
+                if constexpr (kEy == 1) next_shift = ch0 + ct < p.O ? (uint32_t)load_free(shift_of + ch0 + ct) & 31u : 1u;
             };
             auto place = [&](int ch0) {                          // (between two barriers of the group)
                 have = ch0;
