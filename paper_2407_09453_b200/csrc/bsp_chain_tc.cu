@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     wait_for_previous<false>();
+    if (warp == 0) let_next_start();                  // (behind its allocation)
     if (tid == 0) {
         const bool ok = ct_header_ok(p.packed1, p.wtype, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1) && ct_header_ok(p.packed2, p.wtype, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
         const bool placed = (base & 1023u) == 0u;
@@ -161,7 +162,6 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    let_next_start();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tail.tmem, 0);
     const bool run = __shfl_sync(0xFFFFFFFFu, s_fail, 0) == 0u;

@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
         }
     }
     wait_for_previous<false>();
+    if (warp == 0) let_next_start();                  // (behind its allocation)
     if (tid == 0) {
         // the packed buffer must be the one bsp_compact filled for this descriptor, with the masked dense form in it
         const PackedHeader *h = (const PackedHeader *)p.packed;
@@ -167,7 +168,6 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     gt_sync_all<kPair>();                   // (a pair: both CTAs' barriers are initialised before either signals the other)
-    let_next_start();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tail.tmem, 0);
     const bool run = __shfl_sync(0xFFFFFFFFu, s_fail, 0) == 0u;

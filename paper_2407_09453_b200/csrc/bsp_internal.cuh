@@ -79,9 +79,10 @@ inline int gemm_tile_n(int O)
 // one after another without this, the kernels of a stream started in steps of about 2 us.)
 // What an earlier kernel may have written is read by plain loads or __ldcg, through pointers without __restrict__: __ldg and
 // const __restrict__ promise data that nobody writes while the kernel runs, and it runs before wait_for_previous() returns.
-// A kernel that owns tensor memory lets its successor start behind the CTA barrier that follows its allocation.  The first
-// thread of a CTA to signal speaks for the whole CTA: while another of its warps still waits for columns, a CTA of the
-// successor on the same SM could take them and hold them until this kernel ends, and neither would move.
+// In a kernel that owns tensor memory the warp that allocates it signals, behind the allocation, and no other: the first thread
+// of a CTA to signal speaks for the whole CTA, and while the allocating warp still waits for columns, a CTA of the successor on
+// the same SM could take them and hold them until this kernel ends, and neither would move.  (Behind the CTA barrier instead
+// the signal came 0.1 us later, and with it the next kernel.)
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 // kLetNext = false: the next kernel starts when this one has ended (still without the gap between launches), or calls
 // let_next_start() later.

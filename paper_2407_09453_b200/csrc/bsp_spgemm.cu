@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     wait_for_previous<false>();
+    if (warp == kStProducers) let_next_start();        // (behind its allocation)
     // a block row's first and last stored block (rows past the last one are empty)
     auto row_of = [&](int b, int &lo, int &hi) {
         const bool is_a = b < kStARows;
@@ -191,7 +192,6 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
     };
     for (int k = tid; k < kRows * pitch / 8; k += kStThreads) ((uint4 *)s_pos)[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
     __syncthreads();
-    let_next_start();
     for (int b = warp; b < kRows; b += kStProducers + 1) {
         int lo, hi;
         row_of(b, lo, hi);
