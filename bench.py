@@ -371,12 +371,11 @@ def pass_layers(gpu, bsp, torch, layers, dtype, sparsities, pk, ydt, with_setup,
     return out
 
 
-def pass_spgemm(gpu, bsp, torch, reps=5):
+def pass_spgemm(gpu, bsp, torch, pk, reps=5):
     """Block-sparse x block-sparse product C = (Gamma . A)(Omega . B)^t, 2048 x 4096 times (2048 x 4096)^t, bf16 8x8 blocks,
-    magnitude masks at 50 % and 75 %: useful FLOPs are those of the block pairs that both masks keep.  The kernel runs on
-    the general-purpose pipes (index look-ups, ballots; the 8 x 8 x 8 products of bf16 blocks go two at a time through one
-    m16n8k16 tensor-core instruction of the warp), so its yardstick is the fp32 FMA rate: 148 SMs x 128 lanes x 2 x 1.965 GHz."""
-    peak = 148 * 128 * 2 * 1.965e9 / 1e12
+    magnitude masks at 50 % and 75 %: useful FLOPs are those of the block pairs that both masks keep.  At these densities the
+    product runs as dense tiles on the tensor cores, so its yardstick is their bf16 rate, on useful FLOPs."""
+    peak = pk["bf16_tflops"]
     out = []
     g = torch.Generator(device="cuda")
     g.manual_seed(77)
@@ -398,7 +397,7 @@ def pass_spgemm(gpu, bsp, torch, reps=5):
         pairs = float((ga @ gb.t()).sum().item())             # block pairs that both masks keep
         fl = 2.0 * 512 * pairs
         out.append({"sparsity": s, **st, "useful_flops": fl, "tflops": fl / (st["ms"] * 1e-3) / 1e12,
-                    "roofline": {"bound": "alu", "peak": peak, "unit": "TFLOP/s", "frac": fl / (st["ms"] * 1e-3) / 1e12 / peak}})
+                    "roofline": {"bound": "tensor", "peak": peak, "unit": "TFLOP/s", "frac": fl / (st["ms"] * 1e-3) / 1e12 / peak}})
     return out
 
 
@@ -669,7 +668,7 @@ def main():
             "layers": i8, "note": "int8 -> int32, bsp_mask, bsp_compact and the product each timed on their own",
             "sum_ms": {str(s): {k: float(sum(r.get(k, r["conv_ms"]) * r["count"] for r in i8 if r["sparsity"] == s))
                                 for k in ("mask_ms", "compact_ms", "conv_ms", "step_ms", "conv_q8_ms")} for s in (0.5, 0.75)}}
-        sweeps["spgemm_2048x4096_bf16_8x8"] = pass_spgemm(gpu, bsp, torch)
+        sweeps["spgemm_2048x4096_bf16_8x8"] = pass_spgemm(gpu, bsp, torch, pk)
         sweeps["chain_resnet50_tails_b64_bf16_8x8_50"] = pass_chain(gpu, bsp, torch, pk)
     clocks = sampler.stop()
 
