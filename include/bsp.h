@@ -14,8 +14,8 @@
  *    bsp_bcsr structs) are HOST structs read during the call.  The library allocates no device memory:
  *    scratch comes from the caller's workspace `ws` (device, 256-byte aligned), sized by the matching
  *    *_workspace_bytes() call.  The caller zero-fills the first 256 bytes of a workspace once after
- *    allocating it (they hold the latched status word and the counters of the grid-wide barrier that the
- *    single-launch kernels of small layers use); one workspace sized for the largest request may serve all
+ *    allocating it (they hold the latched status word and the counts of arrived CTAs that the single-launch
+ *    kernels of the Gamma builder use); one workspace sized for the largest request may serve all
  *    calls issued on one stream, and a workspace must not be shared by calls running on different streams.
  *  - Alignment: W and the canonical payload must be 4-byte aligned (the set-up kernels read
  *    32-bit words and use 16-byte accesses when the addresses allow it); X, Y and the packed buffer 16-byte

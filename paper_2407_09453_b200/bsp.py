@@ -237,10 +237,10 @@ def conv_kernel_name(wd: WDesc, xd: XDesc) -> str:
 
 
 def launches_per_step(wd: WDesc) -> int:
-    """Kernel launches of one bsp_mask + bsp_compact + bsp_conv2d/bsp_gemm pass.  General path: score, select; the
-    compaction; the product kernel.  Small layers take one launch for the mask (up to 4096 blocks)."""
+    """Kernel launches of one bsp_mask (whole layer) + bsp_compact + bsp_conv2d/bsp_gemm pass: the mask takes one launch for layers of
+    up to 4096 blocks and of more than 24576, in between one for the scores and one for the select; compaction and product one each."""
     nb = (wd.O // wd.bo) * (wd.I // wd.bi)
-    return (1 if nb <= 4096 else 2) + 1 + 1
+    return (2 if 4096 < nb <= 24576 else 1) + 1 + 1
 
 
 class SparseLayer:

@@ -34,21 +34,22 @@ inline int elem_bytes(bsp_dtype t) { return t == BSP_I8 ? 1 : (t == BSP_BF16 ? 2
 
 PackedLayout packed_layout(const bsp_wdesc &wd);
 
-// Workspace: the first 256 bytes hold the latched status word (word 0) and the two words of the grid-wide
-// barrier of the single-launch kernels (words kWsSyncWord, kWsSyncWord + 1); scratch starts after them.
+// Workspace: the first 256 bytes hold the latched status word (word 0) and the counts of CTAs that have arrived and that are done
+// of the single-launch kernels (words kWsSyncWord, kWsSyncWord + 1), zero between launches; scratch starts after them.
 constexpr size_t kWsHeader = 256;
 constexpr int kWsSyncWord = 2;
-// Scratch of the cooperative select after the scores in the mask workspace: 7 x 1024 histogram words, 8 counter and key-span words,
-// one word per CTA and a list of up to 8192 candidate keys.
+// Scratch of the cooperative select after the scores in the mask workspace: 7 x 2048 histogram words, 8 counter words,
+// one word per CTA and a list of up to 8192 candidate keys with the numbers of their blocks.
 constexpr int kSelectMaxCtas = 1024;
-constexpr int kSelectHist = 7 * 1024;
-constexpr size_t kSelectScratch = (kSelectHist + 8 + kSelectMaxCtas) * 4 + 8192 * 8;
+constexpr int kSelectHist = 7 * 2048;
+constexpr int kSelectList = 8192;
+constexpr size_t kSelectScratch = (kSelectHist + 8 + kSelectMaxCtas) * 4 + (size_t)kSelectList * 12;
 
 // Host-side validation of a weight descriptor, shared by every entry point.
 bsp_status check_wdesc(const bsp_wdesc *wd);
 
 bsp_status launch_mask(const bsp_wdesc &wd, const void *W, bsp_norm norm, bsp_scope scope, int64_t n_zero,
-                       uint8_t *gamma, void *scores, void *ws, cudaStream_t st);
+                       uint8_t *gamma, void *scores, bool keep_scores, void *ws, cudaStream_t st);
 bsp_status launch_compact(const bsp_wdesc &wd, const void *W, const uint8_t *gamma, int32_t *row_ptr,
                           int32_t *col_idx, void *payload, void *packed, int64_t capacity_blocks, void *ws,
                           cudaStream_t st);
@@ -105,6 +106,12 @@ __device__ __forceinline__ const T *from_here(const T *p)
 __device__ __forceinline__ uint32_t load_free(const uint32_t *p) { uint32_t v; asm("ld.global.b32 %0, [%1];\n" : "=r"(v) : "l"(p)); return v; }
 __device__ __forceinline__ int32_t load_free(const int32_t *p) { return (int32_t)load_free((const uint32_t *)p); }
 __device__ __forceinline__ uint32_t load_free(const uint8_t *p) { uint32_t v; asm("ld.global.u8 %0, [%1];\n" : "=r"(v) : "l"(p)); return v; }
+__device__ __forceinline__ uint2 load_free(const uint2 *p)
+{
+    uint2 v;
+    asm("ld.global.v2.b32 {%0, %1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ uint4 load_free(const uint4 *p)
 {
     uint4 v;

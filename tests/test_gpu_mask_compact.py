@@ -130,6 +130,40 @@ def test_ties_across_the_ctas_of_a_select(rows, cols):
             assert np.array_equal(g, ref.mask(want, n_zero)), n_zero
 
 
+@pytest.mark.parametrize("rows,cols", [(64, 64), (128, 192), (149, 165), (256, 160)])      # 4096, 24576, 24585 and 40960 blocks
+@pytest.mark.parametrize("what", ["infinite first", "mostly zero", "wide range", "two values"])
+def test_select_of_uneven_scores(rows, cols, what):
+    """Scores that leave most of a histogram's bins empty or lie outside of them, on each kind of select: an infinite weight among the
+    blocks that the range is taken from, weights that were pruned before, forty octaves, two values."""
+    W = make_case(161, rows * 8, cols * 8, 1, 1, "bf16")
+    keep = synth.random_gamma(162, rows, cols, rows * cols // 4).repeat(8, 0).repeat(8, 1).reshape(W.shape)
+    if what == "infinite first":
+        W[0, 0, 0, 0] = np.inf
+    elif what == "mostly zero":
+        W = W * keep
+    elif what == "wide range":
+        W = synth.round_to_bf16((W * np.exp2(np.linspace(-20, 20, rows * 8)).reshape(-1, 1, 1, 1)).astype(np.float32))
+    else:
+        W = np.where(keep != 0, np.float32(0.5), np.float32(0.25))
+    want = ref.scores(W, 8, 8)
+    NB = rows * cols
+    for n_zero in (1, NB // 10, NB // 2, 3 * NB // 4 + 1, NB - 1):
+        g, s, _, _ = gpu_mask(W, 8, 8, "bf16", n_zero)
+        assert np.array_equal(s, want)
+        assert np.array_equal(g, ref.mask(want, n_zero)), n_zero
+
+
+@pytest.mark.parametrize("rows", [(5, 128), (5, 129), (5, 4096), (128, 200), (129, 200)])
+def test_row_scope_in_one_and_two_launches(rows):
+    """Rows that are ranked, selected by the CTA that scores them, and selected in a launch of their own; a few equal keys."""
+    W = synth.uniform_int(163, (rows[0] * 8, 1, 1, rows[1] * 8), -3, 3).astype(np.int8)
+    want = ref.scores(W, 8, 8)
+    for n_zero in (0, 1, rows[1] // 2, rows[1] - 1, rows[1]):
+        g, s, _, _ = gpu_mask(W, 8, 8, "i8", n_zero, scope=bsp.SCOPE_ROW)
+        assert np.array_equal(s, want)
+        assert np.array_equal(g, ref.mask(want, n_zero, ref.SCOPE_ROW)), n_zero
+
+
 @pytest.mark.parametrize("NBo,NBi", [(9, 512), (17, 496), (16, 513), (8, 600), (40, 1024), (1030, 4), (7, 1040)])
 def test_index_without_a_payload(NBo, NBi):
     """row_ptr and col_idx of layers of more than 4096 blocks that keep the packed form only: rows of one and several passes of 512
