@@ -38,12 +38,12 @@ PackedLayout packed_layout(const bsp_wdesc &wd);
 // of the single-launch kernels (words kWsSyncWord, kWsSyncWord + 1), zero between launches; scratch starts after them.
 constexpr size_t kWsHeader = 256;
 constexpr int kWsSyncWord = 2;
-// Scratch of the cooperative select after the scores in the mask workspace: 7 x 2048 histogram words, 8 counter words,
-// one word per CTA and a list of up to 8192 candidate keys with the numbers of their blocks.
+// Scratch of the cooperative select after the scores in the mask workspace: three histograms of 2048 words, 8 counter words,
+// one word per CTA, and in what is left a list of candidate keys with the numbers of their blocks.
 constexpr int kSelectMaxCtas = 1024;
-constexpr int kSelectHist = 7 * 2048;
-constexpr int kSelectList = 8192;
-constexpr size_t kSelectScratch = (kSelectHist + 8 + kSelectMaxCtas) * 4 + (size_t)kSelectList * 12;
+constexpr int kSelectHist = 3 * 2048;
+constexpr size_t kSelectScratch = 98336;
+constexpr int kSelectList = (int)((kSelectScratch - (kSelectHist + 8 + kSelectMaxCtas) * 4) / 12 / 512 * 512);
 
 // Host-side validation of a weight descriptor, shared by every entry point.
 bsp_status check_wdesc(const bsp_wdesc *wd);

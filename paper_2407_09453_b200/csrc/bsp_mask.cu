@@ -598,11 +598,10 @@ __device__ __forceinline__ void select_small(const unsigned long long *keys, int
 constexpr int kCoopThreads = 512;
 constexpr int kFirstShift = 45, kFirstBelow = 14 * 128;      // leading bits of the first pass; its bins below the reference
 constexpr int kCoopBins = 2048, kCoopWidth = 11;
-static_assert(7 * kCoopBins <= kSelectHist, "a histogram for the first pass and one for each eleven bits of a 64-bit key");
-constexpr int kLocalMax = 8192;          // candidates that the CTAs finish on their own, in (dynamic) shared memory
+static_assert(3 * kCoopBins <= kSelectHist, "a histogram in use, one that others may still read, one that is being zeroed");
+constexpr int kLocalMax = kSelectList;   // candidates that the CTAs finish on their own, in (dynamic) shared memory
 constexpr int kSliceMax = 4096;          // keys of a CTA's slice that are kept in shared memory
 constexpr size_t kCoopSmem = (size_t)(kLocalMax + kSliceMax) * sizeof(unsigned long long) + (size_t)kLocalMax * sizeof(unsigned);
-static_assert(kLocalMax <= kSelectList, "the list of candidates");
 
 template <typename A>
 __device__ __forceinline__ unsigned long long key_bits(A score) { return (unsigned long long)__double_as_longlong((double)score); }
@@ -700,9 +699,11 @@ mask_coop_kernel(const uint32_t *W, int I, int HK, int bo, int bi, int NBo, int 
         }
         __syncthreads();
         for (int q = tid; q < kCoopBins; q += kCoopThreads)
-            if (hist[q]) atomicAdd(&ghist[pi * kCoopBins + q], hist[q]);
+            if (hist[q]) atomicAdd(&ghist[pi % 3 * kCoopBins + q], hist[q]);
         if (!meet()) { give_up(); return; }
-        for (int q = tid; q < kCoopBins; q += kCoopThreads) hist[q] = __ldcg(&ghist[pi * kCoopBins + q]);
+        for (int q = tid; q < kCoopBins; q += kCoopThreads) hist[q] = __ldcg(&ghist[pi % 3 * kCoopBins + q]);
+        // (every CTA has read the histogram before this one: it is zeroed for the pass after the next)
+        for (int q = (int)blockIdx.x * kCoopThreads + tid; q < kCoopBins; q += (int)gridDim.x * kCoopThreads) ghist[(pi + 2) % 3 * kCoopBins + q] = 0u;
         __syncthreads();
         select_digit<kCoopThreads, kCoopBins>(hist, warp_sums, prefix, &s_k, &s_prefix, &s_left, width);
         top -= width;
