@@ -98,8 +98,9 @@ __device__ __forceinline__ bool ct_wait_count(const volatile uint32_t *count, ui
     return false;
 }
 
-// kI8: the 8-bit chain; kEy: bytes of an element of Y (compiled apart, so that no form carries another's epilogue code).
-template <bool kI8, int kEy, bool kHalo>
+// kI8: the 8-bit chain; kEy: bytes of an element of Y (compiled apart, so that no form carries another's epilogue code).  kEights: kHalo on tiles of
+// eight columns, as in the product kernel.
+template <bool kI8, int kEy, bool kHalo, bool kEights>
 __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kernel(const __grid_constant__ CtParams p)
 {
     constexpr int kWt = kI8 ? BSP_I8 : BSP_BF16;
@@ -296,10 +297,11 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             // the taps of a kHalo tile (see the product kernel)
             auto taps = [&](auto wide_c, auto first_c, uint32_t d) -> bool {
                 constexpr bool kWide = decltype(wide_c)::value, kFirst = decltype(first_c)::value;
+                constexpr uint64_t shape = kWide ? kGtDesc : kGtDesc32;
                 const uint32_t row16 = kWide ? 8u : 2u, w_tap16 = (uint32_t)(p.O1p * p.kbytes) >> 4, row_step = (uint32_t)(p.halo_w - p.K) * row16;
                 const uint64_t plane_a = (uint64_t)(p.plane_bytes >> 4), plane_b = (uint64_t)(p.O1p * 32 >> 4);
                 const uint32_t two = (uint32_t)p.planes - 1u;
-                uint64_t da = (kWide ? kGtDesc : kGtDesc32) | (uint64_t)a16, db = (kWide ? kGtDesc : kGtDesc32) | (uint64_t)(base >> 4);
+                uint64_t da = (kEights ? gt_desc_groups(shape, (uint32_t)p.halo_w * row16) : shape) | (uint64_t)a16, db = shape | (uint64_t)(base >> 4);
                 uint32_t acc = 0u;
                 int t = 0;
 #pragma unroll 1
@@ -408,10 +410,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             const bool issuer = q == 0 && lane == 0;             // one thread of the group issues its stores
             const int r = q * 32 + lane;                         // this lane's row of a tile
             int row = r;                                         // its row of the staging buffer (kHalo: the place in the box, or none)
-            if constexpr (kHalo) {
-                const int per_image = p.halo_rows * p.halo_w, n = r / per_image, y = (r - n * per_image) / p.halo_w, x = r - n * per_image - y * p.halo_w;
-                row = n < p.Nt && y < p.Ht && x < p.Wt ? (n * p.Ht + y) * p.Wt + x : -1;
-            }
+            if constexpr (kHalo) row = gt_halo_row(r, kEights, p.Wt, p.Ht, p.Nt, p.halo_w, p.halo_rows);
             // constants of a round's channels, fetched one round ahead (thread c holds channel c)
             uint32_t *bias = tail.bias[grp], *half = tail.half[grp];
             uint8_t *shift = tail.shift[grp];
@@ -623,7 +622,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     BSP_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
     if (n_sm[dev] == 0) BSP_CUDA_OK(cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
-    const GtTile Th = gt_pick_halo(xd.N, p.M, p.Nw, wd1.H, wd1.K);
+    const GtHaloTile Th = gt_pick_halo(xd.N, p.M, p.Nw, wd1.H, wd1.K);
     // Where the position tiles fill less than half of the SMs, several CTAs take one: each computes T for itself and its share of
     // layer two's channels.  (Two 128-channel tiles of Y take about 1.2 us one after the other: 7x1 128->64->928 at 11x11 13.0 -> 6.6 us,
     // 3x3 64->80->768 at 22x22 12.3 -> 7.4, 1x1 96->128->592 at 34x34, batch 8, 14.9 -> 11.6.)
@@ -655,7 +654,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     // kHalo: where two boxes of activations, the weights of layer one and at least two chunks of layer two's fit, and the
     // tiles with their border are not many more.  3x3 64->64 then 64->256 at 56x56, batch 64, in a short burst: 44.5 us loaded
     // tap by tap, 33.8 like this (36 in a stream of calls).
-    bool halo = false;
+    bool halo = false, eights = false;
     int w2_slots = 0;
     if (stays) {
         const int kb = row1 <= 32 ? 32 : (row1 <= 64 ? 64 : 128), planes = kb == 128 ? 1 : kb / 32;
@@ -674,7 +673,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
         if (w2_slots >= 2 || w2_slots == p.n_t2 * p.n_c2) {
             halo = true;
             T = Th;
-            p.kbytes = kb; p.planes = planes; p.plane_bytes = plane;
+            p.kbytes = kb; p.planes = planes; p.plane_bytes = plane; eights = Th.eights != 0;
             p.dbt = second ? 1 : 0;
             p.w2_slots = w2_slots; p.w2_stay = w2_slots == p.n_t2 * p.n_c2 ? 1 : 0;
             p.halo_w = T.Wt + wd1.K - 1; p.halo_rows = T.Ht + wd1.H - 1;
@@ -710,13 +709,15 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.off_tail = (uint32_t)at;
     const size_t smem = at + (halo ? sizeof(CtTail<3>) : sizeof(CtTail<2>));
 
-    // kernels by type of the pair, width of Y (32 bits or the narrow form) and kHalo
+    // kernels by type of the pair, width of Y (32 bits or the narrow form) and how layer one is staged
     typedef void (*Kernel)(const CtParams);
-    static const Kernel kernels[2][2][2] = {{{chain_tc_kernel<false, 4, false>, chain_tc_kernel<false, 4, true>}, {chain_tc_kernel<false, 2, false>, chain_tc_kernel<false, 2, true>}},
-                                            {{chain_tc_kernel<true, 4, false>, chain_tc_kernel<true, 4, true>}, {chain_tc_kernel<true, 1, false>, chain_tc_kernel<true, 1, true>}}};
+    static const Kernel kernels[2][2][3] = {{{chain_tc_kernel<false, 4, false, false>, chain_tc_kernel<false, 4, true, false>, chain_tc_kernel<false, 4, true, true>},
+                                             {chain_tc_kernel<false, 2, false, false>, chain_tc_kernel<false, 2, true, false>, chain_tc_kernel<false, 2, true, true>}},
+                                            {{chain_tc_kernel<true, 4, false, false>, chain_tc_kernel<true, 4, true, false>, chain_tc_kernel<true, 4, true, true>},
+                                             {chain_tc_kernel<true, 1, false, false>, chain_tc_kernel<true, 1, true, false>, chain_tc_kernel<true, 1, true, true>}}};
     static bool opted[kGtMaxDevices] = {};
     if (!opted[dev]) {
-        for (int t = 0; t < 8; ++t) BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 4][t / 2 % 2][t % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, kCtSmem));
+        for (int t = 0; t < 12; ++t) BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 6][t / 3 % 2][t % 3], cudaFuncAttributeMaxDynamicSharedMemorySize, kCtSmem));
         opted[dev] = true;
     }
     // bytes of an operand row of layer one in shared memory, and its swizzle
@@ -767,7 +768,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
             return BSP_ERR_CUDA;
     }
     const int grid = p.n_tiles * p.parts < n_sm[dev] ? p.n_tiles * p.parts : n_sm[dev];      // (several parts: one wave)
-    BSP_CUDA_OK(launch_after(kernels[wd1.wtype == BSP_I8 ? 1 : 0][ey == 4 ? 0 : 1][halo ? 1 : 0], dim3((unsigned)grid), dim3(64u + 128u * ct_groups(halo)), smem, st, p));
+    BSP_CUDA_OK(launch_after(kernels[wd1.wtype == BSP_I8 ? 1 : 0][ey == 4 ? 0 : 1][halo ? (eights ? 2 : 1) : 0], dim3((unsigned)grid), dim3(64u + 128u * ct_groups(halo)), smem, st, p));
     return BSP_OK;
 }
 

@@ -88,13 +88,14 @@ __device__ __forceinline__ void gt_tile_origin(const GtParams &p, int mt, int &n
 // tile are loaded once and stay, the activations of a position tile arrive in ONE load with the border that its taps reach,
 // and a tap is a view of that box shifted by whole rows (the swizzle goes by the shared-memory address).  Nine loads of
 // shifted boxes and nine weight tiles per tile had kept such layers at the pace of the TMA unit (about 1.5 cycles per row).
-constexpr int kTaps = 0, kPairs = 1, kHalo = 2;
+// kEights is kHalo on tiles of eight columns (apart, so that kHalo's descriptors stay constants).
+constexpr int kTaps = 0, kPairs = 1, kHalo = 2, kEights = 3;
 template <int kWT, int kEy, int kMode>
 __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_constant__ GtParams p)
 {
     constexpr bool kPair = kMode == kPairs;
     extern __shared__ __align__(1024) uint8_t smem[];
-    GtTail &tail = *(GtTail *)(smem + (kMode == kHalo ? p.w_bytes : 0) + (size_t)p.stages * p.stage_bytes + 8 * kGtStagingBytes);
+    GtTail &tail = *(GtTail *)(smem + (kMode >= kHalo ? p.w_bytes : 0) + (size_t)p.stages * p.stage_bytes + 8 * kGtStagingBytes);
     uint64_t *s_full = tail.full, *s_empty = tail.empty, *s_acc_full = tail.acc_full, *s_acc_empty = tail.acc_empty;
     volatile uint32_t &s_fail = tail.fail;
 
@@ -103,7 +104,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     // 100 cycles of issue and every poll 150, against 48 / 64 / 127 for the MMA itself at 64 / 128 / 256 channels and 90.)
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const int S = p.stages, n_ks = p.n_ks, BN = p.BN;
-    const uint32_t ring = sm32(smem) + (kMode == kHalo ? (uint32_t)p.w_bytes : 0u);
+    const uint32_t ring = sm32(smem) + (kMode >= kHalo ? (uint32_t)p.w_bytes : 0u);
     const uint32_t staging = ring + (uint32_t)(S * p.stage_bytes);
     // Work items: tiles, or for CTA pairs two position tiles side by side on one channel tile (CTA r of the pair takes
     // position tile 2 mp + r; a pair past an odd count loads zeros and stores nothing).
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     const int t_count = kMode == kTaps ? p.n_tiles : kPair ? p.n_tile_pairs : p.n_pos;
     // position tile (of this CTA, in a pair) and channel tile of a work item
     auto tile_of = [&](int tile, int &mt, int &tn) {
-        if constexpr (kMode == kHalo) { mt = tile; tn = (int)blockIdx.x - t_first * ntn; }
+        if constexpr (kMode >= kHalo) { mt = tile; tn = (int)blockIdx.x - t_first * ntn; }
         else {
             gt_divmod(tile, ntn, p.m_ntn, mt, tn);
             if constexpr (kPair) mt = 2 * mt + (int)rank;
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc_full[b])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc_empty[b])), "r"(kPair ? 8 : 4) : "memory");
         }
-        if constexpr (kMode == kHalo)
+        if constexpr (kMode >= kHalo)
             for (int t = 0; t < p.n_ks; ++t) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&tail.w_full[t])), "r"(1) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&p.tmx) : "memory");
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             // (a pair: each CTA loads its own activation box and its half of the weight tile, all four loads announce their
             // bytes on the leader's barrier, which the leader arms with the total)
             const uint32_t stage_bytes = (uint32_t)p.stage_bytes;
-            const uint32_t tx = (uint32_t)(p.a_bytes + (kMode == kHalo ? 0 : BN >> (kPair ? 1 : 0)) * p.kbytes) * (kPair ? 2u : 1u);
+            const uint32_t tx = (uint32_t)(p.a_bytes + (kMode >= kHalo ? 0 : BN >> (kPair ? 1 : 0)) * p.kbytes) * (kPair ? 2u : 1u);
             const int cpt128 = p.cpt * 128, Kw = p.K;
             // (a fresh barrier counts as released: the wait on parity 1 of the first round returns at once)
             uint32_t slot = 0, epar = 1, issued = 0, dst = ring;
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 const int ch0 = tn * BN + (kPair ? (int)rank * (BN >> 1) : 0);
                 int n0, y0, x0;
                 gt_tile_origin(p, mt, n0, y0, x0);
-                if constexpr (kMode == kHalo) {
+                if constexpr (kMode >= kHalo) {
                     if (s_fail) { ok = false; break; }
                     if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; break; }
                     const bool wrap = slot + 1u == (uint32_t)S;
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 atomicExch((uint32_t *)&tail.fail, 1u);
                 // (the follower of a pair has no barrier of its own to watch: its loads announce themselves to the leader;
                 // both CTAs meet at the cluster barrier before they leave)
-                if (kMode == kHalo && issued > 0)
+                if (kMode >= kHalo && issued > 0)
                     for (int t = 0; t < n_ks; ++t) gt_poll(sm32(&tail.w_full[t]), 0u);
                 for (uint32_t back = 0; back < (uint32_t)S && back < issued && rank == 0; ++back) {
                     const uint32_t it = issued - 1u - back;
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 }
             }
         }
-    } else if (kMode == kHalo && warp == 1) {
+    } else if (kMode >= kHalo && warp == 1) {
         // ================= MMA issuer of kHalo =================
         if (run) {
             const uint32_t dfmt = kWT == BSP_I8 ? 2u : 1u, abfmt = kWT == BSP_F32 ? 2u : 1u;
@@ -277,10 +278,11 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             // it cost 10 %.)
             auto issue = [&](auto wide_c, auto first_c, uint32_t d, uint32_t a_tap) -> bool {
                 constexpr bool kWide = decltype(wide_c)::value, kFirst = decltype(first_c)::value;
+                constexpr uint64_t shape = kWide ? kGtDesc : kGtDesc32;
                 const uint32_t row16 = kWide ? 8u : 2u, w_tap16 = (uint32_t)(BN * p.kbytes) >> 4, row_step = (uint32_t)(p.halo_w - p.K) * row16;
                 const uint64_t plane_a = (uint64_t)(p.plane_bytes >> 4), plane_b = (uint64_t)(BN * 32 >> 4);
                 const uint32_t two = (uint32_t)p.planes - 1u;
-                uint64_t da = (kWide ? kGtDesc : kGtDesc32) | (uint64_t)a_tap, db = (kWide ? kGtDesc : kGtDesc32) | (uint64_t)(sm32(smem) >> 4);
+                uint64_t da = (kMode == kEights ? gt_desc_groups(shape, (uint32_t)p.halo_w * row16) : shape) | (uint64_t)a_tap, db = shape | (uint64_t)(sm32(smem) >> 4);
                 uint32_t acc = 0u;
                 int t = 0;
 #pragma unroll 1
@@ -370,10 +372,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             int row = q * 32 + lane;
             if constexpr (kMode == kTaps)                        // (with M = 64, 16 rows in the first half of each quarter)
                 if (p.half_rows) row = lane < 16 ? q * 16 + lane : -1;
-            if constexpr (kMode == kHalo) {
-                const int per_image = p.halo_rows * p.halo_w, n = row / per_image, y = (row - n * per_image) / p.halo_w, x = row - n * per_image - y * p.halo_w;
-                row = n < p.Nt && y < p.Ht && x < p.Wt ? (n * p.Ht + y) * p.Wt + x : -1;
-            }
+            if constexpr (kMode >= kHalo) row = gt_halo_row(row, kMode == kEights, p.Wt, p.Ht, p.Nt, p.halo_w, p.halo_rows);
             // Constants of a round's channels: the group's thread c holds channel c of the next round and puts them into shared
             // memory once the group has read the current ones, so that the trip to memory is never waited for.
             uint32_t *bias = tail.bias[grp], *half = tail.half[grp];
@@ -423,7 +422,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + buf * 256u;
                 // the channels of the round after the last one of this tile: those of the group's next tile
                 int after = n0 + c_first;
-                if (!last && kMode != kHalo && ntn > 1) {
+                if (!last && kMode < kHalo && ntn > 1) {
                     int m2, t2;
                     const int next = tile + 2 * t_step < t_count ? tile + 2 * t_step : tile + t_step;
                     gt_divmod(next, ntn, p.m_ntn, m2, t2);
@@ -546,19 +545,19 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     p.n_ks = HK * p.cpt;
     // kernels by operand type (in the order of bsp_dtype), width of the output (32 bits or the narrow form) and mode
     typedef void (*Kernel)(const GtParams);
-    static const Kernel kernels[3][2][3] = {
-        {{gemm_tc_kernel<BSP_F32, 4, kTaps>, gemm_tc_kernel<BSP_F32, 4, kPairs>, gemm_tc_kernel<BSP_F32, 4, kHalo>},
-         {gemm_tc_kernel<BSP_F32, 2, kTaps>, gemm_tc_kernel<BSP_F32, 2, kPairs>, gemm_tc_kernel<BSP_F32, 2, kHalo>}},
-        {{gemm_tc_kernel<BSP_BF16, 4, kTaps>, gemm_tc_kernel<BSP_BF16, 4, kPairs>, gemm_tc_kernel<BSP_BF16, 4, kHalo>},
-         {gemm_tc_kernel<BSP_BF16, 2, kTaps>, gemm_tc_kernel<BSP_BF16, 2, kPairs>, gemm_tc_kernel<BSP_BF16, 2, kHalo>}},
-        {{gemm_tc_kernel<BSP_I8, 4, kTaps>, gemm_tc_kernel<BSP_I8, 4, kPairs>, gemm_tc_kernel<BSP_I8, 4, kHalo>},
-         {gemm_tc_kernel<BSP_I8, 1, kTaps>, gemm_tc_kernel<BSP_I8, 1, kPairs>, gemm_tc_kernel<BSP_I8, 1, kHalo>}}};
+    static const Kernel kernels[3][2][4] = {
+        {{gemm_tc_kernel<BSP_F32, 4, kTaps>, gemm_tc_kernel<BSP_F32, 4, kPairs>, gemm_tc_kernel<BSP_F32, 4, kHalo>, gemm_tc_kernel<BSP_F32, 4, kEights>},
+         {gemm_tc_kernel<BSP_F32, 2, kTaps>, gemm_tc_kernel<BSP_F32, 2, kPairs>, gemm_tc_kernel<BSP_F32, 2, kHalo>, gemm_tc_kernel<BSP_F32, 2, kEights>}},
+        {{gemm_tc_kernel<BSP_BF16, 4, kTaps>, gemm_tc_kernel<BSP_BF16, 4, kPairs>, gemm_tc_kernel<BSP_BF16, 4, kHalo>, gemm_tc_kernel<BSP_BF16, 4, kEights>},
+         {gemm_tc_kernel<BSP_BF16, 2, kTaps>, gemm_tc_kernel<BSP_BF16, 2, kPairs>, gemm_tc_kernel<BSP_BF16, 2, kHalo>, gemm_tc_kernel<BSP_BF16, 2, kEights>}},
+        {{gemm_tc_kernel<BSP_I8, 4, kTaps>, gemm_tc_kernel<BSP_I8, 4, kPairs>, gemm_tc_kernel<BSP_I8, 4, kHalo>, gemm_tc_kernel<BSP_I8, 4, kEights>},
+         {gemm_tc_kernel<BSP_I8, 1, kTaps>, gemm_tc_kernel<BSP_I8, 1, kPairs>, gemm_tc_kernel<BSP_I8, 1, kHalo>, gemm_tc_kernel<BSP_I8, 1, kEights>}}};
     static_assert(BSP_F32 == 0 && BSP_BF16 == 1 && BSP_I8 == 2, "the table is indexed by type");
     const Kernel *kernel = kernels[wd.wtype][ey == 4 ? 0 : 1];
     static bool opted[kGtMaxDevices] = {};
     if (!opted[dev]) {
-        for (int t = 0; t < 18; ++t)
-            BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 6][t / 3 % 2][t % 3], cudaFuncAttributeMaxDynamicSharedMemorySize, kGtGemmSmem));
+        for (int t = 0; t < 24; ++t)
+            BSP_CUDA_OK(cudaFuncSetAttribute(kernels[t / 8][t / 4 % 2][t % 4], cudaFuncAttributeMaxDynamicSharedMemorySize, kGtGemmSmem));
         opted[dev] = true;
     }
     // Channels per tile: the widest tile keeps the tensor pipe busiest (a stage costs about 256 + 2 BN cycles of operand
@@ -567,7 +566,7 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     // its MMAs (32 + BN / 4 cycles of operand reads or BN / 2 of arithmetic per 32 bytes of K) or, loaded per tap, 1.5
     // cycles per row of its two boxes; kHalo pays only the MMAs, on tiles that the border makes a few more.
     const int staging = 8 * kGtStagingBytes, nk = p.kbytes / 32;
-    const GtTile Th = gt_pick_halo(xd.N, p.M, p.Nw, wd.H, wd.K);
+    const GtHaloTile Th = gt_pick_halo(xd.N, p.M, p.Nw, wd.H, wd.K);
     const bool halo_ok = HK > 1 && HK <= kGtHaloTaps && p.cpt == 1 && p.sh == 1 && p.sw == 1 && Th.tiles > 0;
     // (up to 64 bytes of channels lie in planes of 32-byte rows: MMAs on 64-byte rows took 90 cycles instead of 67 at 128
     // channels and 72 instead of 59 at 64)
@@ -691,7 +690,7 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     }
     int grid = p.n_tiles < n_sm[dev] ? p.n_tiles : n_sm[dev];
     if (mode == kHalo) grid = grid / p.n_tiles_n * p.n_tiles_n;
-    BSP_CUDA_OK(launch_after(kernel[mode], dim3((unsigned)grid), dim3(kGtThreads), smem, st, p));
+    BSP_CUDA_OK(launch_after(kernel[mode == kHalo && Th.eights ? kEights : mode], dim3((unsigned)grid), dim3(kGtThreads), smem, st, p));
     return BSP_OK;
 }
 

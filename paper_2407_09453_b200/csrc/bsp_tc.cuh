@@ -65,6 +65,16 @@ constexpr uint64_t kGtDesc64 = (1ull << 16) | ((uint64_t)(512u >> 4) << 32) | (1
 // Rows of 32 bytes under the 32-byte swizzle (one K-step): 8-row groups 256 bytes apart.
 constexpr uint64_t kGtDesc32 = (1ull << 16) | ((uint64_t)(256u >> 4) << 32) | (1ull << 46) | (6ull << 61);
 
+// A descriptor with another distance between the groups of eight rows, in 16-byte units.
+__device__ __forceinline__ uint64_t gt_desc_groups(uint64_t desc, uint32_t units) { return (desc & ~((uint64_t)0x3FFFu << 32)) | ((uint64_t)units << 32); }
+
+// The place of row r of a kHalo tile's MMA in the tile's box of positions (as TMA stores read it), or -1 for a row between them.
+__device__ __forceinline__ int gt_halo_row(int r, int eights, int Wt, int Ht, int Nt, int halo_w, int halo_rows)
+{
+    const int pitch = eights ? 8 : halo_w, per_image = halo_rows * pitch, n = r / per_image, y = (r - n * per_image) / pitch, x = r - n * per_image - y * pitch;
+    return n < Nt && y < Ht && x < Wt ? (n * Ht + y) * Wt + x : -1;
+}
+
 // The four MMAs of one stage (two when the stage holds 64 bytes of K: `nk`) and the commit that releases the stage,
 // issued by one elected lane of a converged warp.  All lanes execute this statement with the same operands; the MMA of
 // the first K-step overwrites the accumulator when `acc` is 0.
@@ -352,6 +362,8 @@ GtEncodeFn gt_encode()
 // smaller box).  Several images share a tile only when a tile holds whole images.  A box of the tensor map spans
 // Wt * s_w x Ht * s_h input positions and may not exceed 256 in any extent.
 struct GtTile { int Wt, Ht, Nt; long long tiles; };
+// (gt_pick_halo) `eights`: the rows of the MMA go by groups of eight positions of a row of the image.
+struct GtHaloTile : GtTile { int eights; };
 
 // A 1x1 layer without padding or stride is a matrix product over all N L J positions: taken as that many 1x1 images,
 // so that a tile is 128 consecutive positions whatever the image size.
@@ -416,12 +428,23 @@ GtTile gt_pick_packed(GtTile best, int N, int M, int Nw, int sh, int sw)
 }
 
 // Position tile of a stride-1 layer whose activations are staged once per tile, with the H - 1 rows and K - 1 columns that its
-// taps reach beyond it: the rows of the MMA are the 128 consecutive positions of that box from the tap's own offset on, so
-// output (n, y, x) sits in row (n (Ht + H - 1) + y) (Wt + K - 1) + x and the rows between are not used.
-GtTile gt_pick_halo(int N, int M, int Nw, int H, int K)
+// taps reach beyond it.  The rows of the MMA are the 128 consecutive positions of that box from the tap's own offset on, so
+// output (n, y, x) sits in row (n (Ht + H - 1) + y) (Wt + K - 1) + x and the rows between are not used; or, in tiles of eight columns
+// (`eights`), 16 groups of eight positions a row of the box apart (the stride between groups of the matrix descriptor), so that
+// output (n, y, x) sits in row (n (Ht + H - 1) + y) 8 + x and all rows of a tile of 8 x 16 are used: 8-bit 3x3 64->64 at 224x224,
+// batch 32, 85.0 -> 75.3 us.  (Taken where they are fewer; with as many tiles they were up to 2 % slower.)
+GtHaloTile gt_pick_halo(int N, int M, int Nw, int H, int K)
 {
-    GtTile best = {0, 0, 0, -1};
+    GtHaloTile best = {{0, 0, 0, -1}, 0};
     long long best_area = 0;
+    auto offer = [&](int w, int h, int b, int eights) {
+        const int pitch = w + K - 1;
+        const long long cnt = (long long)((N + b - 1) / b) * ((M + h - 1) / h) * ((Nw + w - 1) / w), area = (long long)b * (h + H - 1) * pitch;
+        if (pitch <= 256 && h + H - 1 <= 256 && (best.tiles < 0 || cnt < best.tiles || (cnt == best.tiles && !eights && area < best_area))) {
+            best = {{w, h, b, cnt}, eights};
+            best_area = area;
+        }
+    };
     for (int w = 1; w <= Nw && w <= kGtBM;) {
         const int pitch = w + K - 1, tx = (Nw + w - 1) / w;
         int h = (kGtBM - w) / pitch + 1;
@@ -430,14 +453,17 @@ GtTile gt_pick_halo(int N, int M, int Nw, int H, int K)
         h = (M + ty - 1) / ty;
         int b = 1;
         if (w == Nw && h == M) { b = (kGtBM - ((h - 1) * pitch + w)) / ((h + H - 1) * pitch) + 1; if (b > N) b = N; }
-        const long long cnt = (long long)((N + b - 1) / b) * ty * tx, area = (long long)b * (h + H - 1) * pitch;
-        if (pitch <= 256 && h + H - 1 <= 256 && (best.tiles < 0 || cnt < best.tiles || (cnt == best.tiles && area < best_area))) {
-            best = {w, h, b, cnt};
-            best_area = area;
-        }
+        offer(w, h, b, 0);
         if (tx == 1) break;
         w = (Nw + tx - 2) / (tx - 1);
     }
+    const int w = Nw < 8 ? Nw : 8;
+    int h = M < kGtBM / 8 ? M : kGtBM / 8;
+    const int ty = (M + h - 1) / h;
+    h = (M + ty - 1) / ty;
+    int b = 1;
+    if (h == M) { b = (kGtBM / 8 - M) / (M + H - 1) + 1; if (b > N) b = N; }
+    if (w == 8 || b > 1) offer(w, h, w == Nw ? b : 1, 1);
     return best;
 }
 

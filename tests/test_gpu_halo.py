@@ -34,6 +34,18 @@ def test_taps_and_images(H, K, L, J, N, pad, dtype, out):
     run_conv_case(811, 64, 32, H, K, 8, 8, dtype, (N, L, J, 32), (1, 1), pad, out=out if dtype == "bf16" else "f32")
 
 
+@pytest.mark.parametrize("H,K,L,J,N", [
+    (3, 3, 16, 16, 3),                   # two tiles of 8 x 16 an image
+    (3, 3, 31, 15, 2),                   # a ragged last column and row of tiles
+    (5, 5, 16, 24, 40),                  # more tiles than SMs
+    (1, 7, 16, 16, 2),
+    (3, 3, 7, 7, 64),                    # two images of seven columns a tile, more tiles than images in one
+])
+@pytest.mark.parametrize("dtype,I", [("bf16", 16), ("bf16", 32), ("bf16", 64), ("i8", 64), ("i8", 128), ("f32", 32)])
+def test_tiles_of_eight_columns(H, K, L, J, N, dtype, I):
+    run_conv_case(815, 64, I, H, K, 8, 8, dtype, (N, L, J, I), (1, 1), (H // 2, K // 2))
+
+
 @pytest.mark.parametrize("dtype,O", [("bf16", 48), ("bf16", 200), ("i8", 136), ("f32", 72)])
 def test_channel_tiles(dtype, O):
     """A CTA keeps one channel tile: ragged last tiles, more position tiles than CTAs."""
@@ -79,6 +91,8 @@ def test_requantised_output(O, case):
     (24, 14, 14, 32, 64, 1024, 3, 3, 0), # ... for every three of eight, the last with one past the end
     (2, 22, 22, 192, 80, 176, 3, 3, 1),  # ... with layer one loaded tap by tap
     (60, 17, 17, 192, 64, 160, 3, 3, 0), # tiles of parts of several images
+    (3, 16, 16, 64, 64, 256, 3, 3, 1),   # tiles of eight columns
+    (120, 31, 15, 32, 72, 112, 5, 5, 1), # ... several a CTA, ragged
 ])
 def test_pair_equals_the_two_calls(N, L, J, I, O1, O2, H, K, relu):
     for dtype in ("bf16", "i8"):
