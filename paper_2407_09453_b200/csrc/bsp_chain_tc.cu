@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             const uint32_t idesc2 = (dfmt << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kCtBN2 >> 3) << 17) | ((128u >> 4) << 24);
             const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4;
             uint32_t slot = 0, par = 0, a16 = ring >> 4, tile_i = 0, u2 = 0, slot2 = 0, par2 = 0;
-            bool ok = true, full_now = false;
+            bool ok = true, full_now = false, full2_now = false;
             // the taps of a kHalo tile (see the product kernel)
             auto taps = [&](auto wide_c, auto first_c, uint32_t d) -> bool {
                 constexpr bool kWide = decltype(wide_c)::value, kFirst = decltype(first_c)::value;
@@ -337,13 +337,11 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                     if (++slot == (uint32_t)S) { slot = 0; par ^= 1u; a16 = ring >> 4; } else a16 += stage16;
                 } else {
                     for (int ks = 0; ks < p.n_ks1; ++ks) {
-                        if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
+                        if (!full_now && !gt_poll_stage(full0 + slot * 8u, par)) { ok = false; return; }
                         const bool wrap = slot + 1u == (uint32_t)S;
-                        const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
-                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                         const uint64_t da = kGtDesc | (uint64_t)(a16 & 0x3FFFu), db = kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu);
-                        gt_issue_stage<kWt, false>(d, da, db, idesc1, empty0 + slot * 8u, ks != 0 ? 1u : 0u);
-                        full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+                        full_now = gt_issue_stage<kWt, false>(d, da, db, idesc1, empty0 + slot * 8u, ks != 0 ? 1u : 0u, 4u,
+                                                              full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par) != 0u;
                         if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
                     }
                 }
@@ -367,19 +365,19 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                     for (int c2 = 0; c2 < p.n_c2; ++c2) {
                         const uint64_t da = kGtDesc | (uint64_t)(((tbuf + b * tbytes + (uint32_t)(c2 * kCtChunk)) >> 4) & 0x3FFFu);
                         if constexpr (kHalo) {
-                            if (!__all_sync(0xFFFFFFFFu, gt_poll(sm32(&tail.w2_full[slot2]), par2))) { ok = false; return; }
-                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                            if (!full2_now && !gt_poll_stage(sm32(&tail.w2_full[slot2]), par2)) { ok = false; return; }
+                            const bool wrap = slot2 + 1u == (uint32_t)p.w2_slots;
                             const uint64_t db = kGtDesc | (uint64_t)((base + p.off_w2 + slot2 * (uint32_t)(kCtBN2 * 128)) >> 4);
                             // (weights that stay are never handed back: the arrivals on their barriers go unread)
-                            gt_issue_stage<kWt, false>(d, da, db, idesc2, sm32(&tail.w2_empty[slot2]), c2 != 0 ? 1u : 0u);
-                            if (++slot2 == (uint32_t)p.w2_slots) { slot2 = 0; par2 ^= 1u; }
+                            // (and weights that stay have arrived for good once the first tile is done)
+                            full2_now = gt_issue_stage<kWt, false>(d, da, db, idesc2, sm32(&tail.w2_empty[slot2]), c2 != 0 ? 1u : 0u, 4u,
+                                                                   sm32(&tail.w2_full[wrap ? 0u : slot2 + 1u]), wrap && !p.w2_stay ? par2 ^ 1u : par2) != 0u;
+                            if (wrap) { slot2 = 0; par2 ^= 1u; } else ++slot2;
                         } else {
-                            if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; return; }
+                            if (!full_now && !gt_poll_stage(full0 + slot * 8u, par)) { ok = false; return; }
                             const bool wrap = slot + 1u == (uint32_t)S;
-                            const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
-                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                            gt_issue_stage<kWt, false>(d, da, kGtDesc | (uint64_t)(a16 & 0x3FFFu), idesc2, empty0 + slot * 8u, c2 != 0 ? 1u : 0u);
-                            full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+                            full_now = gt_issue_stage<kWt, false>(d, da, kGtDesc | (uint64_t)(a16 & 0x3FFFu), idesc2, empty0 + slot * 8u, c2 != 0 ? 1u : 0u, 4u,
+                                                                  full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par) != 0u;
                             if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
                         }
                     }

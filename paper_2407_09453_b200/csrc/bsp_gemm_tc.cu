@@ -342,13 +342,11 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t d = tmem + buf * 256u;
                 for (int ks = 0; ks < n_ks; ++ks) {
-                    if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; break; }
+                    if (!full_now && !gt_poll_stage(full0 + slot * 8u, par)) { ok = false; break; }
                     const bool wrap = slot + 1u == (uint32_t)S;
-                    const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint64_t da = desc0 | (uint64_t)(a16 & 0x3FFFu), db = desc0 | (uint64_t)((a16 + astride16) & 0x3FFFu);
-                    gt_issue_stage<kWT, kPair>(d, da, db, idesc, empty0 + slot * 8u, ks != 0 ? 1u : 0u, nk);
-                    full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+                    full_now = gt_issue_stage<kWT, kPair>(d, da, db, idesc, empty0 + slot * 8u, ks != 0 ? 1u : 0u, nk,
+                                                          full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par) != 0u;
                     if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += stage16; }
                 }
                 if (ok) gt_commit_elected<kPair>(sm32(&s_acc_full[buf]));

@@ -271,16 +271,14 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
         uint32_t slot = 0, par = 0, a16 = ring >> 4;
         bool ok = true, full_now = false;
         for (int c = c_lo; c < c_hi; ++c) {
-            if (!full_now && !__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; break; }
+            if (!full_now && !gt_poll_stage(full0 + slot * 8u, par)) { ok = false; break; }
             const bool wrap = slot + 1u == (uint32_t)S;
-            const uint32_t next_full = gt_test(full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par);
             // (the stage's stores come before this thread through its barrier, and before the MMAs by this one fence: a fence in
             // every producer also waited for the loads it had in flight; 2048 x 2048 x 4096 at 50 % 48.9 -> 46.0 us in a burst)
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            gt_issue_stage<BSP_BF16, false>(tmem, kGtDesc | (uint64_t)(a16 & 0x3FFFu), kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu),
-                                            idesc, empty0 + slot * 8u, c != c_lo ? 1u : 0u);
-            full_now = __all_sync(0xFFFFFFFFu, next_full != 0u);
+            full_now = gt_issue_stage<BSP_BF16, false>(tmem, kGtDesc | (uint64_t)(a16 & 0x3FFFu), kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu),
+                                                       idesc, empty0 + slot * 8u, c != c_lo ? 1u : 0u, 4u, full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par) != 0u;
             if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += kStage >> 4; }
         }
         if (ok) gt_commit_elected<false>(sm32(&s_acc));

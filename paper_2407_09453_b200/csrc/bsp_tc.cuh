@@ -34,13 +34,20 @@ __device__ __forceinline__ bool gt_poll(uint32_t bar, uint32_t parity)
 }
 // One look at the barrier, without waiting: non-zero once the phase has completed.  The result of a poll reaches the
 // branch that depends on it after about 90 cycles, so the producer and the MMA warp look at the barrier of the next
-// stage before they issue the current one and fall back to gt_poll only when that look came too early.
+// stage while they issue the current one and fall back to gt_poll only when that look came too early.
 __device__ __forceinline__ uint32_t gt_test(uint32_t bar, uint32_t parity)
 {
     uint32_t done;
     asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.b32 %0, 1, 0, p;\n}\n"
                  : "=r"(done) : "r"(bar), "r"(parity) : "memory");
     return done;
+}
+// The wait of the MMA warp for a stage that its look did not find: all lanes, then the fence that orders the MMAs behind it.
+__device__ __forceinline__ bool gt_poll_stage(uint32_t bar, uint32_t parity)
+{
+    const bool ok = __all_sync(0xFFFFFFFFu, gt_poll(bar, parity));
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    return ok;
 }
 // The same wait for the threads of the epilogue warps: try_wait suspends the thread for a while.
 __device__ __forceinline__ bool gt_wait(uint32_t bar, uint32_t parity)
@@ -75,21 +82,27 @@ __device__ __forceinline__ int gt_halo_row(int r, int eights, int Wt, int Ht, in
     return n < Nt && y < Ht && x < Wt ? (n * Ht + y) * Wt + x : -1;
 }
 
-// The four MMAs of one stage (two when the stage holds 64 bytes of K: `nk`) and the commit that releases the stage,
-// issued by one elected lane of a converged warp.  All lanes execute this statement with the same operands; the MMA of
-// the first K-step overwrites the accumulator when `acc` is 0.
+// The MMAs of one stage (four, or two when the stage holds 64 bytes of K: `nk`), the commit that releases the stage, and a look at
+// the barrier of the next stage, issued by one elected lane of a converged warp.  All lanes execute this statement with the same
+// operands; the MMA of the first K-step overwrites the accumulator when `acc` is 0.  Returns non-zero once the next stage has arrived.
+// The look stands between the second and the third MMA, and its result is taken at the end: the tensor pipe takes one or two
+// instructions ahead, so that what stands before the first MMA of a stage it waits for.  (A stage of four MMAs with M = 64 and 64
+// channels, 128 cycles of arithmetic: 172 cycles with the look before them, 156 with its result taken between them, 132 like this;
+// 32 channels 161, 150 and 132; M = 128 with 64 channels 199, 192 and 192; 128 and more channels take their arithmetic either way.)
 #define GT_ISSUE_STAGE(KIND, CG, COMMIT_TAIL)                                                                       \
-    asm volatile("{\n .reg .pred e, e3, p, t;\n .reg .b64 a1, a2, a3, b1, b2, b3;\n"                                 \
-                 " elect.sync _|e, 0xFFFFFFFF;\n setp.ne.b32 p, %5, 0;\n setp.eq.b32 t, %5, %5;\n"                    \
-                 " setp.gt.u32 e3, %7, 2;\n and.pred e3, e3, e;\n"                                                    \
-                 " add.u64 a1, %1, 2;\n add.u64 a2, %1, 4;\n add.u64 a3, %1, 6;\n"                                    \
-                 " add.u64 b1, %2, 2;\n add.u64 b2, %2, 4;\n add.u64 b3, %2, 6;\n"                                    \
-                 " @e tcgen05.mma.cta_group::" CG ".kind::" KIND " [%0], %1, %2, %3, p;\n"                                 \
-                 " @e tcgen05.mma.cta_group::" CG ".kind::" KIND " [%0], a1, b1, %3, t;\n"                                 \
-                 " @e3 tcgen05.mma.cta_group::" CG ".kind::" KIND " [%0], a2, b2, %3, t;\n"                                \
-                 " @e3 tcgen05.mma.cta_group::" CG ".kind::" KIND " [%0], a3, b3, %3, t;\n"                                \
-                 " @e tcgen05.commit.cta_group::" CG ".mbarrier::arrive::one.shared::cluster" COMMIT_TAIL ";\n}\n"        \
-                 ::"r"(d), "l"(da), "l"(db), "r"(idesc), "r"(bar_empty), "r"(acc), "h"((unsigned short)3), "r"(nk) : "memory")
+    asm volatile("{\n .reg .pred e, e3, p, t, f, v;\n .reg .b64 a1, a2, a3, b1, b2, b3;\n"                           \
+                 " elect.sync _|e, 0xFFFFFFFF;\n setp.ne.b32 p, %6, 0;\n setp.eq.b32 t, %6, %6;\n"                    \
+                 " setp.gt.u32 e3, %8, 2;\n and.pred e3, e3, e;\n"                                                    \
+                 " add.u64 a1, %2, 2;\n add.u64 a2, %2, 4;\n add.u64 a3, %2, 6;\n"                                    \
+                 " add.u64 b1, %3, 2;\n add.u64 b2, %3, 4;\n add.u64 b3, %3, 6;\n"                                    \
+                 " @e tcgen05.mma.cta_group::" CG ".kind::" KIND " [%1], %2, %3, %4, p;\n"                                 \
+                 " @e tcgen05.mma.cta_group::" CG ".kind::" KIND " [%1], a1, b1, %4, t;\n"                                 \
+                 " mbarrier.test_wait.parity.shared::cta.b64 f, [%9], %10;\n"                                              \
+                 " @e3 tcgen05.mma.cta_group::" CG ".kind::" KIND " [%1], a2, b2, %4, t;\n"                                \
+                 " @e3 tcgen05.mma.cta_group::" CG ".kind::" KIND " [%1], a3, b3, %4, t;\n"                                \
+                 " @e tcgen05.commit.cta_group::" CG ".mbarrier::arrive::one.shared::cluster" COMMIT_TAIL ";\n"            \
+                 " vote.sync.all.pred v, f, 0xFFFFFFFF;\n tcgen05.fence::after_thread_sync;\n selp.b32 %0, 1, 0, v;\n}\n"    \
+                 : "=r"(next) : "r"(d), "l"(da), "l"(db), "r"(idesc), "r"(bar_empty), "r"(acc), "h"((unsigned short)3), "r"(nk), "r"(bar_next), "r"(par_next) : "memory")
 
 // The MMAs of one tap without a commit (its activations stay in place for the taps to come): four K-steps inside the span of
 // the 128-byte swizzle, or one or two (`two`) in planes of 32-byte rows, `pa` and `pb` 16-byte units apart.
@@ -129,18 +142,20 @@ __device__ __forceinline__ void gt_issue_planes(uint32_t d, uint64_t da, uint64_
 // tile); the commits then arrive on the barrier at the same shared-memory offset in both CTAs.
 // The operand type is a template argument: a choice at run time costs a branch around every stage.
 template <int kWT, bool kPair>
-__device__ __forceinline__ void gt_issue_stage(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t bar_empty,
-                                               uint32_t acc, uint32_t nk = 4u)
+__device__ __forceinline__ uint32_t gt_issue_stage(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t bar_empty,
+                                                   uint32_t acc, uint32_t nk, uint32_t bar_next, uint32_t par_next)
 {
+    uint32_t next;
     if constexpr (kPair) {
-        if constexpr (kWT == BSP_BF16) GT_ISSUE_STAGE("f16", "2", ".multicast::cluster.b64 [%4], %6");
-        else if constexpr (kWT == BSP_I8) GT_ISSUE_STAGE("i8", "2", ".multicast::cluster.b64 [%4], %6");
-        else GT_ISSUE_STAGE("tf32", "2", ".multicast::cluster.b64 [%4], %6");
+        if constexpr (kWT == BSP_BF16) GT_ISSUE_STAGE("f16", "2", ".multicast::cluster.b64 [%5], %7");
+        else if constexpr (kWT == BSP_I8) GT_ISSUE_STAGE("i8", "2", ".multicast::cluster.b64 [%5], %7");
+        else GT_ISSUE_STAGE("tf32", "2", ".multicast::cluster.b64 [%5], %7");
     } else {
-        if constexpr (kWT == BSP_BF16) GT_ISSUE_STAGE("f16", "1", ".b64 [%4]");
-        else if constexpr (kWT == BSP_I8) GT_ISSUE_STAGE("i8", "1", ".b64 [%4]");
-        else GT_ISSUE_STAGE("tf32", "1", ".b64 [%4]");
+        if constexpr (kWT == BSP_BF16) GT_ISSUE_STAGE("f16", "1", ".b64 [%5]");
+        else if constexpr (kWT == BSP_I8) GT_ISSUE_STAGE("i8", "1", ".b64 [%5]");
+        else GT_ISSUE_STAGE("tf32", "1", ".b64 [%5]");
     }
+    return next;
 }
 // All MMAs issued so far by the elected lane complete -> one arrival on `bar` (in both CTAs of a pair).
 template <bool kPair>
