@@ -51,6 +51,7 @@ struct GtParams {
     uint8_t *Y;
     int ey;
     int half_rows;                    // kTaps: tiles of at most 64 positions, multiplied with M = 64
+    int narrow;                       // kTaps, bfloat16 output: tiles of 32 channels, whose rows of Y are 64 bytes
     int small_acc;                    // int8: the sums of products are at most 2^29
     // kHalo: bytes of the resident weights, pitch and rows of an image's box, position tiles, planes of 32-byte rows and their pitch
     int w_bytes, halo_w, halo_rows, n_pos, planes, plane_bytes;
@@ -224,24 +225,29 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 for (int ks = 0; ks < n_ks; ++ks) {
                     if (!free_now && !__all_sync(0xFFFFFFFFu, gt_poll(empty0 + slot * 8u, epar))) { ok = false; break; }
                     const bool wrap = slot + 1u == (uint32_t)S;
-                    const uint32_t next_free = gt_test(empty0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? epar ^ 1u : epar);
+                    const uint32_t bar_next = empty0 + (wrap ? 0u : slot + 1u) * 8u, par_next = wrap ? epar ^ 1u : epar;
+                    uint32_t next_free;
                     if constexpr (kPair) {
-                        asm volatile("{\n .reg .pred e, l;\n elect.sync _|e, 0xFFFFFFFF;\n setp.eq.u32 l, %12, 0;\n and.pred l, l, e;\n"
-                                     " @l mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
-                                     " @e cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6, %7}], [%13];\n"
-                                     " @e cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%4, %10, %11}], [%13];\n}\n"
-                                     ::"r"(full0 + slot * 8u), "r"(tx), "r"(dst), "l"(&p.tmx), "r"(c128), "r"(kx), "r"(hy), "r"(n0),
-                                       "r"(dst + (uint32_t)p.a_stride), "l"(&p.tmw), "r"(tap), "r"(ch0), "r"(rank), "r"(lead_full0 + slot * 8u) : "memory");
+                        asm volatile("{\n .reg .pred e, l, f, v;\n elect.sync _|e, 0xFFFFFFFF;\n setp.eq.u32 l, %13, 0;\n and.pred l, l, e;\n"
+                                     " @l mbarrier.arrive.expect_tx.shared::cta.b64 _, [%1], %2;\n"
+                                     " @e cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%3], [%4, {%5, %6, %7, %8}], [%14];\n"
+                                     " mbarrier.test_wait.parity.shared::cta.b64 f, [%15], %16;\n"
+                                     " @e cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%9], [%10, {%5, %11, %12}], [%14];\n"
+                                     " vote.sync.all.pred v, f, 0xFFFFFFFF;\n selp.b32 %0, 1, 0, v;\n}\n"
+                                     : "=r"(next_free) : "r"(full0 + slot * 8u), "r"(tx), "r"(dst), "l"(&p.tmx), "r"(c128), "r"(kx), "r"(hy), "r"(n0),
+                                       "r"(dst + (uint32_t)p.a_stride), "l"(&p.tmw), "r"(tap), "r"(ch0), "r"(rank), "r"(lead_full0 + slot * 8u), "r"(bar_next), "r"(par_next) : "memory");
                     } else {
-                        asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xFFFFFFFF;\n"
-                                     " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
-                                     " @e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5, %6, %7}], [%0];\n"
-                                     " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%4, %10, %11}], [%0];\n}\n"
-                                     ::"r"(full0 + slot * 8u), "r"(tx), "r"(dst), "l"(&p.tmx), "r"(c128), "r"(kx), "r"(hy), "r"(n0),
-                                       "r"(dst + (uint32_t)p.a_stride), "l"(&p.tmw), "r"(tap), "r"(ch0) : "memory");
+                        asm volatile("{\n .reg .pred e, f, v;\n elect.sync _|e, 0xFFFFFFFF;\n"
+                                     " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%1], %2;\n"
+                                     " @e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%3], [%4, {%5, %6, %7, %8}], [%1];\n"
+                                     " mbarrier.test_wait.parity.shared::cta.b64 f, [%13], %14;\n"
+                                     " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%9], [%10, {%5, %11, %12}], [%1];\n"
+                                     " vote.sync.all.pred v, f, 0xFFFFFFFF;\n selp.b32 %0, 1, 0, v;\n}\n"
+                                     : "=r"(next_free) : "r"(full0 + slot * 8u), "r"(tx), "r"(dst), "l"(&p.tmx), "r"(c128), "r"(kx), "r"(hy), "r"(n0),
+                                       "r"(dst + (uint32_t)p.a_stride), "l"(&p.tmw), "r"(tap), "r"(ch0), "r"(bar_next), "r"(par_next) : "memory");
                     }
                     ++issued;
-                    free_now = __all_sync(0xFFFFFFFFu, next_free != 0u);
+                    free_now = next_free != 0u;
                     if (wrap) { slot = 0; epar ^= 1u; dst = ring; } else { ++slot; dst += stage_bytes; }
                     // next K-stage: the next 128-byte chunk of channels, then the next tap (columns first)
                     c128 += 128;
@@ -363,6 +369,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             const int q = warp & 3;                              // quarter of the tensor-memory lanes this warp reaches
             const int grp = (warp - 2) >> 2;
             constexpr int cpr = 128 / kEy;                       // output channels per round (128 bytes of a row)
+            const bool narrow = kMode == kTaps && kEy == 2 && p.narrow != 0;
             // the group's staging buffer: 128 rows of 128 bytes
             const uint32_t sg = staging + (uint32_t)(grp * 4 * kGtStagingBytes);
             const bool issuer = q == 0 && lane == 0;             // one thread of the group issues its stores
@@ -442,7 +449,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                     const int left = (p.O - n0 < BN ? p.O - n0 : BN) - c0;          // channels from here on
                     const int next_ch = c0 + c_step < BN ? n0 + c0 + c_step : after;
                     if (next_ch != have) fetch(next_ch);
-                    const uint32_t tcol = tbase + (uint32_t)c0, srow = sg + (uint32_t)row * 128u, sw = (uint32_t)row & 7u;
+                    const uint32_t tcol = tbase + (uint32_t)c0, srow = sg + (uint32_t)row * (narrow ? 64u : 128u), sw = narrow ? ((uint32_t)row >> 1) & 3u : (uint32_t)row & 7u;
                     if constexpr (kEy == 1) {
                         if (c0 != c_first) {
                             if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
@@ -460,7 +467,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                         if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
                         gt_group_sync(1 + grp);
                         if (next_ch != have) place(next_ch);
-                        gt_store_round(srow, sw, row >= 0, out);
+                        gt_store_round(srow, sw, row >= 0, out, narrow ? 4u : 8u);
                     }
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     gt_group_sync(1 + grp);
@@ -611,8 +618,12 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
         T = low;
         taps_cycles = cycles;
     }
+    // ... and tiles of 32 channels, where these still have SMs of their own: half of the weights to load per CTA, and MMAs of 24 cycles
+    // instead of 32.  (A product of 64 positions, 2048->1000, 6.58 -> 6.25 us; fp32, 100 positions, 9.17 -> 8.97.)
+    if (ytype != BSP_I8 && p.BN == 64 && T.Wt * T.Ht * T.Nt <= 64 && T.tiles * ((wd.O + 31) / 32) <= n_sm[dev]) p.BN = 32;
     if (halo_cycles >= 0 && halo_cycles < taps_cycles) { mode = kHalo; p.BN = halo_bn; T = Th; }
     p.half_rows = mode == kTaps && T.Wt * T.Ht * T.Nt <= 64 ? 1 : 0;
+    p.narrow = mode == kTaps && p.BN == 32 && ey == 2 ? 1 : 0;
     p.Wt = T.Wt; p.Ht = T.Ht; p.Nt = T.Nt; p.rows_tile = T.Wt * T.Ht * T.Nt;
     p.tiles_x = (p.Nw + T.Wt - 1) / T.Wt; p.tiles_y = (p.M + T.Ht - 1) / T.Ht;
     p.n_tiles_n = (wd.O + p.BN - 1) / p.BN;
@@ -674,10 +685,10 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
         const cuuint64_t row = (cuuint64_t)wd.O * ey;
         const cuuint64_t gdim[4] = {row, (cuuint64_t)p.Nw, (cuuint64_t)p.M, (cuuint64_t)xd.N};
         const cuuint64_t gstr[3] = {row, row * p.Nw, row * p.Nw * p.M};
-        const cuuint32_t box[4] = {128, (cuuint32_t)T.Wt, (cuuint32_t)T.Ht, (cuuint32_t)T.Nt};
+        const cuuint32_t box[4] = {p.narrow ? 64u : 128u, (cuuint32_t)T.Wt, (cuuint32_t)T.Ht, (cuuint32_t)T.Nt};
         const cuuint32_t estr[4] = {1, 1, 1, 1};
         if (enc(&p.tmy, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, Y, gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                p.narrow ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return BSP_ERR_CUDA;
     }
 

@@ -295,13 +295,14 @@ __device__ __forceinline__ void gt_epilogue_round(uint32_t taddr, const uint32_t
     }
 }
 // ... and from there to the row at `srow` of a tile in shared memory under the 128-byte swizzle (`sw`: the row modulo 8;
-// `live`: the lane has a row).
-__device__ __forceinline__ void gt_store_round(uint32_t srow, uint32_t sw, bool live, const uint32_t (&out)[32])
+// `live`: the lane has a row; `pieces`: 16-byte pieces of the row, 8, or 4 of rows of 64 bytes under the 64-byte swizzle, where `sw` is
+// half the row modulo 4).
+__device__ __forceinline__ void gt_store_round(uint32_t srow, uint32_t sw, bool live, const uint32_t (&out)[32], uint32_t pieces = 8u)
 {
     if (live) {
 #pragma unroll
         for (uint32_t j = 0; j < 8u; ++j)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
+            if (j < 4u || pieces > 4u) asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
                          ::"r"(srow + ((j ^ sw) << 4)), "r"(out[4 * j]), "r"(out[4 * j + 1]), "r"(out[4 * j + 2]), "r"(out[4 * j + 3]) : "memory");
     }
 }
