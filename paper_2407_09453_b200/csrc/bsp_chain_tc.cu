@@ -65,7 +65,7 @@ struct CtTail {
     uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc1_full[2], acc1_empty[2], t_full[2], t_empty[2], acc2_full[2], acc2_empty[2];
     uint64_t w1_full[kCtTaps], w2_full[kCtW2Slots], w2_empty[kCtW2Slots];
     uint64_t before_last;             // layer two of the last tile but one is done (used once)
-    uint32_t tmem, fail;
+    uint32_t tmem, fail, refused;
     uint32_t y_read[2];               // warps that have read accumulator two, counted over all tiles (kGroups > 2 kRpt)
     // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
     __align__(16) uint32_t bias[kGroups][128], half[kGroups][128];
@@ -79,13 +79,6 @@ __device__ __forceinline__ void ct_tile_origin(const CtParams &p, int mt, int &n
     gt_divmod(mt, p.tiles_x, p.m_tx, r, tx);
     gt_divmod(r, p.tiles_y, p.m_ty, ni, ty);
     x0 = tx * p.Wt; y0 = ty * p.Ht; n0 = ni * p.Nt;
-}
-
-__device__ __forceinline__ bool ct_header_ok(const uint8_t *packed, int wtype, int O, int I, int H, int K, int bo, int bi)
-{
-    const PackedHeader *h = (const PackedHeader *)packed;
-    return h->magic == kPackedMagic && h->dtype == wtype && h->O == O && h->I == I && h->H == H && h->K == K && h->bo == bo &&
-           h->bi == bi && (h->forms & kFormDense) != 0;
 }
 
 // Waits (bounded) until a count in shared memory that only grows has reached n.
@@ -152,10 +145,15 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&tail.tmem)), "r"(kGtTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
+    auto header_ok = [&]() {
+        const bool one = gt_header_ok(p.packed1, p.wtype, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1), two = gt_header_ok(p.packed2, p.wtype, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
+        return one && two;
+    };
+    const bool early = tid == 0 && header_ok();
     wait_for_previous<false>();
     if (warp == 0) let_next_start();                  // (behind its allocation)
     if (tid == 0) {
-        const bool ok = ct_header_ok(p.packed1, p.wtype, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1) && ct_header_ok(p.packed2, p.wtype, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
+        const bool ok = early || header_ok();
         const bool placed = (base & 1023u) == 0u;
         s_fail = ok && placed ? 0u : 2u;
         if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
@@ -413,6 +411,8 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             uint32_t *bias = tail.bias[grp], *half = tail.half[grp];
             uint8_t *shift = tail.shift[grp];
             const int ct = ((warp - 2) & 3) * 32 + lane;
+            bool mine = true;                                    // (the look that decides, by one thread, on its way while the tile is made)
+            if (tid == 64) mine = header_ok();
             const uint32_t *bias1 = from_here((const uint32_t *)p.bias1), *bias2 = from_here((const uint32_t *)p.bias2);
             const int32_t *shift1 = from_here(p.shift1), *shift2 = from_here(p.shift2);
             uint32_t next_bias = 0u, next_shift = 1u;
@@ -455,7 +455,12 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             bool ok = true;
             while (rnd >= n_rounds) { rnd -= n_rounds; ++step; }
             if (step < n_local) { fetch(rnd); place(rnd); }
-            gt_group_sync(1 + grp);
+            if (tid == 64) {
+                tail.refused = mine ? 0u : 1u;
+                if (!mine) atomicMax(p.status, (int)BSP_ERR_INDEX);
+            }
+            asm volatile("bar.sync 4, %0;\n" ::"n"(128 * kGroups) : "memory");      // (all groups)
+            const bool store = tail.refused == 0u;
             while (step < n_local) {
                 int next = rnd + groups, next_step = step;
                 while (next >= n_rounds) { next -= n_rounds; ++next_step; }
@@ -542,7 +547,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     gt_group_sync(1 + grp);
                     if (kEy == 1 && change) place(next);
-                    if (issuer && n0 + c0 < p.O2) {
+                    if (issuer && n0 + c0 < p.O2 && store) {
                         int in0, y0, x0;
                         ct_tile_origin(p, t_first + idx * t_step, in0, y0, x0);
                         asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n"

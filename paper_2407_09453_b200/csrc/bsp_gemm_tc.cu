@@ -66,7 +66,7 @@ constexpr int kGtHaloTaps = 30;
 struct GtTail {
     uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc_full[2], acc_empty[2], w_full[kGtHaloTaps];
     uint32_t tmem;
-    uint32_t fail;
+    uint32_t fail, refused;
     // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
     __align__(16) uint32_t bias[2][128], half[2][128];
     __align__(16) uint8_t shift[2][128];
@@ -156,13 +156,13 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
         }
     }
+    auto header_ok = [&]() { return gt_header_ok(p.packed, p.wtype, p.O, p.I, p.H, p.K, p.bo, p.bi); };
+    // (the CTAs of a pair must come to the same decision, and large products have no use for it)
+    const bool early = !kPair && tid == 0 && header_ok();
     wait_for_previous<false>();
     if (warp == 0) let_next_start();                  // (behind its allocation)
     if (tid == 0) {
-        // the packed buffer must be the one bsp_compact filled for this descriptor, with the masked dense form in it
-        const PackedHeader *h = (const PackedHeader *)p.packed;
-        const bool ok = h->magic == kPackedMagic && h->dtype == p.wtype && h->O == p.O && h->I == p.I && h->H == p.H &&
-                        h->K == p.K && h->bo == p.bo && h->bi == p.bi && (h->forms & kFormDense) != 0;
+        const bool ok = early || header_ok();
         const bool placed = (ring & 1023u) == 0u;
         s_fail = ok && placed ? 0u : 2u;
         if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
@@ -383,6 +383,8 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             uint32_t *bias = tail.bias[grp], *half = tail.half[grp];
             uint8_t *shift = tail.shift[grp];
             const int ct = ((warp - 2) & 3) * 32 + lane;
+            bool mine = true;                                    // (the look that decides, by one thread, on its way while the tile is made)
+            if (!kPair && tid == 64) mine = header_ok();
             const uint32_t *bias_of = from_here((const uint32_t *)p.bias);       // raw bits: float32 or int32
             const int32_t *shift_of = from_here(p.shift);
             uint32_t next_bias = 0u, next_shift = 1u;
@@ -403,7 +405,15 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 if constexpr (kEy == 1) { half[ct] = (1u << next_shift) >> 1; shift[ct] = (uint8_t)next_shift; }
             };
             uint32_t tile_i = 0;
-            bool ok = true;
+            bool ok = true, store = true;
+            if constexpr (!kPair) {
+                if (tid == 64) {
+                    tail.refused = mine ? 0u : 1u;
+                    if (!mine) atomicMax(p.status, (int)BSP_ERR_INDEX);
+                }
+                asm volatile("bar.sync 3, 256;\n" ::: "memory");
+                store = tail.refused == 0u;
+            }
             for (int tile = t_first; tile < t_count; tile += t_step, ++tile_i) {
                 const bool last = tile + t_step >= t_count, shared_tile = last && BN > cpr;
                 if (!shared_tile && (int)(tile_i & 1u) != grp) continue;
@@ -474,7 +484,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                     if (kEy == 1 && next_ch != have) place(next_ch);
                     // one store of the tile's box: 128 bytes of every row; what lies past the last channel, column, row or image
                     // of Y is clipped (rows of the buffer beyond the box are not part of the store)
-                    if (issuer && left > 0) {
+                    if (issuer && left > 0 && store) {
                         asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n"
                                      ::"l"(&p.tmy), "r"(sg), "r"((n0 + c0) * kEy), "r"(x0), "r"(y0), "r"(in0) : "memory");
                         asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");

@@ -74,8 +74,8 @@ inline int gemm_tile_n(int O)
 
 // Programmatic dependent launch: a kernel launched by launch_after() may start while the kernel before it on the stream
 // still runs, once every CTA of that one has called let_next_start() or left.  Until wait_for_previous() returns - the
-// kernel before it has then completed and its writes are visible - it touches nothing in global memory (it sets up
-// barriers, tensor memory and descriptors).  It lets its own successor start only after that, so at most two kernels of a
+// kernel before it has then completed and its writes are visible - it takes nothing from global memory (it sets up
+// barriers, tensor memory and descriptors; the tensor-core kernels look at a header, see gt_header_ok).  It lets its own successor start only after that, so at most two kernels of a
 // stream overlap, and no successor can hold a line in L1 that was read before the kernel in between wrote it.  (Launched
 // one after another without this, the kernels of a stream started in steps of about 2 us.)
 // What an earlier kernel may have written is read by plain loads or __ldcg, through pointers without __restrict__: __ldg and

@@ -4,6 +4,7 @@
 // that includes this file gets its own copies (anonymous namespace).
 #pragma once
 #include <cuda.h>
+#include <stddef.h>
 #include "bsp_internal.cuh"
 
 namespace bsp {
@@ -179,6 +180,20 @@ __device__ __forceinline__ void gt_sync_all()
     } else {
         __syncthreads();
     }
+}
+
+// True if `packed` is a buffer that bsp_compact filled for this descriptor, with the masked dense form in it.
+// The kernels look at the header twice.  First before wait_for_previous(), on the side of the kernel that still runs: if that look
+// succeeds, the buffer was once filled for the descriptor, so that loads by it stay inside whatever it holds now, and they need not
+// wait for the look after the wait (a trip to L2, about 0.3 us of a call of 4 to 7).  That one decides whether anything is stored.
+__device__ __forceinline__ bool gt_header_ok(const uint8_t *packed, int wtype, int O, int I, int H, int K, int bo, int bi)
+{
+    static_assert(offsetof(PackedHeader, H) == 16 && offsetof(PackedHeader, forms) == 32, "the header is read in pieces of 16 bytes");
+    int m, t, o, i, h, k, r, c, f;
+    asm volatile("ld.relaxed.gpu.global.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(m), "=r"(t), "=r"(o), "=r"(i) : "l"(packed) : "memory");
+    asm volatile("ld.relaxed.gpu.global.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(h), "=r"(k), "=r"(r), "=r"(c) : "l"(packed + 16) : "memory");
+    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];\n" : "=r"(f) : "l"(packed + 32) : "memory");
+    return (uint32_t)m == kPackedMagic && t == wtype && o == O && i == I && h == H && k == K && r == bo && c == bi && (f & kFormDense) != 0;
 }
 
 // n / d and n % d for 0 <= n < 2^31 by the multiplier m = floor(2^32 / d) (0xFFFFFFFF for d = 1): the product's high
