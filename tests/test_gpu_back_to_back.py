@@ -176,3 +176,43 @@ def test_sparse_operands_that_the_call_before_wrote():
         sa.check(), sb.check()
         return out
     compare(prune)
+
+
+@pytest.mark.parametrize("H", [1, 3])
+def test_packed_buffer_filled_anew_just_before_the_call(H):
+    """A packed buffer that the call before fills for another descriptor (of the same size): whatever a product or a pair saw of it while
+    that call still ran, it stores nothing and reports the buffer; filled again for its own, it gives what it gave."""
+    C, P = 64, 64
+    lays = [bsp.SparseLayer(C, C, H, H, bo, bi, torch.bfloat16) for bo, bi in ((8, 8), (4, 16))]
+    W, X = randn(1, (C, H, H, C), 0.1).bfloat16(), randn(2, (P, 8, 8, C)).bfloat16()
+    lay2 = bsp.SparseLayer(C, C, 1, 1, 8, 8, torch.bfloat16)
+    W2 = randn(3, (C, 1, 1, C), 0.1).bfloat16()
+    for lay, w in ((lays[0], W), (lays[1], W), (lay2, W2)):
+        lay.mask(w, lay.NBo * lay.NBi // 4)
+        lay.compact(w)
+    a, b = lays
+    shared, pad = a.packed, (H // 2, H // 2)
+    xd = bsp.XDesc(P, 8, 8, 1, 1, pad[0], pad[1])
+
+    def calls(Y, Z):
+        a.conv2d(X, None, Y, (1, 1), pad)
+        bsp.bsp_conv2d_chain(a.wd, a.handle(), lay2.wd, lay2.handle(), xd, X, None, 1, None, Z, bsp.F32, a.ws)
+
+    want = [torch.empty((P, 8, 8, C), device="cuda") for _ in range(2)]
+    calls(*want)
+    a.check()
+    for _ in range(20):
+        got = [torch.full((P, 8, 8, C), -7.0, device="cuda") for _ in range(2)]
+        torch.cuda.synchronize()
+        torch.cuda._sleep(1_000_000)
+        bsp.bsp_compact(b.wd, W, b.gamma, b.row_ptr, b.col_idx, None, shared, b.capacity, b.ws)
+        calls(*got)
+        with pytest.raises(bsp.BspError) as e:
+            a.check()
+        assert e.value.status == bsp.ERR_INDEX
+        assert all(bool((g == -7.0).all()) for g in got)
+        torch.cuda._sleep(1_000_000)
+        bsp.bsp_compact(a.wd, W, a.gamma, a.row_ptr, a.col_idx, None, shared, a.capacity, a.ws)
+        calls(*got)
+        a.check()
+        assert all(torch.equal(g, w) for g, w in zip(got, want))
