@@ -125,15 +125,16 @@ spgemm_kernel(const int32_t *a_row_ptr, const int32_t *a_col_idx, const T *a_pay
 // A dropped block must not turn a non-finite weight into NaN (0 * inf): a piece of C whose sums are not all finite is
 // computed again by the sparse form.
 constexpr int kStProducers = 16;
-constexpr int kStThreads = (kStProducers + 1) * 32;
+constexpr int kStFencers = 2;                     // (pairs)
+__host__ __device__ constexpr int st_threads(bool pair) { return (kStProducers + 1 + (pair ? kStFencers : 0)) * 32; }
 constexpr int kStMaxStages = 8;
 constexpr int kStARows = kGtBM / kSpEdge;         // block rows of A per tile
 
 // Groups of producer warps by tile width: a group's chain of wait, store, arrive and load is longer than the MMAs of
 // a chunk, so groups overlap theirs.  2048 x 2048 x 4096 at 50 %, us: one group 52 / 82 / 130 (256 / 128 / 64 columns), two
 // 50 / 72 / 113, four 105 with 64; 16-byte cp.async straight to shared memory instead of registers: 72 / 93 / 143.  (These with
-// a proxy fence in the producers.)  Pairs of CTAs that fill half of B each: 48.3, against 46.0 for 256 columns alone.  (All in
-// short bursts with the same operands; a call in a stream with operands that change takes 51.)
+// a proxy fence in the producers, all in short bursts with the same operands; a call in a stream with operands that change
+// takes 51 with 256 columns.)
 __host__ __device__ constexpr int st_groups(int BN) { return BN == 64 ? 4 : 2; }
 
 struct StParams {
@@ -144,24 +145,35 @@ struct StParams {
     int NBa, NBb, NBk, n_chunks, stages, split;
 };
 
-template <int BN>
-__global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_constant__ StParams p)
+// kPair (BN = 256): the tiles of 2 x 128 rows of A and the same 256 rows of B are taken by a cluster of two CTAs; each fills its own rows of A
+// and half of those of B, and MMAs with M = 256 over the pair read both halves.  A CTA then writes and its MMAs read 32 KB a chunk
+// instead of 48.  The proxy fence between a chunk's stores and its MMAs, about 700 cycles beside the producers' traffic, is taken by warps of
+// its own, ahead of the MMA warp, which had stood still for it: 2048 x 2048 x 4096 at 50 % in a stream of calls 51.0 us alone, 51.6 as
+// pairs with the fence in the MMA warp, 41.7 with two warps that fence, 43.9 with three, 47.3 with six (a fence holds up the producers'
+// loads and stores), 42.4 with one that fences every second chunk; on single CTAs warps that fence made it 54.
+__host__ __device__ constexpr int st_rows(int BN, bool pair) { return kStARows + BN / kSpEdge / (pair ? 2 : 1); }   // block rows that a CTA fills
+template <int BN, bool kPair>
+__global__ void __launch_bounds__(st_threads(kPair), 1) spgemm_tc_kernel(const __grid_constant__ StParams p)
 {
     constexpr int kGroups = st_groups(BN), kDepth = BN == 128 ? 2 : 1;    // (chunks loaded ahead per group: what 120 registers hold)
-    constexpr int kRows = kStARows + BN / kSpEdge;            // block rows of the tile: 16 of A, then those of B
+    constexpr int kRows = st_rows(BN, kPair);                 // block rows of the tile: 16 of A, then those of B
+    constexpr int kThreads = st_threads(kPair);
     constexpr int kW = kStProducers / kGroups;                // warps of a group: they share a chunk
     constexpr int kUnits = kRows * 2 / kW;                    // half block rows (four blocks of a chunk) per warp
     constexpr uint32_t kStage = kRows * 1024u;                // a block row of a chunk: 8 rows of 128 bytes
     extern __shared__ __align__(16) uint8_t st_smem_raw[];
     uint8_t *smem = st_smem_raw + ((1024u - (sm32(st_smem_raw) & 1023u)) & 1023u);
-    __shared__ __align__(8) uint64_t s_full[kStMaxStages], s_empty[kStMaxStages], s_acc;
+    __shared__ __align__(8) uint64_t s_full[kStMaxStages], s_ready[kStMaxStages], s_empty[kStMaxStages], s_acc;
     __shared__ uint32_t s_tmem;
     __shared__ volatile uint32_t s_fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const int S = p.stages, pitch = p.n_chunks * 8;
     const uint32_t ring = sm32(smem);
     int16_t *s_pos = (int16_t *)(smem + (size_t)S * kStage);  // [kRows][pitch]: position within its row's stored blocks, or -1
-    const int i0 = (int)blockIdx.y * kStARows, j0 = (int)blockIdx.x * (BN / kSpEdge);
+    uint32_t rank = 0;
+    if constexpr (kPair) asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
+    const int i0 = (kPair ? (int)(blockIdx.y * 2 + rank) : (int)blockIdx.y) * kStARows, j0 = (kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x) * (BN / kSpEdge);
+    const int jb0 = j0 + (int)rank * (kRows - kStARows);      // the first row of B that this CTA fills
     // this CTA's chunks: all of them, or its share of a split reduction (the CTAs of a tile are a cluster along z)
     const int share = (p.n_chunks + p.split - 1) / p.split;
     const int c_lo = (int)blockIdx.z * share, c_hi = min(p.n_chunks, c_lo + share);
@@ -170,29 +182,35 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
         s_fail = 0u;
         for (int s = 0; s < S; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_full[s])), "r"(kW) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_ready[s])), "r"(2) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_empty[s])), "r"(1) : "memory");
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc)), "r"(1) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == kStProducers) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(BN) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+        if constexpr (kPair) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(BN) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&s_tmem)), "r"(BN) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+        }
     }
     wait_for_previous<false>();
     if (warp == kStProducers) let_next_start();        // (behind its allocation)
     // a block row's first and last stored block (rows past the last one are empty)
     auto row_of = [&](int b, int &lo, int &hi) {
         const bool is_a = b < kStARows;
-        const int g = is_a ? i0 + b : j0 + b - kStARows;
+        const int g = is_a ? i0 + b : jb0 + b - kStARows;
         const int32_t *rp = is_a ? p.a_row_ptr : p.b_row_ptr;
         const bool in = g < (is_a ? p.NBa : p.NBb);
         lo = in ? rp[g] : 0;
         hi = in ? rp[g + 1] : 0;
     };
-    for (int k = tid; k < kRows * pitch / 8; k += kStThreads) ((uint4 *)s_pos)[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    for (int k = tid; k < kRows * pitch / 8; k += kThreads) ((uint4 *)s_pos)[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
     __syncthreads();
-    for (int b = warp; b < kRows; b += kStProducers + 1) {
+    for (int b = warp; b < kRows; b += kThreads / 32) {
         int lo, hi;
         row_of(b, lo, hi);
         const int32_t *ci = b < kStARows ? p.a_col_idx : p.b_col_idx;
@@ -209,7 +227,7 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
+    gt_sync_all<kPair>();                   // (a pair: both CTAs' barriers are initialised before either signals the other)
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, s_tmem, 0);
     const uint32_t full0 = sm32(&s_full[0]), empty0 = sm32(&s_empty[0]);
@@ -265,23 +283,43 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
                 }
         if (!gt_wait(sm32(&s_acc), 0u)) ok = false;
         if (!__all_sync(0xFFFFFFFFu, ok) && lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
-    } else {
-        // ================= MMA issuer =================
-        constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((128u >> 4) << 24);
+    } else if (kPair && warp > kStProducers) {
+        // ================= fences of a pair =================
+        // Two warps take turns with the chunks: wait until one is full, fence, pass it on to the MMA warp of the pair's leader.  (They meet
+        // every second slot of a ring of an even number of stages, so that no other chunk passes a barrier between two of their looks.)
+        const uint32_t first = (uint32_t)(warp - kStProducers - 1);
+        uint32_t ready0, slot = first, par = 0;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(ready0) : "r"(sm32(&s_ready[0])));
+        bool ok = true;
+        for (int c = c_lo + (int)first; c < c_hi; c += kStFencers) {
+            if (!__all_sync(0xFFFFFFFFu, gt_poll(full0 + slot * 8u, par))) { ok = false; break; }
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(ready0 + slot * 8u) : "memory");
+            slot += kStFencers;
+            if (slot >= (uint32_t)S) { slot -= (uint32_t)S; par ^= 1u; }
+        }
+        if (!ok && lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
+    } else if (rank == 0) {
+        // ================= MMA issuer (of a pair, the leader's issues for both CTAs) =================
+        const uint32_t ready0 = kPair ? sm32(&s_ready[0]) : full0;
+        constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | (((kPair ? 256u : 128u) >> 4) << 24);
         uint32_t slot = 0, par = 0, a16 = ring >> 4;
         bool ok = true, full_now = false;
         for (int c = c_lo; c < c_hi; ++c) {
-            if (!full_now && !gt_poll_stage(full0 + slot * 8u, par)) { ok = false; break; }
+            if (!full_now && !gt_poll_stage(ready0 + slot * 8u, par)) { ok = false; break; }
             const bool wrap = slot + 1u == (uint32_t)S;
             // (the stage's stores come before this thread through its barrier, and before the MMAs by this one fence: a fence in
             // every producer also waited for the loads it had in flight; 2048 x 2048 x 4096 at 50 % 48.9 -> 46.0 us in a burst)
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            full_now = gt_issue_stage<BSP_BF16, false>(tmem, kGtDesc | (uint64_t)(a16 & 0x3FFFu), kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu),
-                                                       idesc, empty0 + slot * 8u, c != c_lo ? 1u : 0u, 4u, full0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par) != 0u;
+            if constexpr (!kPair) {
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            }
+            full_now = gt_issue_stage<BSP_BF16, kPair>(tmem, kGtDesc | (uint64_t)(a16 & 0x3FFFu), kGtDesc | (uint64_t)((a16 + (kGtABytes >> 4)) & 0x3FFFu),
+                                                       idesc, empty0 + slot * 8u, c != c_lo ? 1u : 0u, 4u, ready0 + (wrap ? 0u : slot + 1u) * 8u, wrap ? par ^ 1u : par) != 0u;
             if (wrap) { slot = 0; par ^= 1u; a16 = ring >> 4; } else { ++slot; a16 += kStage >> 4; }
         }
-        if (ok) gt_commit_elected<false>(sm32(&s_acc));
+        if (ok) gt_commit_elected<kPair>(sm32(&s_acc));
         else if (lane == 0) atomicExch((uint32_t *)&s_fail, 1u);
     }
     __syncthreads();
@@ -355,29 +393,33 @@ __global__ void __launch_bounds__(kStThreads, 1) spgemm_tc_kernel(const __grid_c
         gt_sync_all<true>();                                   // (no CTA leaves while another still reads its sums)
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
+    gt_sync_all<kPair>();                   // (a pair: neither CTA leaves while the other may still signal its barriers)
     if (!ok && tid == 0) atomicMax(p.status, (int)BSP_ERR_TIMEOUT);
-    if (warp == kStProducers) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(BN) : "memory");
+    if (warp == kStProducers) {
+        if constexpr (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(BN) : "memory");
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(BN) : "memory");
+    }
 }
 
 // Stages that fit beside the position table of a tile (zero: too many block columns).
-int spgemm_tc_stages(int BN, int n_chunks)
+int spgemm_tc_stages(int BN, int n_chunks, bool pair = false)
 {
-    const long long rows = kStARows + BN / kSpEdge;
+    const long long rows = st_rows(BN, pair);
     const long long room = (long long)kGtMaxSmem - 1024 - rows * n_chunks * 16;
     const long long n = room / (rows * 1024);
-    return n < 0 ? 0 : (n > kStMaxStages ? kStMaxStages : (int)n);
+    const int stages = n < 0 ? 0 : (n > kStMaxStages ? kStMaxStages : (int)n);
+    return pair ? stages / kStFencers * kStFencers : stages;
 }
 
 // Tile width and split of the tensor-core form, or BN = 0 where the sparse form is expected to be faster.  Estimates in
 // microseconds, fitted on a B200.  Tensor-core form: a tile costs a start, a share per chunk for the table and the fill of
 // the operands (0.30 / 0.42 / 0.57 a chunk at 64 / 128 / 256 columns, bound by shared memory: stores of the fill, reads
-// of the MMAs), whatever the masks hold.  Sparse form: 28.7 per million pairs of blocks with a common column plus 3.6 per
+// of the MMAs; 0.49 on pairs of 2 x 128 rows and 256 columns), whatever the masks hold.  Sparse form: 28.7 per million pairs of blocks with a common column plus 3.6 per
 // million look-ups, or the chain of one warp where there are few rows.  Measured in bursts, sparse / tensor core: 2048 x 2048 x 4096
 // at 50 % 304 / 46, at 75 % 90 / 43, 512 x 512 x 4096 at 50 % 27 / 14; with the fence in the
 // producers 25 / 44 at 90 %, and 11 / 14 for the smaller one at 75 %.
 // The densities come from the host counts; a wrong count costs time only.
-struct StPlan { int BN, split; };
+struct StPlan { int BN, split, pair; };
 // slots[k] = CTAs of clusters of 2^k that the GPU holds at once (clusters of eight do not reach every SM: 512 x 512 x 4096 on
 // 16 of them took two waves, 28.5 us, against 15.3 on 32 clusters of four).
 StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, int gy, const int (&slots)[4])
@@ -389,7 +431,7 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
     const double pairs = (double)NBa * NBb;
     const double bulk = pairs * (28.7e-6 * common + 3.6e-6 * lookups), chain = rows * (0.14 * common + 0.3 * (int)(lookups / 32 + 1));
     double best = 0.95 * (2.9 + (bulk > chain ? bulk : chain));
-    StPlan plan = {0, 1};
+    StPlan plan = {0, 1, 0};
     const int n_chunks = (NBk + 7) / 8;
     // (the row tiles of A are the grid's y extent, which ends at 65535; the sparse form has a row of A per CTA along x)
     if ((NBa + kStARows - 1) / kStARows > 65535) return plan;
@@ -405,8 +447,13 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
             if ((split - 1) * share >= n_chunks) break;                // (every CTA of a split has at least one chunk)
             const long long waves = (tiles * split + slots[k] - 1) / slots[k];
             const double t = waves * (start + 0.03 * n_chunks + chunk * share) + (split > 1 ? 2.5 : 0.0);
-            if (t < best) { best = t; plan = {BN, split}; }
+            if (t < best) { best = t; plan = {BN, split, 0}; }
         }
+    }
+    if (spgemm_tc_stages(256, n_chunks, true) >= 4 && slots[1] > 0) {
+        const long long tiles = 2ll * ((NBa + 2 * kStARows - 1) / (2 * kStARows)) * ((NBb * kSpEdge + 255) / 256);
+        const double t = (double)((tiles + slots[1] - 1) / slots[1]) * (9.4 + 0.03 * n_chunks + 0.49 * n_chunks);
+        if (t < best) { best = t; plan = {256, 1, 1}; }
     }
     return plan;
 }
@@ -423,18 +470,19 @@ bsp_status spgemm_tc_device(const int (**slots)[4])
     if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
     if (!done[dev].load(std::memory_order_acquire)) {
         const std::lock_guard<std::mutex> lock(once);
-        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
-        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
-        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
+        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
         for (int k = 0; k < 4; ++k) {
             cudaLaunchAttribute attr[1];
             cudaLaunchConfig_t cfg = {};
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1u << k;
             cfg.attrs = attr; cfg.numAttrs = 1;
-            cfg.gridDim = dim3(1, 1, 8); cfg.blockDim = dim3(kStThreads); cfg.dynamicSmemBytes = kGtMaxSmem;
+            cfg.gridDim = dim3(1, 1, 8); cfg.blockDim = dim3(st_threads(false)); cfg.dynamicSmemBytes = kGtMaxSmem;
             int n = 0;
-            BSP_CUDA_OK(cudaOccupancyMaxActiveClusters(&n, spgemm_tc_kernel<64>, &cfg));
+            BSP_CUDA_OK(cudaOccupancyMaxActiveClusters(&n, spgemm_tc_kernel<64, false>, &cfg));
             known[dev][k] = n << k;
         }
         done[dev].store(true, std::memory_order_release);
@@ -443,14 +491,15 @@ bsp_status spgemm_tc_device(const int (**slots)[4])
     return BSP_OK;
 }
 
-template <int BN>
+template <int BN, bool kPair = false>
 bsp_status launch_spgemm_tc(StParams p, cudaStream_t st)
 {
-    constexpr int kRows = kStARows + BN / kSpEdge;
-    p.stages = spgemm_tc_stages(BN, p.n_chunks);
-    const dim3 grid((unsigned)((p.NBb * kSpEdge + BN - 1) / BN), (unsigned)((p.NBa + kStARows - 1) / kStARows), (unsigned)p.split);
+    constexpr int kRows = st_rows(BN, kPair);
+    p.stages = spgemm_tc_stages(BN, p.n_chunks, kPair);
+    unsigned nx = (unsigned)((p.NBb * kSpEdge + BN - 1) / BN), ny = (unsigned)((p.NBa + kStARows - 1) / kStARows);
+    if (kPair) { nx *= 2; ny = (ny + 1) / 2; }
     const size_t smem = 1024 + (size_t)kRows * p.n_chunks * 16 + (size_t)p.stages * kRows * 1024;
-    BSP_CUDA_OK(launch_after_clusters(spgemm_tc_kernel<BN>, grid, dim3(kStThreads), smem, st, 1, p.split, p));
+    BSP_CUDA_OK(launch_after_clusters(spgemm_tc_kernel<BN, kPair>, dim3(nx, ny, (unsigned)p.split), dim3(st_threads(kPair)), smem, st, kPair ? 2 : 1, p.split, p));
     return BSP_OK;
 }
 
@@ -520,6 +569,7 @@ bsp_status bsp_spgemm(const bsp_wdesc *wa, const bsp_bcsr *a, const bsp_wdesc *w
         const StPlan plan = spgemm_plan(NBa, NBb, NBk, a->nnz, b->nnz, gy, *slots);
         const StParams q = {a->row_ptr, a->col_idx, b->row_ptr, b->col_idx, (const uint8_t *)a->payload, (const uint8_t *)b->payload,
                             C, (int *)ws, NBa, NBb, NBk, (NBk + 7) / 8, 0, plan.split};
+        if (plan.pair) return launch_spgemm_tc<256, true>(q, st);
         if (plan.BN == 64) return launch_spgemm_tc<64>(q, st);
         if (plan.BN == 128) return launch_spgemm_tc<128>(q, st);
         if (plan.BN == 256) return launch_spgemm_tc<256>(q, st);

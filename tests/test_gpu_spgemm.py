@@ -51,6 +51,8 @@ def test_spgemm_many_rows_and_long_lists():
     (264, 456, 1032, 0.3, 0.1),          # the same with ragged tiles and a last chunk of one block column
     (2040, 1032, 264, 0.1, 0.1),         # 128 columns, ragged, odd number of chunks
     (2048, 1800, 776, 0.05, 0.05),       # 256 columns, ragged
+    (1840, 1672, 1040, 0.1, 0.1),        # pairs of CTAs, of the last of which one has no rows of A
+    (1160, 2048, 2056, 0.2, 0.1),        # ... a row of blocks, and a last chunk of one block column
 ])
 def test_spgemm_tensor_core_tiles(Oa, Ob, I, fa, fb):
     run_spgemm(931, Oa, Ob, I, "bf16", fa, fb)
@@ -104,6 +106,40 @@ def test_spgemm_dropped_blocks_hide_non_finite_weights():
     A[3 * 8 + 2, 0, 0, 10 * 8 + 1] = 0.0
     want = ref.spgemm(8, ref.compact(A, ga, 8, 8), ref.compact(B, gb, 8, 8))
     assert rel_err(np.where(hit, 0.0, got), np.where(hit, 0.0, want)) <= 2e-5
+
+
+def test_spgemm_pairs_hide_non_finite_weights():
+    """The same on pairs of CTAs, in the rows of either."""
+    O, I = 2048, 1024
+    g = torch.Generator(device="cuda")
+    g.manual_seed(951)
+    lays, full = [], []
+    for k in range(2):
+        W = torch.randn((O, 1, 1, I), device="cuda", generator=g).to(torch.bfloat16)
+        gamma = (torch.rand((O // 8, I // 8), device="cuda", generator=g) < 0.6).to(torch.uint8)
+        if k == 0:
+            gamma[3, 10] = gamma[200, 10] = 1
+            W[3 * 8 + 2, 0, 0, 10 * 8 + 1] = W[200 * 8 + 5, 0, 0, 10 * 8 + 4] = float("inf")
+        else:
+            gamma[:, 10] = 0
+            gamma[7, 10] = gamma[150, 10] = 1
+            W[:, 0, 0, 80:88] = W[:, 0, 0, 80:88].abs() + 1
+        lay = bsp.SparseLayer(O, I, 1, 1, 8, 8, torch.bfloat16)
+        lay.compact(W, gamma)
+        lay.nnz = int(gamma.sum())
+        lays.append(lay)
+        keep = gamma.bool().repeat_interleave(8, 0).repeat_interleave(8, 1)
+        full.append(torch.where(keep, W.reshape(O, I), torch.zeros((), dtype=W.dtype, device="cuda")).double())
+    C = torch.empty((O, O), dtype=torch.float32, device="cuda")
+    bsp.bsp_spgemm(lays[0].wd, lays[0].handle(), lays[1].wd, lays[1].handle(), C, lays[0].ws)
+    lays[0].check()
+    hit = torch.zeros_like(C, dtype=torch.bool)
+    for r in (3 * 8 + 2, 200 * 8 + 5):
+        for b in (7, 150):
+            hit[r, b * 8:b * 8 + 8] = True
+    assert bool(torch.isposinf(C[hit]).all()) and bool(torch.isfinite(C[~hit]).all())
+    want = full[0].nan_to_num(posinf=0.0) @ full[1].T
+    assert float((C.double() - want)[~hit].abs().max() / want.abs().max()) <= 2e-5
 
 
 def test_spgemm_first_calls_from_several_threads():
