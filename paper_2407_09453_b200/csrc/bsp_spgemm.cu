@@ -9,7 +9,8 @@
 // for each of them the warp adds the 8 x 8 x 8 product, lane (r, c) holding C[r][2c], C[r][2c + 1] in fp32 (fp32 blocks:
 // fused multiply-adds; bfloat16 blocks: one m16n8k16 tensor-core instruction per two common columns).  Work and
 // traffic follow the kept blocks only: nothing is read or multiplied where either mask has a zero.  bfloat16 operands whose
-// masks leave enough common columns take the dense form on tcgen05 below.
+// masks leave enough common columns take the dense form on tcgen05 below, fp32 operands tiles of 64 x 64.
+#include <math.h>
 #include <atomic>
 #include <mutex>
 #include "bsp_tc.cuh"
@@ -112,6 +113,121 @@ spgemm_kernel(const int32_t *a_row_ptr, const int32_t *a_col_idx, const T *a_pay
         float acc0 = 0.f, acc1 = 0.f;
         sp_pair<T>(a_payload, b_col_idx, b_payload, load_free(b_row_ptr + j), load_free(b_row_ptr + j + 1), NBk, lane, [&](int k) { return s_pos[k]; }, acc0, acc1, status);
         *(float2 *)(C + ((size_t)i * kSpEdge + r) * ldc + (size_t)j * kSpEdge + c) = make_float2(acc0, acc1);
+    }
+}
+
+// ---- fp32 operands, tiles of 64 x 64 ------------------------------------------------------------------------------------
+// The kernel above reads six 16-byte pieces through L1 for every 16 fused multiply-adds of a thread, which bounds it.  Here a CTA owns
+// eight block rows of A x eight of B.  It walks the block columns in chunks of four: the kept blocks of both are loaded a chunk ahead into
+// registers and written to shared memory transposed, so that a thread, which owns 4 x 4 sums, reads four rows of A and four of B at one
+// column with one 16-byte load each.  A warp owns one block row of A: it passes by the columns that this row dropped, and a lane
+// those that its row of B dropped; nothing is multiplied where either mask has a zero, and the terms of a sum are added in the same order
+// (ascending columns, fused) as above, so that both give the same bits.
+constexpr int kSfThreads = 256;
+constexpr int kSfRows = 8;                        // block rows of A, and of B, per tile
+constexpr int kSfChunk = 4;                       // block columns per chunk
+constexpr int kSfPitch = 8 * 64 + 16;             // floats of one block column of a chunk: [channel][row of the tile] (+ 16: the stores of two columns take different banks)
+constexpr int kSfMaxCols = 1024;                  // block columns (positions of 16 rows in 32 KB)
+struct SfShared {
+    float tile[2][2][kSfChunk * kSfPitch];        // [buffer][A, B]
+};
+
+__global__ void __launch_bounds__(kSfThreads, 2)
+spgemm_f32_kernel(const int32_t *a_row_ptr, const int32_t *a_col_idx, const float *a_payload,
+                  const int32_t *b_row_ptr, const int32_t *b_col_idx, const float *b_payload,
+                  int NBa, int NBb, int NBk, float *C, int *status)
+{
+    __shared__ __align__(16) SfShared sh;
+    extern __shared__ __align__(16) int16_t sf_pos[];          // [16][pitch]: position within its row's stored blocks, or -1
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int i0 = (int)blockIdx.y * kSfRows, j0 = (int)blockIdx.x * kSfRows;
+    const int n_chunks = (NBk + kSfChunk - 1) / kSfChunk, pitch = n_chunks * kSfChunk;
+    for (int k = tid; k < 2 * kSfRows * pitch / 4; k += kSfThreads) ((uint2 *)sf_pos)[k] = make_uint2(~0u, ~0u);
+    wait_for_previous<false>();                                // (the next kernel starts when this one has ended, as above)
+    a_payload = from_here(a_payload); a_col_idx = from_here(a_col_idx); a_row_ptr = from_here(a_row_ptr);
+    b_payload = from_here(b_payload); b_col_idx = from_here(b_col_idx); b_row_ptr = from_here(b_row_ptr);
+    __syncthreads();
+    auto row_of = [&](int b, int &lo, int &hi) {               // a block row's first and last stored block (rows past the last one are empty)
+        const bool is_a = b < kSfRows;
+        const int g = is_a ? i0 + b : j0 + b - kSfRows;
+        const int32_t *rp = is_a ? a_row_ptr : b_row_ptr;
+        const bool in = g < (is_a ? NBa : NBb);
+        lo = in ? load_free(rp + g) : 0;
+        hi = in ? load_free(rp + g + 1) : 0;
+    };
+    for (int b = warp; b < 2 * kSfRows; b += kSfThreads / 32) {
+        int lo, hi;
+        row_of(b, lo, hi);
+        const int32_t *ci = b < kSfRows ? a_col_idx : b_col_idx;
+        for (int n = lo + lane; n < hi; n += 32) {
+            const int k = load_free(ci + n);
+            if (k >= 0 && k < NBk) sf_pos[b * pitch + k] = (int16_t)(n - lo);
+            else atomicMax(status, (int)BSP_ERR_INDEX);        // a column outside the matrix: skipped
+        }
+    }
+    __syncthreads();
+    // loads: four threads per block of the chunk, two rows of it each
+    const int lb = tid >> 4, lk = (tid >> 2) & 3, lr = (tid & 3) * 2;
+    int first, last;
+    row_of(lb, first, last);
+    const float *src = (lb < kSfRows ? a_payload : b_payload) + (size_t)first * 64 + lr * 8;
+    float4 v[4];
+    auto load = [&](int c) {
+        const int n = c < n_chunks ? sf_pos[lb * pitch + c * kSfChunk + lk] : -1;
+        if (n >= 0) {
+            const float4 *p = (const float4 *)(src + (size_t)n * 64);
+            v[0] = load_free(p); v[1] = load_free(p + 1); v[2] = load_free(p + 2); v[3] = load_free(p + 3);
+        }
+    };
+    const int at = lk * kSfPitch + (lb & 7) * 8 + lr;
+    auto put = [&](int buf) {                                  // (what a dropped block leaves there is not read)
+        float *t = sh.tile[buf][lb >> 3] + at;
+        const float lo8[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
+        const float hi8[8] = {v[2].x, v[2].y, v[2].z, v[2].w, v[3].x, v[3].y, v[3].z, v[3].w};
+#pragma unroll
+        for (int q = 0; q < 8; ++q) *(float2 *)(t + q * 64) = make_float2(lo8[q], hi8[q]);
+    };
+    v[0] = v[1] = v[2] = v[3] = make_float4(0.f, 0.f, 0.f, 0.f);
+    load(0);
+    float acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+    const int ay = warp * 8 + (lane >> 4) * 4, bx = (lane & 15) * 4;
+    const int16_t *pos_a = sf_pos + warp * pitch, *pos_b = sf_pos + (kSfRows + ((lane & 15) >> 1)) * pitch;
+    for (int c = 0; c < n_chunks; ++c) {
+        const int buf = c & 1;
+        put(buf);
+        load(c + 1);
+        const short4 na = *(const short4 *)(pos_a + c * kSfChunk), nb = *(const short4 *)(pos_b + c * kSfChunk);
+        __syncthreads();                                       // (buffers are written two chunks apart: one barrier a chunk)
+        const short ka[4] = {na.x, na.y, na.z, na.w}, kb[4] = {nb.x, nb.y, nb.z, nb.w};
+#pragma unroll
+        for (int k = 0; k < kSfChunk; ++k) {
+            if (ka[k] < 0 || kb[k] < 0) continue;
+            const float *pa = sh.tile[buf][0] + k * kSfPitch + ay, *pb = sh.tile[buf][1] + k * kSfPitch + bx;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float4 a = *(const float4 *)(pa + q * 64), b = *(const float4 *)(pb + q * 64);
+                const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) acc[r][t] = fmaf(av[r], bv[t], acc[r][t]);
+            }
+        }
+    }
+    const size_t ldc = (size_t)NBb * kSpEdge;
+    const int row = i0 * kSpEdge + ay, col = j0 * kSpEdge + bx;
+    if (row < NBa * kSpEdge && col < NBb * kSpEdge) {
+        const bool wide = ((uintptr_t)C & 15u) == 0;           // (rows of C are multiples of 32 bytes)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            float *dst = C + (size_t)(row + r) * ldc + col;
+            if (wide) *(float4 *)dst = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+            else { *(float2 *)dst = make_float2(acc[r][0], acc[r][1]); *(float2 *)(dst + 2) = make_float2(acc[r][2], acc[r][3]); }
+        }
     }
 }
 
@@ -458,6 +574,20 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
     return plan;
 }
 
+// Whether fp32 operands take the kernel on tiles.  Estimates in microseconds, fitted on a B200.  By rows of A: 174 per million pairs of blocks
+// with a common column, 3.6 per million look-ups.  On tiles: every chunk of four columns costs a start and the columns that the rows
+// of A kept, twice as much where two CTAs share an SM.  us, rows / tiles: 1024 x 1024 x 2048 at 25 % 408 / 135, at 50 % 183 / 99, at 75 %
+// 49 / 62; 232 x 2048 x 632 at 25 % 76 / 26; 2048 x 2048 x 1024 at 50 % 387 / 174, at 90 % 25 / 75; 512 x 512 x 1024 at 25 % 55 / 42, at 50 % 28 / 32.
+bool spgemm_f32_tiles(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b)
+{
+    auto density = [](long long nnz, double nb) { return nnz <= 0 ? 0.0 : (nnz >= nb ? 1.0 : nnz / nb); };
+    const double da = density(nnz_a, (double)NBa * NBk), db = density(nnz_b, (double)NBb * NBk), pairs = (double)NBa * NBb;
+    const double by_rows = 2.9 + pairs * NBk * db * (174e-6 * da + 3.6e-6);
+    const double ctas = (double)((NBa + kSfRows - 1) / kSfRows) * ((NBb + kSfRows - 1) / kSfRows), chunks = (NBk + kSfChunk - 1) / kSfChunk;
+    const double on_tiles = 4.0 + chunks * (ctas <= 148 ? 0.35 + 1.12 * da : ceil(ctas / 296.0) * (0.45 + 2.1 * da));
+    return on_tiles * 1.1 < by_rows;
+}
+
 // Per device, once: the kernels' shared-memory limit and the slots of spgemm_plan.  Calls come from any thread: who finds the
 // flag set finds the slots, too.
 bsp_status spgemm_tc_device(const int (**slots)[4])
@@ -560,6 +690,21 @@ bsp_status bsp_spgemm(const bsp_wdesc *wa, const bsp_bcsr *a, const bsp_wdesc *w
     const dim3 grid((unsigned)NBa, (unsigned)gy);
     cudaStream_t st = (cudaStream_t)stream;
     if (wa->wtype == BSP_F32) {
+        const dim3 tiles((unsigned)((NBb + kSfRows - 1) / kSfRows), (unsigned)((NBa + kSfRows - 1) / kSfRows));
+        if (NBk <= kSfMaxCols && tiles.y <= 65535u && spgemm_f32_tiles(NBa, NBb, NBk, a->nnz, b->nnz)) {
+            const size_t pos = (size_t)2 * kSfRows * ((NBk + kSfChunk - 1) / kSfChunk * kSfChunk) * sizeof(int16_t);
+            static bool opted[kGtMaxDevices] = {};
+            int dev = 0;
+            BSP_CUDA_OK(cudaGetDevice(&dev));
+            if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
+            if (!opted[dev]) {
+                BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kSfRows * kSfMaxCols * (int)sizeof(int16_t)));
+                opted[dev] = true;
+            }
+            BSP_CUDA_OK(launch_after(spgemm_f32_kernel, tiles, dim3(kSfThreads), pos, st, a->row_ptr, a->col_idx, (const float *)a->payload, b->row_ptr, b->col_idx,
+                                     (const float *)b->payload, NBa, NBb, NBk, C, (int *)ws));
+            return BSP_OK;
+        }
         BSP_CUDA_OK(launch_after(spgemm_kernel<float>, grid, dim3(kSpThreads), smem, st, a->row_ptr, a->col_idx, (const float *)a->payload, b->row_ptr, b->col_idx,
                                                              (const float *)b->payload, NBb, NBk, C, (int *)ws));
     } else {

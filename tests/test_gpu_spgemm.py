@@ -58,6 +58,15 @@ def test_spgemm_tensor_core_tiles(Oa, Ob, I, fa, fb):
     run_spgemm(931, Oa, Ob, I, "bf16", fa, fb)
 
 
+@pytest.mark.parametrize("Oa,Ob,I,fa,fb", [
+    (512, 1024, 520, 0.1, 0.1),          # a CTA an SM, a last chunk of one block column
+    (1288, 1032, 264, 0.2, 0.0),         # ragged tiles of one block row and of one block column, two CTAs an SM
+    (2048, 1800, 256, 0.8, 0.0),         # one operand sparse
+])
+def test_spgemm_fp32_tiles(Oa, Ob, I, fa, fb):
+    run_spgemm(935, Oa, Ob, I, "f32", fa, fb)
+
+
 def test_spgemm_more_rows_than_a_grid_is_high():
     """1048577 block rows of A, one more than 65535 row tiles hold.  Few of them have blocks; the count in the handle says that all
     do, as for a mask that keeps everything (it chooses the kernel)."""
