@@ -324,9 +324,16 @@ __device__ __forceinline__ void gt_store_round(uint32_t srow, uint32_t sw, bool 
 // int8 output: requantised after the bias and written piece by piece, 32 channels at a time in a loop that stays a loop.
 // (Unrolled, a round is a thousand instructions that eight warps fetch in eight places: 4800 cycles a round in the pair
 // 64->64->256 at 56x56, which took 89 us and 47 us like this.)  `small`: 1 <= shift <= 30 for all channels and every sum at
-// most 2^30 (gt_round_shift_small holds, `half` has its 2^(s - 1)).
-template <bool kRelu>
-__device__ __forceinline__ void gt_epilogue_int8(uint32_t taddr, const uint32_t *bias, const uint32_t *half, const uint8_t *shift, bool small, int n, int relu,
+// most 2^30 (gt_round_shift_small holds, `half` has its 2^(s - 1)).  Shifts are words where shared memory has room for them, else bytes,
+// each of which costs an integer operation more.
+__device__ __forceinline__ uint4 gt_shifts(const uint32_t *shift) { return *(const uint4 *)shift; }
+__device__ __forceinline__ uint4 gt_shifts(const uint8_t *shift)
+{
+    const uint32_t s = *(const uint32_t *)shift;
+    return make_uint4(__byte_perm(s, 0u, 0x4440), __byte_perm(s, 0u, 0x4441), __byte_perm(s, 0u, 0x4442), s >> 24);
+}
+template <bool kRelu, typename S>
+__device__ __forceinline__ void gt_epilogue_int8(uint32_t taddr, const uint32_t *bias, const uint32_t *half, const S *shift, bool small, int n, int relu,
                                                  uint32_t srow, uint32_t sw, bool live)
 {
 #pragma unroll 1
@@ -342,19 +349,17 @@ __device__ __forceinline__ void gt_epilogue_int8(uint32_t taddr, const uint32_t 
 #pragma unroll
                 for (int e = 0; e < 32; e += 4) {
                     const uint4 b = *(const uint4 *)(bias + e), h = *(const uint4 *)(half + e);
-                    const uint32_t s = *(const uint32_t *)(shift + e);
-                    out[e / 4] = gt_pack_s8x4(gt_round_shift_small((int)(v[e] + b.x), h.x, __byte_perm(s, 0u, 0x4440)),
-                                              gt_round_shift_small((int)(v[e + 1] + b.y), h.y, __byte_perm(s, 0u, 0x4441)),
-                                              gt_round_shift_small((int)(v[e + 2] + b.z), h.z, __byte_perm(s, 0u, 0x4442)),
-                                              gt_round_shift_small((int)(v[e + 3] + b.w), h.w, s >> 24));
+                    const uint4 s = gt_shifts(shift + e);
+                    out[e / 4] = gt_pack_s8x4(gt_round_shift_small((int)(v[e] + b.x), h.x, s.x), gt_round_shift_small((int)(v[e + 1] + b.y), h.y, s.y),
+                                              gt_round_shift_small((int)(v[e + 2] + b.z), h.z, s.z), gt_round_shift_small((int)(v[e + 3] + b.w), h.w, s.w));
                 }
             } else {
 #pragma unroll
                 for (int e = 0; e < 32; e += 4) {
                     const uint4 b = *(const uint4 *)(bias + e);
-                    const uint32_t s = *(const uint32_t *)(shift + e);
-                    out[e / 4] = gt_pack_s8x4(gt_round_shift((int)(v[e] + b.x), s & 31u), gt_round_shift((int)(v[e + 1] + b.y), (s >> 8) & 31u),
-                                              gt_round_shift((int)(v[e + 2] + b.z), (s >> 16) & 31u), gt_round_shift((int)(v[e + 3] + b.w), s >> 24));
+                    const uint4 s = gt_shifts(shift + e);
+                    out[e / 4] = gt_pack_s8x4(gt_round_shift((int)(v[e] + b.x), s.x), gt_round_shift((int)(v[e + 1] + b.y), s.y),
+                                              gt_round_shift((int)(v[e + 2] + b.z), s.z), gt_round_shift((int)(v[e + 3] + b.w), s.w));
                 }
             }
             if (kRelu && relu) {
