@@ -65,7 +65,7 @@ struct GtParams {
 constexpr int kGtHaloTaps = 30;
 template <typename S>
 struct GtTail {
-    uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc_full[2], acc_empty[2], w_full[kGtHaloTaps];
+    uint64_t full[kGtMaxStages], empty[kGtMaxStages], acc_full[4], acc_empty[4], w_full[kGtHaloTaps];
     uint32_t tmem;
     uint32_t fail, refused;
     // per epilogue group: bias, 2^(shift - 1) and shift of its round's channels
@@ -96,9 +96,9 @@ constexpr int kTaps = 0, kPairs = 1, kHalo = 2, kEights = 3;
 template <int kWT, int kEy, int kMode>
 __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_constant__ GtParams p)
 {
-    constexpr bool kPair = kMode == kPairs;
+    constexpr bool kPair = kMode == kPairs, kFour = kMode >= kHalo && kEy == 1;
     extern __shared__ __align__(1024) uint8_t smem[];
-    using Shift = std::conditional_t<(kMode >= kHalo && kEy == 1), uint32_t, uint8_t>;      // (words: int8 64->64 at 224 x 224, batch 32, 74.9 -> 72.0 us)
+    using Shift = std::conditional_t<kFour, uint32_t, uint8_t>;      // (words: int8 64->64 at 224 x 224, batch 32, 74.9 -> 72.0 us)
     GtTail<Shift> &tail = *(GtTail<Shift> *)(smem + (kMode >= kHalo ? p.w_bytes : 0) + (size_t)p.stages * p.stage_bytes + 8 * kGtStagingBytes);
     uint64_t *s_full = tail.full, *s_empty = tail.empty, *s_acc_full = tail.acc_full, *s_acc_empty = tail.acc_empty;
     volatile uint32_t &s_fail = tail.fail;
@@ -116,6 +116,9 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     if constexpr (kPair) asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
     // kHalo: a CTA keeps one channel tile and walks position tiles.
     const int ntn = p.n_tiles_n;
+    // Two accumulators of 256 columns; kHalo with int8 output: four of 128 where a tile is no wider, because the requantising epilogue
+    // hands one back late (64->128 at 112x112, batch 32, 30.7 -> 28.2 us; other outputs and kTaps gained nothing).
+    const uint32_t acc_log = kFour && BN <= 128 ? 2u : 1u, acc_mask = (1u << acc_log) - 1u;
     const int t_first = kMode == kTaps ? (int)blockIdx.x : kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x / ntn;
     const int t_step = kMode == kTaps ? (int)gridDim.x : kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x / ntn;
     const int t_count = kMode == kTaps ? p.n_tiles : kPair ? p.n_tile_pairs : p.n_pos;
@@ -139,7 +142,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_full[s])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_empty[s])), "r"(1) : "memory");
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < (kFour ? 4 : 2); ++b) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc_full[b])), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(sm32(&s_acc_empty[b])), "r"(kPair ? 8 : 4) : "memory");
         }
@@ -311,7 +314,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             auto run_tiles = [&](auto wide_c) -> bool {
                 uint32_t slot = 0, par = 0, tile_i = 0;
                 for (int tile = t_first; tile < t_count; tile += t_step, ++tile_i) {
-                    const uint32_t buf = tile_i & 1u, use = tile_i >> 1, d = tmem + buf * 256u;
+                    const uint32_t buf = tile_i & acc_mask, use = tile_i >> acc_log, d = tmem + (buf << (9 - acc_log));
                     bool ok = gt_poll(sm32(&s_acc_empty[buf]), (use & 1u) ^ 1u) && gt_poll(full0 + slot * 8u, par) && s_fail == 0u;
                     if (!__all_sync(0xFFFFFFFFu, ok)) return false;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -364,7 +367,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
         }
     } else {
         // ================= epilogue (warps 2-9) =================
-        // Two groups of four warps: group g drains accumulator buffer g, that is every second tile of the CTA, so the
+        // Two groups of four warps: group g drains every second tile of the CTA, so the
         // epilogues of two consecutive tiles run side by side.  The last tile of a CTA (often its only one) is shared, each
         // group taking every second of its 128-byte rounds: 1x1 256->1024 at 14x14, batch 64, 14.1 -> 12.9 us; sharing every
         // tile instead cost 10 % where a CTA has many small ones (8-bit 3x3 64->64 at 224x224, int32 output).
@@ -421,7 +424,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 const bool last = tile + t_step >= t_count, shared_tile = last && BN > cpr;
                 if (!shared_tile && (int)(tile_i & 1u) != grp) continue;
                 const int c_first = shared_tile ? grp * cpr : 0, c_step = shared_tile ? 2 * cpr : cpr;
-                const uint32_t buf = tile_i & 1u, use = tile_i >> 1;
+                const uint32_t buf = tile_i & acc_mask, use = tile_i >> acc_log;
                 int mt, tn;
                 tile_of(tile, mt, tn);
                 const int n0 = tn * BN;
@@ -437,7 +440,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
                 if (kEy == 1 && issuer) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
                 if (kEy == 1 ? !fresh : replace) gt_group_sync(1 + grp);
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + buf * 256u;
+                const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (buf << (9 - acc_log));
                 // the channels of the round after the last one of this tile: those of the group's next tile
                 int after = n0 + c_first;
                 if (!last && kMode < kHalo && ntn > 1) {

@@ -52,6 +52,23 @@ def test_channel_tiles(dtype, O):
     run_conv_case(821, O, 32, 3, 3, 8, 8, dtype, (8, 40, 40, 32), (1, 1), (1, 1))
 
 
+@pytest.mark.parametrize("O,L", [(64, 440), (128, 440), (192, 250), (256, 440), (128, 147)])
+def test_requantised_output_of_many_tiles(O, L):
+    """Tiles of up to 128 channels use four accumulators in turn, wider ones two: one to eleven tiles a CTA."""
+    W = make_case(841, O, 16, 1, 3, "i8")
+    gamma = synth.random_gamma(842, O // 8, 2, O // 8)
+    X = make_x(843, (1, L, 421, 16), "i8")
+    b = make_bias(844, O, "i8")
+    s = synth.uniform_int(845, (O,), 1, 12).astype(np.int32)
+    lay = gpu_layer(W, gamma, 8, 8, "i8")
+    Y = torch.full((1, L, 421, O), -7, dtype=torch.int8, device="cuda")
+    lay.conv2d_q8(torch.from_numpy(X).cuda(), torch.from_numpy(b).cuda(), torch.from_numpy(s).cuda(), Y, (1, 1), (0, 1))
+    lay.check()
+    rp, ci, pl = ref.compact(W, gamma, 8, 8)
+    acc = ref.conv2d(W.shape, 8, 8, rp, ci, pl, X, b, (1, 1), (0, 1))
+    assert np.array_equal(Y.cpu().numpy().reshape(-1, O), ref.requant_i8(acc, s))
+
+
 @pytest.mark.parametrize("O", [64, 128])
 @pytest.mark.parametrize("case", ["plain", "shift 0", "shift 31", "bias"])
 def test_requantised_output(O, case):
