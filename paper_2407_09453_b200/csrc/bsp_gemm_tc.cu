@@ -11,11 +11,11 @@
 // output channels (BN <= 256).  The reduction runs over taps x 128-byte chunks of input channels: per K-stage one
 // thread issues two loads, the activation box shifted by the tap (out-of-bounds positions arrive as zeros: the
 // padding; strides are the tensor map's element strides) and BN x 128 bytes of that tap's weights; one elected lane
-// of the MMA warp issues four MMAs of 128 x BN x 32 bytes; two accumulator buffers of 256 columns let the epilogue of
+// of the MMA warp issues four MMAs of 128 x BN x 32 bytes; two accumulator buffers of 256 columns (or four of 128) let the epilogue of
 // a tile (tensor memory -> registers -> + bias -> convert -> swizzled shared memory -> global memory, by TMA stores of
 // the tile's box) overlap the MMAs of the next one.  Layers that leave most SMs idle take tiles of 64 or 32 positions,
 // multiplied with M = 64; layers of several waves may take boxes of parts of several images; stride-1 layers with taps
-// and few input channels keep their weights in shared memory and load a tile's activations once (kHalo); large products
+// and few input channels keep their weights in shared memory and load a tile's activations once (kHalo, kEights); large products
 // run on pairs of CTAs (kPairs).  The arithmetic skips nothing: a
 // tensor-core instruction covers 128 x BN x 16 entries of the operands at once, far more than a block, and feeding it
 // compact blocks (cp.async expansion of the block-CSR payload in shared memory, or TMA gather loads of 128-byte
