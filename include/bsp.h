@@ -202,8 +202,8 @@ bsp_status bsp_conv2d_q8(const bsp_wdesc *wd, const bsp_bcsr *w, const bsp_xdesc
  *             accumulation and both biases float32 (device, may be NULL), Y [N][M][N_w][O2] F32 or BF16.  T is never
  *             written to memory: a tile of 128 output positions of layer one is its own input tile of layer two.
  *             With more than 128 channels between the layers and about one tile per SM the two separate calls can be the
- *             faster choice (3x3 256->256, 1x1 256->1024 at 14x14, batch 64: 54 us fused, 36 us in two calls; with 64 or 128
- *             channels 40 against 50 us at 56x56, 36 against 40 at 28x28).
+ *             faster choice (3x3 256->256, 1x1 256->1024 at 14x14, batch 64: 51 us fused, 34 us in two calls; with 64 or 128
+ *             channels 39 against 50 us at 56x56, 37 against 38 at 28x28).
  *             w1 / w2: compact forms of the two layers from bsp_compact (`packed` is read; its header is compared with
  *             the descriptors as in bsp_conv2d).  ws: any workspace of at least 256 bytes (status word only).
  * Errors: NULL, SHAPE (second layer not 1x1 on O1 channels, O1 > 256, misaligned buffers), BLOCK, DTYPE (not BF16;
