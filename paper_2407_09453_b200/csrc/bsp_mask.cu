@@ -2,6 +2,7 @@
 // Eq. (1), Eq. (2) and Section "Predetermined Sparsity ratio and Full Training Ahead" of the paper.
 #include <type_traits>
 #include "bsp_internal.cuh"
+#include "bsp_span.cuh"
 
 namespace bsp {
 namespace {
@@ -445,7 +446,8 @@ __device__ __forceinline__ void select_digit(const unsigned *hist, unsigned *war
 // 2048 (4096) equal bins, so that the bin of the threshold holds a few keys whatever the scores look like; it is the next span, until
 // at most kFew keys are left for a warp to rank.  `T` is the threshold key, `ties` how many keys equal to it are still to be
 // zeroed (lowest index first), `same` how many there are.  0 < need <= n; every thread must call it
-// (its first barrier makes the keys visible to all).
+// (its first barrier makes the keys visible to all).  Every round but the first starts on a span of fewer bits than the one before
+// (bsp_span.cuh), and the rounds are counted, so that the loop ends whatever the keys are.
 // (What bounds it is the trip of its instructions to an SM that has not run them before: with the keys in registers and every loop over
 // them unrolled it took 4500 cycles for 4096 keys, digits of ten bits and 128 keys ranked one after the other 7800.)
 constexpr int kRankMax = 4096;
@@ -512,8 +514,8 @@ __device__ __forceinline__ void select_small(const unsigned long long *keys, int
     auto load = [&](int i) { return keys[i]; };
     if (tid == 0) sh.n = 0u;
     unsigned left = (unsigned)n;
-    while (true) {
-        if (lo == hi) { T = lo; ties = need; same = left; break; }
+    T = hi; ties = need; same = left;                      // (a span of one key)
+    for (int round = 0; round < span_rounds(SmallSelect<kT>::kWidth) && lo != hi; ++round) {
         if (left <= (unsigned)kFew) {
             __syncthreads();
             for_keys<kT>(n, load, [&](int, unsigned long long v) {
@@ -539,7 +541,7 @@ __device__ __forceinline__ void select_small(const unsigned long long *keys, int
 #pragma unroll
         for (int q = 0; q < kMine; q += 4) *(uint4 *)(sh.hist + tid * kMine + q) = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
-        const int bits = 64 - __clzll((long long)(hi - lo)), shift = bits > SmallSelect<kT>::kWidth ? bits - SmallSelect<kT>::kWidth : 0;
+        const int shift = span_shift(lo, hi, SmallSelect<kT>::kWidth);
         for_keys<kT>(n, load, [&](int, unsigned long long v) {
             if (v >= lo && v <= hi) atomicAdd(&sh.hist[(unsigned)((v - lo) >> shift)], 1u);
         });
@@ -576,10 +578,8 @@ __device__ __forceinline__ void select_small(const unsigned long long *keys, int
         __syncthreads();
         need = sh.need;
         left = sh.count;
-        lo += (unsigned long long)sh.bin << shift;
-        if (shift == 0) { T = lo; ties = need; same = left; break; }
-        const unsigned long long end = lo + ((1ull << shift) - 1ull);
-        hi = end < hi ? end : hi;
+        span_to_bin(lo, hi, sh.bin, shift);
+        T = hi; ties = need; same = left;                  // (a bin of one key: the loop ends)
     }
 }
 

@@ -153,6 +153,46 @@ def test_select_of_uneven_scores(rows, cols, what):
         assert np.array_equal(g, ref.mask(want, n_zero)), n_zero
 
 
+def by_key_bits(scores, n_zero, scope):
+    """Gamma by the bits of the scores: what the selects order by, NaNs of either sign among them."""
+    seg = scores.view(np.uint64).reshape(1, -1) if scope == bsp.SCOPE_LAYER else scores.view(np.uint64)
+    g = np.ones(seg.shape, dtype=np.uint8)
+    np.put_along_axis(g, np.argsort(seg, axis=1, kind="stable")[:, :n_zero], 0, axis=1)
+    return g.reshape(scores.shape)
+
+
+@pytest.mark.parametrize("rows,cols,scope", [
+    (16, 16, bsp.SCOPE_LAYER),           # one launch, the last arriver selects
+    (65, 64, bsp.SCOPE_LAYER),           # every CTA selects for itself
+    (150, 165, bsp.SCOPE_LAYER),         # the cooperative select
+    (8, 300, bsp.SCOPE_ROW),             # a row per CTA
+    (129, 150, bsp.SCOPE_ROW),           # rows in a launch of their own
+])
+@pytest.mark.parametrize("norm", [bsp.NORM_L2, bsp.NORM_L1, bsp.NORM_VAR])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_select_of_scores_that_are_not_numbers(rows, cols, scope, norm, dtype):
+    """NaNs of both signs and infinities among the weights, few and more than a warp ranks, with the threshold among ordinary scores and
+    among theirs (the last bins of 64 bits)."""
+    W0 = make_case(167, rows * 8, cols * 8, 1, 1, dtype)
+    rng = np.random.default_rng(168)
+    for n_odd in (1, 8, rows * cols // 3):
+        W, bits = to_dev(W0, dtype), torch.int32 if dtype == "f32" else torch.int16
+        raw = W.reshape(rows, 8, cols, 8)[:, 3, :, 5].contiguous().view(bits)
+        odd = [0x7F800000, 0x7FC00000, -0x800000, -0x400000]          # inf, NaN, -inf and a NaN with its sign set
+        values = torch.tensor([odd[k % 4] >> (0 if dtype == "f32" else 16) for k in range(n_odd)], dtype=bits, device="cuda")
+        raw.view(-1)[torch.from_numpy(rng.choice(rows * cols, n_odd, replace=False)).cuda()] = values.flip(0)
+        W.reshape(rows, 8, cols, 8)[:, 3, :, 5] = raw.view(W.dtype)
+        lay = bsp.SparseLayer(rows * 8, cols * 8, 1, 1, 8, 8, TORCH_DT[dtype])
+        sc = torch.empty((rows, cols), dtype=torch.float64, device="cuda")
+        seg = rows * cols if scope == bsp.SCOPE_LAYER else cols
+        for n_zero in sorted({1, seg // 2, seg - min(n_odd, 40), seg - 2, seg - 1}):
+            for keep in (sc, None):
+                lay.mask(W, n_zero, norm, scope, keep)
+                lay.check()
+                assert np.array_equal(from_dev(lay.gamma).reshape(rows, cols), by_key_bits(from_dev(sc), n_zero, scope)), (n_odd, n_zero)
+        assert int((~torch.isfinite(sc)).sum()) == n_odd
+
+
 @pytest.mark.parametrize("rows", [(5, 128), (5, 129), (5, 4096), (128, 200), (129, 200)])
 def test_row_scope_in_one_and_two_launches(rows):
     """Rows that are ranked, selected by the CTA that scores them, and selected in a launch of their own; a few equal keys."""
