@@ -167,8 +167,9 @@ bsp_status bsp_compact(const bsp_wdesc *wd, const void *W, const uint8_t *gamma,
  * `packed`, which holds Gamma (.) W in the layout of W: zeroed blocks cost no arithmetic result and no entry in
  * row_ptr / col_idx / payload, but the tensor-core instruction multiplies them as zeros (an instruction covers
  * 128 x 256 x 16 entries of the operands, far more than a block).
- * The kernel compares the header of `packed` with wd before it loads anything; a buffer that bsp_compact filled for
- * another descriptor latches BSP_ERR_INDEX and leaves Y untouched.  bsp_conv_kernel_name() names the kernel a call
+ * The kernel compares the header of `packed` with wd before it stores anything; a buffer that bsp_compact filled for
+ * another descriptor latches BSP_ERR_INDEX and leaves Y untouched.  (It may have read from such a buffer by then, never
+ * past the end of the allocation that the buffer lies in.)  bsp_conv_kernel_name() names the kernel a call
  * with these descriptors takes (static storage; NULL for descriptors no kernel takes).
  * Errors: NULL, SHAPE, BLOCK, DTYPE, INDEX (nnz out of range; packed buffer does not match wd: latched), CUDA. */
 size_t bsp_conv_workspace_bytes(const bsp_wdesc *wd, const bsp_xdesc *xd);

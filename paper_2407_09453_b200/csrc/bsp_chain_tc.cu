@@ -56,6 +56,7 @@ struct CtParams {
     // kHalo: bytes of K per position, planes and their pitch, pitch and rows of an image's box; slots of layer two's weights
     int kbytes, planes, plane_bytes, halo_w, halo_rows, w2_slots, w2_stay;
     int small1, small2;       // 8-bit: sums of products of either layer at most 2^29
+    int spans;                // memory is mapped as far as the weights of both layers reach (packed_spans)
 };
 
 // Barriers and constants, after everything else in shared memory (all of it dynamic: the base is 1024-byte aligned).
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
         const bool one = gt_header_ok(p.packed1, p.wtype, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1), two = gt_header_ok(p.packed2, p.wtype, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
         return one && two;
     };
-    const bool early = tid == 0 && header_ok();
+    const bool early = tid == 0 && header_ok() && p.spans != 0;
     wait_for_previous<false>();
     if (warp == 0) let_next_start();                  // (behind its allocation)
     if (tid == 0) {
@@ -609,6 +610,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.O2 = wd2.O; p.bo2 = wd2.bo; p.bi2 = wd2.bi; p.relu = relu ? 1 : 0;
     p.tcc = 128 / esz;
     p.O1p = (wd1.O + p.tcc - 1) / p.tcc * p.tcc;
+    p.spans = packed_spans(wd1, packed1) && packed_spans(wd2, packed2) ? 1 : 0;
     p.N = xd.N; p.sh = xd.stride_h; p.sw = xd.stride_w; p.ph = xd.pad_h; p.pw = xd.pad_w;
     p.M = (xd.L + 2 * xd.pad_h - wd1.H) / xd.stride_h + 1;
     p.Nw = (xd.J + 2 * xd.pad_w - wd1.K) / xd.stride_w + 1;

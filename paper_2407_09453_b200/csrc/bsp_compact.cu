@@ -1,6 +1,7 @@
 // Compaction of Gamma (.) W: compressed block rows (row_ptr, col_idx, canonical payload) and the packed form read by
 // the product kernel.  Section "Block Sparsity in a Matrix" (compress block row) and Section "Subvolumes, Data
 // Compression, and Data Movements" of the paper.
+#include <cuda.h>
 #include "bsp_internal.cuh"
 
 namespace bsp {
@@ -13,6 +14,21 @@ PackedLayout packed_layout(const bsp_wdesc &wd)
     L.off_payload = 256;
     L.total_bytes = align_up(L.off_payload + (L.enabled ? (size_t)wd.O * wd.H * wd.K * wd.I * esz : 0) + 256, 256);
     return L;
+}
+
+bool packed_spans(const bsp_wdesc &wd, const void *packed)
+{
+    typedef CUresult (*RangeFn)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const RangeFn range = []() -> RangeFn {
+        void *ptr = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        return cudaGetDriverEntryPoint("cuMemGetAddressRange", &ptr, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess ? (RangeFn)ptr : nullptr;
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    if (range == nullptr || range(&base, &size, (CUdeviceptr)(uintptr_t)packed) != CUDA_SUCCESS) return false;
+    const size_t at = (size_t)((uintptr_t)packed - (uintptr_t)base);
+    return at <= size && packed_layout(wd).total_bytes <= size - at;
 }
 
 namespace {

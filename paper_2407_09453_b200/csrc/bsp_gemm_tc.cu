@@ -51,6 +51,7 @@ struct GtParams {
     uint8_t *Y;
     int ey;
     int half_rows;                    // kTaps: tiles of at most 64 positions, multiplied with M = 64
+    int spans;                        // memory is mapped as far as the weights reach (packed_spans)
     int narrow;                       // kTaps, bfloat16 output: tiles of 32 channels, whose rows of Y are 64 bytes
     int small_acc;                    // int8: the sums of products are at most 2^29
     // kHalo: bytes of the resident weights, pitch and rows of an image's box, position tiles, planes of 32-byte rows and their pitch
@@ -164,7 +165,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
     }
     auto header_ok = [&]() { return gt_header_ok(p.packed, p.wtype, p.O, p.I, p.H, p.K, p.bo, p.bi); };
     // (the CTAs of a pair must come to the same decision, and large products have no use for it)
-    const bool early = !kPair && tid == 0 && header_ok();
+    const bool early = !kPair && tid == 0 && header_ok() && p.spans != 0;
     wait_for_previous<false>();
     if (warp == 0) let_next_start();                  // (behind its allocation)
     if (tid == 0) {
@@ -709,6 +710,7 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
             return BSP_ERR_CUDA;
     }
 
+    p.spans = !pair && packed_spans(wd, packed) ? 1 : 0;
     if (pair) {
         const int pairs = p.n_tile_pairs < n_sm[dev] / 2 ? p.n_tile_pairs : n_sm[dev] / 2;
         BSP_CUDA_OK(launch_after_clusters(kernel[kPairs], dim3((unsigned)(2 * pairs)), dim3(kGtThreads), smem, st, 2, 1, p));

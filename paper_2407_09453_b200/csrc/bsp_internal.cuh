@@ -10,7 +10,7 @@ namespace bsp {
 constexpr uint32_t kPackedMagic = 0x42535032u;   // "BSP2"
 
 // First 256 bytes of the packed buffer, written on the device by bsp_compact and checked by the product kernel
-// before it loads anything.
+// before it stores anything (and before it loads from a buffer that may end before the descriptor's weights do: gt_header_ok).
 struct PackedHeader {
     uint32_t magic;
     int32_t dtype, O, I, H, K, bo, bi;
@@ -33,6 +33,10 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline int elem_bytes(bsp_dtype t) { return t == BSP_I8 ? 1 : (t == BSP_BF16 ? 2 : 4); }
 
 PackedLayout packed_layout(const bsp_wdesc &wd);
+
+// Whether the allocation that `packed` lies in reaches as far as a packed buffer of this descriptor: loads by it then stay in mapped memory,
+// whatever the buffer holds.  (False where the driver cannot say; 0.1 us.)
+bool packed_spans(const bsp_wdesc &wd, const void *packed);
 
 // Workspace: the first 256 bytes hold the latched status word (word 0) and the counts of CTAs that have arrived and that are done
 // of the single-launch kernels (words kWsSyncWord, kWsSyncWord + 1), zero between launches; scratch starts after them.

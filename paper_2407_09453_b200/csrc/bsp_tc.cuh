@@ -183,9 +183,10 @@ __device__ __forceinline__ void gt_sync_all()
 }
 
 // True if `packed` is a buffer that bsp_compact filled for this descriptor, with the masked dense form in it.
-// The kernels look at the header twice.  First before wait_for_previous(), on the side of the kernel that still runs: if that look
-// succeeds, the buffer was once filled for the descriptor, so that loads by it stay inside whatever it holds now, and they need not
-// wait for the look after the wait (a trip to L2, about 0.3 us of a call of 4 to 7).  That one decides whether anything is stored.
+// Where the host knows that memory is mapped as far as the descriptor's weights reach (packed_spans: `spans` of the parameters), the kernels
+// look at the header twice.  First before wait_for_previous(), on the side of the kernel that still runs: if that look succeeds, loads
+// need not wait for the look after the wait, a trip to L2.  That one decides whether anything is stored: the header seen before may have
+// been an old one of memory that held a larger buffer, or one that the kernel before was about to replace.
 __device__ __forceinline__ bool gt_header_ok(const uint8_t *packed, int wtype, int O, int I, int H, int K, int bo, int bi)
 {
     static_assert(offsetof(PackedHeader, H) == 16 && offsetof(PackedHeader, forms) == 32, "the header is read in pieces of 16 bytes");

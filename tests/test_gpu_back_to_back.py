@@ -1,5 +1,7 @@
 """Consecutive kernels of a stream overlap their starts.  Runs of calls in which each reads what the call before wrote, or
 overwrites what it read, give what the same calls give one at a time, bit for bit."""
+import ctypes as C
+
 import pytest
 import torch
 
@@ -176,6 +178,30 @@ def test_sparse_operands_that_the_call_before_wrote():
         sa.check(), sb.check()
         return out
     compare(prune)
+
+
+def test_loads_ahead_only_where_memory_is_mapped():
+    """A header seen before the wait may be an old one of memory that held a larger buffer.  Loads go by it only where the allocation reaches
+    as far as the descriptor's packed form does; the host decides, to the byte."""
+    spans = bsp.lib()._ZN3bsp12packed_spansERK9bsp_wdescPKv
+    spans.restype = C.c_bool
+    wd = bsp.wdesc(256, 512, 3, 3, 8, 8, bsp.BF16)
+    need = bsp.bsp_packed_bytes(wd, 0)
+    cudart, base, size = C.CDLL("libcudart.so.12"), C.c_void_p(0), need + 4096
+    torch.cuda.synchronize()
+    assert cudart.cudaMalloc(C.byref(base), C.c_size_t(size)) == 0
+    try:
+        for offset, want in ((0, True), (4096, True), (4096 + 256, False), (size - 256, False)):
+            assert spans(C.byref(wd), C.c_void_p(base.value + offset)) is want, offset
+        assert not spans(C.byref(bsp.wdesc(264, 512, 3, 3, 8, 8, bsp.BF16)), base)
+        assert not spans(C.byref(bsp.wdesc(1 << 19, 1 << 19, 1, 1, 8, 8, bsp.BF16)), base)
+    finally:
+        assert cudart.cudaFree(base) == 0
+    assert not spans(C.byref(wd), C.c_void_p(256))
+    for dt in (torch.float32, torch.bfloat16, torch.int8):       # (what programs have: tensors)
+        for O, I, H in ((64, 64, 1), (512, 512, 3), (1000, 2048, 1)):
+            lay = bsp.SparseLayer(O, I, H, H, 8, 8, dt)
+            assert spans(C.byref(lay.wd), C.c_void_p(lay.packed.data_ptr()))
 
 
 @pytest.mark.parametrize("H", [1, 3])
