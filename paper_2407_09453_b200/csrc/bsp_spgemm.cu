@@ -536,10 +536,12 @@ int spgemm_tc_stages(int BN, int n_chunks, bool pair = false)
 // producers 25 / 44 at 90 %, and 11 / 14 for the smaller one at 75 %.
 // The densities come from the host counts; a wrong count costs time only.
 struct StPlan { int BN, split, pair; };
-// slots[k] = CTAs of clusters of 2^k that the GPU holds at once (clusters of eight do not reach every SM: 512 x 512 x 4096 on
-// 16 of them took two waves, 28.5 us, against 15.3 on 32 clusters of four).
-StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, int gy, const int (&slots)[4])
+// What the choice needs to know of a GPU.  slots[k] = CTAs of clusters of 2^k that it holds at once (clusters of eight do not reach every
+// SM: 512 x 512 x 4096 on 16 of them took two waves, 28.5 us, against 15.3 on 32 clusters of four); pair_slots = those of pairs.
+struct StDevice { int slots[4], pair_slots; };
+StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, int gy, const StDevice &gpu)
 {
+    const int(&slots)[4] = gpu.slots;
     auto density = [](long long nnz, double nb) { return nnz <= 0 ? 0.0 : (nnz >= nb ? 1.0 : nnz / nb); };
     const double da = density(nnz_a, (double)NBa * NBk), db = density(nnz_b, (double)NBb * NBk);
     const double common = NBk * da * db, lookups = NBk * db;
@@ -566,9 +568,9 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
             if (t < best) { best = t; plan = {BN, split, 0}; }
         }
     }
-    if (spgemm_tc_stages(256, n_chunks, true) >= 4 && slots[1] > 0) {
+    if (spgemm_tc_stages(256, n_chunks, true) >= 4 && gpu.pair_slots > 0) {
         const long long tiles = 2ll * ((NBa + 2 * kStARows - 1) / (2 * kStARows)) * ((NBb * kSpEdge + 255) / 256);
-        const double t = (double)((tiles + slots[1] - 1) / slots[1]) * (9.4 + 0.03 * n_chunks + 0.49 * n_chunks);
+        const double t = (double)((tiles + gpu.pair_slots - 1) / gpu.pair_slots) * (9.4 + 0.03 * n_chunks + 0.49 * n_chunks);
         if (t < best) { best = t; plan = {256, 1, 1}; }
     }
     return plan;
@@ -578,21 +580,21 @@ StPlan spgemm_plan(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, 
 // with a common column, 3.6 per million look-ups.  On tiles: every chunk of four columns costs a start and the columns that the rows
 // of A kept, twice as much where two CTAs share an SM.  us, rows / tiles: 1024 x 1024 x 2048 at 25 % 408 / 135, at 50 % 183 / 99, at 75 %
 // 49 / 62; 232 x 2048 x 632 at 25 % 76 / 26; 2048 x 2048 x 1024 at 50 % 387 / 174, at 90 % 25 / 75; 512 x 512 x 1024 at 25 % 55 / 42, at 50 % 28 / 32.
-bool spgemm_f32_tiles(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b)
+bool spgemm_f32_tiles(int NBa, int NBb, int NBk, long long nnz_a, long long nnz_b, int n_sm)
 {
     auto density = [](long long nnz, double nb) { return nnz <= 0 ? 0.0 : (nnz >= nb ? 1.0 : nnz / nb); };
     const double da = density(nnz_a, (double)NBa * NBk), db = density(nnz_b, (double)NBb * NBk), pairs = (double)NBa * NBb;
     const double by_rows = 2.9 + pairs * NBk * db * (174e-6 * da + 3.6e-6);
     const double ctas = (double)((NBa + kSfRows - 1) / kSfRows) * ((NBb + kSfRows - 1) / kSfRows), chunks = (NBk + kSfChunk - 1) / kSfChunk;
-    const double on_tiles = 4.0 + chunks * (ctas <= 148 ? 0.35 + 1.12 * da : ceil(ctas / 296.0) * (0.45 + 2.1 * da));
+    const double on_tiles = 4.0 + chunks * (ctas <= n_sm ? 0.35 + 1.12 * da : ceil(ctas / (2.0 * n_sm)) * (0.45 + 2.1 * da));
     return on_tiles * 1.1 < by_rows;
 }
 
-// Per device, once: the kernels' shared-memory limit and the slots of spgemm_plan.  Calls come from any thread: who finds the
-// flag set finds the slots, too.
-bsp_status spgemm_tc_device(const int (**slots)[4])
+// Per device, once: the kernels' shared-memory limit and what spgemm_plan needs.  Calls come from any thread: who finds the
+// flag set finds the rest, too.
+bsp_status spgemm_tc_device(const StDevice **gpu)
 {
-    static int known[kGtMaxDevices][4] = {};
+    static StDevice known[kGtMaxDevices] = {};
     static std::atomic<bool> done[kGtMaxDevices] = {};
     static std::mutex once;
     int dev = 0;
@@ -604,20 +606,37 @@ bsp_status spgemm_tc_device(const int (**slots)[4])
         BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
         BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
         BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_tc_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtMaxSmem));
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 5; ++k) {                                  // (the last: pairs)
+            const bool pair = k == 4;
             cudaLaunchAttribute attr[1];
             cudaLaunchConfig_t cfg = {};
             attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1u << k;
+            attr[0].val.clusterDim.x = pair ? 2 : 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = pair ? 1 : 1u << k;
             cfg.attrs = attr; cfg.numAttrs = 1;
-            cfg.gridDim = dim3(1, 1, 8); cfg.blockDim = dim3(st_threads(false)); cfg.dynamicSmemBytes = kGtMaxSmem;
+            cfg.gridDim = pair ? dim3(2) : dim3(1, 1, 8); cfg.blockDim = dim3(st_threads(pair)); cfg.dynamicSmemBytes = kGtMaxSmem;
             int n = 0;
-            BSP_CUDA_OK(cudaOccupancyMaxActiveClusters(&n, spgemm_tc_kernel<64, false>, &cfg));
-            known[dev][k] = n << k;
+            BSP_CUDA_OK(cudaOccupancyMaxActiveClusters(&n, pair ? spgemm_tc_kernel<256, true> : spgemm_tc_kernel<64, false>, &cfg));
+            (pair ? known[dev].pair_slots : known[dev].slots[k]) = pair ? 2 * n : n << k;
         }
         done[dev].store(true, std::memory_order_release);
     }
-    *slots = &known[dev];
+    *gpu = &known[dev];
+    return BSP_OK;
+}
+
+// The same for the fp32 tiles: the kernel's limit, then the number of SMs.  (Two first calls do the same thing twice.)
+bsp_status spgemm_f32_device(int *n_sm)
+{
+    static std::atomic<int> known[kGtMaxDevices] = {};
+    int dev = 0;
+    BSP_CUDA_OK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
+    *n_sm = known[dev].load(std::memory_order_acquire);
+    if (*n_sm == 0) {
+        BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kSfRows * kSfMaxCols * (int)sizeof(int16_t)));
+        BSP_CUDA_OK(cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev));
+        known[dev].store(*n_sm, std::memory_order_release);
+    }
     return BSP_OK;
 }
 
@@ -690,17 +709,12 @@ bsp_status bsp_spgemm(const bsp_wdesc *wa, const bsp_bcsr *a, const bsp_wdesc *w
     const dim3 grid((unsigned)NBa, (unsigned)gy);
     cudaStream_t st = (cudaStream_t)stream;
     if (wa->wtype == BSP_F32) {
+        int n_sm = 0;
+        rc = spgemm_f32_device(&n_sm);
+        if (rc != BSP_OK) return rc;
         const dim3 tiles((unsigned)((NBb + kSfRows - 1) / kSfRows), (unsigned)((NBa + kSfRows - 1) / kSfRows));
-        if (NBk <= kSfMaxCols && tiles.y <= 65535u && spgemm_f32_tiles(NBa, NBb, NBk, a->nnz, b->nnz)) {
+        if (NBk <= kSfMaxCols && tiles.y <= 65535u && spgemm_f32_tiles(NBa, NBb, NBk, a->nnz, b->nnz, n_sm)) {
             const size_t pos = (size_t)2 * kSfRows * ((NBk + kSfChunk - 1) / kSfChunk * kSfChunk) * sizeof(int16_t);
-            static bool opted[kGtMaxDevices] = {};
-            int dev = 0;
-            BSP_CUDA_OK(cudaGetDevice(&dev));
-            if (dev < 0 || dev >= kGtMaxDevices) return BSP_ERR_CUDA;
-            if (!opted[dev]) {
-                BSP_CUDA_OK(cudaFuncSetAttribute(spgemm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kSfRows * kSfMaxCols * (int)sizeof(int16_t)));
-                opted[dev] = true;
-            }
             BSP_CUDA_OK(launch_after(spgemm_f32_kernel, tiles, dim3(kSfThreads), pos, st, a->row_ptr, a->col_idx, (const float *)a->payload, b->row_ptr, b->col_idx,
                                      (const float *)b->payload, NBa, NBb, NBk, C, (int *)ws));
             return BSP_OK;
@@ -708,10 +722,10 @@ bsp_status bsp_spgemm(const bsp_wdesc *wa, const bsp_bcsr *a, const bsp_wdesc *w
         BSP_CUDA_OK(launch_after(spgemm_kernel<float>, grid, dim3(kSpThreads), smem, st, a->row_ptr, a->col_idx, (const float *)a->payload, b->row_ptr, b->col_idx,
                                                              (const float *)b->payload, NBb, NBk, C, (int *)ws));
     } else {
-        const int(*slots)[4] = nullptr;
-        rc = spgemm_tc_device(&slots);
+        const StDevice *gpu = nullptr;
+        rc = spgemm_tc_device(&gpu);
         if (rc != BSP_OK) return rc;
-        const StPlan plan = spgemm_plan(NBa, NBb, NBk, a->nnz, b->nnz, gy, *slots);
+        const StPlan plan = spgemm_plan(NBa, NBb, NBk, a->nnz, b->nnz, gy, *gpu);
         const StParams q = {a->row_ptr, a->col_idx, b->row_ptr, b->col_idx, (const uint8_t *)a->payload, (const uint8_t *)b->payload,
                             C, (int *)ws, NBa, NBb, NBk, (NBk + 7) / 8, 0, plan.split};
         if (plan.pair) return launch_spgemm_tc<256, true>(q, st);

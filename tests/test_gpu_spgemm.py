@@ -67,6 +67,54 @@ def test_spgemm_fp32_tiles(Oa, Ob, I, fa, fb):
     run_spgemm(935, Oa, Ob, I, "f32", fa, fb)
 
 
+@pytest.mark.parametrize("Oa,Ob,I,keep", [
+    (512, 1024, 520, 0.9),               # a CTA an SM, a last chunk of one block column
+    (1288, 1032, 264, 0.8),              # ragged tiles of one block row and of one block column, two CTAs an SM
+    (1024, 1024, 1000, 0.5),
+    (1608, 2000, 128, 0.6),
+])
+def test_spgemm_fp32_tiles_and_rows_give_the_same_bits(Oa, Ob, I, keep):
+    """The count in the handle chooses between the two forms of fp32 operands: tiles for what the masks keep, rows for a count of one.
+    Both add the terms of a sum in the same order, and neither multiplies a dropped block: with infinities and NaNs in blocks that
+    the other operand dropped in the first, a middle and the last column, and in two that are kept."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(961)
+    NBk = I // 8
+    lays = []
+    for k, O in enumerate((Oa, Ob)):
+        W = torch.randn((O, 1, 1, I), device="cuda", generator=g)
+        gamma = (torch.rand((O // 8, NBk), device="cuda", generator=g) < keep).to(torch.uint8)
+        for col in (0, NBk // 2, NBk - 1):
+            gamma[:, col] = k
+            if k == 0:
+                gamma[[0, O // 16, O // 8 - 1], col] = 1          # three rows of A keep the column
+                W[[3, (O // 16) * 8 + 1], 0, 0, col * 8 + 2] = torch.tensor([float("inf"), float("nan")], device="cuda")
+            else:
+                gamma[1::2, col] = 0                             # every second row of B dropped it
+        lay = bsp.SparseLayer(O, I, 1, 1, 8, 8, torch.float32)
+        lay.compact(W, gamma)
+        lay.nnz = int(gamma.sum())
+        lay.check()
+        lays.append((lay, gamma))
+    (la, ga), (lb, gb) = lays
+    got = []
+    for nnz in ((la.nnz, lb.nnz), (1, 1)):
+        la.nnz, lb.nnz = nnz
+        Cm = torch.full((Oa, Ob), -7.0, device="cuda")
+        bsp.bsp_spgemm(la.wd, la.handle(), lb.wd, lb.handle(), Cm, la.ws)
+        la.check()
+        got.append(Cm)
+    finite = torch.isfinite(got[0])
+    assert torch.equal(finite, torch.isfinite(got[1]))
+    assert torch.equal(got[0][finite].view(torch.int32), got[1][finite].view(torch.int32))
+    odd = torch.zeros((Oa // 8, Ob // 8), dtype=torch.bool, device="cuda")
+    odd[0, 0::2] = odd[Oa // 16, 0::2] = True
+    odd = odd.repeat_interleave(8, 0).repeat_interleave(8, 1)
+    rows = torch.zeros(Oa, dtype=torch.bool, device="cuda")
+    rows[[3, (Oa // 16) * 8 + 1]] = True
+    assert torch.equal(~finite, odd & rows[:, None])
+
+
 def test_spgemm_more_rows_than_a_grid_is_high():
     """1048577 block rows of A, one more than 65535 row tiles hold.  Few of them have blocks; the count in the handle says that all
     do, as for a mask that keeps everything (it chooses the kernel)."""
