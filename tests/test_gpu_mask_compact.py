@@ -107,12 +107,15 @@ def test_select_within_one_cta(rows, cols, scope):
 
 @pytest.mark.parametrize("rows,cols", [
     (17, 241),                           # 4097 blocks, the fewest that every CTA selects on for itself
-    (128, 128),                          # 16384, the most
-    (145, 113),                          # 16385, the fewest of the cooperative select
+    (128, 128),
+    (145, 113),
     (129, 128),
-    (157, 157),                          # 24649, the first of int8 with digits of eight bits
-    (256, 256),
-    (256, 512),                          # 131072, where digits of ten bits begin
+    (128, 192),                          # 24576, the most
+    (157, 157),                          # 24649
+    (349, 73),                           # 25477 and
+    (256, 256),                          # more: the cooperative select
+    (256, 512),
+    (24577, 1),                          # the fewest of it
 ])
 def test_ties_across_the_ctas_of_a_select(rows, cols):
     """Layers whose threshold key is held by many blocks, in the shares of many CTAs: few distinct int8 scores, and one score for
@@ -361,10 +364,10 @@ def test_variance_of_int8_weights_is_refused():
 
 
 def test_bounded_wait_runs_out_and_the_workspace_recovers():
-    """A wait that nothing can satisfy ends by itself: the arrival word of the grid barrier in the workspace header is
-    preset (by the host: the contract says it starts at zero) so that no CTA of the one-launch Gamma builder ever counts
-    as the last arriver.  Every CTA's bounded wait expires, the kernel returns, bsp_check reports BSP_ERR_TIMEOUT once and
-    clears the barrier words, and the next call on the same workspace is bit-exact."""
+    """A count of arrivals that cannot be this launch's: the arrival word in the workspace header is preset (by the host: the
+    contract says it starts at zero) so that no CTA of the one-launch Gamma builder, where nobody waits, ever counts
+    as the last arriver.  The kernel returns, bsp_check reports BSP_ERR_TIMEOUT once and clears the words of the
+    counts, and the next call on the same workspace is bit-exact."""
     W = make_case(141, 128, 128, 3, 3, "bf16")
     lay = bsp.SparseLayer(128, 128, 3, 3, 8, 8, torch.bfloat16)
     Wd = to_dev(W, "bf16")
@@ -379,3 +382,71 @@ def test_bounded_wait_runs_out_and_the_workspace_recovers():
     lay.check()
     want = ref.mask(ref.scores(W, 8, 8), 128)
     assert np.array_equal(from_dev(lay.gamma).reshape(16, 16), want)
+
+
+@pytest.mark.parametrize("preset", [
+    0xFFFFFFFF,                          # the count ends one short of the grid: every CTA's wait runs out
+    0x40000000,                          # far more arrivals than any grid has: seen at once
+])
+def test_wait_of_the_cooperative_select_ends_and_the_workspace_recovers(preset):
+    """A wait that nothing can satisfy ends by itself: the arrival word is preset as above, on a layer whose CTAs wait for one another
+    (more than 24576 blocks)."""
+    W = make_case(171, 150 * 8, 165 * 8, 1, 1, "bf16")
+    want = ref.mask(ref.scores(W, 8, 8), 9000)
+    lay = bsp.SparseLayer(150 * 8, 165 * 8, 1, 1, 8, 8, torch.bfloat16)
+    Wd = to_dev(W, "bf16")
+    lay.ws.view(torch.int32)[2] = preset - (1 << 32 if preset >= 1 << 31 else 0)
+    lay.mask(Wd, 9000)
+    with pytest.raises(bsp.BspError) as e:
+        lay.check()
+    assert e.value.status == bsp.ERR_TIMEOUT
+    assert lay.ws.view(torch.int32)[:4].abs().sum().item() == 0
+    lay.mask(Wd, 9000)
+    lay.check()
+    assert np.array_equal(from_dev(lay.gamma).reshape(150, 165), want)
+
+
+@pytest.mark.parametrize("dtype,norm", [("bf16", bsp.NORM_L2), ("bf16", bsp.NORM_L1), ("bf16", bsp.NORM_VAR), ("f32", bsp.NORM_L2),
+                                        ("f32", bsp.NORM_L1), ("f32", bsp.NORM_VAR), ("i8", bsp.NORM_L2), ("i8", bsp.NORM_L1)])
+@pytest.mark.parametrize("rows,cols,H,bo,bi", [
+    (157, 157, 3, 8, 8),                 # taps: b_o threads score a block
+    (150, 165, 1, 8, 8),                 # one tap: a thread does, but for the variance
+    (25, 1000, 2, 16, 4),
+    (1001, 25, 1, 4, 16),
+])
+def test_cooperative_select_by_type_measure_and_block(rows, cols, H, bo, bi, dtype, norm):
+    """Just above 24576 blocks, with the scores asked for and without (they stay on chip then)."""
+    W = make_case(173, rows * bo, cols * bi, H, H, dtype)
+    want = ref.scores(W, bo, bi, norm)
+    NB = rows * cols
+    for n_zero in (1, NB // 2, NB - 1):
+        g, s, lay, Wd = gpu_mask(W, bo, bi, dtype, n_zero, norm)
+        assert np.array_equal(s.view(np.uint64), want.view(np.uint64))
+        assert np.array_equal(g, ref.mask(want, n_zero)), n_zero
+        lay.gamma.fill_(7)
+        lay.mask(Wd, n_zero, norm)
+        lay.check()
+        assert np.array_equal(from_dev(lay.gamma).reshape(rows, cols), g), n_zero
+
+
+@pytest.mark.parametrize("dtype,norm,few", [("bf16", bsp.NORM_L2, False), ("bf16", bsp.NORM_VAR, False), ("i8", bsp.NORM_L2, False), ("i8", bsp.NORM_L1, True)])
+def test_cooperative_select_of_slices_that_shared_memory_does_not_hold(dtype, norm, few):
+    """1048576 blocks: a CTA's share is more than the 4096 keys that it keeps, and the keys are read again from the scores."""
+    O = I = 8192
+    g = torch.Generator()
+    g.manual_seed(181)
+    if dtype == "i8":
+        lim = 1 if few else 127
+        W = torch.randint(-lim, lim + 1, (O, 1, 1, I), generator=g, dtype=torch.int8).numpy()
+    else:
+        W = torch.randn((O, 1, 1, I), generator=g).bfloat16().float().numpy()
+    want = ref.scores(W, 8, 8, norm)
+    NB = want.size
+    for n_zero in (1, NB // 2, NB - 1):
+        g_, s, lay, Wd = gpu_mask(W, 8, 8, dtype, n_zero, norm)
+        assert np.array_equal(s.view(np.uint64), want.view(np.uint64))
+        assert np.array_equal(g_, ref.mask(want, n_zero)), n_zero
+    lay.gamma.fill_(7)
+    lay.mask(Wd, NB // 2, norm)
+    lay.check()
+    assert np.array_equal(from_dev(lay.gamma).reshape(want.shape), ref.mask(want, NB // 2))
