@@ -7,8 +7,8 @@ import torch
 
 from oracle import ref
 from paper_2407_09453_b200 import synth
-from gpu_util import gpu_layer, make_bias, make_case, make_x
-from test_gpu_product import run_conv_case
+from gpu_util import from_dev, gpu_layer, make_bias, make_case, make_x, to_dev
+from test_gpu_product import check, run_conv_case
 
 pytestmark = pytest.mark.gpu
 
@@ -18,6 +18,27 @@ pytestmark = pytest.mark.gpu
 def test_rows_and_channels(P, dtype, out):
     """Quarters of the tile that are empty or partly filled; a last channel tile of 24 channels."""
     run_conv_case(901, 1048, 512, 1, 1, 8, 8, dtype, (P, 1, 1, 512), (1, 1), (0, 0), out=out)
+
+
+@pytest.mark.parametrize("O", [40, 48, 72, 1000])
+@pytest.mark.parametrize("P", [7, 64])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("bias", [True, False])
+def test_tiles_of_32_channels_end_where_y_does(O, P, dtype, bias):
+    """bfloat16 output by rows of 64 bytes: a last tile of 8, 16 or 8 channels of 32, Y in the middle of memory that stays as it was."""
+    I = 512
+    W = make_case(905, O, I, 1, 1, dtype)
+    gamma = synth.random_gamma(906, O // 8, I // 8, O * I // 128)
+    X = make_x(907, (P, I), dtype)
+    b = make_bias(908, O, dtype) if bias else None
+    lay = gpu_layer(W, gamma, 8, 8, dtype)
+    memory = torch.full((4096 + P * O + 4096,), -7, dtype=torch.bfloat16, device="cuda")
+    Y = memory[4096:4096 + P * O].view(P, O)
+    lay.gemm(to_dev(X, dtype), None if b is None else torch.from_numpy(b).cuda(), Y)
+    lay.check()
+    rp, ci, pl = ref.compact(W, gamma, 8, 8)
+    check(from_dev(Y), ref.gemm(O, I, 8, 8, rp, ci, pl.reshape(-1, 8, 8), X, b), dtype, "bf16")
+    assert bool((memory[:4096] == -7).all()) and bool((memory[4096 + P * O:] == -7).all())
 
 
 @pytest.mark.parametrize("O,I,H,K,L,J,N,stride,pad", [
