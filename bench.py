@@ -1,15 +1,16 @@
 #!/usr/bin/env python
 """Benchmark of the block-sparse hot path: Gamma build -> compaction -> block-sparse product with bias.
 
-    python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--workload NAME] [--no-sweeps]
+    python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--workload NAME] [--record FILE]
 
 One step is one pass of the whole path over one batch of synthetic input: bsp_mask (block L2 scores and
 selection to the target block sparsity), bsp_compact (block-CSR + packed forms) and bsp_gemm / bsp_conv2d
 (tensor-core product with fused bias).  The default workload is the largest single-GPU configuration, the
 matrix product O = I = 4096 over P = 8192 positions (bf16, 8x8 blocks at 50 %).  The metric is effective
-TFLOP/s counting only the FLOPs of non-zero blocks.  Rank 0 prints one JSON line; besides the headline it carries
+TFLOP/s counting only the FLOPs of non-zero blocks.  Rank 0 prints one JSON line.  With --record FILE it also runs
 the block-shape / sparsity sweep of that product, a per-layer pass over the ResNet50-shaped layers (batch 64) and
-one over the VGG16 / InceptionV3-shaped int8 layers (batch 32; Gamma build and compaction timed too).
+one over the VGG16 / InceptionV3-shaped int8 layers (batch 32; Gamma build and compaction timed too), and writes
+them to FILE together with the line (on the line, they had made it longer than a log keeps).
 
 With --gpus N > 1 (launched under torch.distributed.run) every rank runs the same workload on its own batch
 (no exchange on the path: output positions are independent), the time is the maximum over ranks and the value
@@ -482,6 +483,20 @@ def pass_chain(gpu, bsp, torch, pk, reps=10):
     return out
 
 
+LINE_BYTES = 3500          # a log that keeps the last 4000 characters of the output shows the line whole
+
+
+def line_of(out):
+    """The one line of a run, within LINE_BYTES: measurements have six figures (names, counts and bytes stay as they are)."""
+    def short(v):
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        if isinstance(v, list):
+            return [short(x) for x in v]
+        return float("%.6g" % v) if isinstance(v, float) else v
+    return json.dumps(short(out))
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -490,7 +505,8 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--workload", default=DEFAULT_WORKLOAD)
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--no-sweeps", action="store_true", help="headline only: skip the block-shape sweep and the layer-table passes")
+    ap.add_argument("--record", metavar="FILE", help="run the block-shape sweep and the layer-table passes, too, and write them with the line to FILE")
+    ap.add_argument("--no-sweeps", action="store_true", help="with --record: the line only")
     ap.add_argument("--only-chain", action="store_true", help="of the extra passes run the fused pairs of layers only (for profiling)")
     ap.add_argument("--no-graph", action="store_true", help="launch the three calls of a step one by one instead of replaying a CUDA graph of them")
     args = ap.parse_args()
@@ -648,7 +664,7 @@ def main():
         del Xd, Y, Wh, Xh, Yh
         torch.cuda.empty_cache()
         sweeps["chain_resnet50_tails_b64_bf16_8x8_50"] = pass_chain(gpu, bsp, torch, pk, reps=2)
-    elif rank == 0 and world == 1 and not args.no_sweeps:
+    elif rank == 0 and world == 1 and args.record and not args.no_sweeps:
         gemm_layer, gdt, _, _, _, gsig = workload("gemm_4096_p8192")
         if layer.name == gemm_layer.name:
             sweeps["sweep_gemm_4096_p8192"] = sweep_product(gpu, bsp, torch, layer, dtype, Wd, Xd, bd, Y, pk)
@@ -704,11 +720,15 @@ def main():
         "gpu_launches": args.steps * bsp.launches_per_step(lay.wd),
         "clocks": clocks,
     }
-    out.update(sweeps)
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         out["cpu_baseline"] = cpu_baseline_subprocess(layer.name)
     if rank == 0:
-        print(json.dumps(out))
+        if args.record:
+            with open(args.record, "w") as f:
+                json.dump({**out, **sweeps}, f)
+        elif sweeps:
+            out.update(sweeps)
+        print(line_of(out))
     if world > 1:
         dist.destroy_process_group()
 
