@@ -41,6 +41,7 @@ struct CtParams {
     const uint8_t *packed1, *packed2;
     int *status;
     int O1, I1, H, K, bo1, bi1, O2, bo2, bi2, relu, wtype;
+    int early_type;           // as in the product kernel, for both packed buffers
     int O1p;                  // O1 rounded up to a whole chunk of T (64 or 128 channels): columns of accumulator one
     int tcc;                  // channels per chunk of T: 64 (bfloat16) or 128 (int8)
     int n_ks1, cpt1, n_c2, n_t2;      // K-stages of layer one, its channel chunks per tap; chunks of T; channel tiles of layer two (of a CTA)
@@ -56,7 +57,6 @@ struct CtParams {
     // kHalo: bytes of K per position, planes and their pitch, pitch and rows of an image's box; slots of layer two's weights
     int kbytes, planes, plane_bytes, halo_w, halo_rows, w2_slots, w2_stay;
     int small1, small2;       // 8-bit: sums of products of either layer at most 2^29
-    int spans;                // memory is mapped as far as the weights of both layers reach (packed_spans)
 };
 
 // Barriers and constants, after everything else in shared memory (all of it dynamic: the base is 1024-byte aligned).
@@ -146,15 +146,15 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sm32(&tail.tmem)), "r"(kGtTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
-    auto header_ok = [&]() {
-        const bool one = gt_header_ok(p.packed1, p.wtype, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1), two = gt_header_ok(p.packed2, p.wtype, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
+    auto header_ok = [&](int type) {
+        const bool one = gt_header_ok(p.packed1, type, p.O1, p.I1, p.H, p.K, p.bo1, p.bi1), two = gt_header_ok(p.packed2, type, p.O2, p.O1, 1, 1, p.bo2, p.bi2);
         return one && two;
     };
-    const bool early = tid == 0 && header_ok() && p.spans != 0;
+    const bool early = tid == 0 && header_ok(p.early_type);
     wait_for_previous<false>();
     if (warp == 0) let_next_start();                  // (behind its allocation)
     if (tid == 0) {
-        const bool ok = early || header_ok();
+        const bool ok = early || header_ok(p.wtype);
         const bool placed = (base & 1023u) == 0u;
         s_fail = ok && placed ? 0u : 2u;
         if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(64 + 128 * ct_groups(kHalo), 1) chain_tc_kerne
             uint8_t *shift = tail.shift[grp];
             const int ct = ((warp - 2) & 3) * 32 + lane;
             bool mine = true;                                    // (the look that decides, by one thread, on its way while the tile is made)
-            if (tid == 64) mine = header_ok();
+            if (tid == 64) mine = header_ok(p.wtype);
             const uint32_t *bias1 = from_here((const uint32_t *)p.bias1), *bias2 = from_here((const uint32_t *)p.bias2);
             const int32_t *shift1 = from_here(p.shift1), *shift2 = from_here(p.shift2);
             uint32_t next_bias = 0u, next_shift = 1u;
@@ -610,7 +610,7 @@ bsp_status launch_chain_tc(const bsp_wdesc &wd1, const void *packed1, const bsp_
     p.O2 = wd2.O; p.bo2 = wd2.bo; p.bi2 = wd2.bi; p.relu = relu ? 1 : 0;
     p.tcc = 128 / esz;
     p.O1p = (wd1.O + p.tcc - 1) / p.tcc * p.tcc;
-    p.spans = packed_spans(wd1, packed1) && packed_spans(wd2, packed2) ? 1 : 0;
+    p.early_type = packed_spans(wd1, packed1) && packed_spans(wd2, packed2) ? (int)wd1.wtype : -1;
     p.N = xd.N; p.sh = xd.stride_h; p.sw = xd.stride_w; p.ph = xd.pad_h; p.pw = xd.pad_w;
     p.M = (xd.L + 2 * xd.pad_h - wd1.H) / xd.stride_h + 1;
     p.Nw = (xd.J + 2 * xd.pad_w - wd1.K) / xd.stride_w + 1;

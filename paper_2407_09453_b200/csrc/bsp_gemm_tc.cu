@@ -41,7 +41,8 @@ struct GtParams {
     const int32_t *shift;     // int8 output only: right shift per output channel, 0..31
     const uint8_t *packed;
     int *status;
-    int O, I, P, H, K, bo, bi, wtype, ytype;
+    int O, I, P, H, K, bo, bi, wtype;
+    int early_type;           // what the look at the header before the wait takes for wtype: -1 where loads may not go by it (packed_spans)
     int BN, n_tiles_n, n_tiles, n_tile_pairs, n_ks;
     int stages, stage_bytes;
     // position tiles: Wt x Ht output positions of Nt images (at most 128), tiles_x x tiles_y of them per Nt images
@@ -51,7 +52,6 @@ struct GtParams {
     uint8_t *Y;
     int ey;
     int half_rows;                    // kTaps: tiles of at most 64 positions, multiplied with M = 64
-    int spans;                        // memory is mapped as far as the weights reach (packed_spans)
     int narrow;                       // kTaps, bfloat16 output: tiles of 32 channels, whose rows of Y are 64 bytes
     int small_acc;                    // int8: the sums of products are at most 2^29
     // kHalo: bytes of the resident weights, pitch and rows of an image's box, position tiles, planes of 32-byte rows and their pitch
@@ -163,13 +163,13 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
         }
     }
-    auto header_ok = [&]() { return gt_header_ok(p.packed, p.wtype, p.O, p.I, p.H, p.K, p.bo, p.bi); };
+    auto header_ok = [&](int type) { return gt_header_ok(p.packed, type, p.O, p.I, p.H, p.K, p.bo, p.bi); };
     // (the CTAs of a pair must come to the same decision, and large products have no use for it)
-    const bool early = !kPair && tid == 0 && header_ok() && p.spans != 0;
+    const bool early = !kPair && tid == 0 && header_ok(p.early_type);
     wait_for_previous<false>();
     if (warp == 0) let_next_start();                  // (behind its allocation)
     if (tid == 0) {
-        const bool ok = early || header_ok();
+        const bool ok = early || header_ok(p.wtype);
         const bool placed = (ring & 1023u) == 0u;
         s_fail = ok && placed ? 0u : 2u;
         if (!ok) atomicMax(p.status, (int)BSP_ERR_INDEX);
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) gemm_tc_kernel(const __grid_con
             Shift *shift = tail.shift[grp];
             const int ct = ((warp - 2) & 3) * 32 + lane;
             bool mine = true;                                    // (the look that decides, by one thread, on its way while the tile is made)
-            if (!kPair && tid == 64) mine = header_ok();
+            if (!kPair && tid == 64) mine = header_ok(p.wtype);
             const uint32_t *bias_of = from_here((const uint32_t *)p.bias);       // raw bits: float32 or int32
             const int32_t *shift_of = from_here(p.shift);
             uint32_t next_bias = 0u, next_shift = 1u;
@@ -546,7 +546,7 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
     p.bias = bias; p.shift = shift; p.packed = (const uint8_t *)packed;
     p.status = (int *)ws;
     p.O = wd.O; p.I = wd.I; p.H = wd.H; p.K = wd.K; p.bo = wd.bo; p.bi = wd.bi;
-    p.wtype = wd.wtype; p.ytype = ytype; p.ey = ey; p.Y = (uint8_t *)Y;
+    p.wtype = wd.wtype; p.ey = ey; p.Y = (uint8_t *)Y;
     p.small_acc = (long long)wd.I * HK * 128 * 128 <= (1 << 29) ? 1 : 0;
     p.N = xd.N; p.sh = xd.stride_h; p.sw = xd.stride_w; p.ph = xd.pad_h; p.pw = xd.pad_w;
     p.M = (xd.L + 2 * xd.pad_h - wd.H) / xd.stride_h + 1;
@@ -710,7 +710,7 @@ bsp_status launch_gemm_tc(const bsp_wdesc &wd, const bsp_xdesc &xd0, const void 
             return BSP_ERR_CUDA;
     }
 
-    p.spans = !pair && packed_spans(wd, packed) ? 1 : 0;
+    p.early_type = !pair && packed_spans(wd, packed) ? (int)wd.wtype : -1;
     if (pair) {
         const int pairs = p.n_tile_pairs < n_sm[dev] / 2 ? p.n_tile_pairs : n_sm[dev] / 2;
         BSP_CUDA_OK(launch_after_clusters(kernel[kPairs], dim3((unsigned)(2 * pairs)), dim3(kGtThreads), smem, st, 2, 1, p));

@@ -183,7 +183,7 @@ __device__ __forceinline__ void gt_sync_all()
 }
 
 // True if `packed` is a buffer that bsp_compact filled for this descriptor, with the masked dense form in it.
-// Where the host knows that memory is mapped as far as the descriptor's weights reach (packed_spans: `spans` of the parameters), the kernels
+// Where the host knows that memory is mapped as far as the descriptor's weights reach (packed_spans), the kernels
 // look at the header twice.  First before wait_for_previous(), on the side of the kernel that still runs: if that look succeeds, loads
 // need not wait for the look after the wait, a trip to L2 (0.1 to 0.5 us a call: fully connected 2048->1000, 64 positions, 5.79 -> 5.47 us,
 // 3x3 128->128 at 28x28 4.85 -> 4.74, 1x1 256->1024 at 14x14, batch 64, 11.56 -> 11.06).  That one decides whether anything is stored:
